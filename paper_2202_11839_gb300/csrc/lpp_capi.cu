@@ -43,7 +43,7 @@ struct lpp_plan_s {
     int nk_pos = 0, nk_neg = 0, nky = 0, nzi = 0;
     FftGeom geom;
     std::vector<int> thr;
-    std::vector<int4> items;        // work list of the combine (combine_items)
+    std::vector<int> items;        // work list of the combine (combine_items)
     std::vector<long long> n_modes;
     std::vector<double> k_mean;
     // channels
@@ -227,7 +227,7 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
         }
     plan->k_mean.assign(nb, 0.0);
     for (int b = 0; b < nb; ++b) plan->k_mean[b] = plan->n_modes[b] ? ksum[b] / plan->n_modes[b] : 0.0;
-    combine_items(n, plan->nk_pos, plan->nk_neg, plan->nky, plan->nzi, tmax, plan->items);
+    combine_items(n, plan->nk_pos, plan->nk_neg, plan->nzi, tmax, plan->items);
 
     // kernel polynomials and quadratures
     build_kernel_polys(plan->kp);
@@ -251,17 +251,20 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
         plan->polys.insert(plan->polys.end(), poly, poly + npoly);
         g.quad = L / 2 - 1;
         plan->groups.push_back(g);
-        for (int part = 0; part <= has_im; ++part)
-            for (int nn = -L; nn <= L; ++nn) {
-                Channel c;
-                c.kind = kind;
-                c.L = L;
-                c.n = nn;
-                c.part = part;
-                c.moment = slot;
-                c.coeff = (part ? g.row_im : g.row_re) + nn + L;
-                plan->channels.push_back(c);
-            }
+        // n = 0, 1, -1, 2, -2, ... with both parts together: the combine's units (n = +-m) are
+        // consecutive channels
+        for (int m = 0; m <= L; ++m)
+            for (int sgn = 0; sgn < (m ? 2 : 1); ++sgn)
+                for (int part = 0; part <= has_im; ++part) {
+                    Channel c;
+                    c.kind = kind;
+                    c.L = L;
+                    c.n = sgn ? -m : m;
+                    c.part = part;
+                    c.moment = slot;
+                    c.coeff = (part ? g.row_im : g.row_re) + c.n + L;
+                    plan->channels.push_back(c);
+                }
     };
     const int crossSlot[3] = {LPP_MOM_CROSS2, LPP_MOM_CROSS4, LPP_MOM_CROSS6};
     for (int i = 0; i < 3; ++i)
@@ -279,11 +282,11 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
     for (int l = 2; l <= 4; l += 2) {
         const int slot = l == 2 ? LPP_MOM_DD2 : LPP_MOM_DD4;
         if (!(m & (1u << slot))) continue;
-        for (int nn = -l; nn <= l; ++nn) {
+        for (int i = 0; i <= 2 * l; ++i) {
             Channel c;
             c.kind = KIND_DENS;
             c.L = l;
-            c.n = nn;
+            c.n = (i & 1) ? (i + 1) / 2 : -i / 2;   // n = 0, 1, -1, 2, -2, ...
             c.part = PART_RE;
             c.moment = slot;
             c.coeff = -1;
@@ -352,7 +355,7 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
     plan->off_tranges = take(two_slot_grid(plan) ? tile_range_bytes(n, plan->fty, plan->ftz) : sizeof(int));
     plan->off_work = take(sizeof(int));
     plan->off_pstat = take(4 * sizeof(int));
-    plan->off_items = take(std::max<size_t>(1, plan->items.size()) * sizeof(int4));
+    plan->off_items = take(std::max<size_t>(1, plan->items.size()) * sizeof(int));
     plan->off_wout = take((size_t)kWindowChannels * 256 * 2 * sizeof(double));
     plan->off_wthr = take(257 * sizeof(int));
     plan->off_partner = take((size_t)std::max(1, plan->n_partner) * n3 * cs);
@@ -399,7 +402,7 @@ static lpp_status write_tables(lpp_plan_t plan) {
         return cudaMemcpyAsync(plan->ws + off, src, bytes, cudaMemcpyHostToDevice, plan->stream);
     };
     LPP_CUDA(put(plan->off_thr, plan->thr.data(), plan->thr.size() * sizeof(int)));
-    if (!plan->items.empty()) LPP_CUDA(put(plan->off_items, plan->items.data(), plan->items.size() * sizeof(int4)));
+    if (!plan->items.empty()) LPP_CUDA(put(plan->off_items, plan->items.data(), plan->items.size() * sizeof(int)));
     // twiddles e^{-2 pi i j / n}
     std::vector<T> tw(2 * n), iw(n), ph(2 * n);
     for (int j = 0; j < n; ++j) {
@@ -733,7 +736,6 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
     cb.grid_stride = (long long)n3;
     cb.n = n;
     cb.interlace = plan->d.interlace;
-    cb.per_grid = plan->d.interlace ? 1 : 2;
     c2<T>* pG1 = partner;
     c2<T>* pG2 = plan->need_g ? partner + n3 : nullptr;
     c2<T>* pD = plan->need_d ? partner + (plan->need_g ? 2 : 0) * n3 : nullptr;
@@ -751,7 +753,7 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
     cb.nzi = plan->nzi;
     cb.out = out;
     cb.err = err;
-    cb.items = plan->items.empty() ? nullptr : (const int4*)(plan->ws + plan->off_items);
+    cb.items = plan->items.empty() ? nullptr : (const int*)(plan->ws + plan->off_items);
     cb.n_items = (int)plan->items.size();
     const int n_ch = (int)plan->channels.size();
     cb.row_dd0 = n_ch;
@@ -889,7 +891,6 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
         cb.partner_mode = 1;
         cb.has_d = plan->need_d;
         cb.has_g = plan->need_g;
-        cb.n_ch = 0;
         if (tm) tm->begin(KK_PARTNER, st);
         LPP_CUDA(launch_combine<T>(cb, plan->n_sm, st));
         nl += 1;
@@ -931,9 +932,9 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
         const int nch = c1 - c0;
         const int ngr = (nch + per_grid - 1) / per_grid;
         fa.n_slots = 0;
-        cb.n_ch = nch;
         cb.has_d = 0;
         cb.has_g = 0;
+        cb.n_runs = 0;
         for (int gi = 0; gi < ngr; ++gi) {
             const int ca0 = c0 + gi * per_grid;
             FusedSlot fs{};
@@ -965,17 +966,28 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
             fs.grid = gi;
             fa.slots[fa.n_slots++] = fs;
         }
+        int n_units = 0;
         for (int ci = 0; ci < nch; ++ci) {
             const Channel& ch = plan->channels[c0 + ci];
-            CombineChan& cc = cb.ch[ci];
-            cc.slot = ci / per_grid;
-            cc.sub = il ? 0 : ci % 2;
-            cc.kind = ch.kind;
-            cc.L = ch.L;
-            cc.n = ch.n;
-            cc.part = ch.part;
-            cc.out_row = c0 + ci;
-            cc.ynorm = ylm_norm_scaled(ch.L, ch.n);
+            const Channel& prev = plan->channels[c0 + std::max(ci, 1) - 1];
+            const int m = ch.n < 0 ? -ch.n : ch.n;
+            const bool new_run = ci == 0 || ch.moment != prev.moment;
+            if (new_run) cb.run[cb.n_runs++] = CombineRun{n_units, n_units, ch.kind, c0 + ci};
+            if (new_run || m != (prev.n < 0 ? -prev.n : prev.n)) {
+                CombineUnit<T>& u = cb.unit[n_units++];
+                u.L = ch.L;
+                u.m = m;
+                u.ynorm = (T)ylm_norm_scaled(ch.L, m);
+                for (int k = 0; k < 4; ++k) {
+                    u.slot[k] = -1;
+                    u.sub[k] = 0;
+                }
+                cb.run[cb.n_runs - 1].u1 = n_units;
+            }
+            CombineUnit<T>& u = cb.unit[n_units - 1];
+            const int k = 2 * (ch.n < 0 ? 1 : 0) + (ch.part == PART_IM ? 1 : 0);
+            u.slot[k] = ci / per_grid;
+            u.sub[k] = il ? 0 : ci % 2;
             if (ch.kind == KIND_CROSS || ch.kind == KIND_DENS) cb.has_d = 1; else cb.has_g = 1;
         }
         const int bits = dens ? slot_bits(fa.slots[0]) : 1 << LPP_SHAPES;

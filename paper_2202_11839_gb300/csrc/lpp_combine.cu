@@ -8,66 +8,66 @@
 // Interlaced fields become F = (A + e^{-i pi (fx+fy+fz)/n} B) / 2, and every field is
 // divided by the assignment window prod_a sinc^p(pi f_a / n) when compensation is on.
 //
-// One CTA walks rows (fz, fy) of kept modes; its lanes cover fx >= 0 (first half)
-// and fx < 0 (second half), so |k| grows monotonically along each warp and equal
-// shells form contiguous lane runs.  Per-mode products are reduced within a warp by a
-// segmented scan, added to FP32 shared-memory partials per row, and folded after every
-// row into compensated (two-float) or FP64 accumulators that the CTA flushes to the
-// global FP64 shell sums once at the end.
+// A lane owns the up to four mode pairs (+-fx, +-fy, fz) with one |k|: they share the shell, the
+// window, Q_L^m(z) and, up to signs, (x + i y)^m.  A warp takes items of 32 consecutive |fx|
+// of one (|fy|, fz), so |k| grows monotonically along the warp and equal shells form
+// contiguous lane runs.  The lanes' products are reduced by a segmented scan; the lane that ends
+// a segment adds it to the warp's own compensated (two-float) or FP64 accumulators in shared
+// memory (every shell occurs in one segment of an item: no atomics, no block barrier), which
+// the CTA adds to the global FP64 shell sums once at the end.
+//
+// The channels of one moment enter its shell sums only through sum_n Y_Ln(khat) F_n(k), and
+// unpacking, interlacing phase, window and partner are linear in the packed values, so a mode
+// pair first contracts its packed values with the harmonics (a run of channels: two real
+// multiply-adds per value) and unpacks, phases, multiplies by the partner and reduces once per
+// run instead of once per channel.
 #include "lpp_internal.h"
 #include "lpp_kernels.h"
 #include "lpp_reduce.cuh"
 
+#include <algorithm>
+
 namespace lpp {
 
+// k-space field at m and -m for sub-field `sub` of a slot from its packed values zm, zp: iw the
+// inverse window at m and -m, ph the interlacing phase at m, whose mirror is ps conj(ph)
+// (ps = -1 for an odd number of indices at the Nyquist frequency, else 1).
 template <typename T>
-struct ModeCtx {
-    c2<T> ph_m, ph_p;   // interlace phases at m and -m
-    T iw_m, iw_p;       // inverse windows
-    long long im, ip;   // linear indices of m and of its mirror
-    bool self;          // m == -m (index-wise)
-};
-
-// DFTs of the two packed fields at m; the values at the mirror are their conjugates.
-template <typename T>
-__device__ __forceinline__ void unpack(const c2<T>* g, const ModeCtx<T>& c, c2<T>& A, c2<T>& B) {
-    const c2<T> zm = g[c.im];
-    const c2<T> zp = g[c.ip];
-    const T h = (T)0.5;
-    A = mk<T>(h * (zm.x + zp.x), h * (zm.y - zp.y));
-    // B = -i (zm - conj zp) / 2
-    const T dr = zm.x - zp.x, di = zm.y + zp.y;
-    B = mk<T>(h * di, -h * dr);
-}
-
-// k-space field at m and -m for sub-field `sub` of a slot, from its packed values.
-template <typename T>
-__device__ __forceinline__ void field_of(c2<T> zm, c2<T> zp, int sub, int interlace, const ModeCtx<T>& c, c2<T>& Fm,
+__device__ __forceinline__ void field_of(c2<T> zm, c2<T> zp, int sub, int interlace, T iw, c2<T> ph, T ps, c2<T>& Fm,
                                          c2<T>& Fp) {
     const T h = (T)0.5;
     const c2<T> A = mk<T>(h * (zm.x + zp.x), h * (zm.y - zp.y));
     const c2<T> B = mk<T>(h * (zm.y + zp.y), -h * (zm.x - zp.x));   // -i (zm - conj zp) / 2
     if (interlace) {
-        Fm = cscale<T>(cadd<T>(A, cmul<T>(c.ph_m, B)), h * c.iw_m);
-        Fp = cscale<T>(cadd<T>(cconj<T>(A), cmul<T>(c.ph_p, cconj<T>(B))), h * c.iw_p);
+        const c2<T> pb = cmul<T>(ph, B);
+        Fm = cscale<T>(cadd<T>(A, pb), h * iw);
+        Fp = cscale<T>(cconj<T>(cadd<T>(A, cscale<T>(pb, ps))), h * iw);
     } else {
         const c2<T> X = sub ? B : A;
-        Fm = cscale<T>(X, c.iw_m);
-        Fp = cscale<T>(cconj<T>(X), c.iw_p);
+        Fm = cscale<T>(X, iw);
+        Fp = cscale<T>(cconj<T>(X), iw);
     }
 }
 
-// k-space field at m and -m for sub-field `sub` of a slot.
+// (x + i y)^m for m = 0 .. 8, once per mode pair
 template <typename T>
-__device__ __forceinline__ void field_at(const c2<T>* g, int sub, int interlace, const ModeCtx<T>& c, c2<T>& Fm,
-                                         c2<T>& Fp) {
-    field_of<T>(g[c.im], g[c.ip], sub, interlace, c, Fm, Fp);
-}
+struct Azimuth {
+    T re[9], im[9];
+    __device__ __forceinline__ void set(T x, T y) {
+        re[0] = (T)1;
+        im[0] = (T)0;
+#pragma unroll
+        for (int m = 1; m <= 8; ++m) {
+            re[m] = re[m - 1] * x - im[m - 1] * y;
+            im[m] = re[m - 1] * y + im[m - 1] * x;
+        }
+    }
+};
 
-// ylm_poly_scaled(L, +-M, x, y, z) with L and M known at compile time: the same recurrence
-// with constant coefficients and no loops; use_im selects the sine part (n < 0).
+// (L - M)! Q_L^M(z) with L and M known at compile time: the recurrence of ylm_poly_scaled with
+// constant coefficients and no loops.
 template <typename T, int L, int M>
-__device__ __forceinline__ T ylm_fixed(T x, T y, T z, bool use_im) {
+__device__ __forceinline__ T q_fixed(T z) {
     T qmm = (T)1;
 #pragma unroll
     for (int i = 1; i <= M; ++i) qmm *= (T)(2 * i - 1);
@@ -82,30 +82,22 @@ __device__ __forceinline__ T ylm_fixed(T x, T y, T z, bool use_im) {
         }
         q = q1;
     }
-    if constexpr (M == 0) {
-        return q;
-    } else {
-        T re = x, im = y;
-#pragma unroll
-        for (int i = 1; i < M; ++i) {
-            const T t = re * x - im * y;
-            im = re * y + im * x;
-            re = t;
-        }
-        return q * (use_im ? im : re);
-    }
+    return q;
 }
 
-// The channel's harmonic (warp-uniform L, n): the estimators' even degrees up to 8 by a
-// compile-time case, anything else by the general recurrence.
+// The harmonics n = +m (yc) and n = -m (ys) of degree L (warp-uniform L, m), without their
+// normalisation: the estimators' even degrees up to 8 by a compile-time case, anything else by
+// the general recurrence.
 template <typename T>
-__device__ __forceinline__ T ylm_channel(int L, int n, T x, T y, T z) {
-    const int m = n < 0 ? -n : n;
-    const bool use_im = n < 0;
+__device__ __forceinline__ void ylm_pair(int L, int m, const Azimuth<T>& az, T z, T& yc, T& ys) {
     switch (L * 16 + m) {
-#define LPP_YCASE(LL, MM) \
-    case LL * 16 + MM:    \
-        return ylm_fixed<T, LL, MM>(x, y, z, use_im);
+#define LPP_YCASE(LL, MM)                       \
+    case LL * 16 + MM: {                        \
+        const T q = q_fixed<T, LL, MM>(z);      \
+        yc = q * az.re[MM];                     \
+        ys = q * az.im[MM];                     \
+        return;                                 \
+    }
         LPP_YCASE(0, 0)
         LPP_YCASE(2, 0) LPP_YCASE(2, 1) LPP_YCASE(2, 2)
         LPP_YCASE(4, 0) LPP_YCASE(4, 1) LPP_YCASE(4, 2) LPP_YCASE(4, 3) LPP_YCASE(4, 4)
@@ -115,60 +107,143 @@ __device__ __forceinline__ T ylm_channel(int L, int n, T x, T y, T z) {
         LPP_YCASE(8, 6) LPP_YCASE(8, 7) LPP_YCASE(8, 8)
 #undef LPP_YCASE
         default:
-            return ylm_poly_scaled<T>(L, n, x, y, z);
+            yc = ylm_poly_scaled<T>(L, m, az.re[1], az.im[1], z);
+            ys = ylm_poly_scaled<T>(L, -m, az.re[1], az.im[1], z);
     }
 }
 
-// COMPACT: walk the work list (a.items, 256 threads, three CTAs per SM); otherwise one pass
-// per whole row (up to 1024 threads)
-template <typename T, bool COMPACT>
-__global__ void __launch_bounds__(COMPACT ? 256 : 1024, COMPACT ? 3 : 1) k_combine(CombineArgs<T> a) {
+// One (|fx|, |fy|, fz) of a lane: what its four mode pairs share.
+template <typename T>
+struct Lane {
+    Azimuth<T> az;   // of (|kx|, |ky|) / |k|
+    T kz, iw, ps;    // fz / |k|, inverse window, mirror sign of the phase (field_of)
+    int nyq;         // bits 0, 1, 2: x, y, z sit at the Nyquist frequency (the mirror keeps them)
+};
+
+// For the pairs (+|fx|, fy) and (-|fx|, fy), q = 0, 1 (fy < 0: yneg): sum_n Y_n(khat) Z_n(m) and
+// sum_n Y_n(khat) Z_n(-m) of a run's channels for the real (s[q][0], s[q][1]) and imaginary
+// (s[q][2], s[q][3]) kernel parts; with two fields per grid the sums are those of the unpacked
+// fields X at m (s[q][0] and s[q][2] alone).  mirror: with the harmonics of the mirror's own
+// vector, which differs from -k in the sign of the Nyquist components.  on[q]: the lane owns
+// the pair; im[q], ip[q] its indices.  A unit is the up to four channels n = +-m x (real,
+// imaginary part) that share Q_L^m: their packed values are loaded together, ahead of the
+// harmonic.
+template <typename T>
+__device__ __forceinline__ void contract_run(const CombineArgs<T>& a, const CombineRun& run, const Lane<T>& c,
+                                             bool yneg, bool mirror, const bool on[2], const unsigned im[2],
+                                             const unsigned ip[2], c2<T> s[2][4]) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[q][k] = mk<T>((T)0, (T)0);
+    for (int ui = run.u0; ui < run.u1; ++ui) {
+        const CombineUnit<T>& u = a.unit[ui];
+        c2<T> zm[4][2], zp[4][2];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const c2<T>* g = a.grids + (long long)max(u.slot[k], 0) * a.grid_stride;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                zm[k][q] = zp[k][q] = mk<T>((T)0, (T)0);
+                if (on[q] && u.slot[k] >= 0) {
+                    zm[k][q] = g[im[q]];
+                    zp[k][q] = g[ip[q]];
+                }
+            }
+        }
+        T yc, ys;
+        ylm_pair<T>(u.L, u.m, c.az, c.kz, yc, ys);
+        yc *= u.ynorm;
+        ys *= u.ynorm;
+        const bool odd = u.m & 1;
+        if (yneg) ys = -ys;
+        if (mirror) {
+            // Y(-k') = Y(k') (L even) with k' = k but for the signs of its Nyquist components
+            const int nx = c.nyq & 1, ny = (c.nyq >> 1) & 1, nz = c.nyq >> 2;
+            if (odd && (nx ^ nz)) { yc = -yc; ys = -ys; }
+            if (nx ^ ny) ys = -ys;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (u.slot[k] < 0) continue;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                // (-x + i y)^m = (-1)^m conj (x + i y)^m
+                const T yk = (k >> 1) ? ((q == 1 && !odd) ? -ys : ys) : ((q == 1 && odd) ? -yc : yc);
+                c2<T> vm = zm[k][q];
+                const c2<T> vp = zp[k][q];
+                const int o = 2 * (k & 1);
+                if (a.interlace) {
+                    s[q][o + 1] = mk<T>(s[q][o + 1].x + yk * vp.x, s[q][o + 1].y + yk * vp.y);
+                } else {
+                    const T h = (T)0.5;
+                    // A = (zm + conj zp) / 2 or B = -i (zm - conj zp) / 2
+                    vm = u.sub[k] ? mk<T>(h * (vm.y + vp.y), -h * (vm.x - vp.x))
+                                  : mk<T>(h * (vm.x + vp.x), h * (vm.y - vp.y));
+                }
+                s[q][o] = mk<T>(s[q][o].x + yk * vm.x, s[q][o].y + yk * vm.y);
+            }
+        }
+    }
+}
+
+// Walks the work list with 8 warps per CTA.  PARTNER: unpack the partner fields and sum their
+// own products instead of the channels.
+//
+// What bounds it: the latency of the scattered rows (both members of every pair, 16 loads in
+// flight per lane; DRAM at 37% of its peak) with 16 warps per SM; instruction issue at 42%.
+// Eight grids of 256^3 to k = 0.995 k_Ny: 0.40 -> 0.23 ms (one mode pair and one reduction per
+// lane and channel before); 1.5 M galaxies on 512^3: 7.1 -> 3.9 ms for the 17 combines.
+constexpr int kCombineWarps = 8;
+template <typename T>
+constexpr int combine_ctas() { return sizeof(T) == 4 ? 2 : 1; }
+
+template <typename T, bool PARTNER>
+__global__ void __launch_bounds__(32 * kCombineWarps, combine_ctas<T>()) k_combine(CombineArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n;
     const int nb = a.nb;
-    const int nacc = a.partner_mode ? 2 : a.n_ch;
+    const int nacc = PARTNER ? 2 : a.n_runs;
     const int E = nacc * nb * 2;
-    T* acc = reinterpret_cast<T*>(smem_raw);                       // [nacc][nb][2] per-row partials
-    T* own = acc + E;                                              // [E][words] owned accumulators
-    T* iw = own + E * Owned<T>::words;                             // [n]
-    c2<T>* ph = reinterpret_cast<c2<T>*>(iw + n + (n & 1));        // [n]
-    int* thr = reinterpret_cast<int*>(ph + n);                     // [nb+1]
+    constexpr int W = Owned<T>::words, NW = kCombineWarps;
+    T* own = reinterpret_cast<T*>(smem_raw);                       // [NW][words][E] accumulators per warp
+    c2<T>* ph = reinterpret_cast<c2<T>*>(own + NW * E * W);        // [n]  (E is even)
+    T* iw = reinterpret_cast<T*>(ph + n);                          // [n]
+    int* thr = reinterpret_cast<int*>(iw + n);                     // [nb+1]
 
     const int tid = threadIdx.x;
-    const int nthr = blockDim.x;
-    for (int i = tid; i < E; i += nthr) acc[i] = (T)0;
-    for (int i = tid; i < E * Owned<T>::words; i += nthr) own[i] = (T)0;
+    constexpr int nthr = 32 * NW;
+    const int warp = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < NW * E * W; i += nthr) own[i] = (T)0;
     for (int i = tid; i < n; i += nthr) { iw[i] = a.inv_w[i]; ph[i] = a.phase[i]; }
     for (int i = tid; i <= nb; i += nthr) thr[i] = a.thr[i];
     __syncthreads();
+    T* mine = own + warp * E * W;
 
-    auto fold = [&]() {
-        __syncthreads();
-        for (int i = tid; i < E; i += nthr) {
-            const T v = acc[i];
-            if (v != (T)0) {
-                Owned<T>::add(own + i, own + E + i, v);
-                acc[i] = (T)0;
-            }
+    const int na = max(a.nk_pos, a.nk_neg) + 1, nseg = (na + 31) / 32;   // |f| values and their segments
+    const int n_work = a.n_items << a.split;
+    for (int wi = blockIdx.x * NW + warp; wi < n_work; wi += gridDim.x * NW) {
+        // split: the pairs of +fy and of -fy by different warps
+        const int it = wi >> a.split;
+        const int sy0 = a.split ? wi & 1 : 0, sy1 = a.split ? sy0 : 1;
+        int row, seg;
+        if (a.items) {
+            row = a.items[it] >> 6;
+            seg = a.items[it] & 63;
+        } else {
+            row = it / nseg;
+            seg = it - row * nseg;
         }
-        __syncthreads();
-    };
-    // The work of one mode pair (m, -m) with m = (fx, y, z) (grid indices y, z); xvalid: the
-    // lane has a mode; half: 0 for fx >= 0, 1 for fx < 0 (shell labels are monotone within a
-    // half, so (half, bin) keys the lane's segment in the warp-segmented sums).  Every lane of
-    // the warp calls it (the shell sums are warp-collective).
-    auto mode_work = [&](bool xvalid, int fx, int z, int y, int half) {
-        // shell label (contiguous along the warp) and whether this lane owns the pair
-        const int x = fx >= 0 ? fx : n + fx;
-        const int xp = (n - x) & (n - 1);
-        const int fxp = freq_of<T>(xp, n);
+        const int zi = row / na;
+        const int ay = row - zi * na;
+        const int ax = 32 * seg + lane;
+        const int z = zi <= a.nk_pos ? zi : n / 2;
         const int zp = (n - z) & (n - 1);
-        const int yp = (n - y) & (n - 1);
-        const int fz = freq_of<T>(z, n), fy = freq_of<T>(y, n);
-        const int fzp = freq_of<T>(zp, n), fyp = freq_of<T>(yp, n);
-        const int q2 = fx * fx + fy * fy + fz * fz;
+        const int fz = z < n / 2 ? z : z - n;
+        // the shell of the lane's four pairs (contiguous along the warp)
+        const int q2 = ax * ax + ay * ay + fz * fz;
         int bin = -1;
-        if (xvalid && q2 > 0 && q2 >= thr[0] && q2 < thr[nb]) {
+        if (ax < na && q2 > 0 && q2 >= thr[0] && q2 < thr[nb]) {
             int lo = 0, hi = nb;  // thr[lo] <= q2 < thr[hi]
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
@@ -176,247 +251,202 @@ __global__ void __launch_bounds__(COMPACT ? 256 : 1024, COMPACT ? 3 : 1) k_combi
             }
             bin = lo;
         }
-        bool own_pair = bin >= 0;
-        ModeCtx<T> c;
-        c.self = false;
-        if (own_pair && z == zp) {
-            // self-conjugate plane: take each pair once, from its lexicographically smaller member
-            if (y > yp || (y == yp && x > xp)) own_pair = false;
-            c.self = (y == yp && x == xp);
-        }
-        T kx = 0, ky = 0, kz = 0, kxp = 0, kyp = 0, kzp = 0;
-        if (own_pair) {
-            c.im = ((long long)z * n + y) * n + x;
-            c.ip = ((long long)zp * n + yp) * n + xp;
-            const long long n3 = (long long)n * n * n;
-            if (!LPP_IN_BOUNDS(c.im >= 0 && c.im < n3 && c.ip >= 0 && c.ip < n3 && bin < nb, a.err)) own_pair = false;
-        }
-        if (own_pair) {
-            c.iw_m = iw[x] * iw[y] * iw[z];
-            c.iw_p = iw[xp] * iw[yp] * iw[zp];
-            c.ph_m = cmul<T>(cmul<T>(ph[x], ph[y]), ph[z]);
-            c.ph_p = cmul<T>(cmul<T>(ph[xp], ph[yp]), ph[zp]);
-            const T inv = (T)1 / sqrt((T)q2);
-            kx = fx * inv; ky = fy * inv; kz = fz * inv;
-            kxp = fxp * inv; kyp = fyp * inv; kzp = fzp * inv;
-        }
-        if (a.partner_mode) {
-            T dd = 0, gg = 0;
-            if (own_pair) {
-                // partner grids: interlaced -> G1 | G2 | D one field per grid;
-                // otherwise (G1, G2) packed in one grid, then (D, -)
-                const c2<T>* g0 = a.grids;
-                int slot = 0;
-                c2<T> Dm = mk<T>(0, 0), Dp = Dm, G1m = Dm, G1p = Dm, G2m = Dm, G2p = Dm;
-                if (a.interlace) {
-                    if (a.has_g) {
-                        field_at<T>(g0 + (slot++) * a.grid_stride, 0, 1, c, G1m, G1p);
-                        field_at<T>(g0 + (slot++) * a.grid_stride, 0, 1, c, G2m, G2p);
-                    }
-                    if (a.has_d) field_at<T>(g0 + slot * a.grid_stride, 0, 1, c, Dm, Dp);
-                } else {
-                    if (a.has_g) {
-                        field_at<T>(g0, 0, 0, c, G1m, G1p);
-                        field_at<T>(g0, 1, 0, c, G2m, G2p);
-                        ++slot;
-                    }
-                    if (a.has_d) field_at<T>(g0 + slot * a.grid_stride, 0, 0, c, Dm, Dp);
-                }
-                if (a.has_d) {
-                    if (a.pD) {   // null: the caller wants only the shell sums
-                        a.pD[c.im] = Dm;
-                        a.pD[c.ip] = Dp;
-                    }
-                    dd = Dm.x * Dm.x + Dm.y * Dm.y;
-                    if (!c.self) dd += Dp.x * Dp.x + Dp.y * Dp.y;
-                }
-                if (a.has_g) {
-                    a.pG1[c.im] = G1m;
-                    a.pG1[c.ip] = G1p;
-                    a.pG2[c.im] = G2m;
-                    a.pG2[c.ip] = G2p;
-                    // G = G1 + i G2: the transform of the complex shear field
-                    const T gr = G1m.x - G2m.y, gi = G1m.y + G2m.x;
-                    gg = gr * gr + gi * gi;
-                    if (!c.self) {
-                        const T hr = G1p.x - G2p.y, hi2 = G1p.y + G2p.x;
-                        gg += hr * hr + hi2 * hi2;
-                    }
-                }
-            }
-            const int key = bin >= 0 ? bin + half * 65536 : -1;
-            warp_bin_add<T>(dd, (T)0, bin, acc, key);
-            warp_bin_add<T>(gg, (T)0, bin, acc + 2 * nb, key);
-        } else {
-            c2<T> Dm = mk<T>(0, 0), Dp = Dm, G1m = Dm, G1p = Dm, G2m = Dm, G2p = Dm;
-            if (own_pair) {
-                if (a.has_d) { Dm = a.pD[c.im]; Dp = a.pD[c.ip]; }
-                if (a.has_g) { G1m = a.pG1[c.im]; G1p = a.pG1[c.ip]; G2m = a.pG2[c.im]; G2p = a.pG2[c.ip]; }
-            }
-            // the mirror is exactly -k unless an index sits at the Nyquist frequency; then an
-            // even-degree harmonic takes the same value at both members of the pair
-            const bool mirror_neg = (fxp == -fx) && (fyp == -fy) && (fzp == -fz);
-            // a warp none of whose lanes owns a mode pair (rows near the last shell) has
-            // nothing to add: it skips the channels (warp-uniform)
-            const bool warp_live = __any_sync(0xffffffffu, own_pair);
-            const SegMask segm = seg_mask(bin >= 0 ? bin + half * 65536 : -1);
-            const int n_slots = warp_live ? (a.n_ch + a.per_grid - 1) / a.per_grid : 0;
-            // four slots at a time: their packed values at m and -m are loaded together
-            for (int s0 = 0; s0 < n_slots; s0 += 4) {
-                c2<T> zm[4], zp[4];
+        if (!LPP_IN_BOUNDS(bin < nb && (bin < 0 || (ax <= n / 2 && ay <= n / 2)), a.err)) bin = -1;
+        if (!__any_sync(0xffffffffu, bin >= 0)) continue;
+        const SegMask segm = seg_mask(bin);
+        Lane<T> c;
+        const T inv = bin >= 0 ? (T)1 / sqrt((T)q2) : (T)0;
+        if constexpr (!PARTNER) c.az.set((T)ax * inv, (T)ay * inv);
+        c.kz = (T)fz * inv;
+        c.nyq = (ax == n / 2 ? 1 : 0) | (ay == n / 2 ? 2 : 0) | (fz == -n / 2 ? 4 : 0);
+        c.ps = (__popc(c.nyq) & 1) ? (T)-1 : (T)1;
+        const int x0 = bin >= 0 ? ax : 0;   // index of +ax (and of -ax at the Nyquist frequency)
+        const int x1 = (n - x0) & (n - 1);
+        c.iw = iw[x0] * iw[ay] * iw[z];
+        const c2<T> phx = ph[x0];
+        const bool anyq = __any_sync(0xffffffffu, bin >= 0 && c.nyq != 0);
+        T dd = 0, gg = 0;
+        // the pairs of +fy and of -fy: whether the lane owns those of +-fx, and their indices
+        auto side = [&](int sy, bool on[2], unsigned im[2], unsigned ip[2], c2<T> phs[2]) {
+            const int y = sy ? (n - ay) & (n - 1) : ay;
+            const int yp = (n - y) & (n - 1);
+            const bool ey = sy ? (ay >= 1 && ay <= a.nk_neg) : ay <= a.nk_pos;
+            // self-conjugate planes: each pair once, from its lexicographically smaller member
+            const bool half = z == zp;
+            const bool row_on = bin >= 0 && ey && !(half && y > yp);
+            on[0] = row_on && ax <= a.nk_pos;
+            on[1] = row_on && ax >= 1 && ax <= a.nk_neg && !(half && y == yp && x1 > x0);
+            const unsigned rm = ((unsigned)z * n + y) * n, rp = ((unsigned)zp * n + yp) * n;
+            im[0] = rm + x0;
+            ip[0] = rp + x1;
+            im[1] = rm + x1;
+            ip[1] = rp + x0;
+            const c2<T> pyz = cmul<T>(ph[y], ph[z]);
+            phs[0] = cmul<T>(phx, pyz);
+            phs[1] = cmul<T>(ax == n / 2 ? phx : cconj<T>(phx), pyz);
+        };
+        if constexpr (PARTNER) {
+            for (int sy = sy0; sy <= sy1; ++sy) {
+                bool on[2];
+                unsigned im[2], ip[2];
+                c2<T> phs[2];
+                side(sy, on, im, ip, phs);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    zm[k] = zp[k] = mk<T>(0, 0);
-                    if (own_pair && s0 + k < n_slots) {
-                        const c2<T>* g = a.grids + (long long)(s0 + k) * a.grid_stride;
-                        zm[k] = g[c.im];
-                        zp[k] = g[c.ip];
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (s0 + k >= n_slots) break;
-                    for (int sub = 0; sub < a.per_grid; ++sub) {
-                        const int ci = (s0 + k) * a.per_grid + sub;
-                        if (ci >= a.n_ch) break;
-                        const CombineChan& ch = a.ch[ci];
-                        T tre = 0, tim = 0;
-                        if (own_pair) {
-                            c2<T> Fm, Fp;
-                            field_of<T>(zm[k], zp[k], ch.sub, a.interlace, c, Fm, Fp);
-                            if (ch.part == PART_IM) {
-                                Fm = mk<T>(-Fm.y, Fm.x);
-                                Fp = mk<T>(-Fp.y, Fp.x);
-                            }
-                            // partner: delta(-k) = conj D; gamma*(-k) = conj G1 - i conj G2;
-                            // gamma(-k) = conj G1 + i conj G2
-                            c2<T> Pm, Pp;
-                            if (ch.kind == KIND_CROSS || ch.kind == KIND_DENS) {
-                                Pm = cconj<T>(Dm);
-                                Pp = cconj<T>(Dp);
-                            } else {
-                                const T s = ch.kind == KIND_PLUS ? (T)-1 : (T)1;
-                                // conj(G1) + s i conj(G2)
-                                Pm = mk<T>(G1m.x + s * G2m.y, -G1m.y + s * G2m.x);
-                                Pp = mk<T>(G1p.x + s * G2p.y, -G1p.y + s * G2p.x);
-                            }
-                            const T yn = (T)ch.ynorm;
-                            const T ym = yn * ylm_channel<T>(ch.L, ch.n, kx, ky, kz);
-                            c2<T> t = cscale<T>(cmul<T>(Fm, Pm), ym);
-                            if (!c.self) {
-                                const T yp2 = (mirror_neg && (ch.L & 1) == 0)
-                                                  ? ym
-                                                  : yn * ylm_channel<T>(ch.L, ch.n, kxp, kyp, kzp);
-                                t = cadd<T>(t, cscale<T>(cmul<T>(Fp, Pp), yp2));
-                            }
-                            tre = t.x;
-                            tim = t.y;
+                for (int q = 0; q < 2; ++q) {
+                    if (!on[q]) continue;
+                    const bool self = im[q] == ip[q];
+                    auto field = [&](int slot, int sub, c2<T>& Fm, c2<T>& Fp) {
+                        const c2<T>* g = a.grids + (long long)slot * a.grid_stride;
+                        field_of<T>(g[im[q]], g[ip[q]], sub, a.interlace, c.iw, phs[q], c.ps, Fm, Fp);
+                    };
+                    // partner grids: interlaced -> G1 | G2 | D one field per grid;
+                    // otherwise (G1, G2) packed in one grid, then (D, -)
+                    int slot = 0;
+                    if (a.has_g) {
+                        c2<T> G1m, G1p, G2m, G2p;
+                        field(0, 0, G1m, G1p);
+                        field(a.interlace ? 1 : 0, a.interlace ? 0 : 1, G2m, G2p);
+                        slot = a.interlace ? 2 : 1;
+                        a.pG1[im[q]] = G1m;
+                        a.pG1[ip[q]] = G1p;
+                        a.pG2[im[q]] = G2m;
+                        a.pG2[ip[q]] = G2p;
+                        // G = G1 + i G2: the transform of the complex shear field
+                        const T gr = G1m.x - G2m.y, gi = G1m.y + G2m.x;
+                        gg += gr * gr + gi * gi;
+                        if (!self) {
+                            const T hr = G1p.x - G2p.y, hi2 = G1p.y + G2p.x;
+                            gg += hr * hr + hi2 * hi2;
                         }
-                        warp_bin_add_seg<T>(tre, tim, bin, segm, acc + ci * 2 * nb);
+                    }
+                    if (a.has_d) {
+                        c2<T> Dm, Dp;
+                        field(slot, 0, Dm, Dp);
+                        if (a.pD) {   // null: the caller wants only the shell sums
+                            a.pD[im[q]] = Dm;
+                            a.pD[ip[q]] = Dp;
+                        }
+                        dd += Dm.x * Dm.x + Dm.y * Dm.y;
+                        if (!self) dd += Dp.x * Dp.x + Dp.y * Dp.y;
                     }
                 }
             }
-        }
-    };
-
-    if constexpr (!COMPACT) {
-        // one pass per row (fz, fy) of the kept cube; lanes cover fx >= 0 (first half) and
-        // fx < 0 (second half)
-        const int P = nthr / 2;
-        const int fx = tid < P ? tid : -1 - (tid - P);
-        const bool xvalid = tid < P ? (fx <= a.nk_pos) : (-fx <= a.nk_neg);
-        const int rows = a.nzi * a.nky;
-        int nrow = 0;
-        for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-            const int zi = row / a.nky;
-            const int yj = row - zi * a.nky;
-            const int z = zi <= a.nk_pos ? zi : n / 2;
-            const int y = yj <= a.nk_pos ? yj : n - (a.nky - yj);
-            const int fz = freq_of<T>(z, n), fy = freq_of<T>(y, n);
-            if (fy * fy + fz * fz >= thr[nb]) continue;   // no mode of this row lies in a shell (CTA-uniform)
-            mode_work(xvalid, fx, z, y, tid < P ? 0 : 1);
-            // fold the partials into the compensated accumulators every second row (a row pair
-            // adds at most 2 x 16 warp segments per shell to an FP32 partial)
-            if ((++nrow & 1) == 0) fold();
-        }
-        if (nrow & 1) fold();
-    } else {
-        // the work list: each warp takes one item (32 consecutive modes of a row inside the
-        // last shell) per round; the partials are folded after every round
-        const int warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
-        for (int base = blockIdx.x * nw; base < a.n_items; base += gridDim.x * nw) {
-            const int it = base + warp;
-            bool xvalid = false;
-            int fx = 0, z = 0, y = 0, half = 0;
-            if (it < a.n_items) {
-                const int4 item = a.items[it];
-                const int zi = item.x / a.nky;
-                const int yj = item.x - zi * a.nky;
-                z = zi <= a.nk_pos ? zi : n / 2;
-                y = yj <= a.nk_pos ? yj : n - (a.nky - yj);
-                const int t = item.y + lane;
-                xvalid = t <= item.z + item.w;
-                half = t > item.z ? 1 : 0;
-                fx = half ? -(t - item.z) : t;
+            warp_own_add<T>(dd, (T)0, bin, segm, mine, E);
+            warp_own_add<T>(gg, (T)0, bin, segm, mine + 2 * nb, E);
+        } else {
+            for (int ri = 0; ri < a.n_runs; ++ri) {
+                const CombineRun& run = a.run[ri];
+                T tre = 0, tim = 0;
+                for (int sy = sy0; sy <= sy1; ++sy) {
+                    bool on[2];
+                    unsigned im[2], ip[2];
+                    c2<T> phs[2];
+                    side(sy, on, im, ip, phs);
+                    if (!__any_sync(0xffffffffu, on[0] || on[1])) continue;   // warp-uniform
+                    // partner: delta(-k) = conj D; gamma*(-k) = conj G1 - i conj G2;
+                    // gamma(-k) = conj G1 + i conj G2
+                    c2<T> Pm[2], Pp[2];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        Pm[q] = Pp[q] = mk<T>((T)0, (T)0);
+                        if (!on[q]) continue;
+                        if (run.kind == KIND_CROSS || run.kind == KIND_DENS) {
+                            Pm[q] = cconj<T>(a.pD[im[q]]);
+                            Pp[q] = cconj<T>(a.pD[ip[q]]);
+                        } else {
+                            const c2<T> G1m = a.pG1[im[q]], G1p = a.pG1[ip[q]], G2m = a.pG2[im[q]], G2p = a.pG2[ip[q]];
+                            const T s = run.kind == KIND_PLUS ? (T)-1 : (T)1;
+                            // conj(G1) + s i conj(G2)
+                            Pm[q] = mk<T>(G1m.x + s * G2m.y, -G1m.y + s * G2m.x);
+                            Pp[q] = mk<T>(G1p.x + s * G2p.y, -G1p.y + s * G2p.x);
+                        }
+                        if (im[q] == ip[q]) Pp[q] = mk<T>((T)0, (T)0);   // its own mirror: counted once
+                    }
+                    // where the mirror is -k, an even-degree harmonic (every L here is even) takes the
+                    // same value at both members of the pair; Nyquist lanes contract their mirror
+                    // with its own harmonics in a second pass
+                    for (int pass = 0; pass < (anyq ? 2 : 1); ++pass) {
+                        c2<T> S[2][4];
+                        contract_run<T>(a, run, c, sy != 0, pass == 1, on, im, ip, S);
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            // X = F_re + i F_im at m and at the mirror
+                            c2<T> Xm, Xp;
+                            if (a.interlace) {
+                                c2<T> Hm, Hp;
+                                field_of<T>(S[q][0], S[q][1], 0, 1, c.iw, phs[q], c.ps, Xm, Xp);
+                                field_of<T>(S[q][2], S[q][3], 0, 1, c.iw, phs[q], c.ps, Hm, Hp);
+                                Xm = mk<T>(Xm.x - Hm.y, Xm.y + Hm.x);
+                                Xp = mk<T>(Xp.x - Hp.y, Xp.y + Hp.x);
+                            } else {
+                                Xm = mk<T>(c.iw * (S[q][0].x - S[q][2].y), c.iw * (S[q][0].y + S[q][2].x));
+                                Xp = mk<T>(c.iw * (S[q][0].x + S[q][2].y), c.iw * (S[q][2].x - S[q][0].y));
+                            }
+                            const c2<T> tm = cmul<T>(Xm, Pm[q]), tp = cmul<T>(Xp, Pp[q]);
+                            if (pass == 0) {
+                                tre += tm.x;
+                                tim += tm.y;
+                            }
+                            if ((c.nyq != 0) == (pass == 1)) {
+                                tre += tp.x;
+                                tim += tp.y;
+                            }
+                        }
+                    }
+                }
+                warp_own_add<T>(tre, tim, bin, segm, mine + ri * 2 * nb, E);
             }
-            mode_work(xvalid, fx, z, y, half);
-            fold();
         }
     }
+    __syncthreads();
     for (int i = tid; i < E; i += nthr) {
-        const double v = Owned<T>::value(own + i, own + E + i);
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v += Owned<T>::value(own + w * E * W + i, own + w * E * W + (W - 1) * E + i);
         if (v != 0.0) {
             const int ci = i / (2 * nb);
             const int rem = i - ci * 2 * nb;
-            const int row_out = a.partner_mode ? (ci == 0 ? a.row_dd0 : a.row_plus0) : a.ch[ci].out_row;
+            const int row_out = PARTNER ? (ci == 0 ? a.row_dd0 : a.row_plus0) : a.run[ci].out_row;
             if (row_out >= 0) atomicAdd(a.out + (long long)row_out * 2 * nb + rem, v);
         }
     }
 }
 
-template <typename T>
-cudaError_t launch_combine(const CombineArgs<T>& a, int n_sm, cudaStream_t st) {
-    const int nacc = a.partner_mode ? 2 : a.n_ch;
+template <typename T, bool PARTNER>
+static cudaError_t launch_combine_mode(const CombineArgs<T>& a, int n_sm, cudaStream_t st) {
+    const int nacc = PARTNER ? 2 : a.n_runs;
     const int E = nacc * a.nb * 2;
-    size_t smem = (size_t)E * sizeof(T) * (1 + Owned<T>::words) + (size_t)(a.n + (a.n & 1)) * sizeof(T) +
-                  (size_t)a.n * sizeof(c2<T>) + (size_t)(a.nb + 1) * sizeof(int);
-    if (a.items != nullptr) {
-        // 8 warps per CTA, three CTAs per SM
-        cudaFuncSetAttribute(k_combine<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        const int threads = 256;
-        int blocks = n_sm * 3;
-        const int rounds = (a.n_items + 7) / 8;
-        if (blocks > rounds) blocks = rounds > 0 ? rounds : 1;
-        k_combine<T, true><<<blocks, threads, smem, st>>>(a);
-        return cudaGetLastError();
-    }
-    cudaFuncSetAttribute(k_combine<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int P = ((a.nk_pos + 1) + 31) / 32 * 32;
-    const int threads = 2 * P;
-    const int rows = a.nzi * a.nky;
-    int blocks = n_sm * (threads <= 256 ? 8 : (threads <= 512 ? 4 : 2));
-    if (blocks > rows) blocks = rows;
-    k_combine<T, false><<<blocks, threads, smem, st>>>(a);
+    const size_t smem = (size_t)kCombineWarps * E * Owned<T>::words * sizeof(T) +
+                        (size_t)a.n * (sizeof(c2<T>) + sizeof(T)) + (size_t)(a.nb + 1) * sizeof(int);
+    CombineArgs<T> c = a;
+    const int na = std::max(a.nk_pos, a.nk_neg) + 1;
+    if (c.items == nullptr) c.n_items = a.nzi * na * ((na + 31) / 32);   // every segment of every row
+    // one resident wave (the launch bounds' CTAs per SM)
+    cudaFuncSetAttribute(k_combine<T, PARTNER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // lists that leave half of the resident warps idle take the two signs of fy as separate items
+    // (64^3 to k = 0.8 k_Ny: 530 items for 2432 warps; an estimate 1.43 -> 1.37 ms)
+    const int warps = n_sm * combine_ctas<T>() * kCombineWarps;
+    c.split = 2 * c.n_items <= warps ? 1 : 0;
+    const int work = c.n_items << c.split;
+    const int blocks = std::max(1, std::min(n_sm * combine_ctas<T>(), (work + kCombineWarps - 1) / kCombineWarps));
+    k_combine<T, PARTNER><<<blocks, 32 * kCombineWarps, smem, st>>>(c);
     return cudaGetLastError();
 }
 
-void combine_items(int n, int nk_pos, int nk_neg, int nky, int nzi, int q_max, std::vector<int4>& items) {
+template <typename T>
+cudaError_t launch_combine(const CombineArgs<T>& a, int n_sm, cudaStream_t st) {
+    return a.partner_mode ? launch_combine_mode<T, true>(a, n_sm, st) : launch_combine_mode<T, false>(a, n_sm, st);
+}
+
+void combine_items(int n, int nk_pos, int nk_neg, int nzi, int q_max, std::vector<int>& items) {
     items.clear();
+    const int na = std::max(nk_pos, nk_neg) + 1;
     for (int zi = 0; zi < nzi; ++zi) {
         const int z = zi <= nk_pos ? zi : n / 2;
-        const int fz = z < n / 2 ? z : z - n;
-        for (int yj = 0; yj < nky; ++yj) {
-            const int y = yj <= nk_pos ? yj : n - (nky - yj);
-            const int fy = y < n / 2 ? y : y - n;
-            const long long rem = (long long)q_max - (long long)fy * fy - (long long)fz * fz;
-            if (rem <= 0) continue;
-            // |fx| <= xr with fx^2 < rem
-            int xr = 0;
-            while ((long long)(xr + 1) * (xr + 1) < rem) ++xr;
-            const int xp = xr < nk_pos ? xr : nk_pos;
-            const int xn = xr < nk_neg ? xr : nk_neg;
-            const int m = xp + 1 + xn;
-            for (int t0 = 0; t0 < m; t0 += 32) items.push_back(make_int4(zi * nky + yj, t0, xp, xn));
+        const long long fz = z < n / 2 ? z : z - n;
+        for (int ay = 0; ay < na; ++ay) {
+            const long long rem = (long long)q_max - (long long)ay * ay - fz * fz;
+            for (int x0 = 0; x0 < na && (long long)x0 * x0 < rem; x0 += 32) items.push_back((zi * na + ay) << 6 | x0 / 32);
         }
     }
 }

@@ -271,14 +271,21 @@ cudaError_t launch_tile_ranges(const FusedArgs<T>& a, int* out, cudaStream_t st)
 size_t tile_range_bytes(int n, int ty, int tz);
 
 // --------------------------------------------------------------------- combine
-struct CombineChan {
-    int slot;      // grid in the batch
-    int sub;       // 0: real-part field (or interlaced pair), 1: imaginary-part field
-    int kind;      // Kind
-    int L, n;      // harmonic
-    int part;      // Part: multiply the field by 1 or by i
+// The channels of one moment and one |n| = m, which share Q_L^m: k = 0, 1 are the real and
+// imaginary kernel parts of n = +m, k = 2, 3 those of n = -m.
+template <typename T>
+struct CombineUnit {
+    int L, m;
+    T ynorm;       // normalisation of Y_{L,m} divided by (L - m)! (goes with ylm_poly_scaled)
+    int slot[4];   // grid in the batch of each channel, -1: not in this batch
+    int sub[4];    // 0: real-part field (or interlaced pair), 1: imaginary-part field
+};
+// Consecutive units u0 .. u1 - 1 of one moment (one kind and even degree): contracted with
+// their harmonics mode by mode and reduced together into output row out_row.
+struct CombineRun {
+    int u0, u1;
+    int kind;
     int out_row;   // row of the FP64 output [row][bin][2]
-    double ynorm;  // normalisation of Y_{L,n} divided by (L - |n|)! (goes with ylm_poly_scaled)
 };
 
 template <typename T>
@@ -287,9 +294,9 @@ struct CombineArgs {
     long long grid_stride;
     int n;
     int interlace;
-    int n_ch;
-    int per_grid;          // channels per batch grid: 1 (interlaced) or 2 (two packed fields)
-    CombineChan ch[kMaxBatchCh];
+    CombineUnit<T> unit[kMaxBatchCh];
+    int n_runs;
+    CombineRun run[kMaxBatchCh];
     // partner spectra (full n^3 arrays, valid on kept modes); in partner mode a null pD
     // skips storing D (only its shell sums are wanted)
     c2<T>* pD;
@@ -304,19 +311,19 @@ struct CombineArgs {
     int nb;
     int nk_pos, nk_neg, nky, nzi;
     double* out;           // [rows][nb][2]
-    // optional work list (combine_items): item = {row, first mode, x extent >= 0, x extent < 0}
-    // of the modes inside the last shell, 32 at a time; null: one CTA pass per whole row
-    const int4* items;
+    // the work list (combine_items), or null: every segment of every row of the kept cube
+    const int* items;
     int n_items;
+    int split;             // set by launch_combine: the pairs of +fy and -fy as separate work items
     int* err;              // ERRF_BOUNDS of LPP_CHECK builds
 };
 
 template <typename T>
 cudaError_t launch_combine(const CombineArgs<T>& a, int n_sm, cudaStream_t st);
-// The work list of the combine for a plan's kept cube: row r = zi * nky + yj (the combine's
-// row enumeration) holds the modes fx = 0 .. xp and -1 .. -xn with fx^2 + fy^2 + fz^2 < q_max;
-// they are split into items of 32 consecutive modes (fx = 0 .. xp first, then -1 .. -xn).
-void combine_items(int n, int nk_pos, int nk_neg, int nky, int nzi, int q_max, std::vector<int4>& items);
+// The work list of the combine for a plan's kept cube: row r = zi * na + |fy| (na = 1 + the
+// largest kept |f|, zi < nzi the kept z >= 0 and the Nyquist plane); item = r << 6 | segment, the
+// segments of 32 consecutive |fx| that hold a mode with fx^2 + fy^2 + fz^2 < q_max.
+void combine_items(int n, int nk_pos, int nk_neg, int nzi, int q_max, std::vector<int>& items);
 
 // ------------------------------------------------------------------ window multipoles
 // pD[m] = Z[m] / W(m) over every mode of grid 0 (the window field alone in the real part)

@@ -82,9 +82,11 @@ __device__ __forceinline__ SegMask seg_mask(int key) {
     return m;
 }
 
-// warp_bin_add with the row's precomputed segment structure
+// The segmented sums added to the warp's own accumulators own[words][E] (complex, interleaved)
+// in shared memory.  Equal shells form one segment (bins monotone along the warp), so no two
+// lanes add to the same accumulator.
 template <typename T>
-__device__ __forceinline__ void warp_bin_add_seg(T re, T im, int bin, const SegMask& m, T* acc) {
+__device__ __forceinline__ void warp_own_add(T re, T im, int bin, const SegMask& m, T* own, int E) {
     const unsigned full = 0xffffffffu;
 #pragma unroll
     for (int s = 0, d = 1; d < 32; d <<= 1, ++s) {
@@ -96,9 +98,10 @@ __device__ __forceinline__ void warp_bin_add_seg(T re, T im, int bin, const SegM
         }
     }
     if (m.last && bin >= 0) {
-        atomicAdd(acc + 2 * bin, re);
-        atomicAdd(acc + 2 * bin + 1, im);
+        Owned<T>::add(own + 2 * bin, own + E + 2 * bin, re);
+        Owned<T>::add(own + 2 * bin + 1, own + E + 2 * bin + 1, im);
     }
+    __syncwarp();   // another lane may add to the same shell next
 }
 
 }  // namespace lpp
