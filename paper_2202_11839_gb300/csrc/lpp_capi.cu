@@ -55,15 +55,12 @@ struct lpp_plan_s {
     int batch = 8;
     int batch_ch = 8;
     // host tables
-    std::vector<double> polys;
-    Quadrature quad[kQuadDegrees];
-    KernelPolys kp;
     // workspace
     char* ws = nullptr;
     size_t ws_bytes = 0;
     size_t ws_need = 0;
     size_t off_sums = 0, off_err = 0, off_out = 0, off_thr = 0, off_tw = 0, off_iw = 0, off_ph = 0;
-    size_t off_quad_dirs[kQuadDegrees] = {0}, off_quad_tab[kQuadDegrees] = {0}, off_polys = 0, off_coeff = 0;
+    size_t off_coeff = 0;
     size_t off_partner = 0, off_grids = 0, off_stage[3] = {0, 0, 0};
     // pencil-sorted catalogues: key, cell coordinates, weights, key offsets; shapes permutation
     size_t off_key[3] = {0, 0, 0}, off_su[3] = {0, 0, 0}, off_sw[3] = {0, 0, 0}, off_koff[3] = {0, 0, 0};
@@ -229,27 +226,21 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
     for (int b = 0; b < nb; ++b) plan->k_mean[b] = plan->n_modes[b] ? ksum[b] / plan->n_modes[b] : 0.0;
     combine_items(n, plan->nk_pos, plan->nk_neg, plan->nzi, tmax, plan->items);
 
-    // kernel polynomials and quadratures
-    build_kernel_polys(plan->kp);
-    for (int qi = 0; qi < kQuadDegrees; ++qi) build_quadrature(2 * (qi + 1), plan->quad[qi]);
 
     // channel groups: (kind, L) -> 2L+1 coefficient rows per projected part
     const unsigned m = d.moments;
     const bool cross_b = (m & LPP_WANT_CROSS_B) != 0;
     int row = 2;  // rows 0, 1: w gamma_1, w gamma_2
-    auto add_group = [&](int kind, int L, int has_im, const double* poly, int npoly, int slot) {
+    auto add_group = [&](int kind, int L, int has_im, int slot) {
+        const int spin = kind == KIND_CROSS ? 2 : kind == KIND_PLUS ? 0 : 4;
         CoeffGroup g;
-        g.kind = kind;
-        g.L = L;
+        g.kernel = 0;
+        while (kernel_spin(g.kernel) != spin || kernel_degree(g.kernel) != L) ++g.kernel;
         g.has_im = has_im;
         g.row_re = row;
         row += 2 * L + 1;
         g.row_im = has_im ? row : -1;
         if (has_im) row += 2 * L + 1;
-        g.poly = (int)plan->polys.size();
-        g.npoly = npoly;
-        plan->polys.insert(plan->polys.end(), poly, poly + npoly);
-        g.quad = L / 2 - 1;
         plan->groups.push_back(g);
         // n = 0, 1, -1, 2, -2, ... with both parts together: the combine's units (n = +-m) are
         // consecutive channels
@@ -268,12 +259,12 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
     };
     const int crossSlot[3] = {LPP_MOM_CROSS2, LPP_MOM_CROSS4, LPP_MOM_CROSS6};
     for (int i = 0; i < 3; ++i)
-        if (m & (1u << crossSlot[i])) add_group(KIND_CROSS, 2 * (i + 1), cross_b ? 1 : 0, plan->kp.cross[i], 2 * i + 1, crossSlot[i]);
-    if (m & (1u << LPP_MOM_PLUS2)) add_group(KIND_PLUS, 2, 1, plan->kp.plus[1], 3, LPP_MOM_PLUS2);
-    if (m & (1u << LPP_MOM_PLUS4)) add_group(KIND_PLUS, 4, 1, plan->kp.plus[2], 5, LPP_MOM_PLUS4);
+        if (m & (1u << crossSlot[i])) add_group(KIND_CROSS, 2 * (i + 1), cross_b ? 1 : 0, crossSlot[i]);
+    if (m & (1u << LPP_MOM_PLUS2)) add_group(KIND_PLUS, 2, 1, LPP_MOM_PLUS2);
+    if (m & (1u << LPP_MOM_PLUS4)) add_group(KIND_PLUS, 4, 1, LPP_MOM_PLUS4);
     const int minusSlot[5] = {LPP_MOM_MINUS4, LPP_MOM_MINUS6, LPP_MOM_MINUS8, LPP_MOM_MINUS10, LPP_MOM_MINUS12};
     for (int i = 0; i < 5; ++i)
-        if (m & (1u << minusSlot[i])) add_group(KIND_MINUS, 4 + 2 * i, 1, plan->kp.minus[i], 2 * i + 1, minusSlot[i]);
+        if (m & (1u << minusSlot[i])) add_group(KIND_MINUS, 4 + 2 * i, 1, minusSlot[i]);
     plan->n_coeff_rows = row;
     plan->n_tensor_ch = (int)plan->channels.size();
     // density multipoles (Eqs. lpp_dens_app, delta_ell): by the addition theorem
@@ -324,11 +315,6 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
     plan->off_tw = take(n * cs);
     plan->off_iw = take(n * es);
     plan->off_ph = take(n * cs);
-    for (int qi = 0; qi < kQuadDegrees; ++qi) {
-        plan->off_quad_dirs[qi] = take(plan->quad[qi].dirs.size() * es);
-        plan->off_quad_tab[qi] = take(plan->quad[qi].table.size() * es);
-    }
-    plan->off_polys = take(std::max<size_t>(1, plan->polys.size()) * es);
     plan->off_coeff = take((size_t)plan->n_coeff_rows * std::max<long long>(1, d.max_shapes) * es);
     {
         int ipt, thr;
@@ -425,16 +411,6 @@ static lpp_status write_tables(lpp_plan_t plan) {
     LPP_CUDA(put(plan->off_tw, keep[0].data(), keep[0].size() * sizeof(T)));
     LPP_CUDA(put(plan->off_iw, keep[1].data(), keep[1].size() * sizeof(T)));
     LPP_CUDA(put(plan->off_ph, keep[2].data(), keep[2].size() * sizeof(T)));
-    for (int qi = 0; qi < kQuadDegrees; ++qi) {
-        keep.emplace_back(plan->quad[qi].dirs.begin(), plan->quad[qi].dirs.end());
-        LPP_CUDA(put(plan->off_quad_dirs[qi], keep.back().data(), keep.back().size() * sizeof(T)));
-        keep.emplace_back(plan->quad[qi].table.begin(), plan->quad[qi].table.end());
-        LPP_CUDA(put(plan->off_quad_tab[qi], keep.back().data(), keep.back().size() * sizeof(T)));
-    }
-    if (!plan->polys.empty()) {
-        keep.emplace_back(plan->polys.begin(), plan->polys.end());
-        LPP_CUDA(put(plan->off_polys, keep.back().data(), keep.back().size() * sizeof(T)));
-    }
     LPP_CUDA(cudaStreamSynchronize(plan->stream));
     plan->tables_ready = true;
     return LPP_OK;
@@ -683,15 +659,7 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
     ca.stride = stride;
     ca.n_groups = (int)plan->groups.size();
     for (int g = 0; g < ca.n_groups; ++g) ca.groups[g] = plan->groups[g];
-    for (int qi = 0; qi < kQuadDegrees; ++qi) {
-        bool used = false;
-        for (const CoeffGroup& g : plan->groups) used = used || g.quad == qi;
-        ca.quad_dirs[qi] = (const T*)(plan->ws + plan->off_quad_dirs[qi]);
-        ca.quad_tab[qi] = (const T*)(plan->ws + plan->off_quad_tab[qi]);
-        ca.quad_S[qi] = used ? plan->quad[qi].S : 0;
-    }
-    ca.polys = (const T*)(plan->ws + plan->off_polys);
-    ca.n_polys = (int)plan->polys.size();
+    for (int i = 0; i < kKernelTable; ++i) ca.tab[i] = (T)kernel_series()[i];
     ca.sums = sums;
     ca.err = err;
     if (sh.shape_kind != LPP_SHAPE_NONE) {

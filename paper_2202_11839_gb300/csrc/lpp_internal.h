@@ -130,16 +130,23 @@ struct Quadrature {
     std::vector<double> table;  // [2L+1][S]
 };
 
-// Polynomial coefficients (power series in mu) of the reduced kernels.
-struct KernelPolys {
-    // cross: Lm2_L / (1 - mu^2);  minus: Lm4_L / (1 - mu^2)^2;  plus: L_l
-    double cross[4][8];   // L = 2,4,6 (index L/2 - 1); up to mu^6
-    double plus[3][8];    // l = 0,2,4 (index l/2)
-    double minus[5][9];   // L = 4,6,8,10,12 (index L/2 - 2); up to mu^8
-};
+// The estimator's kernels as functions of khat: spin s (the power of k.e_theta - i k.e_phi) and
+// degree L, K = (k.e_theta - i k.e_phi)^s d^s P_L(mu)/dmu^s (cross s = 2, plus 0, minus 4).
+constexpr int kKernels = 10;
+__host__ __device__ constexpr int kernel_spin(int k) { return k < 3 ? 2 : (k < 5 ? 0 : 4); }
+__host__ __device__ constexpr int kernel_degree(int k) {
+    return k < 3 ? 2 * (k + 1) : (k < 5 ? 2 * (k - 2) : 2 * (k - 3));
+}
+// First entry of kernel k's (L + 1) x (L + 1) block in the table of kernel_series.
+__host__ __device__ constexpr int kernel_offset(int k) {
+    return k == 0 ? 0 : kernel_offset(k - 1) + (kernel_degree(k - 1) + 1) * (kernel_degree(k - 1) + 1);
+}
+constexpr int kKernelTable = kernel_offset(kKernels);
 
 void build_quadrature(int L, Quadrature& q);
-void build_kernel_polys(KernelPolys& kp);
+// Entry kernel_offset(k) + n (L + 1) + j: the trigonometric series in theta of kernel k's projection
+// onto the harmonics of order n (kKernelTable numbers, see k_coeffs)
+const double* kernel_series();
 void legendre_poly(int l, double* c);  // power-series coefficients, c[0..l]
 void gauss_legendre(int n, double* x, double* w);
 void eb_matrices(double N[2][3], double M[3][3]);

@@ -84,19 +84,14 @@ cudaError_t fft_yz(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGe
 
 // ---------------------------------------------------------- per-particle weights
 constexpr int kMaxGroups = 16;
-constexpr int kQuadDegrees = 6;    // harmonic projection quadratures for L = 2, 4, ..., 12
 constexpr int kMaxSlots = 8;       // complex grids per batch (FftGeom::gmask has as many)
 constexpr int kMaxBatchCh = 16;    // real fields per batch
 
 struct CoeffGroup {
-    int kind;    // Kind
-    int L;
+    int kernel;  // index into kernel_spin, kernel_degree
     int has_im;  // also project the imaginary part of the kernel
     int row_re;  // first coefficient row of the real part (rows row_re + n + L)
     int row_im;  // first row of the imaginary part
-    int poly;    // offset of the mu-polynomial in the poly table
-    int npoly;   // number of coefficients
-    int quad;    // index into the quadrature table list (L/2 - 1)
 };
 
 template <typename T>
@@ -115,11 +110,7 @@ struct CoeffArgs {
     long long stride;
     int n_groups;
     CoeffGroup groups[kMaxGroups];
-    const T* quad_dirs[kQuadDegrees];   // per L = 2,4,...,12: [S][3]
-    const T* quad_tab[kQuadDegrees];    // per L: [2L+1][S]
-    int quad_S[kQuadDegrees];           // 0 for a degree no group of the plan uses
-    const T* polys;          // concatenated mu-polynomial coefficients
-    int n_polys;
+    T tab[kKernelTable];     // kernel_series
     double* sums;            // FP64 reductions (see SumSlot)
     int* err;
 };

@@ -35,31 +35,6 @@ static int derive(double* c, int deg, int m) {
     return deg;
 }
 
-void build_kernel_polys(KernelPolys& kp) {
-    for (int i = 0; i < 4; ++i) for (int j = 0; j < 8; ++j) kp.cross[i][j] = 0.0;
-    for (int i = 0; i < 3; ++i) for (int j = 0; j < 8; ++j) kp.plus[i][j] = 0.0;
-    for (int i = 0; i < 5; ++i) for (int j = 0; j < 9; ++j) kp.minus[i][j] = 0.0;
-    double c[16];
-    // Lm_L(mu)/(1-mu^2)^(m/2) = (-1)^m d^m L_L / dmu^m (m even: sign +1)
-    for (int L = 2; L <= 6; L += 2) {
-        for (int i = 0; i < 16; ++i) c[i] = 0.0;
-        legendre_poly(L, c);
-        const int d = derive(c, L, 2);
-        for (int i = 0; i <= d; ++i) kp.cross[L / 2 - 1][i] = c[i];
-    }
-    for (int l = 0; l <= 4; l += 2) {
-        for (int i = 0; i < 16; ++i) c[i] = 0.0;
-        legendre_poly(l, c);
-        for (int i = 0; i <= l; ++i) kp.plus[l / 2][i] = c[i];
-    }
-    for (int L = 4; L <= 12; L += 2) {
-        for (int i = 0; i < 16; ++i) c[i] = 0.0;
-        legendre_poly(L, c);
-        const int d = derive(c, L, 4);
-        for (int i = 0; i <= d; ++i) kp.minus[L / 2 - 2][i] = c[i];
-    }
-}
-
 // Gauss-Legendre nodes and weights on [-1, 1] by Newton iteration on L_n.
 void gauss_legendre(int n, double* x, double* w) {
     for (int i = 0; i < n; ++i) {
@@ -109,6 +84,59 @@ void build_quadrature(int L, Quadrature& q) {
                 q.table[(size_t)(n + L) * q.S + s] = wt * ylm_norm(L, n) * ylm_poly<double>(L, n, kx, ky, kz);
         }
     }
+}
+
+// For a line of sight (sin t, 0, cos t) with e_theta = (cos t, 0, -sin t), e_phi = y, the projection
+// of kernel k onto the cosine harmonic of order n is real, A_n(t), and onto the sine harmonic
+// imaginary, i B_n(t).  Both are trigonometric polynomials of degree L in t, cosine series for even
+// n and sine series for odd n, A_n with even frequencies j and B_n with odd ones (reflection
+// about z): one row of L + 1 numbers holds both.  The values at 2 L + 4 midpoints come from the
+// exact quadrature, the series from their discrete orthogonality.
+static void build_kernel_series(double* tab) {
+    for (int k = 0; k < kKernels; ++k) {
+        const int L = kernel_degree(k), spin = kernel_spin(k), M = 2 * L + 4;
+        Quadrature q;
+        build_quadrature(L, q);
+        double c[16] = {0};
+        legendre_poly(L, c);
+        const int deg = derive(c, L, spin);
+        double* out = tab + kernel_offset(k);
+        for (int i = 0; i < (L + 1) * (L + 1); ++i) out[i] = 0.0;
+        for (int p = 0; p < M; ++p) {
+            const double t = kPi * (p + 0.5) / M, st = sin(t), ct = cos(t);
+            for (int n = 0; n <= L; ++n) {
+                double A = 0.0, B = 0.0;
+                for (int s = 0; s < q.S; ++s) {
+                    const double kx = q.dirs[3 * s], ky = q.dirs[3 * s + 1], kz = q.dirs[3 * s + 2];
+                    const double mu = kx * st + kz * ct, a = kx * ct - kz * st;
+                    double pm = 0.0;
+                    for (int i = deg; i >= 0; --i) pm = pm * mu + c[i];
+                    double re = 1.0, im = 0.0;   // (a - i ky)^spin
+                    for (int i = 0; i < spin; ++i) {
+                        const double r = re * a + im * ky;
+                        im = im * a - re * ky;
+                        re = r;
+                    }
+                    A += pm * re * q.table[(size_t)(L + n) * q.S + s];
+                    if (n > 0) B += pm * im * q.table[(size_t)(L - n) * q.S + s];
+                }
+                for (int j = 0; j <= L; ++j) {
+                    const double w = (j == 0 ? 1.0 : 2.0) / M;
+                    out[n * (L + 1) + j] += w * ((n & 1) ? sin(j * t) : cos(j * t)) * ((j & 1) ? B : A);
+                }
+            }
+        }
+    }
+}
+
+const double* kernel_series() {
+    // the same numbers for every plan: built on the first use (about 1 ms)
+    static const std::vector<double> tab = [] {
+        std::vector<double> t(kKernelTable);
+        build_kernel_series(t.data());
+        return t;
+    }();
+    return tab.data();
 }
 
 }  // namespace lpp
