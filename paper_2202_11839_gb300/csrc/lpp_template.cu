@@ -6,12 +6,16 @@
 // Both Hankel transforms use the log-Fourier method of Hamilton (2000): A(x) x^-q is
 // expanded in a discrete Fourier series in ln x and each term is transformed with the Mellin
 // transform of j_l,  int_0^inf x^(s-1) j_l(x) dx = 2^(s-2) sqrt(pi) G((l+s)/2) / G((3+l-s)/2).
-// One CTA evaluates one parameter set: the BBKS model and its sigma_8 normalisation, three
-// inverse transforms (L' = 0, 2, 4), then for each of the fourteen output slots (the
-// estimator's order: the density quadrupole and hexadecapole, whose templates are the
-// leakage of the monopole through Q_2 and Q_4, Sec. 4.3, then the minus moments L = 10, 12,
-// which the model leaves zero and only the window fills) the mixture with the window
-// multipoles, one forward transform and the shell averages.  Everything is FP64.
+// Everything is FP64.
+//
+// For one window the whole chain, from the model spectrum to the shell averages of the fourteen
+// output slots (the estimator's order: the density quadrupole and hexadecapole, whose
+// templates are the leakage of the monopole through Q_2 and Q_4, Sec. 4.3, then the minus
+// moments L = 10, 12, which the model leaves zero and only the window fills), is one linear
+// map of the spectrum on the 2048 grid k.  It is formed once per window (k_operator: one row of
+// 2048 weights per slot and shell, by the transposed chain of two to four transforms), and a
+// parameter set costs its model spectrum and one product with the rows (k_template, on the
+// FP64 tensor cores).
 //
 // Grid (shared with the tests): 2048 log-spaced k in [1e-4, 10], zero padding to 4096,
 // k_0 r_0 = exp(-(N-1) Delta), biases 1.5 (inverse) and 0.5 (forward), the input tapered by
@@ -19,6 +23,9 @@
 #include <math.h>
 #include <string.h>
 
+#include <cooperative_groups.h>
+
+#include <algorithm>
 #include <complex>
 #include <vector>
 
@@ -44,16 +51,11 @@ struct SlotDesc {
     int L;
     int n_terms;
     int lp[kMaxTerms];      // L' of each term (0, 2, 4)
-    int coef[kMaxTerms];    // model coefficient id (see model_coef)
+    double coef[kMaxTerms]; // model coefficient (power_for_validation, without A and b_g)
     int qx[kMaxTerms];      // row of the mixed window table Q^X_LL'(r_m)
 };
 
-struct TemplateArgs {
-    const double* params;   // [n][6]: A, b_g, sigma8, tilt, Gamma, shot-noise scale
-    int n_templates;
-    double* out;            // [n][LPP_N_MOMENTS][nb]
-    const double* kin;      // [2048] k_n
-    const double* s8w;      // [2048] sigma_8 quadrature weight w_n k^3 W^2(8k) / (2 pi^2)
+struct OperatorArgs {
     const double* ain;      // [2048] k^3 taper k^-q_inv
     const double2* uinv;    // [3][4096] inverse kernels (1/N folded in)
     const double* rinv;     // [4096] r^-q_inv / (2 pi^2)
@@ -66,8 +68,25 @@ struct TemplateArgs {
     const int* bin_hi;      // [nb] one past the last
     const double* bin_w;    // [2048] k_n^3
     int nb;
-    double shot_plus;
     SlotDesc slots[kSlots];
+    double* op;             // [kSlots][nb][2048]
+};
+
+struct TemplateArgs {
+    const double* params;   // [n][6]: A, b_g, sigma8, tilt, Gamma, shot-noise scale
+    int n_templates;
+    double* out;            // [n][LPP_N_MOMENTS][nb]
+    const double* op;       // [kSlots][nb][2048] the operator's rows
+    const double* kin;      // [2048] k_n
+    const double* lnk;      // [2048] ln k_n
+    const double* s8w;      // [2048] sigma_8 quadrature weight w_n k^3 W^2(8k) / (2 pi^2)
+    const int* bin_lo;      // [nb] first k_n of each shell
+    const int* bin_hi;      // [nb] one past the last
+    int nb;
+    int bins;               // shells per cluster
+    int n_slots;            // slots to compute, in order
+    int slot[kSlots];
+    double shot_plus;
     // optional derived curves gE_0,2, EE_0,2,4, BB_0,2,4 per shell, standardised as
     // (value - ref) / sigma and stored FP32 [n][8][nb]
     float* eb;
@@ -80,53 +99,6 @@ struct TemplateArgs {
     unsigned slot_mask;     // output slots to compute; the others are written as zeros
 };
 
-// BBKS transfer function T(q), q = k / Gamma (Bardeen, Bond, Kaiser & Szalay 1986)
-__device__ __forceinline__ double bbks_transfer(double k, double gam) {
-    const double q = k / gam;
-    return log(1.0 + 2.34 * q) / (2.34 * q) *
-           pow(1.0 + 3.89 * q + (16.1 * q) * (16.1 * q) + (5.46 * q) * (5.46 * q) * (5.46 * q) +
-                   (6.71 * q) * (6.71 * q) * (6.71 * q) * (6.71 * q),
-               -0.25);
-}
-
-// The shape response to spin-2 PNG: P -> [1 + 12 f_NL delta b_IA / M(k)] P for each shape field
-// (Sec. 5), M(k) = (2/3) k^2 T(k) D (c/H0)^2 / Omega_m with D = 1 (z = 0).
-__device__ __forceinline__ double png_factor(double k, double gam, double amp, double len2) {
-    return 1.0 + amp / ((2.0 / 3.0) * k * k * bbks_transfer(k, gam) * len2);
-}
-
-__device__ __forceinline__ double bbks_shape(double k, double gam, double tilt) {
-    const double q = k / gam;
-    const double t = log(1.0 + 2.34 * q) / (2.34 * q) *
-                     pow(1.0 + 3.89 * q + (16.1 * q) * (16.1 * q) + (5.46 * q) * (5.46 * q) * (5.46 * q) +
-                             (6.71 * q) * (6.71 * q) * (6.71 * q) * (6.71 * q),
-                         -0.25);
-    return pow(k, 1.0 + tilt) * t * t;
-}
-
-__device__ __forceinline__ double model_coef(int id, double A, double b) {
-    switch (id) {
-        case 0: return b * b;                  // dd, L' = 0
-        case 1: return -A * b / 6.0;           // cross, L' = 2
-        case 2: return 2.0 * A * A / 15.0;     // plus, L' = 0
-        case 3: return -4.0 * A * A / 21.0;    // plus, L' = 2
-        case 4: return 2.0 * A * A / 35.0;     // plus, L' = 4
-        default: return A * A / 420.0;         // minus, L' = 4
-    }
-}
-
-__device__ double block_sum(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[wid] = v;
-    __syncthreads();
-    double s = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-    __syncthreads();
-    return s;
-}
-
 // wk <- FFT(wk) * u ; FFT again (the log-Fourier transform between the two grids)
 __device__ void log_fourier(double2* wk, const double2* __restrict__ u, const double2* __restrict__ tw) {
     const int tid = threadIdx.x;
@@ -136,123 +108,217 @@ __device__ void log_fourier(double2* wk, const double2* __restrict__ u, const do
     lpp::fft_columns<double, kLogN, false, 1, 1>(wk, 0, tid, tw);
 }
 
-__global__ void __launch_bounds__(512, 1) k_template(TemplateArgs a) {
+// One row (slot, shell) of the operator: out = sum_n op[n] P(k_n).  Forwards, a spectrum is
+// weighted (ain), transformed (T_L' = Re F u F, a real symmetric matrix because u is Hermitian),
+// weighted by the window and the radial powers, transformed again (T_L) and averaged over the
+// shell; the row applies the transposed steps in reverse order to the shell's weights.
+__global__ void __launch_bounds__(512, 1) k_operator(OperatorArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* wk = reinterpret_cast<double2*>(smem_raw);        // [4096]
-    double* xi = reinterpret_cast<double*>(wk + kNfft);        // [3][4096]
-    double* av = xi + 3 * kNfft;                               // [2048]
-    __shared__ double red[32];
+    double* back = reinterpret_cast<double*>(wk + kNfft);      // [4096]
+    double* acc = back + kNfft;                                // [2048]
     const int tid = threadIdx.x, nthr = blockDim.x;
-    const int t = blockIdx.x;
-    if (t >= a.n_templates) return;
-    const double* p = a.params + 6 * (size_t)t;
-    const double A = p[0], b = p[1], s8 = p[2], tilt = p[3], gam = p[4], shot = p[5];
-
-    // model spectrum and its sigma_8 normalisation
-    double loc = 0.0;
-    for (int n = tid; n < kNin; n += nthr) {
-        const double sh = bbks_shape(a.kin[n], gam, tilt);
-        av[n] = sh;
-        loc += a.s8w[n] * sh;
-    }
-    const double s2 = block_sum(loc, red);
-    const double norm = s8 * s8 / s2;
-    for (int n = tid; n < kNin; n += nthr) av[n] *= norm * a.ain[n];
+    const int bb = blockIdx.x % a.nb;
+    const SlotDesc& sd = a.slots[blockIdx.x / a.nb];
+    const int lo = a.bin_lo[bb], hi = a.bin_hi[bb];
+    double den = 0.0;
+    for (int n = lo; n < hi; ++n) den += a.bin_w[n];
+    const double sgn = ((sd.L / 2) & 1) ? -1.0 : 1.0;   // (-i)^L
+    for (int m = tid; m < kNfft; m += nthr)
+        wk[m] = make_double2(m >= lo && m < hi ? sgn * a.bin_w[m] * a.kfwd[m] / den : 0.0, 0.0);
+    for (int m = tid; m < kNin; m += nthr) acc[m] = 0.0;
     __syncthreads();
+    log_fourier(wk, a.ufwd + (size_t)(sd.L / 2) * kNfft, a.tw);
+    for (int m = tid; m < kNfft; m += nthr) back[m] = wk[m].x * a.rfwd[m] * a.rinv[m];
+    __syncthreads();
+    for (int j = 0; j < sd.n_terms; ++j) {
+        const double c = sd.lp[j] == 2 ? -sd.coef[j] : sd.coef[j];   // i^L'
+        for (int m = tid; m < kNfft; m += nthr)
+            wk[m] = make_double2(c * a.qx[(size_t)sd.qx[j] * kNfft + m] * back[m], 0.0);
+        __syncthreads();
+        log_fourier(wk, a.uinv + (size_t)(sd.lp[j] / 2) * kNfft, a.tw);
+        for (int m = tid; m < kNin; m += nthr) acc[m] += wk[m].x;
+        __syncthreads();
+    }
+    double* op = a.op + (size_t)blockIdx.x * kNin;
+    for (int m = tid; m < kNin; m += nthr) op[m] = acc[m] * a.ain[m];
+}
 
-    // xi^(L') = H^-1_L'[P_X], one phase of at most three transforms: Gaussian: P at L' = 0, 2, 4
-    // for every slot; with PNG the shape spectra carry the response factor once (cross, phase 0
-    // with the density's P) or twice (plus and minus, phase 1)
+// c[8][8] += a[8][4] b[4][8] (one warp, FP64 tensor cores): lane l holds a[l / 4][l % 4],
+// b[l % 4][l / 4] and c[l / 4][2 (l % 4) + {0, 1}].
+__device__ __forceinline__ void mma_f64(double c[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};\n"
+                 : "+d"(c[0]), "+d"(c[1])
+                 : "d"(a), "d"(b));
+}
+
+// Templates of eight parameter sets on one cluster of eight CTAs (blockIdx.y: a group of a.bins
+// shells).  CTA c forms the model spectra on its 256 grid k (one thread per k, the sets in turn)
+// and multiplies them with its 256 columns of the operator's rows, 8 sets x 8 rows x 4 columns
+// per tensor instruction; the cluster then adds the eight partial sums through distributed
+// shared memory in a fixed order, CTA c for every eighth shell, normalises to sigma_8 and
+// writes the slots and derived curves.
+//
+// What bounds it: FP64 issue, about half of it the model spectrum (log1p, exp, rsqrt) and half
+// the products; the FP64 mma runs 4.2 times the plain FP64 multiply-add rate on GB300 (2.09
+// against 0.50 T multiply-adds/s), which is why the rows are multiplied by it even for one set
+// (seven of its eight rows idle).  8192 sets, nine slots, 40 shells: 78.0 -> 14.9 ms against one
+// CTA per set running its own transforms (24 FFTs of 4096 points); one set, fourteen slots:
+// 1.99 -> 0.18 ms (the shells spread over the SMs by blockIdx.y).
+constexpr int kCluster = 8, kSets = 8, kSlab = kNin / kCluster, kTiles = 9;
+constexpr int kMaxRows = 8 * 8 * kTiles;   // rows per cluster: 8 warps x kTiles tiles of 8
+constexpr int kSlabPad = kSlab + 2;        // the eight sets' rows start in different banks
+
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(256, 2) k_template(const __grid_constant__ TemplateArgs a) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     const bool png = a.png_amp != 0.0;
-    for (int phase = 0; phase < (png ? 2 : 1); ++phase) {
-    int nrow = 3, rowL[3] = {0, 2, 4}, rowP[3] = {0, 0, 0};
-    if (png && phase == 0) { nrow = 2; rowL[1] = 2; rowP[1] = 1; }
-    if (png && phase == 1) { rowP[0] = rowP[1] = rowP[2] = 2; }
-    for (int r = 0; r < nrow; ++r) {
-        for (int m = tid; m < kNfft; m += nthr) {
-            double v = 0.0;
-            if (m < kNin) {
-                v = av[m];
-                if (rowP[r] > 0) {
-                    const double f = png_factor(a.kin[m], gam, a.png_amp, a.png_len2);
-                    v *= rowP[r] == 1 ? f : f * f;
+    const int n_pow = png ? 3 : 1;   // P, P f, P f^2 with the PNG response f
+    double* spec = reinterpret_cast<double*>(smem_raw);   // [n_pow][kSets][kSlabPad]
+    double* part = spec + n_pow * kSets * kSlabPad;       // [rows][kSets] partial sums
+    __shared__ double s8part[kSets];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int t0 = (int)(blockIdx.x / kCluster) * kSets;
+    const int sets = min(kSets, a.n_templates - t0);
+    const int b0 = blockIdx.y * a.bins, nbl = min(a.bins, a.nb - b0);
+    const int rows = a.n_slots * nbl;
+
+    // model spectra (unnormalised BBKS, Bardeen, Bond, Kaiser & Szalay 1986)
+    {
+        const int n = rank * kSlab + tid;
+        const double k = a.kin[n], lnk = a.lnk[n];
+        for (int t = 0; t < kSets; ++t) {
+            double p = 0.0, f = 0.0;
+            if (t < sets) {
+                const double* th = a.params + 6 * (size_t)(t0 + t);
+                const double tilt = th[3], gam = th[4];
+                const double q = k / gam;
+                const double l = log1p(2.34 * q) / (2.34 * q);
+                const double x = 1.0 + q * (3.89 + q * (16.1 * 16.1 + q * (5.46 * 5.46 * 5.46 +
+                                                                           q * (6.71 * 6.71 * 6.71 * 6.71))));
+                const double rs = rsqrt(x);        // T = l x^(-1/4)
+                p = k * exp(tilt * lnk) * (l * l * rs);
+                // Sec. 5: P -> [1 + 12 f_NL delta b_IA / M(k)] P per shape field,
+                // M(k) = (2/3) k^2 T(k) D (c/H0)^2 / Omega_m with D = 1 (z = 0)
+                if (png) f = 1.0 + a.png_amp / ((2.0 / 3.0) * k * k * (l * sqrt(rs)) * a.png_len2);
+            }
+            spec[t * kSlabPad + tid] = p;
+            if (png) {
+                spec[(kSets + t) * kSlabPad + tid] = p * f;
+                spec[(2 * kSets + t) * kSlabPad + tid] = p * f * f;
+            }
+        }
+    }
+    __syncthreads();
+    // sigma_8^2 of set `warp` over this slab
+    {
+        double s = 0.0;
+        for (int i = lane; i < kSlab; i += 32) s += a.s8w[rank * kSlab + i] * spec[warp * kSlabPad + i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) s8part[warp] = s;
+    }
+    // row r = (slot index) nbl + shell; tile j of the warp: rows 8 (warp + 8 j) ..
+    const int rl = lane >> 2, cl = 2 * (lane & 3);
+    const double* brow[kTiles];
+    const double* arow = spec + rl * kSlabPad + cl;
+    double acc[kTiles][2];
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j) {
+        const int r8 = 8 * (warp + 8 * j);
+        const int r = max(0, min(r8 + rl, rows - 1));   // rows beyond the last repeat it and are not read back
+        const int si = r / nbl;
+        brow[j] = a.op + ((size_t)a.slot[si] * a.nb + b0 + (r - si * nbl)) * kNin + rank * kSlab + cl;
+        acc[j][0] = acc[j][1] = 0.0;
+    }
+    if (!png) {
+        for (int k0 = 0; k0 < kSlab; k0 += 8) {
+            const double2 av = *reinterpret_cast<const double2*>(arow + k0);
+#pragma unroll
+            for (int j = 0; j < kTiles; ++j) {
+                if (8 * (warp + 8 * j) >= rows) break;   // warp-uniform
+                const double2 bv = *reinterpret_cast<const double2*>(brow[j] + k0);
+                mma_f64(acc[j], av.x, bv.x);
+                mma_f64(acc[j], av.y, bv.y);
+            }
+        }
+    } else {
+        // the response enters the density rows not at all, the cross rows once and the plus and
+        // minus rows twice; a tile may straddle two families, so every row takes the product
+        // with its own family's spectrum of the three
+        for (int pw = 0; pw < 3; ++pw) {
+#pragma unroll
+            for (int j = 0; j < kTiles; ++j) {
+                const int r8 = 8 * (warp + 8 * j);
+                if (r8 >= rows) break;
+                const int r = min(r8 + rl, rows - 1);
+                const int sl = a.slot[r / nbl];
+                const int want = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
+                if (!__any_sync(0xffffffffu, want == pw)) continue;   // warp-uniform
+                const double on = want == pw ? 1.0 : 0.0;
+                for (int k0 = 0; k0 < kSlab; k0 += 8) {
+                    const double2 av = *reinterpret_cast<const double2*>(arow + pw * kSets * kSlabPad + k0);
+                    const double2 bv = *reinterpret_cast<const double2*>(brow[j] + k0);
+                    mma_f64(acc[j], av.x, on * bv.x);
+                    mma_f64(acc[j], av.y, on * bv.y);
                 }
             }
-            wk[m] = make_double2(v, 0.0);
-        }
-        __syncthreads();
-        log_fourier(wk, a.uinv + (size_t)(rowL[r] / 2) * kNfft, a.tw);
-        const double sgn = (rowL[r] == 2) ? -1.0 : 1.0;   // i^L'
-        for (int m = tid; m < kNfft; m += nthr) xi[r * kNfft + m] = sgn * wk[m].x * a.rinv[m];
-        __syncthreads();
-    }
-
-    // each output slot of this phase: mixture with the window, forward transform, shell averages
-    for (int s = 0; s < kSlots; ++s) {
-        const SlotDesc& sd = a.slots[s];
-        if (png && (sd.kind >= 2 ? 1 : 0) != phase) continue;
-        if (!((a.slot_mask >> s) & 1u)) {
-            for (int bb = tid; bb < a.nb; bb += nthr) a.out[((size_t)t * kSlots + s) * a.nb + bb] = 0.0;
-            continue;
-        }
-        double cf[kMaxTerms];
-        int row[kMaxTerms];
-        for (int j = 0; j < sd.n_terms; ++j) {
-            cf[j] = model_coef(sd.coef[j], A, b);
-            row[j] = 0;
-            for (int r = 0; r < nrow; ++r)
-                if (rowL[r] == sd.lp[j]) row[j] = r;
-        }
-        for (int m = tid; m < kNfft; m += nthr) {
-            double g = 0.0;
-            for (int j = 0; j < sd.n_terms; ++j)
-                g += cf[j] * a.qx[(size_t)sd.qx[j] * kNfft + m] * xi[row[j] * kNfft + m];
-            wk[m] = make_double2(g * a.rfwd[m], 0.0);
-        }
-        __syncthreads();
-        log_fourier(wk, a.ufwd + (size_t)(sd.L / 2) * kNfft, a.tw);
-        const double sgn = ((sd.L / 2) & 1) ? -1.0 : 1.0;   // (-i)^L
-        const double add = (sd.kind == 2 && sd.L == 0) ? shot * a.shot_plus : 0.0;
-        // one warp per shell
-        const int lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
-        for (int bb = wid; bb < a.nb; bb += nw) {
-            double num = 0.0, den = 0.0;
-            for (int n = a.bin_lo[bb] + lane; n < a.bin_hi[bb]; n += 32) {
-                const double w = a.bin_w[n];
-                num += w * sgn * wk[n].x * a.kfwd[n];
-                den += w;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                num += __shfl_down_sync(0xffffffffu, num, o);
-                den += __shfl_down_sync(0xffffffffu, den, o);
-            }
-            if (lane == 0) a.out[((size_t)t * kSlots + s) * a.nb + bb] = den > 0.0 ? num / den + add : 0.0;
-        }
-        __syncthreads();
-    }
-    }
-    if (a.eb) {
-        // Legendre multipoles of P_gE = Re P_gd and P_EE/BB = (P_+ +- P_-)/2 (Sec. 2.4, Eq. relation_pm_EB)
-        const double* o = a.out + (size_t)t * kSlots * a.nb;
-        for (int bb = tid; bb < a.nb; bb += nthr) {
-            double v[8];
-            for (int li = 0; li < 2; ++li)
-                v[li] = a.N[li][0] * o[1 * a.nb + bb] + a.N[li][1] * o[2 * a.nb + bb] + a.N[li][2] * o[3 * a.nb + bb];
-            for (int li = 0; li < 3; ++li) {
-                const double mm = a.M[li][0] * o[7 * a.nb + bb] + a.M[li][1] * o[8 * a.nb + bb] +
-                                  a.M[li][2] * o[9 * a.nb + bb];
-                const double pl = o[(4 + li) * a.nb + bb];
-                v[2 + li] = 0.5 * (pl + mm);
-                v[5 + li] = 0.5 * (pl - mm);
-            }
-            for (int c = 0; c < 8; ++c) {
-                const int i = c * a.nb + bb;
-                const double ref = a.eb_ref ? a.eb_ref[i] : 0.0;
-                const double sg = a.eb_sigma ? a.eb_sigma[i] : 1.0;
-                a.eb[(size_t)t * 8 * a.nb + i] = (float)((v[c] - ref) / sg);
-            }
         }
     }
+#pragma unroll
+    for (int j = 0; j < kTiles; ++j) {
+        const int r = 8 * (warp + 8 * j) + cl;   // accumulator columns are rows of the operator
+        if (r < rows) part[r * kSets + rl] = acc[j][0];
+        if (r + 1 < rows) part[(r + 1) * kSets + rl] = acc[j][1];
+    }
+    cluster.sync();
+    // sums over the cluster, normalisation and outputs: CTA `rank` takes the shells rank, rank + 8, ..
+    double* val = spec;   // [kSets][kSlots] per shell of this CTA, the spectra are no longer read here
+    for (int bl = rank; bl < nbl; bl += kCluster) {
+        const int b = b0 + bl;
+        for (int i = tid; i < sets * a.n_slots; i += blockDim.x) {
+            const int t = i % sets, si = i / sets, sl = a.slot[si];
+            const double* th = a.params + 6 * (size_t)(t0 + t);
+            double s2 = 0.0, v = 0.0;
+            for (int c = 0; c < kCluster; ++c) {
+                s2 += *cluster.map_shared_rank(&s8part[t], c);
+                v += *cluster.map_shared_rank(part + (si * nbl + bl) * kSets + t, c);
+            }
+            const int kind = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
+            const double amp = kind == 0 ? th[1] * th[1] : (kind == 1 ? th[0] * th[1] : th[0] * th[0]);
+            const bool some = a.bin_lo[b] < a.bin_hi[b];
+            v *= amp * (th[2] * th[2] / s2);
+            if (sl == 4) v += th[5] * a.shot_plus;
+            if (!some) v = 0.0;   // a shell without grid k
+            a.out[((size_t)(t0 + t) * kSlots + sl) * a.nb + b] = v;
+            val[t * kSlots + sl] = v;
+        }
+        for (int i = tid; i < sets * kSlots; i += blockDim.x) {
+            const int t = i / kSlots, sl = i % kSlots;
+            if (!((a.slot_mask >> sl) & 1u)) a.out[((size_t)(t0 + t) * kSlots + sl) * a.nb + b] = 0.0;
+        }
+        __syncthreads();
+        if (a.eb && tid < 8 * sets) {
+            // Legendre multipoles of P_gE = Re P_gd and P_EE/BB = (P_+ +- P_-)/2 (Sec. 2.4, Eq. relation_pm_EB)
+            const int t = tid >> 3, c = tid & 7;
+            const double* o = val + t * kSlots;
+            double v;
+            if (c < 2) {
+                v = a.N[c][0] * o[1] + a.N[c][1] * o[2] + a.N[c][2] * o[3];
+            } else {
+                const int li = (c - 2) % 3;
+                const double mm = a.M[li][0] * o[7] + a.M[li][1] * o[8] + a.M[li][2] * o[9];
+                v = 0.5 * (o[4 + li] + (c < 5 ? mm : -mm));
+            }
+            const int i = c * a.nb + b;
+            const double ref = a.eb_ref ? a.eb_ref[i] : 0.0;
+            const double sg = a.eb_sigma ? a.eb_sigma[i] : 1.0;
+            a.eb[(size_t)(t0 + t) * 8 * a.nb + i] = (float)((v - ref) / sg);
+        }
+        __syncthreads();
+    }
+    cluster.sync();   // the partial sums are read until here
 }
 
 // ------------------------------------------------------------------ host tables
@@ -343,13 +409,13 @@ struct lpp_template_s {
     double png_amp = 0.0, png_len2 = 0.0;   // 12 f_NL delta b_IA and (c/H0)^2 / Omega_m
     unsigned slot_mask = (1u << kSlots) - 1u;
     int qx_rows = 0;
-    std::vector<double> kin, s8w, ain, rinv, rfwd, kfwd, qx, bin_w;
+    std::vector<double> kin, lnk, s8w, ain, rinv, rfwd, kfwd, qx, bin_w;
     std::vector<double2> uinv, ufwd, tw;
     std::vector<int> bin_lo, bin_hi;
     SlotDesc slots[kSlots];
     // device
     char* ws = nullptr;
-    size_t ws_need = 0, o_kin, o_s8w, o_ain, o_uinv, o_rinv, o_ufwd, o_rfwd, o_kfwd, o_qx, o_tw, o_lo, o_hi, o_bw;
+    size_t ws_need = 0, o_kin, o_lnk, o_op, o_s8w, o_ain, o_uinv, o_rinv, o_ufwd, o_rfwd, o_kfwd, o_qx, o_tw, o_lo, o_hi, o_bw;
     bool ready = false;
 };
 
@@ -367,6 +433,7 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
     const double r0 = exp(-(kNfft - 1) * delta) / kKmin;
     const double kr0 = kKmin * r0;
     t->kin.resize(kNin);
+    t->lnk.resize(kNin);
     t->s8w.resize(kNin);
     t->ain.resize(kNin);
     t->kfwd.resize(kNin);
@@ -376,6 +443,7 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
         const double wtr = (n == 0 || n == kNin - 1) ? 0.5 * delta : delta;
         const double th = top_hat(8.0 * k);
         t->kin[n] = k;
+        t->lnk[n] = log(kKmin) + n * delta;
         t->s8w[n] = wtr * k * k * k / (2.0 * kPi * kPi) * th * th;
         t->ain[n] = k * k * k * taper_at(n) * pow(k, -kQinv);
         t->kfwd[n] = 4.0 * kPi * pow(k, -kQfwd);
@@ -421,10 +489,10 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
         sd.kind = kinds[sl];
         sd.L = Ls[sl];
         sd.n_terms = 0;
-        auto add = [&](int lp, int cid) {
+        auto add = [&](int lp, double coef) {
             const int j = sd.n_terms++;
             sd.lp[j] = lp;
-            sd.coef[j] = cid;
+            sd.coef[j] = coef;
             sd.qx[j] = rows++;
             std::vector<double> mix(5);
             for (int lpp = 0; lpp <= 8; lpp += 2) mix[lpp / 2] = mixing(mX[sd.kind], sd.L, lp, lpp);
@@ -434,10 +502,12 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
                 t->qx.push_back(v);
             }
         };
-        if (sd.kind == 0) add(0, 0);
-        else if (sd.kind == 1) add(2, 1);
-        else if (sd.kind == 2) { add(0, 2); add(2, 3); add(4, 4); }
-        else add(4, 5);
+        // P_dd^(0) = b^2 P, P_gd^(2) = -A b P / 6, P_+^(0,2,4) = A^2 (2/15, -4/21, 2/35) P,
+        // P_-^(4) = A^2 P / 420 (the powers of A and b in k_template)
+        if (sd.kind == 0) add(0, 1.0);
+        else if (sd.kind == 1) add(2, -1.0 / 6.0);
+        else if (sd.kind == 2) { add(0, 2.0 / 15.0); add(2, -4.0 / 21.0); add(4, 2.0 / 35.0); }
+        else add(4, 1.0 / 420.0);
     }
     t->qx_rows = rows;
     t->bin_lo.resize(n_bins);
@@ -455,6 +525,8 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
     t->o_kin = take(kNin * 8);
+    t->o_lnk = take(kNin * 8);
+    t->o_op = take((size_t)kSlots * n_bins * kNin * 8);
     t->o_s8w = take(kNin * 8);
     t->o_ain = take(kNin * 8);
     t->o_uinv = take(3 * kNfft * 16);
@@ -491,6 +563,7 @@ extern "C" lpp_status lpp_template_set_workspace(lpp_template_t t, void* dev, si
     };
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = put(t->o_kin, t->kin.data(), kNin * 8);
+    if (e == cudaSuccess) e = put(t->o_lnk, t->lnk.data(), kNin * 8);
     if (e == cudaSuccess) e = put(t->o_s8w, t->s8w.data(), kNin * 8);
     if (e == cudaSuccess) e = put(t->o_ain, t->ain.data(), kNin * 8);
     if (e == cudaSuccess) e = put(t->o_uinv, t->uinv.data(), 3 * kNfft * 16);
@@ -503,6 +576,29 @@ extern "C" lpp_status lpp_template_set_workspace(lpp_template_t t, void* dev, si
     if (e == cudaSuccess) e = put(t->o_lo, t->bin_lo.data(), t->nb * 4);
     if (e == cudaSuccess) e = put(t->o_hi, t->bin_hi.data(), t->nb * 4);
     if (e == cudaSuccess) e = put(t->o_bw, t->bin_w.data(), kNin * 8);
+    if (e == cudaSuccess) {
+        // the operator's rows, once per window
+        OperatorArgs a;
+        memset(&a, 0, sizeof(a));
+        a.ain = (const double*)(t->ws + t->o_ain);
+        a.uinv = (const double2*)(t->ws + t->o_uinv);
+        a.rinv = (const double*)(t->ws + t->o_rinv);
+        a.ufwd = (const double2*)(t->ws + t->o_ufwd);
+        a.rfwd = (const double*)(t->ws + t->o_rfwd);
+        a.kfwd = (const double*)(t->ws + t->o_kfwd);
+        a.qx = (const double*)(t->ws + t->o_qx);
+        a.tw = (const double2*)(t->ws + t->o_tw);
+        a.bin_lo = (const int*)(t->ws + t->o_lo);
+        a.bin_hi = (const int*)(t->ws + t->o_hi);
+        a.bin_w = (const double*)(t->ws + t->o_bw);
+        a.nb = t->nb;
+        for (int s = 0; s < kSlots; ++s) a.slots[s] = t->slots[s];
+        a.op = (double*)(t->ws + t->o_op);
+        const size_t smem = (size_t)kNfft * 16 + (size_t)kNfft * 8 + (size_t)kNin * 8;
+        cudaFuncSetAttribute(k_operator, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_operator<<<kSlots * t->nb, 512, smem, st>>>(a);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return LPP_ERR_CUDA;
     t->ready = true;
@@ -548,31 +644,32 @@ static lpp_status convolve(lpp_template_t t, const double* params, int n_templat
     a.params = params;
     a.n_templates = n_templates;
     a.out = out;
+    a.op = (const double*)(t->ws + t->o_op);
     a.kin = (const double*)(t->ws + t->o_kin);
+    a.lnk = (const double*)(t->ws + t->o_lnk);
     a.s8w = (const double*)(t->ws + t->o_s8w);
-    a.ain = (const double*)(t->ws + t->o_ain);
-    a.uinv = (const double2*)(t->ws + t->o_uinv);
-    a.rinv = (const double*)(t->ws + t->o_rinv);
-    a.ufwd = (const double2*)(t->ws + t->o_ufwd);
-    a.rfwd = (const double*)(t->ws + t->o_rfwd);
-    a.kfwd = (const double*)(t->ws + t->o_kfwd);
-    a.qx = (const double*)(t->ws + t->o_qx);
-    a.tw = (const double2*)(t->ws + t->o_tw);
     a.bin_lo = (const int*)(t->ws + t->o_lo);
     a.bin_hi = (const int*)(t->ws + t->o_hi);
-    a.bin_w = (const double*)(t->ws + t->o_bw);
     a.nb = t->nb;
     a.shot_plus = t->shot_plus;
     a.png_amp = t->png_amp;
     a.png_len2 = t->png_len2;
     a.slot_mask = t->slot_mask;
-    for (int s = 0; s < kSlots; ++s) a.slots[s] = t->slots[s];
+    for (int s = 0; s < kSlots; ++s)
+        if ((t->slot_mask >> s) & 1u) a.slot[a.n_slots++] = s;
     a.eb = eb;
     a.eb_ref = eb_ref;
     a.eb_sigma = eb_sigma;
     lpp::eb_matrices(a.N, a.M);
-    const size_t smem = (size_t)kNfft * 16 + (size_t)3 * kNfft * 8 + (size_t)kNin * 8;
+    // shells per cluster: at most kMaxRows rows, and enough clusters for every SM (2 x 19 clusters of 8)
+    const int clusters = (n_templates + kSets - 1) / kSets, ns = a.n_slots > 0 ? a.n_slots : 1;
+    int groups = std::max((t->nb * ns + kMaxRows - 1) / kMaxRows, std::min(t->nb, (38 + clusters - 1) / clusters));
+    a.bins = (t->nb + groups - 1) / groups;
+    while (a.bins > 1 && a.bins * ns > kMaxRows) --a.bins;
+    groups = (t->nb + a.bins - 1) / a.bins;
+    const size_t smem = ((size_t)(t->png_amp != 0.0 ? 3 : 1) * kSets * kSlabPad +
+                         (size_t)std::max(1, a.n_slots * a.bins) * kSets) * sizeof(double);
     cudaFuncSetAttribute(k_template, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_template<<<n_templates, 512, smem, (cudaStream_t)stream>>>(a);
+    k_template<<<dim3(clusters * kCluster, groups), 256, smem, (cudaStream_t)stream>>>(a);
     return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
 }
