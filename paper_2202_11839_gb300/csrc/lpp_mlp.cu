@@ -1,12 +1,14 @@
 // Template surrogate network: 6 -> [256, GELU] x 4 -> 320, BF16 operands, FP32 accumulation.
 //
-// Every matrix product C = A B^T (A [M x K], B [N x K], both BF16 with K contiguous) runs on
-// the tensor cores (mma.m16n8k16, BF16 in, FP32 accumulate) in 64 x 64 CTA tiles with fused
-// epilogues: bias + GELU for hidden layers (the BF16 activation and, when training, its
-// transpose), bias for the output, plain FP32 for weight gradients, and the GELU derivative
-// for back-propagated gradients.  Adam keeps FP32 master weights and refreshes their BF16
-// copies (and transposes) after every step.  The training loop is native: one call runs all
-// steps of a schedule of minibatch indices.
+// Every matrix product runs on the tensor cores (mma.m16n8k16, BF16 in, FP32 accumulate, the
+// reduction dimension in ascending steps of 16).  The network is a chain of small products:
+// a layer of a 256-row minibatch is 34 MFLOP, less than a microsecond of one launch, so the
+// chain is fused by rows.  A CTA carries its rows through all layers (and, when training, back)
+// with the activations in shared memory while the weight matrices stream through a ring of
+// cp.async stages; a second kernel forms every layer's weight gradient and applies Adam in the
+// epilogue.  Adam keeps FP32 master weights and refreshes their BF16 copies (and transposes)
+// after every step.  The training loop is native: one call runs all steps of a schedule of
+// minibatch indices.
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -26,179 +28,247 @@ constexpr int kOut[kLayers] = {256, 256, 256, 256, 320};
 constexpr int kNout = 320;
 constexpr int kNin = 6;
 
-enum Epi { EPI_HIDDEN = 0, EPI_OUT = 1, EPI_DW = 2, EPI_DA_GELU = 3 };
-
-struct GemmArgs {
-    const bf16* A;
-    int lda;
-    const bf16* B;
-    int ldb;
-    int M, N, K;
-    int epi;
-    const float* bias;
-    float* z;          // hidden: pre-activation; out: output; dW: gradient
-    int ldz;
-    bf16* a16;         // hidden: BF16 GELU(z); da: BF16 gradient
-    int ld16;
-    bf16* a16t;        // transposed BF16 copy (optional)
-    int ld16t;
-    const float* zprev;   // da: pre-activation of the layer below
-    int ldzp;
-    float* g32;           // da: FP32 gradient
-    int ldg;
-};
-
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z) {
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
 }
 
-constexpr int BM = 64, BN = 64, BK = 32, LDS = BK + 8;
+__device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void cp16(void* smem_dst, const void* gmem_src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-__global__ void __launch_bounds__(128) k_gemm(GemmArgs a) {
-    __shared__ __align__(16) bf16 As[BM][LDS];
-    __shared__ __align__(16) bf16 Bs[BN][LDS];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp >> 1, wn = warp & 1;
-    const int g = lane >> 2, t = lane & 3;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
-    for (int k0 = 0; k0 < a.K; k0 += BK) {
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int c = tid + i * 128;   // 256 chunks of 8 BF16 per tile
-            const int row = c >> 2, col = (c & 3) * 8;
-            uint4 va = make_uint4(0, 0, 0, 0), vb = make_uint4(0, 0, 0, 0);
-            if (m0 + row < a.M && k0 + col < a.K)
-                va = *reinterpret_cast<const uint4*>(a.A + (size_t)(m0 + row) * a.lda + k0 + col);
-            if (n0 + row < a.N && k0 + col < a.K)
-                vb = *reinterpret_cast<const uint4*>(a.B + (size_t)(n0 + row) * a.ldb + k0 + col);
-            *reinterpret_cast<uint4*>(&As[row][col]) = va;
-            *reinterpret_cast<uint4*>(&Bs[row][col]) = vb;
+// ---- weight streaming
+// The passes of a row chain: the forward layers 0..4, then (training) the activation gradients
+// through layers 4..1.  Pass p multiplies by w[p] [rows][K], K contiguous, in chunks of 32 K
+// columns (16 for the padded input layer).
+struct Passes {
+    const bf16* w[2 * kLayers - 1];
+};
+__host__ __device__ constexpr int pass_rows(int p) { return p == kLayers - 1 ? kNout : 256; }
+__host__ __device__ constexpr int pass_k(int p) { return p == 0 ? 16 : (p == kLayers ? kNout : 256); }
+
+constexpr int kRowThreads = 256;       // 8 warps: warp w owns the output columns 8 (w NT) ..
+constexpr int kChunkLd = 40;           // BF16 per chunk row: 32 and padding (conflict-free fragments)
+constexpr int kStageElems = kNout * kChunkLd;
+
+// A ring of weight chunks in shared memory: load(c) starts the copy of the c-th chunk of the whole
+// chain (the copies run ahead of the layers).
+template <int kStages>
+struct WeightRing {
+    bf16* ring;
+    int pass = 0, k = 0, n_pass, put = 0, got = 0;
+    __device__ __forceinline__ void load(const Passes& ps) {
+        if (pass < n_pass) {
+            const int rows = pass_rows(pass), K = pass_k(pass);
+            const bf16* w = ps.w[pass];
+            bf16* dst = ring + (put % kStages) * kStageElems;
+            if (K >= 32) {
+                for (int i = threadIdx.x; i < rows * 4; i += kRowThreads)
+                    cp16(dst + (i >> 2) * kChunkLd + (i & 3) * 8, w + (size_t)(i >> 2) * K + k + (i & 3) * 8);
+            } else {
+                for (int i = threadIdx.x; i < rows * 2; i += kRowThreads)
+                    cp16(dst + (i >> 1) * kChunkLd + (i & 1) * 8, w + (size_t)(i >> 1) * K + (i & 1) * 8);
+            }
+            k += 32;
+            if (k >= K) { k = 0; ++pass; }
         }
+        cp_commit();   // an empty group past the end keeps the count of groups in flight
+        ++put;
+    }
+    // The next chunk, once it has landed and every warp has left the chunk before it; starts the
+    // copy that replaces that one.
+    __device__ __forceinline__ const bf16* next(const Passes& ps) {
+        cp_wait<kStages - 2>();
         __syncthreads();
+        load(ps);
+        return ring + (got++ % kStages) * kStageElems;
+    }
+};
+
+// acc[mt][j] += act[16 MT rows][K] . w[columns][K]^T for the warp's NT tiles of 8 columns.
+template <int MT, int NT, int K, int LDA, int ST>
+__device__ __forceinline__ void row_product(WeightRing<ST>& ring, const Passes& ps, const bf16* act,
+                                            float (&acc)[MT][NT][4]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
 #pragma unroll
-        for (int kk = 0; kk < BK; kk += 16) {
-            uint32_t af[2][4], bfr[4][2];
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-            for (int mi = 0; mi < 2; ++mi) {
-                const int r = wm * 32 + mi * 16 + g;
-                af[mi][0] = *reinterpret_cast<const uint32_t*>(&As[r][kk + 2 * t]);
-                af[mi][1] = *reinterpret_cast<const uint32_t*>(&As[r + 8][kk + 2 * t]);
-                af[mi][2] = *reinterpret_cast<const uint32_t*>(&As[r][kk + 2 * t + 8]);
-                af[mi][3] = *reinterpret_cast<const uint32_t*>(&As[r + 8][kk + 2 * t + 8]);
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[mt][j][r] = 0.f;
+    for (int k0 = 0; k0 < K; k0 += 32) {
+        const bf16* w = ring.next(ps);
+#pragma unroll
+        for (int kk = 0; kk < (K < 32 ? K : 32); kk += 16) {
+            uint32_t a[MT][4];
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                const bf16* ap = act + (mt * 16 + g) * LDA + k0 + kk + 2 * t;
+                a[mt][0] = *reinterpret_cast<const uint32_t*>(ap);
+                a[mt][1] = *reinterpret_cast<const uint32_t*>(ap + 8 * LDA);
+                a[mt][2] = *reinterpret_cast<const uint32_t*>(ap + 8);
+                a[mt][3] = *reinterpret_cast<const uint32_t*>(ap + 8 * LDA + 8);
             }
 #pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int n = wn * 32 + ni * 8 + g;
-                bfr[ni][0] = *reinterpret_cast<const uint32_t*>(&Bs[n][kk + 2 * t]);
-                bfr[ni][1] = *reinterpret_cast<const uint32_t*>(&Bs[n][kk + 2 * t + 8]);
+            for (int j = 0; j < NT; ++j) {
+                const bf16* bp = w + (8 * (warp * NT + j) + g) * kChunkLd + kk + 2 * t;
+                const uint32_t b0 = *reinterpret_cast<const uint32_t*>(bp);
+                const uint32_t b1 = *reinterpret_cast<const uint32_t*>(bp + 8);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt][j], a[mt], b0, b1);
             }
-#pragma unroll
-            for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-                for (int ni = 0; ni < 4; ++ni)
-                    asm volatile(
-                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-                        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-                        : "+f"(acc[mi][ni][0]), "+f"(acc[mi][ni][1]), "+f"(acc[mi][ni][2]), "+f"(acc[mi][ni][3])
-                        : "r"(af[mi][0]), "r"(af[mi][1]), "r"(af[mi][2]), "r"(af[mi][3]), "r"(bfr[ni][0]),
-                          "r"(bfr[ni][1]));
         }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-        for (int ni = 0; ni < 4; ++ni)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int row = m0 + wm * 32 + mi * 16 + g + (r >= 2 ? 8 : 0);
-                const int col = n0 + wn * 32 + ni * 8 + 2 * t + (r & 1);
-                if (row >= a.M || col >= a.N) continue;
-                const float v = acc[mi][ni][r];
-                if (a.epi == EPI_HIDDEN) {
-                    const float z = v + a.bias[col];
-                    a.z[(size_t)row * a.ldz + col] = z;
-                    const bf16 h = __float2bfloat16_rn(gelu(z));
-                    a.a16[(size_t)row * a.ld16 + col] = h;
-                    if (a.a16t) a.a16t[(size_t)col * a.ld16t + row] = h;
-                } else if (a.epi == EPI_OUT) {
-                    a.z[(size_t)row * a.ldz + col] = v + a.bias[col];
-                } else if (a.epi == EPI_DW) {
-                    a.z[(size_t)row * a.ldz + col] = v;
-                } else {
-                    const float gv = v * gelu_grad(a.zprev[(size_t)row * a.ldzp + col]);
-                    a.g32[(size_t)row * a.ldg + col] = gv;
-                    const bf16 h = __float2bfloat16_rn(gv);
-                    a.a16[(size_t)row * a.ld16 + col] = h;
-                    a.a16t[(size_t)col * a.ld16t + row] = h;
-                }
-            }
-}
-
-cudaError_t gemm(const GemmArgs& a, cudaStream_t st) {
-    dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM);
-    k_gemm<<<grid, 128, 0, st>>>(a);
-    return cudaGetLastError();
-}
-
-// inputs x [m][6] FP32 -> BF16 [m][16] (zero padded) and, when training, its transpose [16][ld]
-__global__ void k_input(const float* __restrict__ x, const int* __restrict__ idx, int m, bf16* a0, bf16* a0t,
-                        int ldt) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m * 16; i += gridDim.x * blockDim.x) {
-        const int r = i / 16, c = i % 16;
-        const int src = idx ? idx[r] : r;
-        const float v = c < kNin ? x[(size_t)src * kNin + c] : 0.f;
-        const bf16 h = __float2bfloat16_rn(v);
-        a0[i] = h;
-        if (a0t) a0t[(size_t)c * ldt + r] = h;
     }
 }
 
-// dL/d out = 2 (out - y) / (m * 320); loss sum of squares into loss (FP64)
-__global__ void k_loss(const float* __restrict__ out, const float* __restrict__ y, const int* __restrict__ idx, int m,
-                       float* g32, bf16* g16, bf16* g16t, int ldt, double* loss) {
-    double part = 0.0;
-    const float sc = 2.0f / (float)(m * kNout);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m * kNout; i += gridDim.x * blockDim.x) {
-        const int r = i / kNout, c = i % kNout;
-        const int src = idx ? idx[r] : r;
-        const float d = out[i] - y[(size_t)src * kNout + c];
-        part += (double)d * d;
-        const float gv = sc * d;
-        g32[i] = gv;
-        const bf16 h = __float2bfloat16_rn(gv);
-        g16[i] = h;
-        g16t[(size_t)c * ldt + r] = h;
-    }
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-    if ((threadIdx.x & 31) == 0 && part != 0.0) atomicAdd(loss, part / (double)(m * kNout));
+// Ring stages and BF16 per activation row of the training chain (rows of up to 320 gradients) and of
+// the prediction (256 activations); padded for conflict-free fragments.  Two prediction CTAs of 32
+// rows share an SM.
+constexpr int kTrainStages = 4, kActLd = 328;
+constexpr size_t kTrainSmem = ((size_t)kTrainStages * kStageElems + (size_t)2 * 16 * kActLd) * sizeof(bf16);
+constexpr int kPredLd = 264;
+__host__ __device__ constexpr int pred_stages(int mt) { return mt == 1 ? 4 : 3; }
+__host__ __device__ constexpr size_t pred_smem(int mt) {
+    return ((size_t)pred_stages(mt) * kStageElems + (size_t)2 * mt * 16 * kPredLd) * sizeof(bf16);
 }
 
-// db[n] = sum over rows of g[m][n]
-// db[c] = sum_r g[r][c]: 32 columns per CTA (a warp reads 32 consecutive columns of a row),
-// eight warps each over every eighth row, then the eight partial sums in a fixed order
-__global__ void __launch_bounds__(256) k_bias_grad(const float* __restrict__ g, int m, int n, float* db) {
-    __shared__ float part[8][33];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + lane;
-    float s = 0.f;
-    if (c < n)
-        for (int r = w; r < m; r += 8) s += g[(size_t)r * n + c];
-    part[w][lane] = s;
+// [16 rows][cols] of a shared activation tile -> global transpose [cols][ld] at column r0: 16 rows
+// of one column are 32 contiguous bytes.
+__device__ __forceinline__ void store_transposed(const bf16* act, int cols, bf16* dst, int ld, int r0) {
+    for (int c = threadIdx.x; c < cols; c += kRowThreads) {
+        __align__(16) bf16 v[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] = act[r * kActLd + c];
+        uint4* d = reinterpret_cast<uint4*>(dst + (size_t)c * ld + r0);
+        d[0] = reinterpret_cast<const uint4*>(v)[0];
+        d[1] = reinterpret_cast<const uint4*>(v)[1];
+    }
+}
+
+struct TrainRowArgs {
+    Passes ps;
+    const float* bias[kLayers];
+    const float* x;
+    const float* y;
+    const int* idx;            // minibatch rows of x, y
+    int batch;
+    bf16* actt[kLayers];       // layer inputs, transposed [kInPad][batch]
+    bf16* gt[kLayers];         // gradients of the pre-activations, transposed [kOut][batch]
+    float* g32[kLayers];       // and FP32 [batch][kOut]
+    double* loss;
+};
+
+// One training step's row chain: 16 rows of the minibatch per CTA through the forward layers, the
+// loss gradient and the activation gradients, down to every layer's input and pre-activation
+// gradient (transposed, for the weight gradients).  The pre-activations stay in registers: the
+// backward products place their outputs on the same threads.
+//
+// What bounds it: 1.1 MB of weights per CTA through the ring (L2 to shared memory) and the
+// latency of nine dependent products.  A step at batch 256 (both kernels): 199 -> 64 us against
+// one launch per product, bias gradient, loss and update (22 launches).
+__global__ void __launch_bounds__(kRowThreads, 1) k_train_rows(const __grid_constant__ TrainRowArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    WeightRing<kTrainStages> ring;
+    ring.ring = reinterpret_cast<bf16*>(smem_raw);
+    ring.n_pass = 2 * kLayers - 1;
+    bf16* buf[2];
+    buf[0] = ring.ring + kTrainStages * kStageElems;
+    buf[1] = buf[0] + 16 * kActLd;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int r0 = blockIdx.x * 16;
+    for (int c = 0; c < kTrainStages - 1; ++c) ring.load(a.ps);
+    {   // inputs: BF16 [16][16], zero padded
+        const int r = tid >> 4, c = tid & 15;
+        const float v = c < kNin ? a.x[(size_t)a.idx[r0 + r] * kNin + c] : 0.f;
+        buf[0][r * kActLd + c] = __float2bfloat16_rn(v);
+    }
     __syncthreads();
-    if (w == 0 && c < n) {
-        float t = 0.f;
+    store_transposed(buf[0], pass_k(0), a.actt[0], a.batch, r0);
+    float z[kLayers - 1][4][4];
+    int cur = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) t += part[k][lane];
-        db[c] = t;
+    for (int l = 0; l < kLayers - 1; ++l) {
+        float acc[1][4][4];
+        if (l == 0) row_product<1, 4, 16, kActLd>(ring, a.ps, buf[cur], acc);
+        else row_product<1, 4, 256, kActLd>(ring, a.ps, buf[cur], acc);
+        bf16* nx = buf[cur ^ 1];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = 8 * (warp * 4 + j) + 2 * t;
+            const float2 b = *reinterpret_cast<const float2*>(a.bias[l] + c);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) z[l][j][r] = acc[0][j][r] + ((r & 1) ? b.y : b.x);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                *reinterpret_cast<__nv_bfloat162*>(nx + (g + 8 * h) * kActLd + c) =
+                    __nv_bfloat162(__float2bfloat16_rn(gelu(z[l][j][2 * h])), __float2bfloat16_rn(gelu(z[l][j][2 * h + 1])));
+        }
+        cur ^= 1;
+        __syncthreads();
+        store_transposed(buf[cur], 256, a.actt[l + 1], a.batch, r0);
+    }
+    // output layer, loss and its gradient 2 (out - y) / (batch * 320)
+    {
+        float acc[1][5][4];
+        row_product<1, 5, 256, kActLd>(ring, a.ps, buf[cur], acc);
+        const float sc = 2.0f / (float)(a.batch * kNout);
+        double part = 0.0;
+        bf16* nx = buf[cur ^ 1];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const int c = 8 * (warp * 5 + j) + 2 * t;
+            const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + c);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = r0 + g + 8 * h;
+                const float2 yv = *reinterpret_cast<const float2*>(a.y + (size_t)a.idx[r] * kNout + c);
+                const float d0 = (acc[0][j][2 * h] + b.x) - yv.x, d1 = (acc[0][j][2 * h + 1] + b.y) - yv.y;
+                part += (double)d0 * d0 + (double)d1 * d1;
+                const float2 gv = make_float2(sc * d0, sc * d1);
+                *reinterpret_cast<float2*>(a.g32[kLayers - 1] + (size_t)r * kNout + c) = gv;
+                *reinterpret_cast<__nv_bfloat162*>(nx + (g + 8 * h) * kActLd + c) =
+                    __nv_bfloat162(__float2bfloat16_rn(gv.x), __float2bfloat16_rn(gv.y));
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
+        if (lane == 0 && part != 0.0) atomicAdd(a.loss, part / (double)(a.batch * kNout));
+        cur ^= 1;
+        __syncthreads();
+        store_transposed(buf[cur], kNout, a.gt[kLayers - 1], a.batch, r0);
+    }
+    // g_{l-1} = (g_l W_l) * GELU'(z_{l-1})
+#pragma unroll
+    for (int l = kLayers - 1; l > 0; --l) {
+        float acc[1][4][4];
+        if (l == kLayers - 1) row_product<1, 4, kNout, kActLd>(ring, a.ps, buf[cur], acc);
+        else row_product<1, 4, 256, kActLd>(ring, a.ps, buf[cur], acc);
+        bf16* nx = buf[cur ^ 1];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = 8 * (warp * 4 + j) + 2 * t;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 gv = make_float2(acc[0][j][2 * h] * gelu_grad(z[l - 1][j][2 * h]),
+                                              acc[0][j][2 * h + 1] * gelu_grad(z[l - 1][j][2 * h + 1]));
+                *reinterpret_cast<float2*>(a.g32[l - 1] + (size_t)(r0 + g + 8 * h) * 256 + c) = gv;
+                *reinterpret_cast<__nv_bfloat162*>(nx + (g + 8 * h) * kActLd + c) =
+                    __nv_bfloat162(__float2bfloat16_rn(gv.x), __float2bfloat16_rn(gv.y));
+            }
+        }
+        cur ^= 1;
+        __syncthreads();
+        store_transposed(buf[cur], 256, a.gt[l - 1], a.batch, r0);
     }
 }
 
@@ -212,39 +282,129 @@ struct AdamArgs {
     float lr, b1, b2, eps, bc1, bc2;
 };
 
-__global__ void k_adam(AdamArgs a) {
-    const int layer = blockIdx.y;
-    const AdamLayer& L = a.L[layer];
-    const int nw = L.out * L.inp;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + L.out; i += gridDim.x * blockDim.x) {
-        float *p, *m, *v;
-        float gr;
-        if (i < nw) {
-            const int c = i % L.inp;
-            if (c >= L.in) continue;   // padded input columns stay zero
-            p = L.w + i;
-            m = L.mw + i;
-            v = L.vw + i;
-            gr = L.dw[i];
-        } else {
-            const int j = i - nw;
-            p = L.b + j;
-            m = L.mb + j;
-            v = L.vb + j;
-            gr = L.db[j];
+// The weight and bias gradients of a step and their Adam update.
+struct TrainWeightArgs {
+    AdamArgs adam;
+    const bf16* actt[kLayers];   // layer inputs, transposed [kInPad][batch]
+    const bf16* gt[kLayers];     // pre-activation gradients, transposed [kOut][batch]
+    const float* g32[kLayers];   // and FP32 [batch][kOut]
+    int batch;
+    int update;                  // 0: store the gradients (AdamLayer::dw, db) and change nothing else
+};
+
+// One Adam step of a parameter: the new value.
+__device__ __forceinline__ float adam_step(const AdamArgs& a, float p, float& m, float& v, float gr) {
+    const float mm = a.b1 * m + (1.f - a.b1) * gr;
+    const float vv = a.b2 * v + (1.f - a.b2) * gr * gr;
+    m = mm;
+    v = vv;
+    const float upd = a.lr * (mm / a.bc1) / (sqrtf(vv / a.bc2) + a.eps);
+    return p - upd;
+}
+
+// dW_l = g_l^T a_l in tiles of 32 outputs x 64 inputs per CTA (144 CTAs, one wave) with Adam in the
+// epilogue, and the bias gradients, 32 columns per CTA: a row's columns by one warp, eight
+// partial sums over the rows r = w (mod 8) added in a fixed order.
+constexpr int kTileM = 32, kTileN = 64, kPanel = 256, kPanelLd = kPanel + 8;
+constexpr int kWeightTiles = 8 + 3 * 8 * 4 + 10 * 4;    // layer 0, layers 1..3, layer 4
+constexpr int kBiasTiles = 4 * 8 + 10;
+constexpr size_t kWeightSmem = (size_t)(kTileM + kTileN) * kPanelLd * sizeof(bf16);
+
+__global__ void __launch_bounds__(128) k_train_weights(const __grid_constant__ TrainWeightArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int b = blockIdx.x;
+    if (b >= kWeightTiles) {
+        b -= kWeightTiles;
+        const int l = b < 32 ? b >> 3 : kLayers - 1;
+        const int c = (b - 8 * l) * 32 + lane, n = kOut[0] + (l == kLayers - 1 ? kNout - 256 : 0);
+        float* part = reinterpret_cast<float*>(smem_raw);   // [8][33]
+        for (int w = warp; w < 8; w += 4) {
+            float s = 0.f;
+#pragma unroll 8
+            for (int r = w; r < a.batch; r += 8) s += a.g32[l][(size_t)r * n + c];
+            part[w * 33 + lane] = s;
         }
-        const float mm = a.b1 * *m + (1.f - a.b1) * gr;
-        const float vv = a.b2 * *v + (1.f - a.b2) * gr * gr;
-        *m = mm;
-        *v = vv;
-        const float upd = a.lr * (mm / a.bc1) / (sqrtf(vv / a.bc2) + a.eps);
-        const float nwv = *p - upd;
-        *p = nwv;
-        if (i < nw) {
-            const int r = i / L.inp, c = i % L.inp;
-            const bf16 h = __float2bfloat16_rn(nwv);
-            L.w16[i] = h;
-            L.w16t[(size_t)c * L.out + r] = h;
+        __syncthreads();
+        if (warp == 0) {
+            float gr = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) gr += part[k * 33 + lane];
+            const AdamLayer& L = a.adam.L[l];
+            if (a.update) L.b[c] = adam_step(a.adam, L.b[c], L.mb[c], L.vb[c], gr);
+            else L.db[c] = gr;
+        }
+        return;
+    }
+    int l = 0, tn = 1;
+    if (b >= 8) {
+        b -= 8;
+        l = b < 96 ? 1 + (b >> 5) : kLayers - 1;
+        b -= 32 * (l - 1);
+        tn = 4;
+    }
+    const int m0 = (b / tn) * kTileM, n0 = (b % tn) * kTileN;
+    const AdamLayer& L = a.adam.L[l];
+    const int inp = L.inp, rows_b = min(kTileN, inp - n0);
+    bf16* As = reinterpret_cast<bf16*>(smem_raw);
+    bf16* Bs = As + kTileM * kPanelLd;
+    const int wm = warp >> 1, wn = warp & 1, g = lane >> 2, t = lane & 3;
+    float acc[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[j][r] = 0.f;
+    for (int k0 = 0; k0 < a.batch; k0 += kPanel) {
+        const int kp = min(kPanel, a.batch - k0);   // a multiple of 32
+        const int seg = kp / 8;
+        __syncthreads();
+        for (int i = tid; i < (kTileM + rows_b) * seg; i += 128) {
+            const int r = i / seg, c = (i - r * seg) * 8;
+            if (r < kTileM) cp16(As + r * kPanelLd + c, a.gt[l] + (size_t)(m0 + r) * a.batch + k0 + c);
+            else cp16(Bs + (r - kTileM) * kPanelLd + c, a.actt[l] + (size_t)(n0 + r - kTileM) * a.batch + k0 + c);
+        }
+        cp_commit();
+        cp_wait<0>();
+        __syncthreads();
+        for (int k = 0; k < kp; k += 16) {
+            const bf16* ap = As + (wm * 16 + g) * kPanelLd + k + 2 * t;
+            uint32_t af[4];
+            af[0] = *reinterpret_cast<const uint32_t*>(ap);
+            af[1] = *reinterpret_cast<const uint32_t*>(ap + 8 * kPanelLd);
+            af[2] = *reinterpret_cast<const uint32_t*>(ap + 8);
+            af[3] = *reinterpret_cast<const uint32_t*>(ap + 8 * kPanelLd + 8);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (wn * 32 + 8 * j >= rows_b) break;   // warp-uniform (the input layer has 16 columns)
+                const bf16* bp = Bs + (wn * 32 + 8 * j + g) * kPanelLd + k + 2 * t;
+                mma_bf16(acc[j], af, *reinterpret_cast<const uint32_t*>(bp), *reinterpret_cast<const uint32_t*>(bp + 8));
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (wn * 32 + 8 * j >= rows_b) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = m0 + wm * 16 + g + 8 * h, col = n0 + wn * 32 + 8 * j + 2 * t;
+            const size_t i = (size_t)row * inp + col;
+            if (!a.update) {
+                *reinterpret_cast<float2*>(L.dw + i) = make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
+                continue;
+            }
+            if (col >= L.in) continue;   // padded input columns stay zero (L.in is even)
+            float2 p = *reinterpret_cast<const float2*>(L.w + i);
+            float2 m = *reinterpret_cast<const float2*>(L.mw + i);
+            float2 v = *reinterpret_cast<const float2*>(L.vw + i);
+            p.x = adam_step(a.adam, p.x, m.x, v.x, acc[j][2 * h]);
+            p.y = adam_step(a.adam, p.y, m.y, v.y, acc[j][2 * h + 1]);
+            *reinterpret_cast<float2*>(L.w + i) = p;
+            *reinterpret_cast<float2*>(L.mw + i) = m;
+            *reinterpret_cast<float2*>(L.vw + i) = v;
+            const __nv_bfloat162 q(__float2bfloat16_rn(p.x), __float2bfloat16_rn(p.y));
+            *reinterpret_cast<__nv_bfloat162*>(L.w16 + i) = q;
+            L.w16t[(size_t)col * L.out + row] = q.x;
+            L.w16t[(size_t)(col + 1) * L.out + row] = q.y;
         }
     }
 }
@@ -264,6 +424,7 @@ __global__ void k_refresh(AdamArgs a) {
 
 // parameters -> network inputs and network outputs -> curves (see lpp_surrogate_map)
 constexpr int kMaxNodes = 8;
+constexpr int kBadExponent = 1 << 20;   // a row or column with an infinity or NaN
 struct MapArgs {
     float scale[kNin], shift[kNin];   // x_c = theta_c * scale_c + shift_c (0, 0 when not fed)
     double dscale[kNin], dshift[kNin];
@@ -275,10 +436,11 @@ struct MapArgs {
     const double* base;               // [nodes^2][320] or null
     int nodes, base_in[2];
     double N[2][3], M[3][3];          // native moments -> derived multipoles
-    // the decoding's copy of base as float pairs (hi + lo = base to 2^-48), and the Lobatto
-    // nodes with the Lagrange normalisations 1 / prod_{j != i} (x_i - x_j), for k_decode
-    const float* base_hi;
-    const float* base_lo;
+    // the decoding's copy of base: kDigits signed base-256 digits per value relative to 2^column
+    // exponent (digit_fragments), the exponents, and the Lobatto nodes with the Lagrange
+    // normalisations 1 / prod_{j != i} (x_i - x_j)
+    const uint4* digits;
+    const int* exponent;    // [kNout]
     double xs[kMaxNodes], cw[kMaxNodes];
 };
 
@@ -311,14 +473,63 @@ __device__ __forceinline__ void lobatto_basis_fast(double x, const MapArgs& a, d
     }
 }
 
-// base -> (hi, lo) float pairs, hi = rn(b), lo = rn(b - hi)
-__global__ void k_split_base(const double* __restrict__ base, int count, float* __restrict__ hi,
-                             float* __restrict__ lo) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-        const double b = base[i];
-        const float h = (float)b;
-        hi[i] = h;
-        lo[i] = (float)(b - (double)h);
+// ---- exact products of the baseline on the tensor cores
+// The baseline sum_q w_q base_qj cancels: it needs more than the FP32 digits of its terms, and
+// GB300 runs FP64 at 1/64 of the FP32 rate.  Both factors are therefore written as kDigits signed
+// base-256 digits of a 48-bit fixed-point number (weights relative to the row's largest, base
+// values to the column's largest).  A digit is an integer of at most 128, exact in BF16; a sum of
+// 64 products of digits is an integer below 2^20, and one of up to six such sums below 2^23,
+// exact in the FP32 accumulators.  Products of digits i and j have weight 2^(-8 (i + j)): the sums
+// of equal i + j <= 6 share an accumulator (26 of the 36 products; the rest are below 2^-48 of
+// the largest term), and the seven accumulators are added in float pairs.
+constexpr int kDigits = 6, kOrders = 7;
+constexpr int kBaseKsteps = kMaxNodes * kMaxNodes / 16;            // 16 baseline terms per mma
+constexpr int kDigitWords = kDigits * (kNout / 8) * (kBaseKsteps / 2) * 32;   // uint4 of digit fragments
+
+// x in [-1, 1] -> its kDigits digits d_i: x = sum_i d_i 2^(-8 i - 7) to 2^-48
+__device__ __forceinline__ void fixed_digits(double x, int* d) {
+    long long v = llrint(x * 140737488355328.0);   // 2^47
+#pragma unroll
+    for (int i = kDigits - 1; i > 0; --i) {
+        d[i] = (int)((v + 128) & 255) - 128;
+        v = (v - d[i]) >> 8;
+    }
+    d[0] = (int)v;
+}
+
+// base -> digits in the order in which a lane reads its operand fragments: word
+// ((digit 40 + column tile) 2 + k half) 32 + lane holds terms q = 32 half + {2t, 2t+1, 2t+8, 2t+9} + {0, 16}
+// of column 8 tile + g (g = lane / 4, t = lane % 4); one warp per column.
+__global__ void k_base_digits(const double* __restrict__ base, int nn, uint4* __restrict__ digits,
+                              int* __restrict__ exponent) {
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (j >= kNout) return;
+    double v[2], m = 0.0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int q = lane + 32 * h;
+        v[h] = q < nn ? base[(size_t)q * kNout + j] : 0.0;
+        m = fmax(m, fabs(v[h]));
+        if (!(fabs(v[h]) < INFINITY)) m = INFINITY;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const bool finite = m < INFINITY;
+    int e = 0;
+    if (finite && m > 0.0) frexp(m, &e);   // |v| <= 2^e
+    if (lane == 0) exponent[j] = finite ? e : kBadExponent;
+    bf16* out = reinterpret_cast<bf16*>(digits);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        int d[kDigits];
+        fixed_digits(finite ? ldexp(v[h], -e) : 0.0, d);
+        // term q = 32 h + lane: k step of 16, position in it -> fragment register and half
+        const int s16 = lane >> 4, p = lane & 15, t = (p & 7) >> 1;
+        const int word = 2 * s16 + (p >> 3);   // of the uint4: {b0, b1} of two k steps
+        for (int i = 0; i < kDigits; ++i) {
+            const size_t w = ((size_t)(i * (kNout / 8) + j / 8) * 2 + h) * 32 + (j & 7) * 4 + t;
+            out[w * 8 + word * 2 + (p & 1)] = __float2bfloat16_rn((float)d[i]);
+        }
     }
 }
 
@@ -335,76 +546,281 @@ __device__ double baseline(const MapArgs& a, const double* t, int j) {
     return u;
 }
 
-// network outputs y [m][320] -> standardised curves (pre_c (baseline + sd y) + theta_5 s - ref) / sigma.
-// One CTA of kNout threads per kDecodeRows parameter rows at a time: the rows' Lagrange weights
-// l_a(x_p) l_b(x_q) are formed once in FP64 in shared memory and split into float pairs; thread
-// j loads its base column once for the rows and sums each row's baseline output in float-float
-// arithmetic (error-free products and sums, Dekker and Knuth): the FP64 sum of baseline() to
-// about 2^-44 relative, on the FP32 pipes (GB300 runs FP64 at a small fraction of the FP32 rate).
-constexpr int kDecodeRows = 4;
-__global__ void __launch_bounds__(kNout) k_decode(const double* __restrict__ theta, int m, const float* __restrict__ y,
-                                                  float* __restrict__ out, MapArgs a) {
-    constexpr int nb = kNout / 8, R = kDecodeRows;
-    __shared__ double la[R][kMaxNodes], lb[R][kMaxNodes];
-    __shared__ float whi[R][kMaxNodes * kMaxNodes], wlo[R][kMaxNodes * kMaxNodes];
-    const int j = threadIdx.x;
-    const int nn = a.base ? a.nodes * a.nodes : 0;
-    for (int r0 = blockIdx.x * R; r0 < m; r0 += gridDim.x * R) {
-        const int nr = m - r0 < R ? m - r0 : R;
-        if (a.base) {
-            if (j < 2 * R && (j >> 1) < nr) {
-                const int rr = j >> 1, c = a.base_in[j & 1];
-                const double* t = theta + (size_t)(r0 + rr) * kNin;
-                lobatto_basis_fast(t[c] * a.dscale[c] + a.dshift[c], a, (j & 1) ? lb[rr] : la[rr]);
+// ---- float pairs (hi + lo, |lo| <= ulp(hi) / 2): sums and products to about 2^-46
+struct fpair {
+    float hi, lo;
+};
+__device__ __forceinline__ fpair two_sum(float a, float b) {   // exact (Knuth)
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
+}
+__device__ __forceinline__ fpair fast_two_sum(float a, float b) {   // exact for |a| >= |b| (Dekker)
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ fpair pair_of(double v) {
+    const float h = (float)v;
+    return {h, (float)(v - (double)h)};
+}
+__device__ __forceinline__ fpair pair_add(fpair a, fpair b) {
+    fpair s = two_sum(a.hi, b.hi);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+}
+__device__ __forceinline__ fpair pair_mul(fpair a, fpair b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    float e = fmaf(a.hi, b.hi, -p);
+    e = fmaf(a.hi, b.lo, e);
+    e = fmaf(a.lo, b.hi, e);
+    return fast_two_sum(p, e);
+}
+__device__ __forceinline__ fpair pair_mul(fpair a, float b) {
+    const float p = __fmul_rn(a.hi, b);
+    return fast_two_sum(p, fmaf(a.lo, b, fmaf(a.hi, b, -p)));
+}
+__device__ __forceinline__ float exp2i(int e) {   // 2^e for -126 <= e <= 127
+    return __int_as_float((e + 127) << 23);
+}
+
+__device__ __forceinline__ float scale2(float v, int e) {   // v 2^e
+    return e > -100 && e < 100 ? v * exp2i(e) : ldexpf(v, e);
+}
+
+struct PredictArgs {
+    Passes ps;
+    const float* bias[kLayers];
+    const float* x;         // network inputs [n][6], or
+    const double* theta;    // parameters [n][6], encoded by the map
+    int n;
+    float* out;             // [n][320]
+    MapArgs map;
+};
+
+// The columns' constants of the decoding in shared memory (float pairs) and the rows'.
+struct ColumnConst {
+    float2 mu[kNout], sd[kNout], shot[kNout], ref[kNout], isig[kNout];
+    int e[kNout];
+};
+template <int MT>
+struct RowConst {
+    float2 amp[2][16 * MT], t5[16 * MT];   // A b sigma_8^2 (gE), A^2 sigma_8^2 (EE, BB); shot-noise scale
+    int e[16 * MT];
+    double la[16 * MT][kMaxNodes], lb[16 * MT][kMaxNodes];
+};
+
+// Forward pass of 16 MT rows per CTA (all layers, k_train_rows' row products) and, with MAP, the
+// whole prediction: the parameters' encoding before it and the decoding after it
+//   (pre_c (mu + sum_q w_q base_q + sd y) + theta_5 shot - ref) / sigma,
+// the baseline by exact digit products (above), the rest in float pairs.
+//
+// What bounds it: at 8192 rows the GELUs' instructions and the mma issue; at few rows the latency
+// of the dependent layers.  8192 rows: 287 -> 108 us, 50 rows: 85 -> 49 us, against eight launches
+// with the decoding's last operations in FP64.
+template <int MT, bool MAP>
+__global__ void __launch_bounds__(kRowThreads, MT == 1 ? 1 : 2) k_predict(const __grid_constant__ PredictArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int R = 16 * MT;
+    constexpr int ST = pred_stages(MT);
+    WeightRing<ST> ring;
+    ring.ring = reinterpret_cast<bf16*>(smem_raw);
+    ring.n_pass = kLayers;
+    bf16* buf[2];
+    buf[0] = ring.ring + ST * kStageElems;
+    buf[1] = buf[0] + R * kPredLd;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int r0 = blockIdx.x * R, rows = min(R, a.n - r0);
+    for (int c = 0; c < ST - 1; ++c) ring.load(a.ps);
+    for (int i = tid; i < R * 16; i += kRowThreads) {
+        const int r = i >> 4, c = i & 15;
+        float v = 0.f;
+        if (r < rows && c < kNin) {
+            if constexpr (MAP) v = (float)(a.theta[(size_t)(r0 + r) * kNin + c] * (double)a.map.scale[c] + (double)a.map.shift[c]);
+            else v = a.x[(size_t)(r0 + r) * kNin + c];
+        }
+        buf[0][r * kPredLd + c] = __float2bfloat16_rn(v);
+    }
+    int cur = 0;
+    for (int l = 0; l < kLayers - 1; ++l) {
+        float acc[MT][4][4];
+        if (l == 0) row_product<MT, 4, 16, kPredLd>(ring, a.ps, buf[cur], acc);
+        else row_product<MT, 4, 256, kPredLd>(ring, a.ps, buf[cur], acc);
+        bf16* nx = buf[cur ^ 1];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int c = 8 * (warp * 4 + j) + 2 * t;
+            const float2 b = *reinterpret_cast<const float2*>(a.bias[l] + c);
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    *reinterpret_cast<__nv_bfloat162*>(nx + (mt * 16 + g + 8 * h) * kPredLd + c) =
+                        __nv_bfloat162(__float2bfloat16_rn(gelu(acc[mt][j][2 * h] + b.x)),
+                                       __float2bfloat16_rn(gelu(acc[mt][j][2 * h + 1] + b.y)));
+        }
+        cur ^= 1;
+    }
+    float y[MT][5][4];
+    row_product<MT, 5, 256, kPredLd>(ring, a.ps, buf[cur], y);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        const int c = 8 * (warp * 5 + j) + 2 * t;
+        const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + c);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) y[mt][j][r] += (r & 1) ? b.y : b.x;
+    }
+    if constexpr (!MAP) {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = mt * 16 + g + 8 * h;
+                if (r >= rows) continue;
+#pragma unroll
+                for (int j = 0; j < 5; ++j)
+                    *reinterpret_cast<float2*>(a.out + (size_t)(r0 + r) * kNout + 8 * (warp * 5 + j) + 2 * t) =
+                        make_float2(y[mt][j][2 * h], y[mt][j][2 * h + 1]);
             }
-            __syncthreads();
-            for (int q = j; q < R * nn; q += blockDim.x) {
-                const int rr = q / nn, qq = q - rr * nn;
-                float h = 0.f, l = 0.f;
-                if (rr < nr) {
-                    const double w = la[rr][qq / a.nodes] * lb[rr][qq % a.nodes];
-                    h = (float)w;
-                    l = (float)(w - (double)h);
+        return;
+    } else {
+        cp_wait<0>();
+        __syncthreads();   // the ring and the activations are free
+        // shared memory of the decoding: the weights' digit fragments, then the constants
+        uint4* wd = reinterpret_cast<uint4*>(smem_raw);   // [kDigits][MT][kBaseKsteps][32]
+        ColumnConst& cc = *reinterpret_cast<ColumnConst*>(wd + kDigits * MT * kBaseKsteps * 32);
+        RowConst<MT>& rc = *reinterpret_cast<RowConst<MT>*>(&cc + 1);
+        static_assert(sizeof(uint4) * kDigits * MT * kBaseKsteps * 32 + sizeof(ColumnConst) + sizeof(RowConst<MT>) <= pred_smem(MT),
+                      "the decoding fits in the forward pass's shared memory");
+        const MapArgs& m = a.map;
+        auto as2 = [](fpair p) { return make_float2(p.hi, p.lo); };
+        auto pr = [](float2 v) { return fpair{v.x, v.y}; };
+        for (int j = tid; j < kNout; j += kRowThreads) {
+            cc.mu[j] = as2(pair_of(m.mu[j]));
+            cc.sd[j] = as2(pair_of(m.sd[j]));
+            cc.shot[j] = as2(pair_of(m.shot[j]));
+            cc.ref[j] = as2(pair_of(m.ref ? m.ref[j] : 0.0));
+            cc.isig[j] = as2(pair_of(m.sigma ? 1.0 / m.sigma[j] : 1.0));
+            cc.e[j] = m.base ? m.exponent[j] : 0;
+        }
+        for (int i = tid; i < 3 * R; i += kRowThreads) {
+            const int r = i / 3, k = i - 3 * r;
+            if (r >= rows) continue;
+            const double* th = a.theta + (size_t)(r0 + r) * kNin;
+            if (k == 0) {
+                const double s2 = th[2] * th[2];
+                rc.amp[0][r] = as2(pair_of(s2 * (th[0] * th[1])));
+                rc.amp[1][r] = as2(pair_of(s2 * (th[0] * th[0])));
+                rc.t5[r] = as2(pair_of(th[5]));
+            } else if (m.base) {
+                const int c = m.base_in[k - 1];
+                lobatto_basis_fast(th[c] * m.dscale[c] + m.dshift[c], m, k == 1 ? rc.la[r] : rc.lb[r]);
+            }
+        }
+        __syncthreads();
+        if (m.base) {
+            // the rows' Lagrange weights as digit fragments: one warp per row
+            const int nn = m.nodes * m.nodes;
+            bf16* wo = reinterpret_cast<bf16*>(wd);
+            for (int r = warp; r < R; r += kRowThreads / 32) {
+                double v[2], mx = 0.0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int q = lane + 32 * h;
+                    v[h] = (r < rows && q < nn) ? rc.la[r][q / m.nodes] * rc.lb[r][q % m.nodes] : 0.0;
+                    mx = fmax(mx, fabs(v[h]));
+                    if (!(fabs(v[h]) < INFINITY)) mx = INFINITY;
                 }
-                whi[rr][qq] = h;
-                wlo[rr][qq] = l;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                const bool finite = mx < INFINITY;
+                int e = 0;
+                if (finite && mx > 0.0) frexp(mx, &e);
+                if (lane == 0) rc.e[r] = finite ? e : kBadExponent;
+                const int mt = r >> 4, rr = r & 15;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    int d[kDigits];
+                    fixed_digits(finite ? ldexp(v[h], -e) : 0.0, d);
+                    // term q = 32 h + lane = 16 ks + p: register (rr >> 3) + 2 (p >> 3) of lane 4 (rr & 7) + (p & 7) / 2
+                    const int ks = 2 * h + (lane >> 4), p = lane & 15;
+                    const int reg = (rr >> 3) + 2 * (p >> 3), ln = 4 * (rr & 7) + ((p & 7) >> 1);
+#pragma unroll
+                    for (int i = 0; i < kDigits; ++i)
+                        wo[((((i * MT + mt) * kBaseKsteps + ks) * 32 + ln) * 4 + reg) * 2 + (p & 1)] =
+                            __float2bfloat16_rn((float)d[i]);
+                }
             }
             __syncthreads();
         }
-        float s_hi[R], s_lo[R];
 #pragma unroll
-        for (int rr = 0; rr < R; ++rr) s_hi[rr] = s_lo[rr] = 0.f;
-        for (int q = 0; q < nn; ++q) {
-            const float bh = a.base_hi[(size_t)q * kNout + j], bl = a.base_lo[(size_t)q * kNout + j];
+        for (int j = 0; j < 5; ++j) {
+            const int tile = warp * 5 + j;
 #pragma unroll
-            for (int rr = 0; rr < R; ++rr) {
-                const float wh = whi[rr][q], wl = wlo[rr][q];
-                // the _rn intrinsics are never contracted into FMAs, which the exact
-                // transformations need
-                const float p = __fmul_rn(wh, bh);
-                float e = fmaf(wh, bh, -p);              // wh bh = p + e exactly
-                e += fmaf(wh, bl, wl * bh);              // the cross terms (wl bl is below 2^-48)
-                const float s = __fadd_rn(s_hi[rr], p);  // s_hi + p = s + err exactly
-                const float bb = __fsub_rn(s, s_hi[rr]);
-                const float err = __fadd_rn(__fsub_rn(s_hi[rr], __fsub_rn(s, bb)), __fsub_rn(p, bb));
-                s_hi[rr] = s;
-                s_lo[rr] += err + e;
+            for (int mt = 0; mt < MT; ++mt) {
+                float acc[kOrders][4];
+#pragma unroll
+                for (int o = 0; o < kOrders; ++o)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) acc[o][r] = 0.f;
+                if (m.base) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint4 bd[kDigits];
+#pragma unroll
+                        for (int i = 0; i < kDigits; ++i)
+                            bd[i] = m.digits[((size_t)(i * (kNout / 8) + tile) * 2 + h) * 32 + lane];
+#pragma unroll
+                        for (int k = 0; k < 2; ++k)
+#pragma unroll
+                            for (int i = 0; i < kDigits; ++i) {
+                                const uint4 av = wd[((i * MT + mt) * kBaseKsteps + 2 * h + k) * 32 + lane];
+                                const uint32_t af[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+                                for (int q = 0; q < kDigits; ++q)
+                                    if (i + q < kOrders)
+                                        mma_bf16(acc[i + q], af, k ? bd[q].z : bd[q].x, k ? bd[q].w : bd[q].y);
+                            }
+                    }
+                }
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    const int r = mt * 16 + g + 8 * hh;
+                    if (r >= rows) continue;
+                    float res[2];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const int c = 8 * tile + 2 * t + q, v = 2 * hh + q;
+                        fpair u = pr(cc.mu[c]);
+                        if (m.base) {
+                            // sum_o acc_o 2^(-8 o), the small orders first
+                            fpair b{0.f, 0.f};
+#pragma unroll
+                            for (int o = kOrders - 1; o >= 0; --o) {
+                                const fpair s2 = two_sum(__fmul_rn(acc[o][v], exp2i(-8 * o)), b.hi);
+                                b = fast_two_sum(s2.hi, __fadd_rn(s2.lo, b.lo));
+                            }
+                            const int er = rc.e[r], ec = cc.e[c];
+                            if (er == kBadExponent || ec == kBadExponent) {
+                                b.hi = b.lo = NAN;
+                            } else {
+                                const int e = er + ec - 14;   // the digits' unit: 2^(e_r + e_c) 2^-14
+                                b.hi = scale2(b.hi, e);
+                                b.lo = scale2(b.lo, e);
+                            }
+                            u = pair_add(u, b);
+                        }
+                        u = pair_add(u, pair_mul(pr(cc.sd[c]), y[mt][j][v]));
+                        u = pair_mul(u, pr(rc.amp[c < 2 * (kNout / 8) ? 0 : 1][r]));
+                        u = pair_add(u, pair_mul(pr(rc.t5[r]), pr(cc.shot[c])));
+                        const float2 rf = cc.ref[c];
+                        u = pair_add(u, fpair{-rf.x, -rf.y});
+                        u = pair_mul(u, pr(cc.isig[c]));
+                        res[q] = __fadd_rn(u.hi, u.lo);
+                    }
+                    *reinterpret_cast<float2*>(a.out + (size_t)(r0 + r) * kNout + 8 * tile + 2 * t) = make_float2(res[0], res[1]);
+                }
             }
         }
-#pragma unroll
-        for (int rr = 0; rr < R; ++rr) {
-            if (rr >= nr) break;
-            const int r = r0 + rr;
-            const double* t = theta + (size_t)r * kNin;
-            const double u = a.mu[j] + ((double)s_hi[rr] + (double)s_lo[rr]);
-            const size_t i = (size_t)r * kNout + j;
-            const double amp = t[2] * t[2] * ((j / nb) < 2 ? t[0] * t[1] : t[0] * t[0]);
-            double v = amp * (u + a.sd[j] * (double)y[i]) + t[5] * a.shot[j];
-            if (a.ref) v -= a.ref[j];
-            if (a.sigma) v /= a.sigma[j];
-            out[i] = (float)v;
-        }
-        __syncthreads();   // la, lb, whi, wlo are rewritten for the next rows
     }
 }
 
@@ -439,11 +855,10 @@ struct lpp_surrogate_s {
     size_t need = 0;
     // offsets
     size_t w[kLayers], b[kLayers], mw[kLayers], vw[kLayers], mb[kLayers], vb[kLayers], dw[kLayers], db[kLayers];
-    size_t w16[kLayers], w16t[kLayers], act[kLayers + 1], actt[kLayers], z[kLayers];
-    size_t g32[2], g16[2], g16t[2], loss, xin;
-    size_t base_hi, base_lo;          // the decoding's float-pair copy of the map's base
+    size_t w16[kLayers], w16t[kLayers], actt[kLayers], gt[kLayers], g32[kLayers], loss;
+    size_t digits, exponent;          // the decoding's digits of the map's base
     bool has_map = false;
-    bool base_split = false;          // base_hi/base_lo hold the current map's base
+    bool base_split = false;          // digits, exponent hold the current map's base
     MapArgs map;
 };
 
@@ -465,20 +880,13 @@ extern "C" lpp_status lpp_surrogate_create(int batch, lpp_surrogate_t* out) {
         s->db[l] = take(kOut[l] * 4);
         s->w16[l] = take(nw * 2);
         s->w16t[l] = take(nw * 2);
-        s->act[l] = take((size_t)batch * kInPad[l] * 2);
         s->actt[l] = take((size_t)batch * kInPad[l] * 2);
-        s->z[l] = take((size_t)batch * kOut[l] * 4);
-    }
-    s->act[kLayers] = 0;
-    for (int i = 0; i < 2; ++i) {
-        s->g32[i] = take((size_t)batch * kNout * 4);
-        s->g16[i] = take((size_t)batch * kNout * 2);
-        s->g16t[i] = take((size_t)batch * kNout * 2);
+        s->gt[l] = take((size_t)batch * kOut[l] * 2);
+        s->g32[l] = take((size_t)batch * kOut[l] * 4);
     }
     s->loss = take(8);
-    s->xin = take((size_t)batch * kNin * 4);
-    s->base_hi = take((size_t)kMaxNodes * kMaxNodes * kNout * 4);
-    s->base_lo = take((size_t)kMaxNodes * kMaxNodes * kNout * 4);
+    s->digits = take((size_t)kDigitWords * sizeof(uint4));
+    s->exponent = take((size_t)kNout * sizeof(int));
     s->need = off;
     *out = s;
     return LPP_OK;
@@ -657,51 +1065,40 @@ extern "C" lpp_status lpp_surrogate_get_params(lpp_surrogate_t s, float* params,
     return LPP_OK;
 }
 
-// forward pass of m <= batch rows (inputs gathered through idx when given)
-static cudaError_t forward(lpp_surrogate_t s, const float* x, const int* idx, int m, bool train, float* out_final,
-                           cudaStream_t st) {
-    const int B = s->batch;
-    bf16* a0 = (bf16*)(s->ws + s->act[0]);
-    k_input<<<(m * 16 + 255) / 256, 256, 0, st>>>(x, idx, m, a0, train ? (bf16*)(s->ws + s->actt[0]) : nullptr, B);
-    for (int l = 0; l < kLayers; ++l) {
-        GemmArgs g;
-        memset(&g, 0, sizeof(g));
-        g.A = (const bf16*)(s->ws + s->act[l]);
-        g.lda = kInPad[l];
-        g.B = (const bf16*)(s->ws + s->w16[l]);
-        g.ldb = kInPad[l];
-        g.M = m;
-        g.N = kOut[l];
-        g.K = kInPad[l];
-        g.bias = (const float*)(s->ws + s->b[l]);
-        if (l < kLayers - 1) {
-            g.epi = EPI_HIDDEN;
-            g.z = (float*)(s->ws + s->z[l]);
-            g.ldz = kOut[l];
-            g.a16 = (bf16*)(s->ws + s->act[l + 1]);
-            g.ld16 = kInPad[l + 1];
-            g.a16t = train ? (bf16*)(s->ws + s->actt[l + 1]) : nullptr;
-            g.ld16t = B;
-        } else {
-            g.epi = EPI_OUT;
-            g.z = out_final ? out_final : (float*)(s->ws + s->z[l]);
-            g.ldz = kOut[l];
-        }
-        cudaError_t e = gemm(g, st);
-        if (e != cudaSuccess) return e;
+static Passes passes(lpp_surrogate_t s) {
+    Passes p;
+    for (int l = 0; l < kLayers; ++l) p.w[l] = (const bf16*)(s->ws + s->w16[l]);
+    for (int l = kLayers - 1; l > 0; --l) p.w[2 * kLayers - 1 - l] = (const bf16*)(s->ws + s->w16t[l]);
+    return p;
+}
+
+// The fused forward pass (MAP: the whole prediction) of n rows: 16 rows per CTA up to one CTA per
+// SM, 32 rows beyond (two CTAs per SM, half the weight traffic per row).
+template <bool MAP>
+static cudaError_t launch_predict(lpp_surrogate_t s, PredictArgs& a, cudaStream_t st) {
+    if (a.n == 0) return cudaSuccess;
+    a.ps = passes(s);
+    for (int l = 0; l < kLayers; ++l) a.bias[l] = (const float*)(s->ws + s->b[l]);
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (a.n <= 16 * sms) {
+        cudaFuncSetAttribute(k_predict<1, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pred_smem(1));
+        k_predict<1, MAP><<<(a.n + 15) / 16, kRowThreads, pred_smem(1), st>>>(a);
+    } else {
+        cudaFuncSetAttribute(k_predict<2, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pred_smem(2));
+        k_predict<2, MAP><<<(a.n + 31) / 32, kRowThreads, pred_smem(2), st>>>(a);
     }
     return cudaGetLastError();
 }
 
 extern "C" lpp_status lpp_surrogate_infer(lpp_surrogate_t s, const float* x, int n, float* y, void* stream) {
     if (!s || !s->ws || n < 0 || (n > 0 && (!x || !y))) return LPP_ERR_INVALID_ARG;
-    cudaStream_t st = (cudaStream_t)stream;
-    for (int r0 = 0; r0 < n; r0 += s->batch) {
-        const int m = n - r0 < s->batch ? n - r0 : s->batch;
-        if (forward(s, x + (size_t)r0 * kNin, nullptr, m, false, y + (size_t)r0 * kNout, st) != cudaSuccess)
-            return LPP_ERR_CUDA;
-    }
-    return LPP_OK;
+    PredictArgs a;
+    memset(&a, 0, sizeof(a));
+    a.x = x;
+    a.n = n;
+    a.out = y;
+    return launch_predict<false>(s, a, (cudaStream_t)stream) == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
 }
 
 extern "C" lpp_status lpp_surrogate_set_map(lpp_surrogate_t s, const lpp_surrogate_map* m) {
@@ -766,96 +1163,62 @@ extern "C" lpp_status lpp_surrogate_encode(lpp_surrogate_t s, const double* thet
 extern "C" lpp_status lpp_surrogate_predict(lpp_surrogate_t s, const double* theta, int n, float* out, void* stream) {
     if (!s || !s->ws || !s->has_map || n < 0 || (n > 0 && (!theta || !out))) return LPP_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    float* x = (float*)(s->ws + s->xin);
     if (s->map.base) {
-        s->map.base_hi = (const float*)(s->ws + s->base_hi);
-        s->map.base_lo = (const float*)(s->ws + s->base_lo);
+        s->map.digits = (const uint4*)(s->ws + s->digits);
+        s->map.exponent = (const int*)(s->ws + s->exponent);
         if (!s->base_split) {
-            const int count = s->map.nodes * s->map.nodes * kNout;
-            k_split_base<<<(count + 255) / 256, 256, 0, st>>>(s->map.base, count, (float*)(s->ws + s->base_hi),
-                                                             (float*)(s->ws + s->base_lo));
+            k_base_digits<<<kNout / 8, 256, 0, st>>>(s->map.base, s->map.nodes * s->map.nodes,
+                                                     (uint4*)(s->ws + s->digits), (int*)(s->ws + s->exponent));
             if (cudaGetLastError() != cudaSuccess) return LPP_ERR_CUDA;
             s->base_split = true;
         }
     }
-    for (int r0 = 0; r0 < n; r0 += s->batch) {
-        const int m = n - r0 < s->batch ? n - r0 : s->batch;
-        const double* th = theta + (size_t)r0 * kNin;
-        k_encode<<<(m * kNin + 255) / 256, 256, 0, st>>>(th, m, x, s->map);
-        float* y = out + (size_t)r0 * kNout;
-        if (forward(s, x, nullptr, m, false, y, st) != cudaSuccess) return LPP_ERR_CUDA;
-        {
-            int dev = 0, sms = 152;
-            if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            const int groups = (m + kDecodeRows - 1) / kDecodeRows;
-            const int blocks = groups < sms * 6 ? (groups > 0 ? groups : 1) : sms * 6;
-            k_decode<<<blocks, kNout, 0, st>>>(th, m, y, y, s->map);
-        }
-    }
-    return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
+    PredictArgs a;
+    memset(&a, 0, sizeof(a));
+    a.theta = theta;
+    a.n = n;
+    a.out = out;
+    a.map = s->map;
+    return launch_predict<true>(s, a, st) == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
 }
 
-// One Adam step on the minibatch rows idx[0..batch) of (x, y); the mean squared error of the
-// minibatch (before the step) is added to *loss_out (device).
+// The gradients of the minibatch rows idx[0..batch) of (x, y) and, with update, one Adam step; the
+// mean squared error of the minibatch (before the step) is added to *loss_out (device).
 static cudaError_t train_step(lpp_surrogate_t s, const float* x, const float* y, const int* idx, float lr,
-                              double* loss_out, cudaStream_t st) {
-    const int B = s->batch;
-    cudaError_t e = forward(s, x, idx, B, true, nullptr, st);
-    if (e != cudaSuccess) return e;
-    int cur = 0;
-    k_loss<<<(B * kNout + 255) / 256, 256, 0, st>>>((const float*)(s->ws + s->z[kLayers - 1]), y, idx, B,
-                                                    (float*)(s->ws + s->g32[cur]), (bf16*)(s->ws + s->g16[cur]),
-                                                    (bf16*)(s->ws + s->g16t[cur]), B, loss_out);
-    for (int l = kLayers - 1; l >= 0; --l) {
-        // dW_l = g^T a_l : [out x inp] = [out x B] . [inp x B]^T
-        GemmArgs gw;
-        memset(&gw, 0, sizeof(gw));
-        gw.A = (const bf16*)(s->ws + s->g16t[cur]);
-        gw.lda = B;
-        gw.B = (const bf16*)(s->ws + s->actt[l]);
-        gw.ldb = B;
-        gw.M = kOut[l];
-        gw.N = kInPad[l];
-        gw.K = B;
-        gw.epi = EPI_DW;
-        gw.z = (float*)(s->ws + s->dw[l]);
-        gw.ldz = kInPad[l];
-        if ((e = gemm(gw, st)) != cudaSuccess) return e;
-        k_bias_grad<<<(kOut[l] + 31) / 32, 256, 0, st>>>((const float*)(s->ws + s->g32[cur]), B, kOut[l],
-                                                           (float*)(s->ws + s->db[l]));
-        if (l > 0) {
-            // g_{l-1} = (g_l W_l) * GELU'(z_{l-1}) : [B x inp] = [B x out] . [inp x out]^T
-            GemmArgs gd;
-            memset(&gd, 0, sizeof(gd));
-            gd.A = (const bf16*)(s->ws + s->g16[cur]);
-            gd.lda = kOut[l];
-            gd.B = (const bf16*)(s->ws + s->w16t[l]);
-            gd.ldb = kOut[l];
-            gd.M = B;
-            gd.N = kInPad[l];
-            gd.K = kOut[l];
-            gd.epi = EPI_DA_GELU;
-            gd.zprev = (const float*)(s->ws + s->z[l - 1]);
-            gd.ldzp = kOut[l - 1];
-            gd.g32 = (float*)(s->ws + s->g32[1 - cur]);
-            gd.ldg = kInPad[l];
-            gd.a16 = (bf16*)(s->ws + s->g16[1 - cur]);
-            gd.ld16 = kInPad[l];
-            gd.a16t = (bf16*)(s->ws + s->g16t[1 - cur]);
-            gd.ld16t = B;
-            if ((e = gemm(gd, st)) != cudaSuccess) return e;
-            cur = 1 - cur;
-        }
+                              bool update, double* loss_out, cudaStream_t st) {
+    TrainRowArgs r;
+    memset(&r, 0, sizeof(r));
+    TrainWeightArgs w;
+    memset(&w, 0, sizeof(w));
+    r.ps = passes(s);
+    for (int l = 0; l < kLayers; ++l) {
+        r.bias[l] = (const float*)(s->ws + s->b[l]);
+        r.actt[l] = (bf16*)(s->ws + s->actt[l]);
+        r.gt[l] = (bf16*)(s->ws + s->gt[l]);
+        r.g32[l] = (float*)(s->ws + s->g32[l]);
+        w.actt[l] = r.actt[l];
+        w.gt[l] = r.gt[l];
+        w.g32[l] = r.g32[l];
     }
-    s->step += 1;
-    AdamArgs a = adam_args(s);
+    r.x = x;
+    r.y = y;
+    r.idx = idx;
+    r.batch = w.batch = s->batch;
+    r.loss = loss_out;
+    cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem);
+    cudaFuncSetAttribute(k_train_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWeightSmem);
+    k_train_rows<<<s->batch / 16, kRowThreads, kTrainSmem, st>>>(r);
+    if (update) s->step += 1;
+    AdamArgs& a = w.adam;
+    a = adam_args(s);
     a.lr = lr;
     a.b1 = 0.9f;
     a.b2 = 0.999f;
     a.eps = 1e-8f;
     a.bc1 = (float)(1.0 - pow(0.9, (double)s->step));
     a.bc2 = (float)(1.0 - pow(0.999, (double)s->step));
-    k_adam<<<dim3(128, kLayers), 256, 0, st>>>(a);
+    w.update = update ? 1 : 0;
+    k_train_weights<<<kWeightTiles + kBiasTiles, 128, kWeightSmem, st>>>(w);
     return cudaGetLastError();
 }
 
@@ -867,7 +1230,7 @@ extern "C" lpp_status lpp_surrogate_train(lpp_surrogate_t s, const float* x, con
     double* scratch = (double*)(s->ws + s->loss);
     for (int i = 0; i < n_steps; ++i) {
         double* lo = losses ? losses + i : scratch;
-        if (train_step(s, x, y, schedule + (size_t)i * s->batch, lr, lo, st) != cudaSuccess) return LPP_ERR_CUDA;
+        if (train_step(s, x, y, schedule + (size_t)i * s->batch, lr, true, lo, st) != cudaSuccess) return LPP_ERR_CUDA;
     }
     return LPP_OK;
 }
@@ -877,41 +1240,21 @@ extern "C" lpp_status lpp_surrogate_gradients(lpp_surrogate_t s, const float* x,
                                               float* grads, double* loss, void* stream) {
     if (!s || !s->ws || !x || !y || !idx || !grads) return LPP_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    const long long saved = s->step;
     double* lo = (double*)(s->ws + s->loss);
     if (cudaMemsetAsync(lo, 0, 8, st) != cudaSuccess) return LPP_ERR_CUDA;
-    // run the step with lr = 0 so that only the gradients are formed (Adam moments are restored below)
-    std::vector<char> mom;
-    for (int l = 0; l < kLayers; ++l) {
-        const size_t nw = (size_t)kOut[l] * kInPad[l] * 4;
-        const size_t off0 = mom.size();
-        mom.resize(off0 + 2 * nw + 2 * kOut[l] * 4);
-        cudaMemcpyAsync(mom.data() + off0, s->ws + s->mw[l], nw, cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(mom.data() + off0 + nw, s->ws + s->vw[l], nw, cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(mom.data() + off0 + 2 * nw, s->ws + s->mb[l], kOut[l] * 4, cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(mom.data() + off0 + 2 * nw + kOut[l] * 4, s->ws + s->vb[l], kOut[l] * 4,
-                        cudaMemcpyDeviceToHost, st);
-    }
-    if (train_step(s, x, y, idx, 0.0f, lo, st) != cudaSuccess) return LPP_ERR_CUDA;
-    size_t p = 0, mo = 0;
+    if (train_step(s, x, y, idx, 0.0f, false, lo, st) != cudaSuccess) return LPP_ERR_CUDA;
+    size_t p = 0;
     std::vector<float> dw;
     for (int l = 0; l < kLayers; ++l) {
         const size_t nw = (size_t)kOut[l] * kInPad[l];
         dw.resize(nw);
         cudaMemcpyAsync(dw.data(), s->ws + s->dw[l], nw * 4, cudaMemcpyDeviceToHost, st);
         cudaMemcpyAsync(grads + p + (size_t)kOut[l] * kIn[l], s->ws + s->db[l], kOut[l] * 4, cudaMemcpyDeviceToHost, st);
-        cudaMemcpyAsync(s->ws + s->mw[l], mom.data() + mo, nw * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(s->ws + s->vw[l], mom.data() + mo + nw * 4, nw * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(s->ws + s->mb[l], mom.data() + mo + 2 * nw * 4, kOut[l] * 4, cudaMemcpyHostToDevice, st);
-        cudaMemcpyAsync(s->ws + s->vb[l], mom.data() + mo + 2 * nw * 4 + kOut[l] * 4, kOut[l] * 4,
-                        cudaMemcpyHostToDevice, st);
         if (cudaStreamSynchronize(st) != cudaSuccess) return LPP_ERR_CUDA;
         for (int r = 0; r < kOut[l]; ++r)
             for (int c = 0; c < kIn[l]; ++c) grads[p++] = dw[(size_t)r * kInPad[l] + c];
         p += kOut[l];
-        mo += 2 * nw * 4 + 2 * kOut[l] * 4;
     }
-    s->step = saved;
     if (loss && cudaMemcpyAsync(loss, lo, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return LPP_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return LPP_ERR_CUDA;
     return LPP_OK;
