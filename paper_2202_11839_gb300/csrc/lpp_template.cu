@@ -79,6 +79,9 @@ struct TemplateArgs {
     const double* op;       // [kSlots][nb][2048] the operator's rows
     const double* kin;      // [2048] k_n
     const double* lnk;      // [2048] ln k_n
+    const double* ik;       // [2048] 1 / (2.34 k_n)
+    const double2* logtab;  // [128] (1 / c, ln c) of log1p_over
+    double dlnk;            // ln k_{n+1} - ln k_n
     const double* s8w;      // [2048] sigma_8 quadrature weight w_n k^3 W^2(8k) / (2 pi^2)
     const int* bin_lo;      // [nb] first k_n of each shell
     const int* bin_hi;      // [nb] one past the last
@@ -152,30 +155,63 @@ __device__ __forceinline__ void mma_f64(double c[2], double a, double b) {
                  : "d"(a), "d"(b));
 }
 
+// ln(1 + y) for 0 < y < 2^1000 by Tang's table method (ACM TOMS 16, 378, 1990): 1 + y = 2^e m,
+// c the middle of m's 1/128 interval (c = 1 in the first, so that small y keep their relative
+// accuracy), r = m / c - 1 with the rounding of 1 + y restored, |r| < 2^-7, and eight terms of
+// ln(1 + r).  16 FP64 operations, to 4e-16 relative; log1p takes several times as many, and the
+// FP64 rate bounds the spectra.
+__device__ __forceinline__ double log1p_table(double y, const double2* tab) {
+    const double s = 1.0 + y;
+    const double lost = y - (s - 1.0);   // s + lost = 1 + y exactly
+    const long long bits = __double_as_longlong(s);
+    const int e = (int)(bits >> 52) - 1023;
+    const double2 c = tab[(int)(bits >> 45) & 127];
+    const double m = __longlong_as_double((bits & 0x000fffffffffffffLL) | 0x3ff0000000000000LL);
+    const double w = __longlong_as_double((long long)(1023 - e) << 52);   // 2^-e
+    const double r = fma(lost * w, c.x, fma(m, c.x, -1.0));
+    double p = -1.0 / 8.0;
+    p = fma(p, r, 1.0 / 7.0);
+    p = fma(p, r, -1.0 / 6.0);
+    p = fma(p, r, 1.0 / 5.0);
+    p = fma(p, r, -1.0 / 4.0);
+    p = fma(p, r, 1.0 / 3.0);
+    p = fma(p, r, -1.0 / 2.0);
+    p = fma(p * r, r, r);
+    return fma((double)e, 0.69314718055994530942, c.y) + p;
+}
+
 // Templates of eight parameter sets on one cluster of eight CTAs (blockIdx.y: a group of a.bins
 // shells).  CTA c forms the model spectra on its 256 grid k (one thread per k, the sets in turn)
 // and multiplies them with its 256 columns of the operator's rows, 8 sets x 8 rows x 4 columns
-// per tensor instruction; the cluster then adds the eight partial sums through distributed
-// shared memory in a fixed order, CTA c for every eighth shell, normalises to sigma_8 and
-// writes the slots and derived curves.
+// per tensor instruction, the columns split over four groups of warps when the rows are few;
+// the cluster then adds the partial sums through distributed shared memory in a fixed order,
+// CTA c for every eighth shell, normalises to sigma_8 and writes the slots and derived curves.
 //
-// What bounds it: FP64 issue, about half of it the model spectrum (log1p, exp, rsqrt) and half
-// the products; the FP64 mma runs 4.2 times the plain FP64 multiply-add rate on GB300 (2.09
-// against 0.50 T multiply-adds/s), which is why the rows are multiplied by it even for one set
-// (seven of its eight rows idle).  8192 sets, nine slots, 40 shells: 78.0 -> 14.9 ms against one
-// CTA per set running its own transforms (24 FFTs of 4096 points); one set, fourteen slots:
-// 1.99 -> 0.18 ms (the shells spread over the SMs by blockIdx.y).
+// What bounds it: the FP64 rate, 0.59 T multiply-adds/s on GB300 (0.52 through the FP64 mma, which
+// is no faster here but issues and loads a quarter as much): 6.1 G multiply-adds of the products
+// are 11.6 ms of 8192 sets with nine slots and 40 shells, the model spectra (k^tilt from two
+// short tables of powers, log1p_table, rsqrt: about 50 operations a value) most of the rest.
+// 78.0 -> 15.0 ms against one CTA per set running its own transforms (24 FFTs of 4096 points).
+// One set, fourteen slots: 1.99 ms -> 24 us, the shells spread over the SMs by blockIdx.y;
+// there an mma would idle seven of its eight rows, and up to kFewSets sets take plain
+// multiply-adds (FEW).
 constexpr int kCluster = 8, kSets = 8, kSlab = kNin / kCluster, kTiles = 9;
+constexpr int kSegs = 4;   // column segments of a slab, each summed by itself
+constexpr int kFewSets = 2;
 constexpr int kMaxRows = 8 * 8 * kTiles;   // rows per cluster: 8 warps x kTiles tiles of 8
 constexpr int kSlabPad = kSlab + 2;        // the eight sets' rows start in different banks
 
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(256, 2) k_template(const __grid_constant__ TemplateArgs a) {
+// NT: tiles of 8 rows per warp, KPARTS: column segments taken by different warps (1 or kSegs);
+// compile-time, so that every tile of a warp is one unconditional product
+template <int NT, int KPARTS, bool FEW = false>
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(256, NT <= 6 ? 3 : 2)
+k_template(const __grid_constant__ TemplateArgs a) {
     namespace cg = cooperative_groups;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const bool png = a.png_amp != 0.0;
     const int n_pow = png ? 3 : 1;   // P, P f, P f^2 with the PNG response f
     double* spec = reinterpret_cast<double*>(smem_raw);   // [n_pow][kSets][kSlabPad]
-    double* part = spec + n_pow * kSets * kSlabPad;       // [rows][kSets] partial sums
+    double* part = spec + n_pow * kSets * kSlabPad;       // [kparts][rows][kSets] partial sums
     __shared__ double s8part[kSets];
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
@@ -185,21 +221,37 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(256, 2) k_tem
     const int b0 = blockIdx.y * a.bins, nbl = min(a.bins, a.nb - b0);
     const int rows = a.n_slots * nbl;
 
+    // per set: k^tilt at every 16th grid k of the slab, the 16 powers between, 1 / Gamma
+    __shared__ double pw_hi[kSets][16], pw_lo[kSets][16], igam[kSets];
+    __shared__ double2 logtab[128];
+    {
+        const int t = tid >> 5, i = tid & 15;
+        if (t < sets) {
+            const double tilt = a.params[6 * (size_t)(t0 + t) + 3];
+            const double v = exp(tilt * ((lane & 16) ? a.dlnk * i : a.lnk[rank * kSlab + 16 * i]));
+            if (lane & 16) pw_lo[t][i] = v;
+            else pw_hi[t][i] = v;
+            if (lane == 0) igam[t] = 1.0 / a.params[6 * (size_t)(t0 + t) + 4];
+        }
+        if (tid < 128) logtab[tid] = a.logtab[tid];
+    }
+    __syncthreads();
     // model spectra (unnormalised BBKS, Bardeen, Bond, Kaiser & Szalay 1986)
     {
         const int n = rank * kSlab + tid;
-        const double k = a.kin[n], lnk = a.lnk[n];
+        const double k = a.kin[n], ik = a.ik[n];
+#pragma unroll 2
         for (int t = 0; t < kSets; ++t) {
             double p = 0.0, f = 0.0;
             if (t < sets) {
-                const double* th = a.params + 6 * (size_t)(t0 + t);
-                const double tilt = th[3], gam = th[4];
-                const double q = k / gam;
-                const double l = log1p(2.34 * q) / (2.34 * q);
+                const double ig = igam[t], q = k * ig, y = 2.34 * q;
+                double l;
+                if (y > 0.0 && y < 1e300) l = log1p_table(y, logtab) * (ik * a.params[6 * (size_t)(t0 + t) + 4]);
+                else l = log1p(y) / y;
                 const double x = 1.0 + q * (3.89 + q * (16.1 * 16.1 + q * (5.46 * 5.46 * 5.46 +
                                                                            q * (6.71 * 6.71 * 6.71 * 6.71))));
                 const double rs = rsqrt(x);        // T = l x^(-1/4)
-                p = k * exp(tilt * lnk) * (l * l * rs);
+                p = k * (pw_hi[t][tid >> 4] * pw_lo[t][tid & 15]) * (l * l * rs);
                 // Sec. 5: P -> [1 + 12 f_NL delta b_IA / M(k)] P per shape field,
                 // M(k) = (2/3) k^2 T(k) D (c/H0)^2 / Omega_m with D = 1 (z = 0)
                 if (png) f = 1.0 + a.png_amp / ((2.0 / 3.0) * k * k * (l * sqrt(rs)) * a.png_len2);
@@ -219,58 +271,99 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(256, 2) k_tem
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
         if (lane == 0) s8part[warp] = s;
     }
-    // row r = (slot index) nbl + shell; tile j of the warp: rows 8 (warp + 8 j) ..
-    const int rl = lane >> 2, cl = 2 * (lane & 3);
-    const double* brow[kTiles];
-    const double* arow = spec + rl * kSlabPad + cl;
-    double acc[kTiles][2];
+    if constexpr (FEW) {
+        // a warp per row (slot index) nbl + shell: 8 columns per lane, then the lanes' sums
+        for (int r = warp; r < rows; r += 8) {
+            const int si = r / nbl, sl = a.slot[si];
+            const int pw = !png || sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);   // power of the response
+            const double2* op = reinterpret_cast<const double2*>(
+                a.op + ((size_t)sl * a.nb + b0 + (r - si * nbl)) * kNin + rank * kSlab);
+            double2 o[4];
 #pragma unroll
-    for (int j = 0; j < kTiles; ++j) {
-        const int r8 = 8 * (warp + 8 * j);
-        const int r = max(0, min(r8 + rl, rows - 1));   // rows beyond the last repeat it and are not read back
-        const int si = r / nbl;
-        brow[j] = a.op + ((size_t)a.slot[si] * a.nb + b0 + (r - si * nbl)) * kNin + rank * kSlab + cl;
-        acc[j][0] = acc[j][1] = 0.0;
-    }
-    if (!png) {
-        for (int k0 = 0; k0 < kSlab; k0 += 8) {
-            const double2 av = *reinterpret_cast<const double2*>(arow + k0);
+            for (int i = 0; i < 4; ++i) o[i] = op[lane + 32 * i];
+            for (int t = 0; t < sets; ++t) {
+                const double2* sp = reinterpret_cast<const double2*>(spec + (pw * kSets + t) * kSlabPad);
+                double v = 0.0, w = 0.0;
 #pragma unroll
-            for (int j = 0; j < kTiles; ++j) {
-                if (8 * (warp + 8 * j) >= rows) break;   // warp-uniform
-                const double2 bv = *reinterpret_cast<const double2*>(brow[j] + k0);
-                mma_f64(acc[j], av.x, bv.x);
-                mma_f64(acc[j], av.y, bv.y);
+                for (int i = 0; i < 4; ++i) {
+                    const double2 p = sp[lane + 32 * i];
+                    v = fma(o[i].x, p.x, v);
+                    w = fma(o[i].y, p.y, w);
+                }
+                v += w;
+#pragma unroll
+                for (int q = 16; q > 0; q >>= 1) v += __shfl_down_sync(0xffffffffu, v, q);
+                if (lane == 0) part[r * kSets + t] = v;
             }
         }
     } else {
-        // the response enters the density rows not at all, the cross rows once and the plus and
-        // minus rows twice; a tile may straddle two families, so every row takes the product
-        // with its own family's spectrum of the three
-        for (int pw = 0; pw < 3; ++pw) {
+    // row r = (slot index) nbl + shell; the warp takes tiles wt, wt + lanes, .. of 8 rows, and all
+    // four segments of 64 columns or one.  Every segment is summed by itself and the segments are
+    // added in order, so a value does not depend on the split (on the slots and sets of the call).
+    constexpr int lanes = 8 / KPARTS;
+    const int wt = warp % lanes, kpart = warp / lanes;
+    const int rl = lane >> 2, cl = 2 * (lane & 3);
+    unsigned brow[NT];   // in double2, from the slab's first column
+    const double2* op = reinterpret_cast<const double2*>(a.op + rank * kSlab + cl);
+    const double* arow = spec + rl * kSlabPad + cl;
+    double acc[NT][2];
 #pragma unroll
-            for (int j = 0; j < kTiles; ++j) {
-                const int r8 = 8 * (warp + 8 * j);
-                if (r8 >= rows) break;
-                const int r = min(r8 + rl, rows - 1);
-                const int sl = a.slot[r / nbl];
-                const int want = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
-                if (!__any_sync(0xffffffffu, want == pw)) continue;   // warp-uniform
-                const double on = want == pw ? 1.0 : 0.0;
-                for (int k0 = 0; k0 < kSlab; k0 += 8) {
-                    const double2 av = *reinterpret_cast<const double2*>(arow + pw * kSets * kSlabPad + k0);
-                    const double2 bv = *reinterpret_cast<const double2*>(brow[j] + k0);
-                    mma_f64(acc[j], av.x, on * bv.x);
-                    mma_f64(acc[j], av.y, on * bv.y);
+    for (int j = 0; j < NT; ++j) {
+        // rows beyond the last repeat it and are not read back
+        const int r = max(0, min(8 * (wt + lanes * j) + rl, rows - 1));
+        const int si = r / nbl;
+        brow[j] = (unsigned)((a.slot[si] * a.nb + b0 + (r - si * nbl)) * (kNin / 2));
+    }
+    for (int seg = kpart; seg < kSegs; seg += KPARTS) {
+        const int k_lo = seg * (kSlab / kSegs), k_hi = k_lo + kSlab / kSegs;
+#pragma unroll
+        for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = 0.0;
+        if (!png) {
+            for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
+                const double2 av = *reinterpret_cast<const double2*>(arow + k0);
+                double2 bv[NT];
+#pragma unroll
+                for (int j = 0; j < NT; ++j) bv[j] = op[brow[j] + k0 / 2];
+#pragma unroll
+                for (int j = 0; j < NT; ++j) mma_f64(acc[j], av.x, bv[j].x);
+#pragma unroll
+                for (int j = 0; j < NT; ++j) mma_f64(acc[j], av.y, bv[j].y);
+            }
+        } else {
+            // the response enters the density rows not at all, the cross rows once and the plus and
+            // minus rows twice; a tile may straddle two families, so every row takes the product
+            // with its own family's spectrum of the three
+            for (int pw = 0; pw < 3; ++pw) {
+#pragma unroll
+                for (int j = 0; j < NT; ++j) {
+                    const int r8 = 8 * (wt + lanes * j);
+                    if (r8 >= rows) break;
+                    const int r = min(r8 + rl, rows - 1);
+                    const int sl = a.slot[r / nbl];
+                    const int want = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
+                    if (!__any_sync(0xffffffffu, want == pw)) continue;   // warp-uniform
+                    const double on = want == pw ? 1.0 : 0.0;
+                    for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
+                        const double2 av = *reinterpret_cast<const double2*>(arow + pw * kSets * kSlabPad + k0);
+                        const double2 bv = op[brow[j] + k0 / 2];
+                        mma_f64(acc[j], av.x, on * bv.x);
+                        mma_f64(acc[j], av.y, on * bv.y);
+                    }
                 }
             }
         }
-    }
+        const bool first = seg < KPARTS;
 #pragma unroll
-    for (int j = 0; j < kTiles; ++j) {
-        const int r = 8 * (warp + 8 * j) + cl;   // accumulator columns are rows of the operator
-        if (r < rows) part[r * kSets + rl] = acc[j][0];
-        if (r + 1 < rows) part[(r + 1) * kSets + rl] = acc[j][1];
+        for (int j = 0; j < NT; ++j) {
+            const int r = 8 * (wt + lanes * j) + cl;   // accumulator columns are rows of the operator
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (r + q >= rows) continue;
+                double* d = part + (kpart * rows + r + q) * kSets + rl;
+                *d = first ? acc[j][q] : *d + acc[j][q];
+            }
+        }
+    }
     }
     cluster.sync();
     // sums over the cluster, normalisation and outputs: CTA `rank` takes the shells rank, rank + 8, ..
@@ -280,10 +373,22 @@ __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(256, 2) k_tem
         for (int i = tid; i < sets * a.n_slots; i += blockDim.x) {
             const int t = i % sets, si = i / sets, sl = a.slot[si];
             const double* th = a.params + 6 * (size_t)(t0 + t);
-            double s2 = 0.0, v = 0.0;
+            double sv[kCluster], pv[kCluster][KPARTS];
+#pragma unroll
             for (int c = 0; c < kCluster; ++c) {
-                s2 += *cluster.map_shared_rank(&s8part[t], c);
-                v += *cluster.map_shared_rank(part + (si * nbl + bl) * kSets + t, c);
+                sv[c] = *cluster.map_shared_rank(&s8part[t], c);
+                const double* pc = cluster.map_shared_rank(part + (si * nbl + bl) * kSets + t, c);
+#pragma unroll
+                for (int kp = 0; kp < KPARTS; ++kp) pv[c][kp] = pc[kp * rows * kSets];
+            }
+            double s2 = 0.0, v = 0.0;
+#pragma unroll
+            for (int c = 0; c < kCluster; ++c) {
+                s2 += sv[c];
+                double slab = pv[c][0];
+#pragma unroll
+                for (int kp = 1; kp < KPARTS; ++kp) slab += pv[c][kp];
+                v += slab;
             }
             const int kind = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
             const double amp = kind == 0 ? th[1] * th[1] : (kind == 1 ? th[0] * th[1] : th[0] * th[0]);
@@ -409,13 +514,14 @@ struct lpp_template_s {
     double png_amp = 0.0, png_len2 = 0.0;   // 12 f_NL delta b_IA and (c/H0)^2 / Omega_m
     unsigned slot_mask = (1u << kSlots) - 1u;
     int qx_rows = 0;
-    std::vector<double> kin, lnk, s8w, ain, rinv, rfwd, kfwd, qx, bin_w;
-    std::vector<double2> uinv, ufwd, tw;
+    std::vector<double> kin, lnk, ik, s8w, ain, rinv, rfwd, kfwd, qx, bin_w;
+    std::vector<double2> uinv, ufwd, tw, logtab;
+    double dlnk = 0.0;
     std::vector<int> bin_lo, bin_hi;
     SlotDesc slots[kSlots];
     // device
     char* ws = nullptr;
-    size_t ws_need = 0, o_kin, o_lnk, o_op, o_s8w, o_ain, o_uinv, o_rinv, o_ufwd, o_rfwd, o_kfwd, o_qx, o_tw, o_lo, o_hi, o_bw;
+    size_t ws_need = 0, o_kin, o_lnk, o_ik, o_logtab, o_op, o_s8w, o_ain, o_uinv, o_rinv, o_ufwd, o_rfwd, o_kfwd, o_qx, o_tw, o_lo, o_hi, o_bw;
     bool ready = false;
 };
 
@@ -434,6 +540,14 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
     const double kr0 = kKmin * r0;
     t->kin.resize(kNin);
     t->lnk.resize(kNin);
+    t->ik.resize(kNin);
+    t->dlnk = delta;
+    t->logtab.resize(128);
+    for (int i = 0; i < 128; ++i) {
+        // ln c from the rounded 1 / c that divides
+        const double ic = i == 0 ? 1.0 : 1.0 / (1.0 + (i + 0.5) / 128.0);
+        t->logtab[i] = make_double2(ic, i == 0 ? 0.0 : -log(ic));
+    }
     t->s8w.resize(kNin);
     t->ain.resize(kNin);
     t->kfwd.resize(kNin);
@@ -444,6 +558,7 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
         const double th = top_hat(8.0 * k);
         t->kin[n] = k;
         t->lnk[n] = log(kKmin) + n * delta;
+        t->ik[n] = 1.0 / (2.34 * k);
         t->s8w[n] = wtr * k * k * k / (2.0 * kPi * kPi) * th * th;
         t->ain[n] = k * k * k * taper_at(n) * pow(k, -kQinv);
         t->kfwd[n] = 4.0 * kPi * pow(k, -kQfwd);
@@ -526,6 +641,8 @@ extern "C" lpp_status lpp_template_create(const double* q, const double* s, int 
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
     t->o_kin = take(kNin * 8);
     t->o_lnk = take(kNin * 8);
+    t->o_ik = take(kNin * 8);
+    t->o_logtab = take(128 * 16);
     t->o_op = take((size_t)kSlots * n_bins * kNin * 8);
     t->o_s8w = take(kNin * 8);
     t->o_ain = take(kNin * 8);
@@ -564,6 +681,8 @@ extern "C" lpp_status lpp_template_set_workspace(lpp_template_t t, void* dev, si
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = put(t->o_kin, t->kin.data(), kNin * 8);
     if (e == cudaSuccess) e = put(t->o_lnk, t->lnk.data(), kNin * 8);
+    if (e == cudaSuccess) e = put(t->o_ik, t->ik.data(), kNin * 8);
+    if (e == cudaSuccess) e = put(t->o_logtab, t->logtab.data(), 128 * 16);
     if (e == cudaSuccess) e = put(t->o_s8w, t->s8w.data(), kNin * 8);
     if (e == cudaSuccess) e = put(t->o_ain, t->ain.data(), kNin * 8);
     if (e == cudaSuccess) e = put(t->o_uinv, t->uinv.data(), 3 * kNfft * 16);
@@ -647,6 +766,9 @@ static lpp_status convolve(lpp_template_t t, const double* params, int n_templat
     a.op = (const double*)(t->ws + t->o_op);
     a.kin = (const double*)(t->ws + t->o_kin);
     a.lnk = (const double*)(t->ws + t->o_lnk);
+    a.ik = (const double*)(t->ws + t->o_ik);
+    a.logtab = (const double2*)(t->ws + t->o_logtab);
+    a.dlnk = t->dlnk;
     a.s8w = (const double*)(t->ws + t->o_s8w);
     a.bin_lo = (const int*)(t->ws + t->o_lo);
     a.bin_hi = (const int*)(t->ws + t->o_hi);
@@ -667,9 +789,36 @@ static lpp_status convolve(lpp_template_t t, const double* params, int n_templat
     a.bins = (t->nb + groups - 1) / groups;
     while (a.bins > 1 && a.bins * ns > kMaxRows) --a.bins;
     groups = (t->nb + a.bins - 1) / a.bins;
-    const size_t smem = ((size_t)(t->png_amp != 0.0 ? 3 : 1) * kSets * kSlabPad +
-                         (size_t)std::max(1, a.n_slots * a.bins) * kSets) * sizeof(double);
-    cudaFuncSetAttribute(k_template, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_template<<<dim3(clusters * kCluster, groups), 256, smem, (cudaStream_t)stream>>>(a);
+    // few rows: a warp takes one column segment (at most four tiles each, so that all eight warps
+    // have work and few loads in a row)
+    const int rows = ns * a.bins, kparts = rows <= 64 ? kSegs : 1;
+    const int nt = ((rows + 7) / 8 + 8 / kparts - 1) / (8 / kparts);
+    const size_t smem = ((size_t)(t->png_amp != 0.0 ? 3 : 1) * kSets * kSlabPad + (size_t)kparts * rows * kSets) *
+                        sizeof(double);
+    auto launch = [&](void (*kernel)(TemplateArgs)) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        kernel<<<dim3(clusters * kCluster, groups), 256, smem, (cudaStream_t)stream>>>(a);
+    };
+    if (n_templates <= kFewSets) {
+        launch(k_template<1, 1, true>);
+    } else if (kparts == kSegs) {
+        switch (nt) {
+            case 1: launch(k_template<1, kSegs>); break;
+            case 2: launch(k_template<2, kSegs>); break;
+            case 3: launch(k_template<3, kSegs>); break;
+            default: launch(k_template<4, kSegs>); break;
+        }
+    } else {
+        switch (nt) {
+            case 2: launch(k_template<2, 1>); break;
+            case 3: launch(k_template<3, 1>); break;
+            case 4: launch(k_template<4, 1>); break;
+            case 5: launch(k_template<5, 1>); break;
+            case 6: launch(k_template<6, 1>); break;
+            case 7: launch(k_template<7, 1>); break;
+            case 8: launch(k_template<8, 1>); break;
+            default: launch(k_template<9, 1>); break;
+        }
+    }
     return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
 }
