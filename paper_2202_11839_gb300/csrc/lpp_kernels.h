@@ -325,8 +325,12 @@ template <typename T>
 cudaError_t launch_window_mult(c2<T>* grids, long long grid_stride, int n_grids, const c2<T>* pD, const T* inv_w,
                                int n, cudaStream_t st);
 struct SbinChan {
-    int grid, sub, l, m, out_row;
-    double ynorm;
+    int grid, sub, l, m;
+    double ynorm;   // normalisation of Y_{l,m} divided by (l - |m|)! (goes with ylm_poly_scaled)
+};
+// Consecutive channels c0 .. c1 - 1 of one degree, reduced together into output row out_row.
+struct SbinRun {
+    int c0, c1, out_row;
 };
 template <typename T>
 struct SbinArgs {
@@ -334,6 +338,8 @@ struct SbinArgs {
     long long grid_stride;
     int n, n_ch;
     SbinChan ch[kMaxBatchCh];
+    int n_runs;
+    SbinRun run[kMaxBatchCh];
     const int* thr;   // [nb+1] thresholds on the integer |s|^2 / h^2
     int nb;
     int ns_pos, ns_neg, nks;

@@ -26,41 +26,10 @@ template <> struct Owned<double> {
     static constexpr int words = 1;
 };
 
-template <typename T>
-__device__ __forceinline__ int freq_of(int i, int n) { return i < n / 2 ? i : i - n; }
-
-// segmented inclusive scan of (re, im) over lanes with equal segment keys, the keys monotone
-// along the warp (equal keys form one contiguous run); the last lane of each run adds the run
-// total to acc[bin][2].  key = bin when the shell labels themselves are monotone.
-template <typename T>
-__device__ __forceinline__ void warp_bin_add(T re, T im, int bin, T* acc, int key) {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int ok = __shfl_up_sync(full, key, d);
-        const T ore = __shfl_up_sync(full, re, d);
-        const T oim = __shfl_up_sync(full, im, d);
-        if (lane >= d && ok == key) {
-            re += ore;
-            im += oim;
-        }
-    }
-    const int nk = __shfl_down_sync(full, key, 1);
-    const bool last = (lane == 31) || (nk != key);
-    if (last && bin >= 0) {
-        atomicAdd(acc + 2 * bin, re);
-        atomicAdd(acc + 2 * bin + 1, im);
-    }
-}
-template <typename T>
-__device__ __forceinline__ void warp_bin_add(T re, T im, int bin, T* acc) {
-    warp_bin_add<T>(re, im, bin, acc, bin);
-}
-
-// The shell labels of a row are the same for every channel: the steps of the segmented scan
-// that add (bit s: lane >= 2^s and the lane 2^s below is in the same shell) and whether the
-// lane ends its segment are computed once per row.
+// Segmented inclusive scans over lanes with equal shells, the shells monotone along the warp
+// (equal shells form one contiguous run).  The steps that add (bit s: lane >= 2^s and the lane
+// 2^s below is in the same shell) and whether the lane ends its segment are the same for every
+// value of an item and computed once.
 struct SegMask {
     unsigned add;   // bit s set: add the value shuffled up by 2^s
     bool last;      // the lane holds its segment's sum after the scan

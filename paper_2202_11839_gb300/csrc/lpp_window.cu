@@ -8,6 +8,9 @@
 #include "lpp_internal.h"
 #include "lpp_kernels.h"
 #include "lpp_reduce.cuh"
+#include "lpp_ylm.cuh"
+
+#include <algorithm>
 
 namespace lpp {
 
@@ -73,34 +76,41 @@ cudaError_t launch_window_mult(c2<T>* grids, long long grid_stride, int n_grids,
     return cudaGetLastError();
 }
 
-// Shell sums over separations: rows (sz, sy) of the kept cube; lanes cover sx >= 0 and
-// sx < 0 in two halves so that |s| grows monotonically along each warp.
+// Shell sums over separations.  A warp takes 32 consecutive sx >= 0 or sx < 0 of one row (sz, sy)
+// of the kept cube, so that |s| grows monotonically along it.  The channels of one degree l enter
+// Q_l only through sum_n Y_ln(shat) C_n(s): they are contracted separation by separation and
+// reduced once per degree (a.run), into the warp's own accumulators (warp_own_add).
+// (One reduction, a harmonic with divisions and block barriers per channel and row before: 3.75 ms
+// of the 16 ms of kernels of a 256^3 call to 115 grid spacings.)
+constexpr int kSbinWarps = 8;
+
 template <typename T>
-__global__ void __launch_bounds__(1024) k_sbin(SbinArgs<T> a) {
+__global__ void __launch_bounds__(32 * kSbinWarps, sizeof(T) == 4 ? 3 : 2) k_sbin(const __grid_constant__ SbinArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n, nb = a.nb;
-    const int E = a.n_ch * nb * 2;
-    T* acc = reinterpret_cast<T*>(smem_raw);
-    T* own = acc + E;
-    int* thr = reinterpret_cast<int*>(own + E * Owned<T>::words);
-    const int tid = threadIdx.x, nthr = blockDim.x;
-    for (int i = tid; i < E; i += nthr) acc[i] = (T)0;
-    for (int i = tid; i < E * Owned<T>::words; i += nthr) own[i] = (T)0;
-    for (int i = tid; i <= nb; i += nthr) thr[i] = a.thr[i];
+    const int E = a.n_runs * nb * 2;
+    constexpr int W = Owned<T>::words, NW = kSbinWarps;
+    T* own = reinterpret_cast<T*>(smem_raw);                 // [NW][words][E]
+    int* thr = reinterpret_cast<int*>(own + NW * E * W);     // [nb+1]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int i = tid; i < NW * E * W; i += 32 * NW) own[i] = (T)0;
+    for (int i = tid; i <= nb; i += 32 * NW) thr[i] = a.thr[i];
     __syncthreads();
-    const int P = nthr / 2;
-    const int fx = tid < P ? tid : -1 - (tid - P);
-    const bool xvalid = tid < P ? (fx <= a.ns_pos) : (-fx <= a.ns_neg);
-    const int x = fx >= 0 ? fx : n + fx;
-    const int rows = a.nks * a.nks;
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
+    T* mine = own + warp * E * W;
+    const int npos = (a.ns_pos + 32) / 32, nseg = npos + (a.ns_neg + 31) / 32;
+    const int items = a.nks * a.nks * nseg;
+    for (int it = blockIdx.x * NW + warp; it < items; it += gridDim.x * NW) {
+        const int row = it / nseg, seg = it - row * nseg;
         const int zj = row / a.nks, yj = row - zj * a.nks;
         const int z = zj <= a.ns_pos ? zj : n - (a.nks - zj);
         const int y = yj <= a.ns_pos ? yj : n - (a.nks - yj);
         const int fz = z < n / 2 ? z : z - n, fy = y < n / 2 ? y : y - n;
+        const bool neg = seg >= npos;
+        const int ax = neg ? 32 * (seg - npos) + lane + 1 : 32 * seg + lane;   // |sx|
+        const int fx = neg ? -ax : ax;
         const int q2 = fx * fx + fy * fy + fz * fz;
         int bin = -1;
-        if (xvalid && q2 > 0 && q2 >= thr[0] && q2 < thr[nb]) {
+        if (ax <= (neg ? a.ns_neg : a.ns_pos) && q2 > 0 && q2 >= thr[0] && q2 < thr[nb]) {
             int lo = 0, hi = nb;
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
@@ -108,55 +118,56 @@ __global__ void __launch_bounds__(1024) k_sbin(SbinArgs<T> a) {
             }
             bin = lo;
         }
-        T sxh = 0, syh = 0, szh = 0;
-        long long idx = 0;
-        if (bin >= 0) {
-            const T inv = (T)1 / sqrt((T)q2);
-            sxh = fx * inv;
-            syh = fy * inv;
-            szh = fz * inv;
-            idx = ((long long)z * n + y) * n + x;
-        }
-        for (int ci = 0; ci < a.n_ch; ++ci) {
-            const SbinChan& ch = a.ch[ci];
+        if (!__any_sync(0xffffffffu, bin >= 0)) continue;
+        const SegMask segm = seg_mask(bin);
+        const T inv = bin >= 0 ? (T)1 / sqrt((T)q2) : (T)0;
+        Azimuth<T> az;
+        az.set((T)fx * inv, (T)fy * inv);
+        const T sz = (T)fz * inv;
+        const unsigned idx = bin >= 0 ? ((unsigned)z * n + y) * n + (fx >= 0 ? fx : n + fx) : 0u;
+        for (int ri = 0; ri < a.n_runs; ++ri) {
             T v = 0;
-            if (bin >= 0) {
-                const c2<T> c = a.grids[(long long)ch.grid * a.grid_stride + idx];
-                const T corr = (ch.sub ? c.y : c.x) * (T)a.scale;
-                v = (T)ch.ynorm * ylm_poly<T>(ch.l, ch.m, sxh, syh, szh) * corr;
+            for (int ci = a.run[ri].c0; ci < a.run[ri].c1; ci += 2) {
+                // channels n = +m and -m of one degree (m = 0: one)
+                const SbinChan &p = a.ch[ci], &q = a.ch[min(ci + 1, a.run[ri].c1 - 1)];
+                T cp = 0, cq = 0;
+                if (bin >= 0) {
+                    const c2<T> u = a.grids[(long long)p.grid * a.grid_stride + idx];
+                    const c2<T> w = a.grids[(long long)q.grid * a.grid_stride + idx];
+                    cp = p.sub ? u.y : u.x;
+                    cq = q.sub ? w.y : w.x;
+                }
+                const bool pair = ci + 1 < a.run[ri].c1 && q.m == -p.m && p.m != 0;
+                T yc, ys;
+                ylm_pair<T>(p.l, p.m < 0 ? -p.m : p.m, az, sz, yc, ys);
+                v += (T)p.ynorm * (p.m < 0 ? ys : yc) * cp;
+                if (pair) v += (T)q.ynorm * (q.m < 0 ? ys : yc) * cq;
+                else --ci;   // one channel this time
             }
-            warp_bin_add<T>(v, (T)0, bin, acc + ci * 2 * nb);
+            warp_own_add<T>(v * (T)a.scale, (T)0, bin, segm, mine + ri * 2 * nb, E);
         }
-        __syncthreads();
-        for (int i = tid; i < E; i += nthr) {
-            const T v = acc[i];
-            if (v != (T)0) {
-                Owned<T>::add(own + i, own + E + i, v);
-                acc[i] = (T)0;
-            }
-        }
-        __syncthreads();
     }
-    for (int i = tid; i < E; i += nthr) {
-        const double v = Owned<T>::value(own + i, own + E + i);
+    __syncthreads();
+    for (int i = tid; i < E; i += 32 * NW) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v += Owned<T>::value(own + w * E * W + i, own + w * E * W + (W - 1) * E + i);
         if (v != 0.0) {
-            const int ci = i / (2 * nb);
-            atomicAdd(a.out + (long long)a.ch[ci].out_row * 2 * nb + (i - ci * 2 * nb), v);
+            const int ri = i / (2 * nb);
+            atomicAdd(a.out + (long long)a.run[ri].out_row * 2 * nb + (i - ri * 2 * nb), v);
         }
     }
 }
 
 template <typename T>
 cudaError_t launch_sbin(const SbinArgs<T>& a, int n_sm, cudaStream_t st) {
-    const int P = ((a.ns_pos + 1) + 31) / 32 * 32;
-    const int threads = 2 * P;
-    const int E = a.n_ch * a.nb * 2;
-    const size_t smem = (size_t)E * sizeof(T) * (1 + Owned<T>::words) + (size_t)(a.nb + 1) * sizeof(int);
+    const int E = a.n_runs * a.nb * 2;
+    const size_t smem = (size_t)kSbinWarps * E * Owned<T>::words * sizeof(T) + (size_t)(a.nb + 1) * sizeof(int);
     cudaFuncSetAttribute(k_sbin<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int rows = a.nks * a.nks;
-    int blocks = n_sm * (threads <= 256 ? 8 : (threads <= 512 ? 4 : 2));
-    if (blocks > rows) blocks = rows;
-    k_sbin<T><<<blocks, threads, smem, st>>>(a);
+    const long long items = (long long)a.nks * a.nks * ((a.ns_pos + 32) / 32 + (a.ns_neg + 31) / 32);
+    const int blocks = (int)std::max(1LL, std::min<long long>((long long)n_sm * (sizeof(T) == 4 ? 3 : 2),
+                                                              (items + kSbinWarps - 1) / kSbinWarps));
+    k_sbin<T><<<blocks, 32 * kSbinWarps, smem, st>>>(a);
     return cudaGetLastError();
 }
 
