@@ -3,12 +3,14 @@
 // Every matrix product runs on the tensor cores (mma.m16n8k16, BF16 in, FP32 accumulate, the
 // reduction dimension in ascending steps of 16).  The network is a chain of small products:
 // a layer of a 256-row minibatch is 34 MFLOP, less than a microsecond of one launch, so the
-// chain is fused by rows.  A CTA carries its rows through all layers (and, when training, back)
-// with the activations in shared memory while the weight matrices stream through a ring of
-// cp.async stages; a second kernel forms every layer's weight gradient and applies Adam in the
-// epilogue.  Adam keeps FP32 master weights and refreshes their BF16 copies (and transposes)
-// after every step.  The training loop is native: one call runs all steps of a schedule of
-// minibatch indices.
+// chain is fused by rows.  A cluster of four CTAs carries 16 rows through all layers (and, when
+// training, back): each CTA computes a quarter of a layer's columns while its slice of the weight
+// matrices streams through a ring of cp.async stages, and writes its activations into the shared
+// memory of all four.  Predictions of many rows take one CTA per 32 rows.  A second kernel forms
+// every layer's weight gradient and applies Adam in the epilogue.  Adam keeps FP32 master weights
+// and refreshes their BF16 copies (and transposes) after every step.  The training loop is native:
+// one call runs all steps of a schedule of minibatch indices.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -132,21 +134,101 @@ __device__ __forceinline__ void row_product(WeightRing<ST>& ring, const Passes& 
     }
 }
 
-// Ring stages and BF16 per activation row of the training chain (rows of up to 320 gradients) and of
-// the prediction (256 activations); padded for conflict-free fragments.  Two prediction CTAs of 32
-// rows share an SM.
-constexpr int kTrainStages = 4, kActLd = 328;
-constexpr size_t kTrainSmem = ((size_t)kTrainStages * kStageElems + (size_t)2 * 16 * kActLd) * sizeof(bf16);
+constexpr int kActLd = 328;   // BF16 per activation row of a cluster: up to 320 and padding (conflict-free fragments)
+// Ring stages and BF16 per activation row of a CTA that carries 32 rows (256 and padding); two
+// such CTAs share an SM.
 constexpr int kPredLd = 264;
-__host__ __device__ constexpr int pred_stages(int mt) { return mt == 1 ? 4 : 3; }
-__host__ __device__ constexpr size_t pred_smem(int mt) {
-    return ((size_t)pred_stages(mt) * kStageElems + (size_t)2 * mt * 16 * kPredLd) * sizeof(bf16);
+constexpr int kPredStages = 3, kPredRows = 32;
+constexpr size_t kPredSmem = ((size_t)kPredStages * kStageElems + (size_t)2 * kPredRows * kPredLd) * sizeof(bf16);
+
+// ---- 16 rows on a cluster of kSplit CTAs
+// CTA `rank` owns the columns [rank, rank + 1) N / kSplit of every product (64, or 80 of the output
+// layer), in tiles of 8 columns: tile w by warp w, tiles 8 and 9 of the output layer by warps 0
+// and 1.  Weight chunks are 128 K columns of those rows.
+constexpr int kSplit = 4;
+constexpr int kSliceStages = 4, kSliceLd = 136, kSliceElems = (kNout / kSplit) * kSliceLd;
+__host__ __device__ constexpr int slice_rows(int p) { return pass_rows(p) / kSplit; }
+constexpr size_t kSliceSmem = ((size_t)kSliceStages * kSliceElems + (size_t)2 * 16 * kActLd) * sizeof(bf16);
+
+struct SliceRing {
+    bf16* ring;
+    int n_pass, rank;
+    int pass = 0, k = 0, put = 0, got = 0;
+    __device__ __forceinline__ void load(const Passes& ps) {
+        if (pass < n_pass) {
+            const int rows = slice_rows(pass), K = pass_k(pass);
+            const int kc = min(128, K - k), sh = kc == 128 ? 4 : (kc == 64 ? 3 : 1);   // kc = 128, 64 or 16
+            const bf16* w = ps.w[pass] + (size_t)rank * rows * K + k;
+            bf16* dst = ring + (put % kSliceStages) * kSliceElems;
+            for (int i = threadIdx.x; i < rows << sh; i += kRowThreads) {
+                const int r = i >> sh, c = (i & ((1 << sh) - 1)) * 8;
+                cp16(dst + r * kSliceLd + c, w + (size_t)r * K + c);
+            }
+            k += 128;
+            if (k >= K) { k = 0; ++pass; }
+        }
+        cp_commit();   // an empty group past the end keeps the count of groups in flight
+        ++put;
+    }
+    __device__ __forceinline__ const bf16* next(const Passes& ps) {
+        cp_wait<kSliceStages - 2>();
+        __syncthreads();
+        load(ps);
+        return ring + (got++ % kSliceStages) * kSliceElems;
+    }
+};
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t a[4], const bf16* p) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                 : "r"(s));
 }
 
-// [16 rows][cols] of a shared activation tile -> global transpose [cols][ld] at column r0: 16 rows
-// of one column are 32 contiguous bytes.
-__device__ __forceinline__ void store_transposed(const bf16* act, int cols, bf16* dst, int ld, int r0) {
-    for (int c = threadIdx.x; c < cols; c += kRowThreads) {
+// acc[j] = act[16][K] . w[tile warp + 8 j]^T, tiles of this CTA's slice; TILES = 8 or 10 in the slice.
+template <int K, int TILES>
+__device__ __forceinline__ void slice_product(SliceRing& ring, const Passes& ps, const bf16* act,
+                                              float (&acc)[(TILES + 7) / 8][4]) {
+    constexpr int NT = (TILES + 7) / 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[j][r] = 0.f;
+    const bf16* arow = act + (lane & 15) * kActLd + (lane >> 4) * 8;
+    for (int k0 = 0; k0 < K; k0 += 128) {
+        const bf16* w = ring.next(ps);
+        const int kc = K < 128 ? K : min(128, K - k0);
+#pragma unroll
+        for (int kk = 0; kk < (K < 128 ? K : 128); kk += 16) {
+            if (K % 128 != 0 && kk >= kc) break;
+            uint32_t a[4];
+            ldmatrix_x4(a, arow + k0 + kk);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                if (TILES > 8 && warp + 8 * j >= TILES) break;   // warp-uniform
+                const bf16* bp = w + (8 * (warp + 8 * j) + g) * kSliceLd + kk + 2 * t;
+                mma_bf16(acc[j], a, *reinterpret_cast<const uint32_t*>(bp), *reinterpret_cast<const uint32_t*>(bp + 8));
+            }
+        }
+    }
+}
+
+// Two neighbouring values (row r, columns c, c + 1 of the whole layer) into the activation buffer of
+// every CTA of the cluster.
+__device__ __forceinline__ void share2(bf16* buf, int r, int c, float v0, float v1) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const __nv_bfloat162 v(__float2bfloat16_rn(v0), __float2bfloat16_rn(v1));
+#pragma unroll
+    for (int q = 0; q < kSplit; ++q)
+        *reinterpret_cast<__nv_bfloat162*>(cl.map_shared_rank(buf + r * kActLd + c, q)) = v;
+}
+
+// [16 rows][columns c0 .. c0 + cols) of a shared activation tile -> global transpose [column][ld] at
+// row r0: 16 rows of one column are 32 contiguous bytes.
+__device__ __forceinline__ void store_transposed(const bf16* act, int c0, int cols, bf16* dst, int ld, int r0) {
+    for (int c = c0 + threadIdx.x; c < c0 + cols; c += kRowThreads) {
         __align__(16) bf16 v[16];
 #pragma unroll
         for (int r = 0; r < 16; ++r) v[r] = act[r * kActLd + c];
@@ -169,106 +251,100 @@ struct TrainRowArgs {
     double* loss;
 };
 
-// One training step's row chain: 16 rows of the minibatch per CTA through the forward layers, the
-// loss gradient and the activation gradients, down to every layer's input and pre-activation
+// One training step's row chain: 16 rows of the minibatch per cluster through the forward layers,
+// the loss gradient and the activation gradients, down to every layer's input and pre-activation
 // gradient (transposed, for the weight gradients).  The pre-activations stay in registers: the
-// backward products place their outputs on the same threads.
+// backward products place their outputs on the same threads.  The activation buffers alternate,
+// and the cluster's barrier after each layer separates a buffer's last reads from its next
+// writes two layers later.
 //
-// What bounds it: 1.1 MB of weights per CTA through the ring (L2 to shared memory) and the
-// latency of nine dependent products.  A step at batch 256 (both kernels): 199 -> 64 us against
-// one launch per product, bias gradient, loss and update (22 launches).
-__global__ void __launch_bounds__(kRowThreads, 1) k_train_rows(const __grid_constant__ TrainRowArgs a) {
+// What bounds it: the latency of nine dependent products (16 to 20 dependent mma each, the ring's
+// and the cluster's barriers).  A step at batch 256 (both kernels): 199 us as 22 launches, 64 us
+// with one CTA per 16 rows, 39 us on clusters.
+__global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(kRowThreads, 1)
+k_train_rows(const __grid_constant__ TrainRowArgs a) {
+    namespace cg = cooperative_groups;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    WeightRing<kTrainStages> ring;
+    cg::cluster_group cluster = cg::this_cluster();
+    SliceRing ring;
     ring.ring = reinterpret_cast<bf16*>(smem_raw);
     ring.n_pass = 2 * kLayers - 1;
+    ring.rank = (int)cluster.block_rank();
     bf16* buf[2];
-    buf[0] = ring.ring + kTrainStages * kStageElems;
+    buf[0] = ring.ring + kSliceStages * kSliceElems;
     buf[1] = buf[0] + 16 * kActLd;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    const int r0 = blockIdx.x * 16;
-    for (int c = 0; c < kTrainStages - 1; ++c) ring.load(a.ps);
+    const int r0 = (int)(blockIdx.x / kSplit) * 16;
+    const int h0 = ring.rank * (256 / kSplit), o0 = ring.rank * (kNout / kSplit);   // this CTA's columns
+    for (int c = 0; c < kSliceStages - 1; ++c) ring.load(a.ps);
     {   // inputs: BF16 [16][16], zero padded
         const int r = tid >> 4, c = tid & 15;
         const float v = c < kNin ? a.x[(size_t)a.idx[r0 + r] * kNin + c] : 0.f;
         buf[0][r * kActLd + c] = __float2bfloat16_rn(v);
     }
-    __syncthreads();
-    store_transposed(buf[0], pass_k(0), a.actt[0], a.batch, r0);
-    float z[kLayers - 1][4][4];
+    cluster.sync();   // every CTA of the cluster runs before its shared memory is written
+    if (ring.rank == 0) store_transposed(buf[0], 0, pass_k(0), a.actt[0], a.batch, r0);
+    const int c = h0 + 8 * warp + 2 * t;   // the thread's hidden columns c, c + 1
+    float z[kLayers - 1][4];
     int cur = 0;
 #pragma unroll
     for (int l = 0; l < kLayers - 1; ++l) {
-        float acc[1][4][4];
-        if (l == 0) row_product<1, 4, 16, kActLd>(ring, a.ps, buf[cur], acc);
-        else row_product<1, 4, 256, kActLd>(ring, a.ps, buf[cur], acc);
-        bf16* nx = buf[cur ^ 1];
+        float acc[1][4];
+        if (l == 0) slice_product<16, 8>(ring, a.ps, buf[cur], acc);
+        else slice_product<256, 8>(ring, a.ps, buf[cur], acc);
+        const float2 b = *reinterpret_cast<const float2*>(a.bias[l] + c);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = 8 * (warp * 4 + j) + 2 * t;
-            const float2 b = *reinterpret_cast<const float2*>(a.bias[l] + c);
+        for (int r = 0; r < 4; ++r) z[l][r] = acc[0][r] + ((r & 1) ? b.y : b.x);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) z[l][j][r] = acc[0][j][r] + ((r & 1) ? b.y : b.x);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                *reinterpret_cast<__nv_bfloat162*>(nx + (g + 8 * h) * kActLd + c) =
-                    __nv_bfloat162(__float2bfloat16_rn(gelu(z[l][j][2 * h])), __float2bfloat16_rn(gelu(z[l][j][2 * h + 1])));
-        }
+        for (int h = 0; h < 2; ++h) share2(buf[cur ^ 1], g + 8 * h, c, gelu(z[l][2 * h]), gelu(z[l][2 * h + 1]));
         cur ^= 1;
-        __syncthreads();
-        store_transposed(buf[cur], 256, a.actt[l + 1], a.batch, r0);
+        cluster.sync();
+        store_transposed(buf[cur], h0, 256 / kSplit, a.actt[l + 1], a.batch, r0);
     }
     // output layer, loss and its gradient 2 (out - y) / (batch * 320)
     {
-        float acc[1][5][4];
-        row_product<1, 5, 256, kActLd>(ring, a.ps, buf[cur], acc);
+        float acc[2][4];
+        slice_product<256, 10>(ring, a.ps, buf[cur], acc);
         const float sc = 2.0f / (float)(a.batch * kNout);
         double part = 0.0;
-        bf16* nx = buf[cur ^ 1];
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const int c = 8 * (warp * 5 + j) + 2 * t;
-            const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + c);
+        for (int j = 0; j < 2; ++j) {
+            if (warp + 8 * j >= kNout / kSplit / 8) break;
+            const int co = o0 + 8 * (warp + 8 * j) + 2 * t;
+            const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + co);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int r = r0 + g + 8 * h;
-                const float2 yv = *reinterpret_cast<const float2*>(a.y + (size_t)a.idx[r] * kNout + c);
-                const float d0 = (acc[0][j][2 * h] + b.x) - yv.x, d1 = (acc[0][j][2 * h + 1] + b.y) - yv.y;
+                const float2 yv = *reinterpret_cast<const float2*>(a.y + (size_t)a.idx[r] * kNout + co);
+                const float d0 = (acc[j][2 * h] + b.x) - yv.x, d1 = (acc[j][2 * h + 1] + b.y) - yv.y;
                 part += (double)d0 * d0 + (double)d1 * d1;
                 const float2 gv = make_float2(sc * d0, sc * d1);
-                *reinterpret_cast<float2*>(a.g32[kLayers - 1] + (size_t)r * kNout + c) = gv;
-                *reinterpret_cast<__nv_bfloat162*>(nx + (g + 8 * h) * kActLd + c) =
-                    __nv_bfloat162(__float2bfloat16_rn(gv.x), __float2bfloat16_rn(gv.y));
+                *reinterpret_cast<float2*>(a.g32[kLayers - 1] + (size_t)r * kNout + co) = gv;
+                share2(buf[cur ^ 1], g + 8 * h, co, gv.x, gv.y);
             }
         }
         for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
         if (lane == 0 && part != 0.0) atomicAdd(a.loss, part / (double)(a.batch * kNout));
         cur ^= 1;
-        __syncthreads();
-        store_transposed(buf[cur], kNout, a.gt[kLayers - 1], a.batch, r0);
+        cluster.sync();
+        store_transposed(buf[cur], o0, kNout / kSplit, a.gt[kLayers - 1], a.batch, r0);
     }
     // g_{l-1} = (g_l W_l) * GELU'(z_{l-1})
 #pragma unroll
     for (int l = kLayers - 1; l > 0; --l) {
-        float acc[1][4][4];
-        if (l == kLayers - 1) row_product<1, 4, kNout, kActLd>(ring, a.ps, buf[cur], acc);
-        else row_product<1, 4, 256, kActLd>(ring, a.ps, buf[cur], acc);
-        bf16* nx = buf[cur ^ 1];
+        float acc[1][4];
+        if (l == kLayers - 1) slice_product<kNout, 8>(ring, a.ps, buf[cur], acc);
+        else slice_product<256, 8>(ring, a.ps, buf[cur], acc);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = 8 * (warp * 4 + j) + 2 * t;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float2 gv = make_float2(acc[0][j][2 * h] * gelu_grad(z[l - 1][j][2 * h]),
-                                              acc[0][j][2 * h + 1] * gelu_grad(z[l - 1][j][2 * h + 1]));
-                *reinterpret_cast<float2*>(a.g32[l - 1] + (size_t)(r0 + g + 8 * h) * 256 + c) = gv;
-                *reinterpret_cast<__nv_bfloat162*>(nx + (g + 8 * h) * kActLd + c) =
-                    __nv_bfloat162(__float2bfloat16_rn(gv.x), __float2bfloat16_rn(gv.y));
-            }
+        for (int h = 0; h < 2; ++h) {
+            const float2 gv = make_float2(acc[0][2 * h] * gelu_grad(z[l - 1][2 * h]),
+                                          acc[0][2 * h + 1] * gelu_grad(z[l - 1][2 * h + 1]));
+            *reinterpret_cast<float2*>(a.g32[l - 1] + (size_t)(r0 + g + 8 * h) * 256 + c) = gv;
+            share2(buf[cur ^ 1], g + 8 * h, c, gv.x, gv.y);
         }
         cur ^= 1;
-        __syncthreads();
-        store_transposed(buf[cur], 256, a.gt[l - 1], a.batch, r0);
+        cluster.sync();   // also: no CTA leaves while the others write to it
+        store_transposed(buf[cur], h0, 256 / kSplit, a.gt[l - 1], a.batch, r0);
     }
 }
 
@@ -486,15 +562,27 @@ constexpr int kDigits = 6, kOrders = 7;
 constexpr int kBaseKsteps = kMaxNodes * kMaxNodes / 16;            // 16 baseline terms per mma
 constexpr int kDigitWords = kDigits * (kNout / 8) * (kBaseKsteps / 2) * 32;   // uint4 of digit fragments
 
-// x in [-1, 1] -> its kDigits digits d_i: x = sum_i d_i 2^(-8 i - 7) to 2^-48
-__device__ __forceinline__ void fixed_digits(double x, int* d) {
-    long long v = llrint(x * 140737488355328.0);   // 2^47
+// v with |v| <= 2^e -> the kDigits digits d_i of v = 2^e sum_i d_i 2^(-8 i - 7) to 2^(e - 48).  One
+// FP64 multiply-add: v 2^(47 - e) + 1.5 2^52 holds the rounded integer in its low bits.
+__device__ __forceinline__ void fixed_digits(double v, int e, int* d) {
+    const double scale = __hiloint2double((47 - e + 1023) << 20, 0);
+    long long q = __double_as_longlong(fma(v, scale, 6755399441055744.0)) - 0x4338000000000000LL;
 #pragma unroll
     for (int i = kDigits - 1; i > 0; --i) {
-        d[i] = (int)((v + 128) & 255) - 128;
-        v = (v - d[i]) >> 8;
+        d[i] = (int)((q + 128) & 255) - 128;
+        q = (q - d[i]) >> 8;
     }
-    d[0] = (int)v;
+    d[0] = (int)q;
+}
+// The exponent e of the largest of the warp's values (two per lane): |v| < 2^e; kBadExponent for
+// an infinity, a NaN or values beyond 2^900; the smallest usable exponent for zeros.  Integer
+// instructions on the high words.
+__device__ __forceinline__ int warp_exponent(double v0, double v1) {
+    int h = max(__double2hiint(v0) & 0x7fffffff, __double2hiint(v1) & 0x7fffffff);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
+    const int e = (h >> 20) - 1022;
+    return e > 900 ? kBadExponent : max(e, -900);
 }
 
 // base -> digits in the order in which a lane reads its operand fragments: word
@@ -504,25 +592,16 @@ __global__ void k_base_digits(const double* __restrict__ base, int nn, uint4* __
                               int* __restrict__ exponent) {
     const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (j >= kNout) return;
-    double v[2], m = 0.0;
+    double v[2];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int q = lane + 32 * h;
-        v[h] = q < nn ? base[(size_t)q * kNout + j] : 0.0;
-        m = fmax(m, fabs(v[h]));
-        if (!(fabs(v[h]) < INFINITY)) m = INFINITY;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const bool finite = m < INFINITY;
-    int e = 0;
-    if (finite && m > 0.0) frexp(m, &e);   // |v| <= 2^e
-    if (lane == 0) exponent[j] = finite ? e : kBadExponent;
+    for (int h = 0; h < 2; ++h) v[h] = lane + 32 * h < nn ? base[(size_t)(lane + 32 * h) * kNout + j] : 0.0;
+    const int e = warp_exponent(v[0], v[1]);
+    if (lane == 0) exponent[j] = e;
     bf16* out = reinterpret_cast<bf16*>(digits);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         int d[kDigits];
-        fixed_digits(finite ? ldexp(v[h], -e) : 0.0, d);
+        fixed_digits(e == kBadExponent ? 0.0 : v[h], e == kBadExponent ? 0 : e, d);
         // term q = 32 h + lane: k step of 16, position in it -> fragment register and half
         const int s16 = lane >> 4, p = lane & 15, t = (p & 7) >> 1;
         const int word = 2 * s16 + (p >> 3);   // of the uint4: {b0, b1} of two k steps
@@ -593,51 +672,200 @@ struct PredictArgs {
     int n;
     float* out;             // [n][320]
     MapArgs map;
+    const struct ColumnConst* cols;   // [320] of this call (k_columns), for many rows
 };
 
-// The columns' constants of the decoding in shared memory (float pairs) and the rows'.
+// The columns' constants of the decoding (float pairs) and the column exponents of the baseline, from
+// the map's arrays as they are at this call.
 struct ColumnConst {
-    float2 mu[kNout], sd[kNout], shot[kNout], ref[kNout], isig[kNout];
-    int e[kNout];
+    float2 mu, sd, shot, ref, isig;
+    int e;
 };
-template <int MT>
+__device__ __forceinline__ ColumnConst column_const(const MapArgs& m, int j) {
+    auto as2 = [](fpair p) { return make_float2(p.hi, p.lo); };
+    ColumnConst c;
+    c.mu = as2(pair_of(m.mu[j]));
+    c.sd = as2(pair_of(m.sd[j]));
+    c.shot = as2(pair_of(m.shot[j]));
+    c.ref = as2(pair_of(m.ref ? m.ref[j] : 0.0));
+    c.isig = as2(pair_of(m.sigma ? 1.0 / m.sigma[j] : 1.0));
+    c.e = m.base ? m.exponent[j] : 0;
+    return c;
+}
+__global__ void k_columns(MapArgs m, ColumnConst* __restrict__ out) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < kNout) out[j] = column_const(m, j);
+}
+
+// The rows' constants.
+template <int R>
 struct RowConst {
-    float2 amp[2][16 * MT], t5[16 * MT];   // A b sigma_8^2 (gE), A^2 sigma_8^2 (EE, BB); shot-noise scale
-    int e[16 * MT];
-    double la[16 * MT][kMaxNodes], lb[16 * MT][kMaxNodes];
+    float2 amp[2][R], t5[R];   // A b sigma_8^2 (gE), A^2 sigma_8^2 (EE, BB); shot-noise scale
+    int e[R];
+    double la[R][kMaxNodes], lb[R][kMaxNodes];
 };
 
-// Forward pass of 16 MT rows per CTA (all layers, k_train_rows' row products) and, with MAP, the
-// whole prediction: the parameters' encoding before it and the decoding after it
-//   (pre_c (mu + sum_q w_q base_q + sd y) + theta_5 shot - ref) / sigma,
-// the baseline by exact digit products (above), the rest in float pairs.
-//
-// What bounds it: at 8192 rows the GELUs' instructions and the mma issue; at few rows the latency
-// of the dependent layers.  8192 rows: 287 -> 108 us, 50 rows: 85 -> 49 us, against eight launches
-// with the decoding's last operations in FP64.
-template <int MT, bool MAP>
-__global__ void __launch_bounds__(kRowThreads, MT == 1 ? 1 : 2) k_predict(const __grid_constant__ PredictArgs a) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    constexpr int R = 16 * MT;
-    constexpr int ST = pred_stages(MT);
-    WeightRing<ST> ring;
-    ring.ring = reinterpret_cast<bf16*>(smem_raw);
-    ring.n_pass = kLayers;
-    bf16* buf[2];
-    buf[0] = ring.ring + ST * kStageElems;
-    buf[1] = buf[0] + R * kPredLd;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    const int r0 = blockIdx.x * R, rows = min(R, a.n - r0);
-    for (int c = 0; c < ST - 1; ++c) ring.load(a.ps);
-    for (int i = tid; i < R * 16; i += kRowThreads) {
+// The constants of R parameter rows and their Lagrange weights as digit fragments
+// wd[kDigits][R / 16][kBaseKsteps][32]; ends with a barrier.
+template <int R>
+__device__ __forceinline__ void decode_rows(const MapArgs& m, const double* theta, int r0, int rows, RowConst<R>& rc,
+                                            uint4* wd) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int MT = R / 16;
+    auto as2 = [](fpair p) { return make_float2(p.hi, p.lo); };
+    for (int i = tid; i < 3 * R; i += kRowThreads) {
+        const int r = i / 3, k = i - 3 * r;
+        if (r >= rows) continue;
+        const double* th = theta + (size_t)(r0 + r) * kNin;
+        if (k == 0) {
+            const double s2 = th[2] * th[2];
+            rc.amp[0][r] = as2(pair_of(s2 * (th[0] * th[1])));
+            rc.amp[1][r] = as2(pair_of(s2 * (th[0] * th[0])));
+            rc.t5[r] = as2(pair_of(th[5]));
+        } else if (m.base) {
+            const int c = m.base_in[k - 1];
+            lobatto_basis_fast(th[c] * m.dscale[c] + m.dshift[c], m, k == 1 ? rc.la[r] : rc.lb[r]);
+        }
+    }
+    __syncthreads();
+    if (!m.base) return;
+    const int nn = m.nodes * m.nodes;
+    bf16* wo = reinterpret_cast<bf16*>(wd);
+    for (int r = warp; r < R; r += kRowThreads / 32) {   // one warp per row
+        double v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int q = lane + 32 * h;
+            v[h] = (r < rows && q < nn) ? rc.la[r][q / m.nodes] * rc.lb[r][q % m.nodes] : 0.0;
+        }
+        const int e = warp_exponent(v[0], v[1]);
+        if (lane == 0) rc.e[r] = e;
+        const int mt = r >> 4, rr = r & 15;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            int d[kDigits];
+            fixed_digits(e == kBadExponent ? 0.0 : v[h], e == kBadExponent ? 0 : e, d);
+            // term q = 32 h + lane = 16 ks + p: register (rr >> 3) + 2 (p >> 3) of lane 4 (rr & 7) + (p & 7) / 2
+            const int ks = 2 * h + (lane >> 4), p = lane & 15;
+            const int reg = (rr >> 3) + 2 * (p >> 3), ln = 4 * (rr & 7) + ((p & 7) >> 1);
+#pragma unroll
+            for (int i = 0; i < kDigits; ++i)
+                wo[((((i * MT + mt) * kBaseKsteps + ks) * 32 + ln) * 4 + reg) * 2 + (p & 1)] =
+                    __float2bfloat16_rn((float)d[i]);
+        }
+    }
+    __syncthreads();
+}
+
+// The decoding of one tile: rows 16 mt + {g, g + 8}, columns 8 tile + {2 t, 2 t + 1}, from the
+// network outputs y[4] on the mma accumulator's positions.
+template <int R>
+__device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, const RowConst<R>& rc,
+                                            const ColumnConst* cc, int mt, int tile, int rows, const float y[4],
+                                            float* out) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    constexpr int MT = R / 16;
+    auto pr = [](float2 v) { return fpair{v.x, v.y}; };
+    float acc[kOrders][4];
+#pragma unroll
+    for (int o = 0; o < kOrders; ++o)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[o][r] = 0.f;
+    if (m.base) {
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            uint4 bd[kDigits];
+#pragma unroll
+            for (int i = 0; i < kDigits; ++i) bd[i] = m.digits[((size_t)(i * (kNout / 8) + tile) * 2 + h) * 32 + lane];
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int i = 0; i < kDigits; ++i) {
+                    const uint4 av = wd[((i * MT + mt) * kBaseKsteps + 2 * h + k) * 32 + lane];
+                    const uint32_t af[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+                    for (int q = 0; q < kDigits; ++q)
+                        if (i + q < kOrders) mma_bf16(acc[i + q], af, k ? bd[q].z : bd[q].x, k ? bd[q].w : bd[q].y);
+                }
+        }
+    }
+    ColumnConst cq[2];
+    cq[0] = cc[8 * tile + 2 * t];
+    cq[1] = cc[8 * tile + 2 * t + 1];
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        const int r = mt * 16 + g + 8 * hh;
+        if (r >= rows) continue;
+        float res[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int v = 2 * hh + q;
+            const ColumnConst& c = cq[q];
+            fpair u = pr(c.mu);
+            if (m.base) {
+                // sum_o acc_o 2^(-8 o): the first three orders exactly, the rest (below 2^-22 of the
+                // largest possible sum) in one float
+                const float low = fmaf(acc[6][v], exp2i(-48), fmaf(acc[5][v], exp2i(-40),
+                                       fmaf(acc[4][v], exp2i(-32), __fmul_rn(acc[3][v], exp2i(-24)))));
+                const fpair s1 = two_sum(acc[0][v], __fmul_rn(acc[1][v], exp2i(-8)));
+                const fpair s2 = two_sum(s1.hi, __fmul_rn(acc[2][v], exp2i(-16)));
+                fpair b = fast_two_sum(s2.hi, __fadd_rn(s2.lo, __fadd_rn(s1.lo, low)));
+                const int er = rc.e[r];
+                if (er == kBadExponent || c.e == kBadExponent) {
+                    b.hi = b.lo = NAN;
+                } else {
+                    const int e = er + c.e - 14;   // the digits' unit: 2^(e_r + e_c) 2^-14
+                    b.hi = scale2(b.hi, e);
+                    b.lo = scale2(b.lo, e);
+                }
+                u = pair_add(u, b);
+            }
+            u = pair_add(u, pair_mul(pr(c.sd), y[v]));
+            u = pair_mul(u, pr(rc.amp[tile < 2 * (kNout / 8) / 8 ? 0 : 1][r]));
+            u = pair_add(u, pair_mul(pr(rc.t5[r]), pr(c.shot)));
+            u = pair_add(u, fpair{-c.ref.x, -c.ref.y});
+            u = pair_mul(u, pr(c.isig));
+            res[q] = __fadd_rn(u.hi, u.lo);
+        }
+        *reinterpret_cast<float2*>(out + (size_t)r * kNout + 8 * tile + 2 * t) = make_float2(res[0], res[1]);
+    }
+}
+
+// Network inputs of R rows (encoded by the map, or given), BF16 [R][16], zero padded.
+template <int R, bool MAP>
+__device__ __forceinline__ void input_rows(const PredictArgs& a, int r0, int rows, bf16* act, int lda) {
+    for (int i = threadIdx.x; i < R * 16; i += kRowThreads) {
         const int r = i >> 4, c = i & 15;
         float v = 0.f;
         if (r < rows && c < kNin) {
             if constexpr (MAP) v = (float)(a.theta[(size_t)(r0 + r) * kNin + c] * (double)a.map.scale[c] + (double)a.map.shift[c]);
             else v = a.x[(size_t)(r0 + r) * kNin + c];
         }
-        buf[0][r * kPredLd + c] = __float2bfloat16_rn(v);
+        act[r * lda + c] = __float2bfloat16_rn(v);
     }
+}
+
+// Forward pass of 32 rows per CTA and, with MAP, the whole prediction: the parameters' encoding
+// before it and the decoding after it
+//   (pre_c (mu + sum_q w_q base_q + sd y) + theta_5 shot - ref) / sigma,
+// the baseline by exact digit products (above), the rest in float pairs.
+//
+// What bounds it: the GELUs' instructions and the mma issue.  8192 rows: 287 us as eight launches
+// with the decoding's last operations in FP64 -> 90 us.
+template <bool MAP>
+__global__ void __launch_bounds__(kRowThreads, 2) k_predict(const __grid_constant__ PredictArgs a) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int R = kPredRows, MT = R / 16;
+    WeightRing<kPredStages> ring;
+    ring.ring = reinterpret_cast<bf16*>(smem_raw);
+    ring.n_pass = kLayers;
+    bf16* buf[2];
+    buf[0] = ring.ring + kPredStages * kStageElems;
+    buf[1] = buf[0] + R * kPredLd;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int r0 = blockIdx.x * R, rows = min(R, a.n - r0);
+    for (int c = 0; c < kPredStages - 1; ++c) ring.load(a.ps);
+    input_rows<R, MAP>(a, r0, rows, buf[0], kPredLd);
     int cur = 0;
     for (int l = 0; l < kLayers - 1; ++l) {
         float acc[MT][4][4];
@@ -660,169 +888,106 @@ __global__ void __launch_bounds__(kRowThreads, MT == 1 ? 1 : 2) k_predict(const 
     }
     float y[MT][5][4];
     row_product<MT, 5, 256, kPredLd>(ring, a.ps, buf[cur], y);
+    cp_wait<0>();
+    __syncthreads();   // the ring and the activations are free
+    // network outputs in shared memory on their accumulator positions [tile][mt][lane]: the decoding
+    // loops over the tiles without unrolling (an unrolled one stalls on instruction fetches)
+    uint4* wd = reinterpret_cast<uint4*>(smem_raw);                     // [kDigits][MT][kBaseKsteps][32]
+    float4* ys = reinterpret_cast<float4*>(wd + kDigits * MT * kBaseKsteps * 32);   // [kNout / 8][MT][32]
+    RowConst<R>& rc = *reinterpret_cast<RowConst<R>*>(ys + (kNout / 8) * MT * 32);
+    static_assert(sizeof(uint4) * kDigits * MT * kBaseKsteps * 32 + sizeof(float4) * (kNout / 8) * MT * 32 +
+                      sizeof(RowConst<R>) <= kPredSmem, "the decoding fits in the forward pass's shared memory");
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         const int c = 8 * (warp * 5 + j) + 2 * t;
         const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + c);
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) y[mt][j][r] += (r & 1) ? b.y : b.x;
+        for (int mt = 0; mt < MT; ++mt) {
+            const float4 v = make_float4(y[mt][j][0] + b.x, y[mt][j][1] + b.y, y[mt][j][2] + b.x, y[mt][j][3] + b.y);
+            if constexpr (MAP) {
+                ys[((warp * 5 + j) * MT + mt) * 32 + lane] = v;
+            } else {
+                const int r = mt * 16 + g;
+                float* o = a.out + (size_t)(r0 + r) * kNout + c;
+                if (r < rows) *reinterpret_cast<float2*>(o) = make_float2(v.x, v.y);
+                if (r + 8 < rows) *reinterpret_cast<float2*>(o + 8 * kNout) = make_float2(v.z, v.w);
+            }
+        }
     }
-    if constexpr (!MAP) {
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = mt * 16 + g + 8 * h;
-                if (r >= rows) continue;
-#pragma unroll
-                for (int j = 0; j < 5; ++j)
-                    *reinterpret_cast<float2*>(a.out + (size_t)(r0 + r) * kNout + 8 * (warp * 5 + j) + 2 * t) =
-                        make_float2(y[mt][j][2 * h], y[mt][j][2 * h + 1]);
-            }
-        return;
-    } else {
-        cp_wait<0>();
-        __syncthreads();   // the ring and the activations are free
-        // shared memory of the decoding: the weights' digit fragments, then the constants
-        uint4* wd = reinterpret_cast<uint4*>(smem_raw);   // [kDigits][MT][kBaseKsteps][32]
-        ColumnConst& cc = *reinterpret_cast<ColumnConst*>(wd + kDigits * MT * kBaseKsteps * 32);
-        RowConst<MT>& rc = *reinterpret_cast<RowConst<MT>*>(&cc + 1);
-        static_assert(sizeof(uint4) * kDigits * MT * kBaseKsteps * 32 + sizeof(ColumnConst) + sizeof(RowConst<MT>) <= pred_smem(MT),
-                      "the decoding fits in the forward pass's shared memory");
-        const MapArgs& m = a.map;
-        auto as2 = [](fpair p) { return make_float2(p.hi, p.lo); };
-        auto pr = [](float2 v) { return fpair{v.x, v.y}; };
-        for (int j = tid; j < kNout; j += kRowThreads) {
-            cc.mu[j] = as2(pair_of(m.mu[j]));
-            cc.sd[j] = as2(pair_of(m.sd[j]));
-            cc.shot[j] = as2(pair_of(m.shot[j]));
-            cc.ref[j] = as2(pair_of(m.ref ? m.ref[j] : 0.0));
-            cc.isig[j] = as2(pair_of(m.sigma ? 1.0 / m.sigma[j] : 1.0));
-            cc.e[j] = m.base ? m.exponent[j] : 0;
-        }
-        for (int i = tid; i < 3 * R; i += kRowThreads) {
-            const int r = i / 3, k = i - 3 * r;
-            if (r >= rows) continue;
-            const double* th = a.theta + (size_t)(r0 + r) * kNin;
-            if (k == 0) {
-                const double s2 = th[2] * th[2];
-                rc.amp[0][r] = as2(pair_of(s2 * (th[0] * th[1])));
-                rc.amp[1][r] = as2(pair_of(s2 * (th[0] * th[0])));
-                rc.t5[r] = as2(pair_of(th[5]));
-            } else if (m.base) {
-                const int c = m.base_in[k - 1];
-                lobatto_basis_fast(th[c] * m.dscale[c] + m.dshift[c], m, k == 1 ? rc.la[r] : rc.lb[r]);
-            }
-        }
-        __syncthreads();
-        if (m.base) {
-            // the rows' Lagrange weights as digit fragments: one warp per row
-            const int nn = m.nodes * m.nodes;
-            bf16* wo = reinterpret_cast<bf16*>(wd);
-            for (int r = warp; r < R; r += kRowThreads / 32) {
-                double v[2], mx = 0.0;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int q = lane + 32 * h;
-                    v[h] = (r < rows && q < nn) ? rc.la[r][q / m.nodes] * rc.lb[r][q % m.nodes] : 0.0;
-                    mx = fmax(mx, fabs(v[h]));
-                    if (!(fabs(v[h]) < INFINITY)) mx = INFINITY;
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                const bool finite = mx < INFINITY;
-                int e = 0;
-                if (finite && mx > 0.0) frexp(mx, &e);
-                if (lane == 0) rc.e[r] = finite ? e : kBadExponent;
-                const int mt = r >> 4, rr = r & 15;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    int d[kDigits];
-                    fixed_digits(finite ? ldexp(v[h], -e) : 0.0, d);
-                    // term q = 32 h + lane = 16 ks + p: register (rr >> 3) + 2 (p >> 3) of lane 4 (rr & 7) + (p & 7) / 2
-                    const int ks = 2 * h + (lane >> 4), p = lane & 15;
-                    const int reg = (rr >> 3) + 2 * (p >> 3), ln = 4 * (rr & 7) + ((p & 7) >> 1);
-#pragma unroll
-                    for (int i = 0; i < kDigits; ++i)
-                        wo[((((i * MT + mt) * kBaseKsteps + ks) * 32 + ln) * 4 + reg) * 2 + (p & 1)] =
-                            __float2bfloat16_rn((float)d[i]);
-                }
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const int tile = warp * 5 + j;
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-                float acc[kOrders][4];
-#pragma unroll
-                for (int o = 0; o < kOrders; ++o)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) acc[o][r] = 0.f;
-                if (m.base) {
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint4 bd[kDigits];
-#pragma unroll
-                        for (int i = 0; i < kDigits; ++i)
-                            bd[i] = m.digits[((size_t)(i * (kNout / 8) + tile) * 2 + h) * 32 + lane];
-#pragma unroll
-                        for (int k = 0; k < 2; ++k)
-#pragma unroll
-                            for (int i = 0; i < kDigits; ++i) {
-                                const uint4 av = wd[((i * MT + mt) * kBaseKsteps + 2 * h + k) * 32 + lane];
-                                const uint32_t af[4] = {av.x, av.y, av.z, av.w};
-#pragma unroll
-                                for (int q = 0; q < kDigits; ++q)
-                                    if (i + q < kOrders)
-                                        mma_bf16(acc[i + q], af, k ? bd[q].z : bd[q].x, k ? bd[q].w : bd[q].y);
-                            }
-                    }
-                }
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    const int r = mt * 16 + g + 8 * hh;
-                    if (r >= rows) continue;
-                    float res[2];
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const int c = 8 * tile + 2 * t + q, v = 2 * hh + q;
-                        fpair u = pr(cc.mu[c]);
-                        if (m.base) {
-                            // sum_o acc_o 2^(-8 o), the small orders first
-                            fpair b{0.f, 0.f};
-#pragma unroll
-                            for (int o = kOrders - 1; o >= 0; --o) {
-                                const fpair s2 = two_sum(__fmul_rn(acc[o][v], exp2i(-8 * o)), b.hi);
-                                b = fast_two_sum(s2.hi, __fadd_rn(s2.lo, b.lo));
-                            }
-                            const int er = rc.e[r], ec = cc.e[c];
-                            if (er == kBadExponent || ec == kBadExponent) {
-                                b.hi = b.lo = NAN;
-                            } else {
-                                const int e = er + ec - 14;   // the digits' unit: 2^(e_r + e_c) 2^-14
-                                b.hi = scale2(b.hi, e);
-                                b.lo = scale2(b.lo, e);
-                            }
-                            u = pair_add(u, b);
-                        }
-                        u = pair_add(u, pair_mul(pr(cc.sd[c]), y[mt][j][v]));
-                        u = pair_mul(u, pr(rc.amp[c < 2 * (kNout / 8) ? 0 : 1][r]));
-                        u = pair_add(u, pair_mul(pr(rc.t5[r]), pr(cc.shot[c])));
-                        const float2 rf = cc.ref[c];
-                        u = pair_add(u, fpair{-rf.x, -rf.y});
-                        u = pair_mul(u, pr(cc.isig[c]));
-                        res[q] = __fadd_rn(u.hi, u.lo);
-                    }
-                    *reinterpret_cast<float2*>(a.out + (size_t)(r0 + r) * kNout + 8 * tile + 2 * t) = make_float2(res[0], res[1]);
-                }
-            }
+    if constexpr (MAP) {
+        decode_rows<R>(a.map, a.theta, r0, rows, rc, wd);   // begins after the stores above: other addresses, and a barrier inside
+#pragma unroll 1
+        for (int i = warp * 5 * MT; i < (warp + 1) * 5 * MT; ++i) {
+            const float4 v = ys[i * 32 + lane];
+            const float yv[4] = {v.x, v.y, v.z, v.w};
+            decode_tile<R>(a.map, wd, rc, a.cols, i % MT, i / MT, rows, yv, a.out + (size_t)r0 * kNout);
         }
     }
 }
+
+// The same for few rows: 16 rows on a cluster of kSplit CTAs, each a quarter of every layer's columns
+// and of the outputs.  What bounds it: the latency of the dependent layers.  50 rows: 85 us as eight
+// launches, 49 us with one CTA per 16 rows -> 25 us.
+template <bool MAP>
+__global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(kRowThreads, 1)
+k_predict_few(const __grid_constant__ PredictArgs a) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cg::cluster_group cluster = cg::this_cluster();
+    SliceRing ring;
+    ring.ring = reinterpret_cast<bf16*>(smem_raw);
+    ring.n_pass = kLayers;
+    ring.rank = (int)cluster.block_rank();
+    bf16* buf[2];
+    buf[0] = ring.ring + kSliceStages * kSliceElems;
+    buf[1] = buf[0] + 16 * kActLd;
+    // the decoding's rows and columns are prepared while the first weights arrive
+    constexpr int R = 16;
+    uint4* wd = reinterpret_cast<uint4*>(smem_raw + kSliceSmem);                     // [kDigits][1][kBaseKsteps][32]
+    RowConst<R>& rc = *reinterpret_cast<RowConst<R>*>(wd + kDigits * kBaseKsteps * 32);
+    ColumnConst* cols = reinterpret_cast<ColumnConst*>(&rc + 1);                     // [kNout / kSplit]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int r0 = (int)(blockIdx.x / kSplit) * R, rows = min(R, a.n - r0);
+    const int h0 = ring.rank * (256 / kSplit), o0 = ring.rank * (kNout / kSplit);
+    for (int c = 0; c < kSliceStages - 1; ++c) ring.load(a.ps);
+    input_rows<R, MAP>(a, r0, rows, buf[0], kActLd);
+    if constexpr (MAP) {
+        if (tid < kNout / kSplit) cols[tid] = column_const(a.map, o0 + tid);
+        decode_rows<R>(a.map, a.theta, r0, rows, rc, wd);
+    }
+    cluster.sync();   // every CTA of the cluster runs before its shared memory is written
+    const int c = h0 + 8 * warp + 2 * t;
+    int cur = 0;
+    for (int l = 0; l < kLayers - 1; ++l) {
+        float acc[1][4];
+        if (l == 0) slice_product<16, 8>(ring, a.ps, buf[cur], acc);
+        else slice_product<256, 8>(ring, a.ps, buf[cur], acc);
+        const float2 b = *reinterpret_cast<const float2*>(a.bias[l] + c);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            share2(buf[cur ^ 1], g + 8 * h, c, gelu(acc[0][2 * h] + b.x), gelu(acc[0][2 * h + 1] + b.y));
+        cur ^= 1;
+        cluster.sync();   // after the last layer: no CTA leaves while the others write to it
+    }
+    float y[2][4];
+    slice_product<256, 10>(ring, a.ps, buf[cur], y);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        if (warp + 8 * j >= kNout / kSplit / 8) break;   // warp-uniform
+        const int tile = o0 / 8 + warp + 8 * j, co = 8 * tile + 2 * t;
+        const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + co);
+        const float v[4] = {y[j][0] + b.x, y[j][1] + b.y, y[j][2] + b.x, y[j][3] + b.y};
+        if constexpr (MAP) {
+            decode_tile<R>(a.map, wd, rc, cols - o0, 0, tile, rows, v, a.out + (size_t)r0 * kNout);
+        } else {
+            float* o = a.out + (size_t)(r0 + g) * kNout + co;
+            if (g < rows) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
+            if (g + 8 < rows) *reinterpret_cast<float2*>(o + 8 * kNout) = make_float2(v[2], v[3]);
+        }
+    }
+}
+constexpr size_t kFewSmem = kSliceSmem + sizeof(uint4) * kDigits * kBaseKsteps * 32 + sizeof(RowConst<16>) +
+                            sizeof(ColumnConst) * (kNout / kSplit);
 
 // training targets: derived curves u of native template slots [n][LPP_N_MOMENTS][40] (FP64, unit
 // amplitude, no shot noise), y = (u - baseline) / sd
@@ -857,6 +1022,7 @@ struct lpp_surrogate_s {
     size_t w[kLayers], b[kLayers], mw[kLayers], vw[kLayers], mb[kLayers], vb[kLayers], dw[kLayers], db[kLayers];
     size_t w16[kLayers], w16t[kLayers], actt[kLayers], gt[kLayers], g32[kLayers], loss;
     size_t digits, exponent;          // the decoding's digits of the map's base
+    size_t cols;                      // and the columns' constants of a call
     bool has_map = false;
     bool base_split = false;          // digits, exponent hold the current map's base
     MapArgs map;
@@ -887,6 +1053,7 @@ extern "C" lpp_status lpp_surrogate_create(int batch, lpp_surrogate_t* out) {
     s->loss = take(8);
     s->digits = take((size_t)kDigitWords * sizeof(uint4));
     s->exponent = take((size_t)kNout * sizeof(int));
+    s->cols = take((size_t)kNout * sizeof(ColumnConst));
     s->need = off;
     *out = s;
     return LPP_OK;
@@ -1072,8 +1239,8 @@ static Passes passes(lpp_surrogate_t s) {
     return p;
 }
 
-// The fused forward pass (MAP: the whole prediction) of n rows: 16 rows per CTA up to one CTA per
-// SM, 32 rows beyond (two CTAs per SM, half the weight traffic per row).
+// The fused forward pass (MAP: the whole prediction) of n rows: clusters of four CTAs per 16 rows
+// while they fit the SMs at once (608 rows on 152 SMs), one CTA per 32 rows beyond.
 template <bool MAP>
 static cudaError_t launch_predict(lpp_surrogate_t s, PredictArgs& a, cudaStream_t st) {
     if (a.n == 0) return cudaSuccess;
@@ -1081,12 +1248,17 @@ static cudaError_t launch_predict(lpp_surrogate_t s, PredictArgs& a, cudaStream_
     for (int l = 0; l < kLayers; ++l) a.bias[l] = (const float*)(s->ws + s->b[l]);
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (a.n <= 16 * sms) {
-        cudaFuncSetAttribute(k_predict<1, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pred_smem(1));
-        k_predict<1, MAP><<<(a.n + 15) / 16, kRowThreads, pred_smem(1), st>>>(a);
+    const int groups = (a.n + 15) / 16;
+    if (groups * kSplit <= sms) {
+        cudaFuncSetAttribute(k_predict_few<MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmem);
+        k_predict_few<MAP><<<groups * kSplit, kRowThreads, kFewSmem, st>>>(a);
     } else {
-        cudaFuncSetAttribute(k_predict<2, MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pred_smem(2));
-        k_predict<2, MAP><<<(a.n + 31) / 32, kRowThreads, pred_smem(2), st>>>(a);
+        if (MAP) {
+            a.cols = (const ColumnConst*)(s->ws + s->cols);
+            k_columns<<<(kNout + 63) / 64, 64, 0, st>>>(a.map, (ColumnConst*)(s->ws + s->cols));
+        }
+        cudaFuncSetAttribute(k_predict<MAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPredSmem);
+        k_predict<MAP><<<(a.n + kPredRows - 1) / kPredRows, kRowThreads, kPredSmem, st>>>(a);
     }
     return cudaGetLastError();
 }
@@ -1205,9 +1377,9 @@ static cudaError_t train_step(lpp_surrogate_t s, const float* x, const float* y,
     r.idx = idx;
     r.batch = w.batch = s->batch;
     r.loss = loss_out;
-    cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem);
+    cudaFuncSetAttribute(k_train_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSliceSmem);
     cudaFuncSetAttribute(k_train_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWeightSmem);
-    k_train_rows<<<s->batch / 16, kRowThreads, kTrainSmem, st>>>(r);
+    k_train_rows<<<s->batch / 16 * kSplit, kRowThreads, kSliceSmem, st>>>(r);
     if (update) s->step += 1;
     AdamArgs& a = w.adam;
     a = adam_args(s);
