@@ -225,7 +225,7 @@ struct FusedArgs {
     const int* trows;                    // z-tile rows to visit (persistent grid), or null (all tiles)
     const int* trow_count;
     int skip_empty;                      // empty tiles store nothing (the y pass fills their zeros)
-    int dual;                            // FP32 n = 256/512: two slots per CTA (see k_assign_xfft2)
+    int dual;                            // FP32 n = 64..512: two slots per CTA (see k_assign_xfft2)
     const int* tranges;                  // two-slot launches: per-tile range records, or null
     int* work;                           // one-slot launches over trows: item counter, zeroed
                                          // before the launch (dynamic schedule), or null

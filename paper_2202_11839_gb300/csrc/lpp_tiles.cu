@@ -871,7 +871,8 @@ __device__ __forceinline__ void fused_tile2(const FusedArgs<T>& a, int tile_y, i
 // With range records (a.tranges) warp 0 loads the next tile's record into registers while
 // the CTA works on the current tile and stores it into the other record buffer at the end.
 template <typename T, int LOGN>
-__global__ void __launch_bounds__(2 * FusedShape<T, LOGN>::THREADS, 1) k_assign_xfft2(FusedArgs<T> a) {
+__global__ void __launch_bounds__(2 * FusedShape<T, LOGN>::THREADS, 1024 / (2 * FusedShape<T, LOGN>::THREADS))
+k_assign_xfft2(FusedArgs<T> a) {
     using S = FusedShape<T, LOGN>;
     static_assert(S::MAXR <= kRecPref - kRecBegin && S::MAXR + 1 <= kRecSrc - kRecPref && S::MAXR <= kRec - kRecSrc,
                   "range record layout");
@@ -1018,7 +1019,7 @@ static cudaError_t launch_fused_n(const FusedArgs<T>& a, int n_tiles, cudaStream
     if (a.ty != S::TY || a.tz != S::TZ) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)(S::N + S::TILE + S::TWR) * sizeof(c2<T>);
     cudaFuncSetAttribute(k_assign_xfft<T, LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if constexpr (sizeof(T) == 4 && (LOGN == 8 || LOGN == 9)) {
+    if constexpr (sizeof(T) == 4 && LOGN >= 6 && LOGN <= 9) {
         if (a.dual) {
             // two slots per CTA (FusedArgs::dual: even slot count, interlaced single-source
             // coefficient slots, a tile-row list)
@@ -1026,8 +1027,9 @@ static cudaError_t launch_fused_n(const FusedArgs<T>& a, int n_tiles, cudaStream
             cudaFuncSetAttribute(k_assign_xfft2<T, LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
             int dev = 0, sms = 152;
             if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            const int pairs = a.n_slots / 2;
-            const int g2 = std::max(1, std::min(n_tiles, 2 * sms / pairs));
+            // about two waves of the resident CTAs (1024 threads per SM by the launch bounds)
+            const int pairs = a.n_slots / 2, per_sm = 1024 / (2 * S::THREADS);
+            const int g2 = std::max(1, std::min(n_tiles, 2 * per_sm * sms / pairs));
             k_assign_xfft2<T, LOGN><<<dim3(g2, pairs), 2 * S::THREADS, smem2, st>>>(a);
             return cudaGetLastError();
         }

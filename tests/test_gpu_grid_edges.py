@@ -73,6 +73,8 @@ def test_one_slot_matches_two_slot_small_grids(n):
     cfg = _cfg(n, 512.0, 3, True, 8)
     two = U.run_gpu(cfg, cat, L.LPP_FP32)
     one = U.run_gpu(dict(cfg, fused_slots=1), cat, L.LPP_FP32)
+    assert two.extra["path"]["two_slot_launches"] > 0
+    assert one.extra["path"]["two_slot_launches"] == 0
     pp = np.abs(one.raw[U.O.M_INDEX[("plus", 0)]].real) / one.norm_auto
     pd = np.abs(one.raw[U.O.M_INDEX[("dd", 0)]].real) / one.norm_dd
     sc = np.abs(one.p) + np.sqrt(pp * pd)[None, :]
