@@ -2,7 +2,8 @@
 //
 // Each CTA transforms a tile of W pencils (n complex points each) with a mixed-radix
 // Stockham FFT (radix 8 stages, one leading radix-2 or -4 stage), every thread holding
-// 8 points per stage, and writes the pencils back in place.  Pencils along y and z are
+// 8 points per stage (FP32 grids of 64^3 and more: 8 points of two pencils, lpp_fft_pair.cuh), and
+// writes the pencils back in place.  Pencils along y and z are
 // read as rows of W consecutive x values, so every global access is a contiguous
 // W-element segment; the first stage takes its operands straight from those rows and
 // the last stage stores straight to them, so shared memory holds only the stages in
@@ -17,6 +18,7 @@
 #include "lpp_internal.h"
 #include "lpp_kernels.h"
 #include "lpp_fft_dev.cuh"
+#include "lpp_fft_pair.cuh"
 
 namespace lpp {
 
@@ -170,6 +172,108 @@ __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LO
     }
 }
 
+// ---- FP32 passes on pencil pairs (lpp_fft_pair.cuh), 64 <= n <= 1024
+// One y (MODE 1) or z (MODE 2) tile of one grid, as pencil_tile.
+template <int LOGN, bool INV, int MODE>
+__device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair* tw, cpair* tile, const FftGeom& g,
+                                          int tile_id, int gi) {
+    using S = PairShape<LOGN>;
+    constexpr int N = S::N, W = S::W;
+    const int tid = threadIdx.x;
+    const unsigned N2 = (unsigned)N * N;
+    const int o = tile_id / g.ntx;
+    const int i = tile_id - o * g.ntx;
+    const int x0 = (g.ntx == N / W || i < g.nlo) ? i * W : N - (g.ntx - i) * W;
+    if (!LPP_IN_BOUNDS(o >= 0 && o < (MODE == 1 ? N : g.nky) && x0 >= 0 && x0 + W <= N, g.err)) return;
+    float2* base = grid;
+    if (MODE == 1) {
+        base += (size_t)o * N2 + x0;  // o = z
+    } else {
+        const int y = (o <= g.nk_pos) ? o : N - (g.nky - o);
+        if (g.q_max > 0) {
+            // columns outside the last shell in (fx, fy) for every fz: nothing to transform
+            const int fy = y < N / 2 ? y : y - N;
+            // the smallest |fx| of the tile: x0 itself or its upper end (tiles do not straddle N / 2)
+            const int fx = x0 < N / 2 ? x0 : N - (x0 + W - 1);
+            if (fx * fx + fy * fy >= g.q_max) return;
+        }
+        base += (size_t)y * N + x0;
+    }
+    const int c = tid & (S::CP - 1), u = tid >> S::LOGC;
+    constexpr unsigned ES = MODE == 1 ? (unsigned)N : (unsigned)N * N;
+    float4* gp = reinterpret_cast<float4*>(base + 2 * c);   // x0 even: 16-byte aligned
+    static_assert(S::PER <= 32, "one liveness bit per operand");
+    // operands on rows that no particle of the grid's roles reaches are zero and not loaded
+    unsigned live = 0xffffffffu;
+    const int gm = g.gmask[gi];
+    if (gm && (MODE == 1 ? g.plive != nullptr : g.pmask != nullptr)) {
+        live = 0u;
+#pragma unroll
+        for (int b = 0; b < S::PER; ++b) {
+            const int e = lead_row<LOGN, S::IPT>(u, b);
+            int hit = 0;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                if (gm & (1 << r))
+                    hit |= MODE == 1 ? __ldg(g.plive + (size_t)r * N * N + (size_t)o * N + e)
+                                     : __ldg(g.pmask + r * N + e);
+            }
+            live |= (hit ? 1u : 0u) << b;
+        }
+    }
+    auto twiddle = [](float2 w) { return cpair{pk2(w.x, w.x), pk2(-w.y, -w.y)}; };
+    if (twg)
+        for (int k = tid; k < N; k += S::THREADS) tw[k] = twiddle(twg[k]);
+    fft_pairs_io<LOGN, INV>(
+        tile, c, u, tw,
+        [&](int b, int e) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if ((live >> b) & 1u) v = gp[(size_t)e * (ES / 2)];
+            return cpair{pk2(v.x, v.z), pk2(v.y, v.w)};
+        },
+        [&](int e, cpair v) {
+            if (!kept(e, N, g.nk_pos, g.nk_neg)) return;
+            float4 w;
+            unpk2(v.re, w.x, w.z);
+            unpk2(v.im, w.y, w.w);
+            gp[(size_t)e * (ES / 2)] = w;
+        });
+}
+
+template <int LOGN, bool INV, int MODE>
+__global__ void __launch_bounds__(PairShape<LOGN>::THREADS, PairShape<LOGN>::MINB)
+k_fft_pair(float2* __restrict__ data, const float2* __restrict__ twg, const __grid_constant__ FftGeom g) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cpair* tw = reinterpret_cast<cpair*>(smem_raw);
+    constexpr size_t N = PairShape<LOGN>::N;
+    // a z plane that no particle of the grid's roles reaches is neither stored by the fused
+    // assignment nor by this pass
+    if (MODE == 1 && !plane_live(g, blockIdx.y, blockIdx.x / g.ntx, (int)N)) return;
+    pair_tile<LOGN, INV, MODE>(data + blockIdx.y * N * N * N, twg, tw, tw + N, g, blockIdx.x, blockIdx.y);
+}
+
+// The y pass as a persistent grid (see k_fft_ypass).
+template <int LOGN, bool INV>
+__global__ void __launch_bounds__(PairShape<LOGN>::THREADS, PairShape<LOGN>::MINB)
+k_fft_ypair(float2* __restrict__ data, const float2* __restrict__ twg, const __grid_constant__ FftGeom g, int n_grids) {
+    using S = PairShape<LOGN>;
+    constexpr int N = S::N;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cpair* tw = reinterpret_cast<cpair*>(smem_raw);
+    for (int i = threadIdx.x; i < N; i += S::THREADS) {   // first read after a barrier
+        const float2 w = twg[i];
+        tw[i] = cpair{pk2(w.x, w.x), pk2(-w.y, -w.y)};
+    }
+    const int per_grid = g.ntx * N;
+    const int items = per_grid * n_grids;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int gi = it / per_grid, tile_id = it - gi * per_grid;
+        if (!plane_live(g, gi, tile_id / g.ntx, N)) continue;
+        pair_tile<LOGN, INV, 1>(data + (size_t)gi * N * N * N, nullptr, tw, tw + N, g, tile_id, gi);
+        __syncthreads();   // the next item's first stage rewrites the tile
+    }
+}
+
 int fft_tile_width(int n) {
     int w = 8192 / n;
     if (w > 32) w = 32;
@@ -200,8 +304,6 @@ static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, cons
     const size_t smem = (size_t)(N + N * S::LD) * sizeof(c2<T>);
     // the attribute is per device and function: set it on every call (cheap, host-only)
     cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const double es = (double)sizeof(c2<T>);
     const double n3 = (double)N * N * N;
     const double keep = (double)(g.nky) / N;               // kept fraction of one axis
@@ -214,26 +316,47 @@ static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, cons
     if (timer) timer->begin(KK_FFT, st);
     bool skip = false;
     for (int i = 0; i < n_grids && i < 8; ++i) skip = skip || (g.pmask && g.gmask[i]);
-    if (skip) {
-        // one wave of resident CTAs (the occupancy the launch bounds give), at most one per item
+    // one wave of resident CTAs (the occupancy the launch bounds give), at most one per item
+    auto wave = [&](auto kernel, int threads, size_t bytes) {
         int dev = 0, sms = 0, ps = 0;
-        cudaFuncSetAttribute(k_fft_ypass<T, LOGN, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_fft_ypass<T, LOGN, INV>, S::THREADS, smem);
-        if (ps < 1) ps = 1;
-        if (sms < 1) sms = 1;
-        const long long items = (long long)g.ntx * N * n_grids;
-        const int blocks = (int)std::min<long long>(items, (long long)ps * sms);
-        k_fft_ypass<T, LOGN, INV><<<blocks, S::THREADS, smem, st>>>(data, tw, g, n_grids);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kernel, threads, bytes);
+        return (int)std::min<long long>((long long)g.ntx * N * n_grids, (long long)std::max(ps, 1) * std::max(sms, 1));
+    };
+    if constexpr (sizeof(T) == 4 && LOGN >= 6) {
+        using P = PairShape<LOGN>;
+        auto attr = [&](auto kernel) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
+        };
+        if (skip) {
+            attr(k_fft_ypair<LOGN, INV>);
+            k_fft_ypair<LOGN, INV><<<wave(k_fft_ypair<LOGN, INV>, P::THREADS, P::SMEM), P::THREADS, P::SMEM, st>>>(
+                data, tw, g, n_grids);
+        } else {
+            attr(k_fft_pair<LOGN, INV, 1>);
+            k_fft_pair<LOGN, INV, 1><<<dim3(g.ntx * N, n_grids), P::THREADS, P::SMEM, st>>>(data, tw, g);
+        }
+    } else if (skip) {
+        cudaFuncSetAttribute(k_fft_ypass<T, LOGN, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_fft_ypass<T, LOGN, INV><<<wave(k_fft_ypass<T, LOGN, INV>, S::THREADS, smem), S::THREADS, smem, st>>>(
+            data, tw, g, n_grids);
     } else {
+        cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         k_fft_pass<T, LOGN, INV, 1><<<dim3(g.ntx * N, n_grids), S::THREADS, smem, st>>>(data, tw, g);
     }
     // y: only the reached planes are read and written; z: their entries are read, all written
     if (timer)
         timer->end(KK_FFT, st, n_grids * n3 * es * xcols * ((double)g.ylive_frac + (double)g.yread_frac * keep));
     if (timer) timer->begin(KK_FFT, st);
-    k_fft_pass<T, LOGN, INV, 2><<<dim3(g.ntx * g.nky, n_grids), S::THREADS, smem, st>>>(data, tw, g);
+    if constexpr (sizeof(T) == 4 && LOGN >= 6) {
+        using P = PairShape<LOGN>;
+        cudaFuncSetAttribute(k_fft_pair<LOGN, INV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
+        k_fft_pair<LOGN, INV, 2><<<dim3(g.ntx * g.nky, n_grids), P::THREADS, P::SMEM, st>>>(data, tw, g);
+    } else {
+        cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_fft_pass<T, LOGN, INV, 2><<<dim3(g.ntx * g.nky, n_grids), S::THREADS, smem, st>>>(data, tw, g);
+    }
     if (timer) {
         // the z pass transforms the columns that some shell can use
         double zfrac = 1.0;
