@@ -7,8 +7,9 @@
 // 8, a shared-memory access 16 bytes for two pencils, and a twiddle is read once for both.  The
 // tile holds N rows of W / 2 pairs {re0, re1, im0, im1}; eight consecutive lanes read 128
 // contiguous bytes of one row, so no padding is needed.  Same factorisation and order of
-// operations as lpp_fft_dev.cuh.  Eight grids of 256^3 to k = 0.8 k_Ny, y pass 414 -> 383 us (2.08 GB,
-// 5.4 TB/s: now bound by DRAM), z pass 368 -> 320 us (1.80 GB, 5.6 TB/s).  Grids below 64^3 keep one
+// operations as lpp_fft_dev.cuh.  Eight grids of 256^3 to k = 0.995 k_Ny, y pass 414 -> 383 us, z pass 368 -> 320 us;
+// with the stores of ColumnBound and tiles of 16 columns 320 us (1.9 GB, 6.0 TB/s: bound by DRAM) and 246
+// us (1.4 GB, 5.7 TB/s).  512^3 stays bound by the latency of its five steps per tile, 32 warps per SM.  Grids below 64^3 keep one
 // pencil per thread: their passes take a few microseconds and have too few pencils to pair.
 #pragma once
 
@@ -108,12 +109,15 @@ __device__ __forceinline__ void pdft8(cpair* v) {
     }
 }
 
-// Pass shape: the tile width of PassShape, half as many pencil pairs; one butterfly slot (eight values
-// of a pair: 32 registers) per thread, as two would spill at the 64 registers of 1024 threads per SM.
+// Pass shape: W pencils (128-byte segments; 64 bytes at n = 1024), half as many pencil pairs; one
+// butterfly slot (eight values of a pair: 32 registers) per thread, as two would spill at the 64
+// registers of 1024 threads per SM.  Small CTAs overlap one tile's stores with another's loads: at
+// 256^3, 32 -> 16 columns, y pass 375 -> 320 us, z pass 280 -> 246 us (at 512^3, 16 -> 8 columns, 454 ->
+// 465 us: half segments); 64^3 keeps 32 (16: y pass 5.1 -> 5.5 us, its persistent CTAs get no work).
 template <int LOGN>
 struct PairShape {
     static constexpr int N = 1 << LOGN;
-    static constexpr int W = PassShape<LOGN>::W;
+    static constexpr int W = LOGN == 6 ? 32 : (LOGN < 10 ? 16 : 8);
     static constexpr int CP = W / 2;
     static constexpr int LOGC = ilog2(CP);
     static constexpr int IPT = 1;

@@ -63,8 +63,8 @@ struct FftGeom {
     int gmask[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     float yread_frac = 1.0f;   // host bookkeeping: fraction of z planes the y pass writes
     float ylive_frac = 1.0f;   // host bookkeeping: fraction of x pencils the y pass reads
-    // z pass: skip (kx, ky) columns whose every mode has |f|^2 >= q_max (beyond the last
-    // shell; never read by the combine); 0 transforms every column
+    // modes with |f|^2 >= q_max are beyond the last shell and never read by the combine: the y and z
+    // passes leave out what only they need; 0 transforms and stores every kept mode
     int q_max = 0;
     // optional per-pencil reach [3][n*n] bytes (role, z * n + y): the y pass reads zeros for
     // x pencils that no particle of the grid's roles reaches (the fused pass stores nothing there)
