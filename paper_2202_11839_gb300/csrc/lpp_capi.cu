@@ -1159,6 +1159,22 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
     FftGeom gs = fft_geometry(n, ns_pos, ns_neg);
     gfull.err = err;
     gs.err = err;
+    // what the randoms reach: the assignment visits only those tiles (dynamically: their counts
+    // differ) and the y pass reads only those pencils (1 M randoms of a polar cap on a padded 256^3
+    // grid: the assignment 4.32 -> 3.82 ms, the forward y passes 0.93 -> 0.23 ms)
+    const int ran_bit = 1 << LPP_RANDOMS;
+    const int* koff = (const int*)(plan->ws + plan->off_koff[LPP_RANDOMS]);
+    int* pmask = (int*)(plan->ws + plan->off_pmask);
+    unsigned char* plive = (unsigned char*)(plan->ws + plan->off_plive);
+    int* trows = (int*)(plan->ws + plan->off_trows);
+    int* work = (int*)(plan->ws + plan->off_work);
+    const bool use_rows = n / plan->ftz <= 256;
+    LPP_CUDA(launch_plane_mask(koff, koff, koff, 0, 0, 1, n, pmask, st));
+    LPP_CUDA(launch_pencil_live(koff, koff, koff, 0, 0, 1, n, plive, st));
+    if (use_rows) LPP_CUDA(launch_tile_rows(pmask, ran_bit, n, plan->ftz, trows, trows + 512, st));
+    gfull.pmask = pmask;
+    gfull.plive = plive;
+    for (int i = 0; i < 8; ++i) gfull.gmask[i] = ran_bit;
     FusedArgs<T> fa;
     memset(&fa, 0, sizeof(fa));
     fa.err = err;
@@ -1173,6 +1189,18 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
     fa.tz = plan->ftz;
     fa.scheme = plan->d.scheme;
     fa.interlace = 0;
+    fa.pmask = pmask;
+    fa.skip_empty = 1;
+    if (use_rows) {
+        fa.trows = trows;
+        fa.trow_count = trows + 512;
+        fa.work = work;
+    }
+    auto assign = [&]() -> lpp_status {
+        if (fa.work) LPP_CUDA(cudaMemsetAsync(work, 0, sizeof(int), st));
+        LPP_CUDA(launch_assign_xfft<T>(fa, st));
+        return LPP_OK;
+    };
     fa.nk_pos = n / 2 - 1;
     fa.nk_neg = n / 2;
     fa.tw = tw;
@@ -1187,7 +1215,7 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
     ws.grid = 0;
     ws.yl_a = ws.yl_b = -1;
     fa.slots[0] = ws;
-    LPP_CUDA(launch_assign_xfft<T>(fa, st));
+    { lpp_status s0 = assign(); if (s0 != LPP_OK) return s0; }
     LPP_CUDA(fft_yz<T>(grids, 1, n, tw, gfull, false, st, nullptr));
     LPP_CUDA(launch_window_partner<T>(grids, pW, iw, n, st));
     // channels (l, m), two per grid
@@ -1244,7 +1272,7 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
                 sb.run[sb.n_runs - 1].c1 = sb.n_ch;
             }
         }
-        LPP_CUDA(launch_assign_xfft<T>(fa, st));
+        { lpp_status s0 = assign(); if (s0 != LPP_OK) return s0; }
         LPP_CUDA(fft_yz<T>(grids, ngr, n, tw, gfull, false, st, nullptr));
         LPP_CUDA(launch_window_mult<T>(grids, (long long)n3, ngr, pW, iw, n, st));
         LPP_CUDA(fft3d<T>(grids, ngr, n, tw, gs, true, st, nullptr));
