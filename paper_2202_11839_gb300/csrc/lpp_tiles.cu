@@ -266,17 +266,23 @@ __device__ __forceinline__ void fold_halo(c2<T>* tile, int c, int i, bool fixed)
     *src = mk<T>((T)0, (T)0);
 }
 
-// Tile of TY x TZ pencils: TY = 4 (TY = 2 when the FP64 1024-point tile would not fit).
+// Tile of TY x TZ pencils: TY = 4 (TY = 2 when the FP64 1024-point tile would not fit).  FP32 grids of
+// 128^3 and 256^3 take 8 x 4 pencils: a particle is visited by (1 + 3/TY)(1 + 3/TZ) tiles, 2.4 instead of
+// 3.1 (TSC, 2 M galaxies, all channels of an estimate at 256^3: 14.5 -> 12.4 ms; 60,000 to 250,000 on
+// 128^3: 7.7 -> 6.8 ms for four).  64^3 has too few tiles for that (266 -> 291 us); two tiles of 512^3
+// would not fit in shared memory.
+constexpr int kWideLo = 7;
 template <typename T, int LOGN>
 struct FusedShape {
     static constexpr int N = 1 << LOGN;
-    static constexpr int TY = (sizeof(T) == 8 && LOGN >= 10) ? 2 : 4;
+    static constexpr bool WIDE = sizeof(T) == 4 && LOGN >= kWideLo && LOGN <= 8;
+    static constexpr int TY = WIDE ? 8 : ((sizeof(T) == 8 && LOGN >= 10) ? 2 : 4);
     static constexpr int TZ = 4;
     static constexpr int W = TY * TZ;
     static constexpr int LD = W + 1;
     static constexpr int ROWS = N + 3;   // x = -1 .. n + 1 (scatter)
     static constexpr int TILE = ROWS * LD;
-    static constexpr int IPT = (W * N / 8) <= 512 ? 1 : ((W * N / 8) <= 1024 ? 2 : 4);
+    static constexpr int IPT = (W * N / 8) <= (WIDE ? 256 : 512) ? 1 : ((W * N / 8) <= 1024 ? 2 : 4);
     static constexpr int THREADS = W * N / (8 * IPT);
     static constexpr int MAXR = 2 * 2 * (TZ + 3);   // key ranges: sources x z rows x (1 or 2)
     // resident CTAs per SM the register budget is sized for (shared memory allows 3 at
@@ -285,10 +291,10 @@ struct FusedShape {
     // the last x stage runs one warp per pencil and stores straight to the grid when a
     // warp's 32 lanes cover the N/8 butterfly slots (N >= 256); it reads the per-leg
     // twiddle table of TWR entries after the tiles
-    static constexpr bool WARP_OUT = (N / 8 == 32 * IPT) && (THREADS == 32 * W);
+    static constexpr bool WARP_OUT = N == 256 || N == 512 || ((N / 8 == 32 * IPT) && (THREADS == 32 * W));
     // n = 256, 512: the whole x transform of a pencil by one warp (fft_pencil_warp), with
     // its twiddle tables in the TWR entries
-    static constexpr bool WARP_FFT = WARP_OUT && (N == 256 || N == 512);
+    static constexpr bool WARP_FFT = N == 256 || N == 512;
     static constexpr int TWR = WARP_FFT ? PencilWarpTw<LOGN>::SIZE : (WARP_OUT ? 7 * (N / 8) : 0);
 };
 
@@ -453,28 +459,30 @@ __device__ __forceinline__ void x_transform(c2<T>* tile, int t, const c2<T>* tw,
     using S = FusedShape<T, LOGN>;
     constexpr int N = S::N, W = S::W, LD = S::LD, IPT = S::IPT, TY = S::TY, R0 = LeadRadix<LOGN>::R;
     if constexpr (S::WARP_FFT) {
-        // one warp per pencil
-        const int pc = t >> 5, lane = t & 31;
-        if (lane < 3) fold_halo<T, N, LD>(tile, pc, lane, fixed);
-        __syncwarp();
-        c2<T>* po = out + ((size_t)(pc / TY) * N + (pc & (TY - 1))) * N;
-        auto store = [&](int e, c2<T> v) {
-            if (kept(e, N, nk_pos, nk_neg)) po[e] = v;
-        };
+        // a pencil by one warp
+        const int lane = t & 31;
         constexpr int T1 = PencilWarpTw<LOGN>::T1;
-        if constexpr (sizeof(T) == 4) {
-            if (fixed) {
-                const int2* ti = reinterpret_cast<const int2*>(tile) + pc;
-                fft_pencil_warp<T, LOGN, false, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) {
-                    const int2 q = ti[e * LD];
-                    return mk<T>((T)((float)q.x * unit), (T)((float)q.y * unit));
-                }, store);
-                return;
+        for (int pc = t >> 5; pc < W; pc += S::THREADS / 32) {
+            if (lane < 3) fold_halo<T, N, LD>(tile, pc, lane, fixed);
+            __syncwarp();
+            c2<T>* po = out + ((size_t)(pc / TY) * N + (pc & (TY - 1))) * N;
+            auto store = [&](int e, c2<T> v) {
+                if (kept(e, N, nk_pos, nk_neg)) po[e] = v;
+            };
+            if constexpr (sizeof(T) == 4) {
+                if (fixed) {
+                    const int2* ti = reinterpret_cast<const int2*>(tile) + pc;
+                    fft_pencil_warp<T, LOGN, false, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) {
+                        const int2 q = ti[e * LD];
+                        return mk<T>((T)((float)q.x * unit), (T)((float)q.y * unit));
+                    }, store);
+                    continue;
+                }
             }
+            const c2<T>* col = tile + pc;
+            fft_pencil_warp<T, LOGN, false, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) { return col[e * LD]; },
+                                                      store);
         }
-        const c2<T>* col = tile + pc;
-        fft_pencil_warp<T, LOGN, false, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) { return col[e * LD]; },
-                                                  store);
     } else {
         const int c = t & (W - 1), u = t >> ilog2(W);
         for (int i = t; i < 3 * W; i += S::THREADS) fold_halo<T, N, LD>(tile, i % W, i / W, fixed);
@@ -718,14 +726,15 @@ cudaError_t launch_plane_mask(const int* off0, const int* off1, const int* off2,
 // Tile shape (TY, TZ), pencils per thread, threads and shared memory of the fused kernel
 // (mirrors FusedShape).
 void fused_geometry(int n, size_t elem_bytes, int* ty, int* tz, int* ipt, int* threads, size_t* smem) {
-    *ty = (elem_bytes == 8 && n >= 1024) ? 2 : 4;
+    const bool wide = elem_bytes == 4 && n >= (1 << kWideLo) && n <= 256;
+    *ty = wide ? 8 : ((elem_bytes == 8 && n >= 1024) ? 2 : 4);
     *tz = 4;
     const int w = *ty * *tz;
     const int t1 = w * n / 8;
-    *ipt = t1 <= 512 ? 1 : (t1 <= 1024 ? 2 : 4);
+    *ipt = t1 <= (wide ? 256 : 512) ? 1 : (t1 <= 1024 ? 2 : 4);
     *threads = t1 / *ipt;
-    const bool warp_out = n / 8 == 32 * *ipt && *threads == 32 * w;
-    const bool warp_fft = warp_out && (n == 256 || n == 512);
+    const bool warp_fft = n == 256 || n == 512;
+    const bool warp_out = warp_fft || (n / 8 == 32 * *ipt && *threads == 32 * w);
     // PencilWarpTw<LOGN>::SIZE: two-pass tables at n = 512, three-pass at n = 256
     const int twr = warp_fft ? (n / 64 - 1) * 64 + 56 : (warp_out ? 7 * (n / 8) : 0);
     *smem = (size_t)(n + (n + 3) * (w + 1) + twr) * 2 * elem_bytes;
