@@ -583,9 +583,10 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
     if (plan->cat[LPP_DENSITY].set) { lpp_status s0 = sort_cat(LPP_DENSITY, de); if (s0 != LPP_OK) return s0; }
     if (has_rand) { lpp_status s0 = sort_cat(LPP_RANDOMS, ra); if (s0 != LPP_OK) return s0; }
     int* pmask = (int*)(plan->ws + plan->off_pmask);
+    const Reach reach = stencil_reach(plan->d.scheme, plan->d.interlace);
     LPP_CUDA(launch_plane_mask((const int*)(plan->ws + plan->off_koff[0]), (const int*)(plan->ws + plan->off_koff[1]),
                                (const int*)(plan->ws + plan->off_koff[2]), 1, plan->cat[LPP_DENSITY].set ? 1 : 0,
-                               has_rand ? 1 : 0, n, pmask, st));
+                               has_rand ? 1 : 0, n, reach, pmask, st));
     nl += 1;
     // the z-tile rows the fused passes visit: channel slots (shapes) and the partner slots
     int* trows = (int*)(plan->ws + plan->off_trows);
@@ -601,7 +602,7 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
     unsigned char* plive = (unsigned char*)(plan->ws + plan->off_plive);
     LPP_CUDA(launch_pencil_live((const int*)(plan->ws + plan->off_koff[0]), (const int*)(plan->ws + plan->off_koff[1]),
                                 (const int*)(plan->ws + plan->off_koff[2]), 1, plan->cat[LPP_DENSITY].set ? 1 : 0,
-                                has_rand ? 1 : 0, n, plive, st));
+                                has_rand ? 1 : 0, n, reach, plive, st));
     nl += 1;
     // timing only: which planes are reached, for the byte counts of the skipping kernels
     // (one small synchronisation per estimate)
@@ -1169,8 +1170,8 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
     int* trows = (int*)(plan->ws + plan->off_trows);
     int* work = (int*)(plan->ws + plan->off_work);
     const bool use_rows = n / plan->ftz <= 256;
-    LPP_CUDA(launch_plane_mask(koff, koff, koff, 0, 0, 1, n, pmask, st));
-    LPP_CUDA(launch_pencil_live(koff, koff, koff, 0, 0, 1, n, plive, st));
+    LPP_CUDA(launch_plane_mask(koff, koff, koff, 0, 0, 1, n, stencil_reach(plan->d.scheme, 0), pmask, st));
+    LPP_CUDA(launch_pencil_live(koff, koff, koff, 0, 0, 1, n, stencil_reach(plan->d.scheme, 0), plive, st));
     if (use_rows) LPP_CUDA(launch_tile_rows(pmask, ran_bit, n, plan->ftz, trows, trows + 512, st));
     gfull.pmask = pmask;
     gfull.plive = plive;

@@ -244,10 +244,19 @@ cudaError_t launch_tile_rows(const int* pmask, int bits, int n, int tz, int* row
 // plive[r][z * n + y] = 1 when a particle of role r (set[r] != 0) sits in a key row
 // (fy, fz) with y - 2 <= fy <= y + 1 and z - 2 <= fz <= z + 1 (mod n): the x pencils that
 // its CIC/TSC stencils (interlaced or not) reach
+// Keys y - lo .. y + hi (and the same along z) hold the particles whose stencils reach pencil y: with
+// u in [f, f + 1), CIC covers f .. f + 1 (and f - 1 .. f + 1 with the half-cell shifted grid), TSC
+// f - 1 .. f + 2 (shifted f - 1 .. f + 1).
+struct Reach {
+    int lo, hi;
+};
+__host__ __device__ constexpr Reach stencil_reach(int scheme, int interlace) {
+    return Reach{scheme >= 3 ? 2 : 1, scheme >= 3 || interlace ? 1 : 0};
+}
 cudaError_t launch_pencil_live(const int* off0, const int* off1, const int* off2, int set0, int set1, int set2, int n,
-                               unsigned char* plive, cudaStream_t st);
+                               Reach reach, unsigned char* plive, cudaStream_t st);
 cudaError_t launch_plane_mask(const int* off0, const int* off1, const int* off2, int set0, int set1, int set2, int n,
-                              int* pmask, cudaStream_t st);
+                              Reach reach, int* pmask, cudaStream_t st);
 template <typename T>
 cudaError_t launch_pencil_sort(const T* pos, const T* w, long long count, long long cap, int n, double box,
                                const double origin[3], int* key, int* counts, int* off, int* cursor, int* scan_tmp,

@@ -5,10 +5,11 @@
 // scatter) stores the cell coordinates u and the weight of each particle in key order.
 //
 // Fused kernel.  One CTA owns a tile of TY x TZ x-pencils (all n points along x) of one
-// batch grid.  CIC and TSC stencils, on the grid and on the half-cell shifted grid,
-// reach the rows floor(u) - 1 .. floor(u) + 2, so the particles that touch the tile are
-// exactly those with keys in rows [y0 - 2, y0 + TY] x [z0 - 2, z0 + TZ]: TZ + 3
-// contiguous key ranges of the sorted arrays.  The CTA scatters them into the tile with
+// batch grid.  With the stencils' reach (lo, hi) (stencil_reach) the particles that touch the
+// tile are exactly those with keys in rows [y0 - lo, y0 + TY - 1 + hi] x [z0 - lo, z0 + TZ - 1 + hi]:
+// TZ + lo + hi <= TZ + 3 contiguous key ranges of the sorted arrays (the window of TSC for every
+// scheme made CIC tiles visit twice as many particles: 4 x 4 tiles, FP64 64^3, 50,000 galaxies, ten
+// launches 1.67 -> 1.40 ms).  The CTA scatters them into the tile with
 // shared-memory atomics (sub-grid 0 into the real part and the shifted sub-grid into the
 // imaginary part, or two fields), runs the x-FFT of its pencils in place and writes only
 // the kept x frequencies.  The grid is never zeroed, never touched by global atomics and
@@ -324,9 +325,9 @@ __device__ __forceinline__ void fill_twr(const c2<T>* tw, c2<T>* twr, int first,
 }
 
 // The particle ranges of the tile at (y0, z0) for the sources of slot `sl`, found by one
-// warp (all 32 lanes): TZ+3 z rows of keys y0-2 .. y0+TY per source, one or two contiguous
+// warp (all 32 lanes): the z rows of keys in reach per source, one or two contiguous
 // ranges each (the y window may wrap).  Lane l takes row l (source l / (TZ+3)); a warp scan
-// places the ranges.  With want_wmax, also the largest 4 x 4 key-row window count of source
+// places the ranges.  With want_wmax, also the largest key-row window count of one pencil of source
 // 0 (the fixed-point bound).  rcount: the warp's scratch.
 template <typename T, int LOGN>
 __device__ __forceinline__ void warp_ranges(const FusedArgs<T>& a, const FusedSlot& sl, int y0, int z0, int lane,
@@ -334,13 +335,14 @@ __device__ __forceinline__ void warp_ranges(const FusedArgs<T>& a, const FusedSl
                                             int (*rcount)[FusedShape<T, LOGN>::TY + 3], int& wmax, bool want_wmax) {
     using S = FusedShape<T, LOGN>;
     constexpr int N = S::N, TY = S::TY, TZ = S::TZ;
+    const Reach rc = stencil_reach(a.scheme, a.interlace);
     int bb[2] = {0, 0}, ee[2] = {0, 0}, m = 0, s_idx = 0;
-    if (lane < sl.n_src * (TZ + 3)) {
+    const int dz = lane % (TZ + 3);
+    if (lane < sl.n_src * (TZ + 3) && dz < TZ + rc.lo + rc.hi) {
         s_idx = lane / (TZ + 3);
-        const int dz = lane - s_idx * (TZ + 3);
         const int* off = a.cat[sl.src[s_idx].cat].off;
-        const int zr = (z0 - 2 + dz) & (N - 1);
-        const int ylo = y0 - 2, yhi = y0 + TY;   // inclusive
+        const int zr = (z0 - rc.lo + dz) & (N - 1);
+        const int ylo = y0 - rc.lo, yhi = y0 + TY - 1 + rc.hi;   // inclusive
         bb[m] = off[zr * N + (ylo < 0 ? 0 : ylo)];
         ee[m++] = off[zr * N + (yhi >= N ? N - 1 : yhi) + 1];
         if (ylo < 0) { bb[m] = off[zr * N + N + ylo]; ee[m++] = off[zr * N + N]; }
@@ -370,25 +372,26 @@ __device__ __forceinline__ void warp_ranges(const FusedArgs<T>& a, const FusedSl
         n_ranges = nr_inc;
     }
     if (want_wmax) {
-        // a cell (y, z) of the tile receives only from the key rows y-2..y+1, z-2..z+1:
-        // the largest such 4 x 4 window sum bounds the contributions of any one cell
+        // a cell (y, z) of the tile receives only from the key rows y-lo..y+hi, z-lo..z+hi:
+        // the largest such window sum bounds the contributions of any one cell
         if (lane < TZ + 3) {
             const int* off = a.cat[sl.src[0].cat].off;
-            const int zr = (z0 - 2 + lane) & (N - 1);
+            const int zr = (z0 - rc.lo + lane) & (N - 1);
 #pragma unroll
             for (int dy = 0; dy < TY + 3; ++dy) {
-                const int yr = (y0 - 2 + dy) & (N - 1);
+                const int yr = (y0 - rc.lo + dy) & (N - 1);
                 rcount[lane][dy] = off[zr * N + yr + 1] - off[zr * N + yr];
             }
         }
         __syncwarp();
         int wsum = 0;
         if (lane < TY * TZ) {
-            const int ly = lane % TY, lz = lane / TY;   // cell (y0 + ly, z0 + lz): rows ly..ly+3
+            const int ly = lane % TY, lz = lane / TY;   // cell (y0 + ly, z0 + lz): rows ly..ly+lo+hi
 #pragma unroll
             for (int a2 = 0; a2 < 4; ++a2)
 #pragma unroll
-                for (int b2 = 0; b2 < 4; ++b2) wsum += rcount[lz + a2][ly + b2];
+                for (int b2 = 0; b2 < 4; ++b2)
+                    if (a2 <= rc.lo + rc.hi && b2 <= rc.lo + rc.hi) wsum += rcount[lz + a2][ly + b2];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wsum = max(wsum, __shfl_down_sync(0xffffffffu, wsum, o));
@@ -410,12 +413,13 @@ __device__ __forceinline__ void tile_setup(const FusedArgs<T>& a, const FusedSlo
     if (NT < 64) {
         // tiny tiles (n <= 16): one thread finds the ranges, everybody clears the tile
         if (tid == 0) {
+            const Reach rc = stencil_reach(a.scheme, a.interlace);
             int nr = 0, acc = 0;
             for (int sidx = 0; sidx < sl.n_src; ++sidx) {
                 const int* off = a.cat[sl.src[sidx].cat].off;
-                for (int dz = 0; dz < TZ + 3; ++dz) {
-                    const int zr = (z0 - 2 + dz) & (N - 1);
-                    const int ylo = y0 - 2, yhi = y0 + TY;
+                for (int dz = 0; dz < TZ + rc.lo + rc.hi; ++dz) {
+                    const int zr = (z0 - rc.lo + dz) & (N - 1);
+                    const int ylo = y0 - rc.lo, yhi = y0 + TY - 1 + rc.hi;
                     int bb[2], ee[2], m = 0;
                     bb[m] = off[zr * N + (ylo < 0 ? 0 : ylo)];
                     ee[m++] = off[zr * N + (yhi >= N ? N - 1 : yhi) + 1];
@@ -578,7 +582,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T>& a, int slot, int 
     const int P = a.scheme;
     const T* vb_ptr = (!a.interlace && sl.vals_b) ? static_cast<const T*>(sl.vals_b) : nullptr;
     // fixed-point accumulation (FP32 channel slots): a cell sums at most wmax contributions
-    // (particles of its 4 x 4 key-row window) of magnitude <= amax (the TSC/CIC weights are
+    // (particles of its key-row window) of magnitude <= amax (the TSC/CIC weights are
     // <= 1), so 2^30 / (max(wmax, kMinWindow) amax) units keep every cell and its rounding
     // (<= wmax units, two sub-grid stencils) inside int32 and every contribution within
     // 2^21 units (fixed_round).  The tile takes it only
@@ -667,7 +671,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs<T>& a, int slot, int 
 }
 
 __global__ void k_plane_mask(const int* __restrict__ off0, const int* __restrict__ off1, const int* __restrict__ off2,
-                             int set0, int set1, int set2, int n, int* __restrict__ pmask) {
+                             int set0, int set1, int set2, int n, Reach reach, int* __restrict__ pmask) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * n) return;
     const int r = i / n, z = i - r * n;
@@ -675,7 +679,7 @@ __global__ void k_plane_mask(const int* __restrict__ off0, const int* __restrict
     const int set = r == 0 ? set0 : (r == 1 ? set1 : set2);
     int hit = 0;
     if (set) {
-        for (int d = -2; d <= 1; ++d) {
+        for (int d = -reach.lo; d <= reach.hi; ++d) {
             const int f = (z + d) & (n - 1);
             hit |= off[(size_t)(f + 1) * n] > off[(size_t)f * n];
         }
@@ -684,7 +688,7 @@ __global__ void k_plane_mask(const int* __restrict__ off0, const int* __restrict
 }
 
 __global__ void k_pencil_live(const int* __restrict__ off0, const int* __restrict__ off1,
-                              const int* __restrict__ off2, int set0, int set1, int set2, int n,
+                              const int* __restrict__ off2, int set0, int set1, int set2, int n, Reach reach,
                               unsigned char* __restrict__ plive) {
     const long long nn = (long long)n * n;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < 3 * nn;
@@ -696,9 +700,9 @@ __global__ void k_pencil_live(const int* __restrict__ off0, const int* __restric
         const int set = r == 0 ? set0 : (r == 1 ? set1 : set2);
         int hit = 0;
         if (set) {
-            for (int dz = -2; dz <= 1 && !hit; ++dz) {
+            for (int dz = -reach.lo; dz <= reach.hi && !hit; ++dz) {
                 const int fz = (z + dz) & (n - 1);
-                for (int dy = -2; dy <= 1; ++dy) {
+                for (int dy = -reach.lo; dy <= reach.hi; ++dy) {
                     const int key = fz * n + ((y + dy) & (n - 1));
                     if (off[key + 1] > off[key]) { hit = 1; break; }
                 }
@@ -709,17 +713,17 @@ __global__ void k_pencil_live(const int* __restrict__ off0, const int* __restric
 }
 
 cudaError_t launch_pencil_live(const int* off0, const int* off1, const int* off2, int set0, int set1, int set2, int n,
-                               unsigned char* plive, cudaStream_t st) {
+                               Reach reach, unsigned char* plive, cudaStream_t st) {
     const long long total = 3LL * n * n;
     long long blocks = (total + 255) / 256;
     if (blocks > 152 * 32) blocks = 152 * 32;
-    k_pencil_live<<<(int)blocks, 256, 0, st>>>(off0, off1, off2, set0, set1, set2, n, plive);
+    k_pencil_live<<<(int)blocks, 256, 0, st>>>(off0, off1, off2, set0, set1, set2, n, reach, plive);
     return cudaGetLastError();
 }
 
 cudaError_t launch_plane_mask(const int* off0, const int* off1, const int* off2, int set0, int set1, int set2, int n,
-                              int* pmask, cudaStream_t st) {
-    k_plane_mask<<<(3 * n + 255) / 256, 256, 0, st>>>(off0, off1, off2, set0, set1, set2, n, pmask);
+                              Reach reach, int* pmask, cudaStream_t st) {
+    k_plane_mask<<<(3 * n + 255) / 256, 256, 0, st>>>(off0, off1, off2, set0, set1, set2, n, reach, pmask);
     return cudaGetLastError();
 }
 
