@@ -352,7 +352,7 @@ static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, cons
     }
     if (timer) timer->begin(KK_FFT, st);
     bool skip = false;
-    for (int i = 0; i < n_grids && i < 8; ++i) skip = skip || (g.pmask && g.gmask[i]);
+    for (int i = 0; i < n_grids && i < kMaxSlots; ++i) skip = skip || (g.pmask && g.gmask[i]);
     // one wave of resident CTAs (the occupancy the launch bounds give), at most one per item
     auto wave = [&](auto kernel, int threads, size_t bytes) {
         int dev = 0, sms = 0, ps = 0;

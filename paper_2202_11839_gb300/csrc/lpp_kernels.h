@@ -60,7 +60,7 @@ struct FftGeom {
     // nonzero where a particle of that role can reach plane z) and, per grid of the call,
     // the bit set of roles assigned to it (0: never skip)
     const int* pmask = nullptr;
-    int gmask[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    int gmask[16] = {};
     float yread_frac = 1.0f;   // host bookkeeping: fraction of z planes the y pass writes
     float ylive_frac = 1.0f;   // host bookkeeping: fraction of x pencils the y pass reads
     // modes with |f|^2 >= q_max are beyond the last shell and never read by the combine: the y and z
@@ -84,7 +84,7 @@ cudaError_t fft_yz(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGe
 
 // ---------------------------------------------------------- per-particle weights
 constexpr int kMaxGroups = 16;
-constexpr int kMaxSlots = 8;       // complex grids per batch (FftGeom::gmask has as many)
+constexpr int kMaxSlots = 16;      // complex grids per batch (FftGeom::gmask has as many)
 constexpr int kMaxBatchCh = 16;    // real fields per batch
 
 struct CoeffGroup {
