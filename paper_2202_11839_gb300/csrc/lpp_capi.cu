@@ -877,7 +877,7 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
         double fl = 0.0;
         for (int i = 0; i < fa.n_slots; ++i) fl += pencil_frac(gp.gmask[fa.slots[i].grid]);
         gp.ylive_frac = fa.n_slots ? (float)(fl / fa.n_slots) : 1.0f;
-        LPP_CUDA(fft_yz<T>(grids, pgrids, n, tw, gp, false, st, tm));
+        LPP_CUDA(fft_yz<T>(grids, pgrids, n, tw, gp, st, tm));
         nl += 2;
         cb.partner_mode = 1;
         cb.has_d = plan->need_d;
@@ -998,7 +998,7 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
         gc.yread_frac = (float)plane_frac(bits);
         gc.plive = plive;
         gc.ylive_frac = (float)pencil_frac(bits);
-        LPP_CUDA(fft_yz<T>(grids, ngr, n, tw, gc, false, st, tm));
+        LPP_CUDA(fft_yz<T>(grids, ngr, n, tw, gc, st, tm));
         if (tm) tm->begin(KK_COMBINE, st);
         LPP_CUDA(launch_combine<T>(cb, plan->n_sm, st));
         nl += 3;
@@ -1158,7 +1158,7 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
                                    (int*)(plan->ws + plan->off_cursor), (int*)(plan->ws + plan->off_scan),
                                    (T*)(plan->ws + plan->off_su[LPP_RANDOMS]),
                                    (T*)(plan->ws + plan->off_sw[LPP_RANDOMS]), nullptr, err, st));
-    // forward transforms keep every frequency; the inverse keeps the separations of the shells
+    // the fields' transforms keep every frequency; the correlations' keep the separations of the shells
     FftGeom gfull = fft_geometry(n, n / 2 - 1, n / 2);
     FftGeom gs = fft_geometry(n, ns_pos, ns_neg);
     gfull.err = err;
@@ -1211,7 +1211,7 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
     fa.sums = sums;
     for (int a = 0; a < 3; ++a) { fa.observer[a] = plan->d.observer[a]; fa.origin[a] = plan->d.origin[a]; }
     fa.h = h;
-    // the window field W itself: transformed and deconvolved into the partner array
+    // the window field W itself: its transform and deconvolution into the partner array
     fa.n_slots = 1;
     FusedSlot ws{};
     ws.n_src = 1;
@@ -1220,8 +1220,9 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
     ws.yl_a = ws.yl_b = -1;
     fa.slots[0] = ws;
     { lpp_status s0 = assign(); if (s0 != LPP_OK) return s0; }
-    LPP_CUDA(fft_yz<T>(grids, 1, n, tw, gfull, false, st, nullptr));
+    LPP_CUDA(fft_yz<T>(grids, 1, n, tw, gfull, st, nullptr));
     LPP_CUDA(launch_window_partner<T>(grids, pW, iw, n, st));
+    gfull.mult = pW;   // the channels' z passes write the correlation's transform
     // channels (l, m), two per grid
     int chl[kWindowChannels], chm[kWindowChannels], nchan = 0;
     for (int l = 0; l <= 8; l += 2)
@@ -1277,9 +1278,8 @@ static lpp_status run_window(lpp_plan_t plan, int nb, const double* s_edges, dou
             }
         }
         { lpp_status s0 = assign(); if (s0 != LPP_OK) return s0; }
-        LPP_CUDA(fft_yz<T>(grids, ngr, n, tw, gfull, false, st, nullptr));
-        LPP_CUDA(launch_window_mult<T>(grids, (long long)n3, ngr, pW, iw, n, st));
-        LPP_CUDA(fft3d<T>(grids, ngr, n, tw, gs, true, st, nullptr));
+        LPP_CUDA(fft_yz<T>(grids, ngr, n, tw, gfull, st, nullptr));
+        LPP_CUDA(fft3d<T>(grids, ngr, n, tw, gs, st, nullptr));
         LPP_CUDA(launch_sbin<T>(sb, plan->n_sm, st));
     }
     std::vector<double> h_out((size_t)kWindowChannels * nb * 2);

@@ -68,7 +68,7 @@ struct ColumnBound {
 // loaded into tw here, after the column test and beside the operand loads (they are first
 // read after the first stage's barrier); null when tw already holds them.  Every return is
 // CTA-uniform; the tile is free again after the caller's next barrier.
-template <typename T, int LOGN, bool INV, int MODE>
+template <typename T, int LOGN, int MODE>
 __device__ __forceinline__ void pencil_tile(c2<T>* grid, const c2<T>* twg, c2<T>* tw, c2<T>* tile, const FftGeom& g,
                                             int tile_id, int gi) {
     using S = PassShape<LOGN>;
@@ -129,15 +129,17 @@ __device__ __forceinline__ void pencil_tile(c2<T>* grid, const c2<T>* twg, c2<T>
     }
     if (twg)
         for (int k = tid; k < N; k += S::THREADS) tw[k] = twg[k];
-    fft_columns_io<T, LOGN, INV, S::IPT, LD>(
+    fft_columns_io<T, LOGN, false, S::IPT, LD>(
         tile, c, u, tw,
         [&](int b, int e) { return ((live >> b) & 1u) ? gp[(size_t)e * ES] : mk<T>((T)0, (T)0); },
         [&](int e, c2<T> v) {
-            if (col.stores(g, e)) gp[(size_t)e * ES] = v;
+            if (!col.stores(g, e)) return;
+            if (MODE == 2 && g.mult) v = cmul<T>(v, static_cast<const c2<T>*>(g.mult)[(gp - grid) + (size_t)e * ES]);
+            gp[(size_t)e * ES] = v;
         });
 }
 
-template <typename T, int LOGN, bool INV, int MODE>
+template <typename T, int LOGN, int MODE>
 __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LOGN == 9 ? 3 : 2) : 1) k_fft_pass(c2<T>* __restrict__ data,
                                                                       const c2<T>* __restrict__ twg, FftGeom g) {
     using S = PassShape<LOGN>;
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LO
             tile[e * LD + c] = base[e + c * N];
         }
         __syncthreads();
-        fft_columns<T, LOGN, INV, S::IPT, LD>(tile, tid & (W - 1), tid >> S::LOGW, tw);
+        fft_columns<T, LOGN, false, S::IPT, LD>(tile, tid & (W - 1), tid >> S::LOGW, tw);
 #pragma unroll
         for (int k = 0; k < S::PER; ++k) {
             const int idx = tid + k * S::THREADS;
@@ -173,14 +175,14 @@ __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LO
         // a z plane that no particle of the grid's roles reaches: its pencils are zero;
         // neither the fused assignment nor this pass stores it
         if (MODE == 1 && !plane_live(g, blockIdx.y, tile_id / g.ntx, N)) return;
-        pencil_tile<T, LOGN, INV, MODE>(grid, twg, tw, tile, g, tile_id, blockIdx.y);
+        pencil_tile<T, LOGN, MODE>(grid, twg, tw, tile, g, tile_id, blockIdx.y);
     }
 }
 
 // The y pass as a persistent grid over the (grid, plane, x tile) items of the call, for calls
 // that skip unreached planes: the items of unreached planes cost a mask test instead of a
 // CTA launch (with its shared memory held), and the twiddles are loaded once per CTA.
-template <typename T, int LOGN, bool INV>
+template <typename T, int LOGN>
 __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LOGN == 9 ? 3 : 2) : 1) k_fft_ypass(c2<T>* __restrict__ data,
                                                                        const c2<T>* __restrict__ twg, FftGeom g, int n_grids) {
     using S = PassShape<LOGN>;
@@ -194,14 +196,14 @@ __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LO
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int gi = it / per_grid, tile_id = it - gi * per_grid;
         if (!plane_live(g, gi, tile_id / g.ntx, N)) continue;
-        pencil_tile<T, LOGN, INV, 1>(data + (size_t)gi * N * N * N, nullptr, tw, tile, g, tile_id, gi);
+        pencil_tile<T, LOGN, 1>(data + (size_t)gi * N * N * N, nullptr, tw, tile, g, tile_id, gi);
         __syncthreads();   // the next item's first stage rewrites the tile
     }
 }
 
 // ---- FP32 passes on pencil pairs (lpp_fft_pair.cuh), 64 <= n <= 1024
 // One y (MODE 1) or z (MODE 2) tile of one grid, as pencil_tile.
-template <int LOGN, bool INV, int MODE>
+template <int LOGN, int MODE, bool MULT>
 __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair* tw, cpair* tile, const FftGeom& g,
                                           int tile_id, int gi) {
     using S = PairShape<LOGN>;
@@ -255,7 +257,7 @@ __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair
     auto twiddle = [](float2 w) { return cpair{pk2(w.x, w.x), pk2(-w.y, -w.y)}; };
     if (twg)
         for (int k = tid; k < N; k += S::THREADS) tw[k] = twiddle(twg[k]);
-    fft_pairs_io<LOGN, INV>(
+    fft_pairs_io<LOGN, false>(
         tile, c, u, tw,
         [&](int b, int e) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -264,6 +266,11 @@ __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair
         },
         [&](int e, cpair v) {
             if (!col.stores(g, e)) return;
+            if constexpr (MULT) {
+                const float4 f = static_cast<const float4*>(
+                    g.mult)[(gp - reinterpret_cast<float4*>(grid)) + (size_t)e * (ES / 2)];
+                v = pmul<true>(v, cpair{pk2(f.x, f.z), pk2(f.y, f.w)});
+            }
             float4 w;
             unpk2(v.re, w.x, w.z);
             unpk2(v.im, w.y, w.w);
@@ -271,7 +278,7 @@ __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair
         });
 }
 
-template <int LOGN, bool INV, int MODE>
+template <int LOGN, int MODE, bool MULT = false>
 __global__ void __launch_bounds__(PairShape<LOGN>::THREADS, PairShape<LOGN>::MINB)
 k_fft_pair(float2* __restrict__ data, const float2* __restrict__ twg, const __grid_constant__ FftGeom g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -280,11 +287,14 @@ k_fft_pair(float2* __restrict__ data, const float2* __restrict__ twg, const __gr
     // a z plane that no particle of the grid's roles reaches is neither stored by the fused
     // assignment nor by this pass
     if (MODE == 1 && !plane_live(g, blockIdx.y, blockIdx.x / g.ntx, (int)N)) return;
-    pair_tile<LOGN, INV, MODE>(data + blockIdx.y * N * N * N, twg, tw, tw + N, g, blockIdx.x, blockIdx.y);
+    // MULT: the grids' CTAs of one tile side by side (they share its factors in L2)
+    const int ng = MULT ? (int)gridDim.x / (g.ntx * g.nky) : 1;
+    const int gi = MULT ? (int)blockIdx.x % ng : (int)blockIdx.y, tile_id = (int)blockIdx.x / ng;
+    pair_tile<LOGN, MODE, MULT>(data + gi * N * N * N, twg, tw, tw + N, g, tile_id, gi);
 }
 
 // The y pass as a persistent grid (see k_fft_ypass).
-template <int LOGN, bool INV>
+template <int LOGN>
 __global__ void __launch_bounds__(PairShape<LOGN>::THREADS, PairShape<LOGN>::MINB)
 k_fft_ypair(float2* __restrict__ data, const float2* __restrict__ twg, const __grid_constant__ FftGeom g, int n_grids) {
     using S = PairShape<LOGN>;
@@ -300,7 +310,7 @@ k_fft_ypair(float2* __restrict__ data, const float2* __restrict__ twg, const __g
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
         const int gi = it / per_grid, tile_id = it - gi * per_grid;
         if (!plane_live(g, gi, tile_id / g.ntx, N)) continue;
-        pair_tile<LOGN, INV, 1>(data + (size_t)gi * N * N * N, nullptr, tw, tw + N, g, tile_id, gi);
+        pair_tile<LOGN, 1, false>(data + (size_t)gi * N * N * N, nullptr, tw, tw + N, g, tile_id, gi);
         __syncthreads();   // the next item's first stage rewrites the tile
     }
 }
@@ -331,7 +341,7 @@ FftGeom fft_geometry(int n, int nk_pos, int nk_neg) {
     return g;
 }
 
-template <typename T, int LOGN, bool INV>
+template <typename T, int LOGN>
 static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, const FftGeom& geom, bool with_x,
                                  cudaStream_t st, Timer* timer) {
     using S = PassShape<LOGN>;
@@ -341,13 +351,13 @@ static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, cons
     if (sizeof(T) == 4 && LOGN >= 6) set_tiles(g, N, PairShape<LOGN>::W);
     const size_t smem = (size_t)(N + N * S::LD) * sizeof(c2<T>);
     // the attribute is per device and function: set it on every call (cheap, host-only)
-    cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_fft_pass<T, LOGN, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const double es = (double)sizeof(c2<T>);
     const double n3 = (double)N * N * N;
     const double keep = (double)(g.nky) / N;               // kept fraction of one axis
     if (with_x) {
         if (timer) timer->begin(KK_FFT, st);
-        k_fft_pass<T, LOGN, INV, 0><<<dim3((N / W) * N, n_grids), S::THREADS, smem, st>>>(data, tw, g);
+        k_fft_pass<T, LOGN, 0><<<dim3((N / W) * N, n_grids), S::THREADS, smem, st>>>(data, tw, g);
         if (timer) timer->end(KK_FFT, st, n_grids * n3 * es * (1.0 + keep));
     }
     if (timer) timer->begin(KK_FFT, st);
@@ -367,20 +377,20 @@ static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, cons
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
         };
         if (skip) {
-            attr(k_fft_ypair<LOGN, INV>);
-            k_fft_ypair<LOGN, INV><<<wave(k_fft_ypair<LOGN, INV>, P::THREADS, P::SMEM), P::THREADS, P::SMEM, st>>>(
+            attr(k_fft_ypair<LOGN>);
+            k_fft_ypair<LOGN><<<wave(k_fft_ypair<LOGN>, P::THREADS, P::SMEM), P::THREADS, P::SMEM, st>>>(
                 data, tw, g, n_grids);
         } else {
-            attr(k_fft_pair<LOGN, INV, 1>);
-            k_fft_pair<LOGN, INV, 1><<<dim3(g.ntx * N, n_grids), P::THREADS, P::SMEM, st>>>(data, tw, g);
+            attr(k_fft_pair<LOGN, 1>);
+            k_fft_pair<LOGN, 1><<<dim3(g.ntx * N, n_grids), P::THREADS, P::SMEM, st>>>(data, tw, g);
         }
     } else if (skip) {
-        cudaFuncSetAttribute(k_fft_ypass<T, LOGN, INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_fft_ypass<T, LOGN, INV><<<wave(k_fft_ypass<T, LOGN, INV>, S::THREADS, smem), S::THREADS, smem, st>>>(
+        cudaFuncSetAttribute(k_fft_ypass<T, LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_fft_ypass<T, LOGN><<<wave(k_fft_ypass<T, LOGN>, S::THREADS, smem), S::THREADS, smem, st>>>(
             data, tw, g, n_grids);
     } else {
-        cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_fft_pass<T, LOGN, INV, 1><<<dim3(g.ntx * N, n_grids), S::THREADS, smem, st>>>(data, tw, g);
+        cudaFuncSetAttribute(k_fft_pass<T, LOGN, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_fft_pass<T, LOGN, 1><<<dim3(g.ntx * N, n_grids), S::THREADS, smem, st>>>(data, tw, g);
     }
     // the fractions of the grid's columns and modes that the passes move (ColumnBound)
     double circle = keep * keep, sphere = keep * keep * keep;
@@ -406,25 +416,32 @@ static cudaError_t launch_passes(c2<T>* data, int n_grids, const c2<T>* tw, cons
     if (timer) timer->begin(KK_FFT, st);
     if constexpr (sizeof(T) == 4 && LOGN >= 6) {
         using P = PairShape<LOGN>;
-        cudaFuncSetAttribute(k_fft_pair<LOGN, INV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
-        k_fft_pair<LOGN, INV, 2><<<dim3(g.ntx * g.nky, n_grids), P::THREADS, P::SMEM, st>>>(data, tw, g);
+        auto attr = [&](auto kernel) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::SMEM);
+        };
+        if (g.mult) {
+            attr(k_fft_pair<LOGN, 2, true>);
+            k_fft_pair<LOGN, 2, true><<<g.ntx * g.nky * n_grids, P::THREADS, P::SMEM, st>>>(data, tw, g);
+        } else {
+            attr(k_fft_pair<LOGN, 2>);
+            k_fft_pair<LOGN, 2><<<dim3(g.ntx * g.nky, n_grids), P::THREADS, P::SMEM, st>>>(data, tw, g);
+        }
     } else {
-        cudaFuncSetAttribute(k_fft_pass<T, LOGN, INV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_fft_pass<T, LOGN, INV, 2><<<dim3(g.ntx * g.nky, n_grids), S::THREADS, smem, st>>>(data, tw, g);
+        cudaFuncSetAttribute(k_fft_pass<T, LOGN, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_fft_pass<T, LOGN, 2><<<dim3(g.ntx * g.nky, n_grids), S::THREADS, smem, st>>>(data, tw, g);
     }
     if (timer) timer->end(KK_FFT, st, n_grids * n3 * es * (circle * (double)g.yread_frac + sphere));
     return cudaGetLastError();
 }
 
 template <typename T>
-static cudaError_t fft_dispatch(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, bool inverse,
+static cudaError_t fft_dispatch(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g,
                                 bool with_x, cudaStream_t st, Timer* timer) {
     int logn = 0;
     while ((1 << logn) < n) ++logn;
 #define LPP_FFT_CASE(LG)                                                                          \
     case LG:                                                                                      \
-        return inverse ? launch_passes<T, LG, true>(data, n_grids, tw, g, with_x, st, timer)     \
-                       : launch_passes<T, LG, false>(data, n_grids, tw, g, with_x, st, timer);
+        return launch_passes<T, LG>(data, n_grids, tw, g, with_x, st, timer);
     switch (logn) {
         LPP_FFT_CASE(3)
         LPP_FFT_CASE(4)
@@ -441,20 +458,20 @@ static cudaError_t fft_dispatch(c2<T>* data, int n_grids, int n, const c2<T>* tw
 }
 
 template <typename T>
-cudaError_t fft3d(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, bool inverse,
+cudaError_t fft3d(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g,
                   cudaStream_t st, Timer* timer) {
-    return fft_dispatch<T>(data, n_grids, n, tw, g, inverse, true, st, timer);
+    return fft_dispatch<T>(data, n_grids, n, tw, g, true, st, timer);
 }
 
 template <typename T>
-cudaError_t fft_yz(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, bool inverse,
+cudaError_t fft_yz(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g,
                    cudaStream_t st, Timer* timer) {
-    return fft_dispatch<T>(data, n_grids, n, tw, g, inverse, false, st, timer);
+    return fft_dispatch<T>(data, n_grids, n, tw, g, false, st, timer);
 }
 
-template cudaError_t fft3d<float>(c2<float>*, int, int, const c2<float>*, const FftGeom&, bool, cudaStream_t, Timer*);
-template cudaError_t fft3d<double>(c2<double>*, int, int, const c2<double>*, const FftGeom&, bool, cudaStream_t, Timer*);
-template cudaError_t fft_yz<float>(c2<float>*, int, int, const c2<float>*, const FftGeom&, bool, cudaStream_t, Timer*);
-template cudaError_t fft_yz<double>(c2<double>*, int, int, const c2<double>*, const FftGeom&, bool, cudaStream_t, Timer*);
+template cudaError_t fft3d<float>(c2<float>*, int, int, const c2<float>*, const FftGeom&, cudaStream_t, Timer*);
+template cudaError_t fft3d<double>(c2<double>*, int, int, const c2<double>*, const FftGeom&, cudaStream_t, Timer*);
+template cudaError_t fft_yz<float>(c2<float>*, int, int, const c2<float>*, const FftGeom&, cudaStream_t, Timer*);
+template cudaError_t fft_yz<double>(c2<double>*, int, int, const c2<double>*, const FftGeom&, cudaStream_t, Timer*);
 
 }  // namespace lpp

@@ -70,17 +70,19 @@ struct FftGeom {
     // x pencils that no particle of the grid's roles reaches (the fused pass stores nothing there)
     const unsigned char* plive = nullptr;
     int* err = nullptr;   // ERRF_BOUNDS of LPP_CHECK builds
+    // z pass: a factor per mode (c2<T>[n^3]) that every grid's results take; null: none
+    const void* mult = nullptr;
 };
 
 int fft_tile_width(int n);
 FftGeom fft_geometry(int n, int nk_pos, int nk_neg);
 template <typename T>
-cudaError_t fft3d(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, bool inverse,
-                  cudaStream_t st, Timer* timer);
+cudaError_t fft3d(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, cudaStream_t st,
+                  Timer* timer);
 // y and z passes only (the x pass fused into the assignment kernel)
 template <typename T>
-cudaError_t fft_yz(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, bool inverse,
-                   cudaStream_t st, Timer* timer);
+cudaError_t fft_yz(c2<T>* data, int n_grids, int n, const c2<T>* tw, const FftGeom& g, cudaStream_t st,
+                   Timer* timer);
 
 // ---------------------------------------------------------- per-particle weights
 constexpr int kMaxGroups = 16;
@@ -326,13 +328,9 @@ cudaError_t launch_combine(const CombineArgs<T>& a, int n_sm, cudaStream_t st);
 void combine_items(int n, int nk_pos, int nk_neg, int nzi, int q_max, std::vector<int>& items);
 
 // ------------------------------------------------------------------ window multipoles
-// pD[m] = Z[m] / W(m) over every mode of grid 0 (the window field alone in the real part)
+// pD[m] = conj(Z[m]) / W(m)^2 over every mode of grid 0 (the window field alone in the real part)
 template <typename T>
 cudaError_t launch_window_partner(const c2<T>* grid, c2<T>* pD, const T* inv_w, int n, cudaStream_t st);
-// per mode pair, Z <- conj(A/W) pD + i conj(B/W) pD for the two packed fields of every grid
-template <typename T>
-cudaError_t launch_window_mult(c2<T>* grids, long long grid_stride, int n_grids, const c2<T>* pD, const T* inv_w,
-                               int n, cudaStream_t st);
 struct SbinChan {
     int grid, sub, l, m;
     double ynorm;   // normalisation of Y_{l,m} divided by (l - |m|)! (goes with ylm_poly_scaled)

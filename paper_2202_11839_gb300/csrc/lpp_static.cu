@@ -151,7 +151,7 @@ lpp_status run_static(char* base, const Layout& lay, int n, double box, const do
     aa.err = err;
     LPP_STATIC_CUDA(launch_assign<T>(aa, scheme, interlace, st));
     const FftGeom geom = fft_geometry(n, nk_pos, nk_neg);
-    LPP_STATIC_CUDA(fft3d<T>(grid, 1, n, reinterpret_cast<const c2<T>*>(base + lay.tw), geom, false, st, nullptr));
+    LPP_STATIC_CUDA(fft3d<T>(grid, 1, n, reinterpret_cast<const c2<T>*>(base + lay.tw), geom, st, nullptr));
     CombineArgs<T> cb;
     memset(&cb, 0, sizeof(cb));
     cb.grids = grid;

@@ -3,8 +3,11 @@
 // With the addition theorem L_l(s.x) = 4 pi / (2l+1) sum_n Y_{l,n}(s) Y_{l,n}(x) (real
 // harmonics), Q_l(s) = 4 pi < sum_n Y_{l,n}(s) C_n(s) >_shell / I with the
 // cross-correlations C_n(s) = int_x A_n(x) W(x+s) of A_n = W Y_{l,n}(x) and W.  Each C_n is
-// IFFT[conj(A_n(k)) W(k)]; two real fields share one complex grid, so a pass packs
-// C_a + i C_b and the inverse transform returns both correlations at once.
+// IFFT[conj(A_n(k)) W(k)]; two real fields share one complex grid Z = A_a + i A_b.  For real fields
+// conj(A_a(k)) + i conj(A_b(k)) = Z(-k), so C_a + i C_b = IFFT[Z(-k) W(k)] = FFT[Z(k) conj(W(k))] / n^3:
+// the z pass of Z's transform multiplies its results by conj(W) (deconvolved twice) and a second
+// forward transform returns both correlations at once.  (As a kernel of its own over the pairs (k, -k)
+// the products took 1.44 of 12.5 ms of kernels of a 256^3 call.)
 #include "lpp_internal.h"
 #include "lpp_kernels.h"
 #include "lpp_reduce.cuh"
@@ -21,58 +24,14 @@ __global__ void k_window_partner(const c2<T>* __restrict__ grid, c2<T>* __restri
     for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < n3;
          m += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(m % n), y = (int)((m / n) % n), z = (int)(m / ((long long)n * n));
-        pD[m] = cscale<T>(grid[m], inv_w[x] * inv_w[y] * inv_w[z]);
+        const T w = inv_w[x] * inv_w[y] * inv_w[z];
+        pD[m] = cscale<T>(cconj<T>(grid[m]), w * w);
     }
 }
 
 template <typename T>
 cudaError_t launch_window_partner(const c2<T>* grid, c2<T>* pD, const T* inv_w, int n, cudaStream_t st) {
     k_window_partner<T><<<152 * 8, 256, 0, st>>>(grid, pD, inv_w, n);
-    return cudaGetLastError();
-}
-
-// One thread per mode pair (m, -m): rows (z, y) with z in [0, n/2]; in the self-conjugate
-// planes z = 0 and z = n/2 the pair is taken from its lexicographically smaller member.
-template <typename T>
-__global__ void k_window_mult(c2<T>* __restrict__ grids, long long grid_stride, const c2<T>* __restrict__ pD,
-                              const T* __restrict__ inv_w, int n) {
-    c2<T>* g = grids + (long long)blockIdx.y * grid_stride;
-    const int rows = (n / 2 + 1) * n;
-    for (int row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int z = row / n, y = row - z * n;
-        const int zp = (n - z) & (n - 1), yp = (n - y) & (n - 1);
-        for (int x = threadIdx.x; x < n; x += blockDim.x) {
-            const int xp = (n - x) & (n - 1);
-            if (z == zp && (y > yp || (y == yp && x > xp))) continue;
-            const long long im = ((long long)z * n + y) * n + x;
-            const long long ip = ((long long)zp * n + yp) * n + xp;
-            const c2<T> zm = g[im], zq = g[ip];
-            const T h = (T)0.5;
-            const c2<T> A = mk<T>(h * (zm.x + zq.x), h * (zm.y - zq.y));        // (Z(m) + conj Z(-m)) / 2
-            const c2<T> B = mk<T>(h * (zm.y + zq.y), -h * (zm.x - zq.x));       // -i (Z(m) - conj Z(-m)) / 2
-            const T wm = inv_w[x] * inv_w[y] * inv_w[z];
-            const T wp = inv_w[xp] * inv_w[yp] * inv_w[zp];
-            const c2<T> Pm = pD[im], Pp = pD[ip];
-            // conj(F/W) P at m; the fields at -m are conj A, conj B
-            const c2<T> ca = cmul<T>(cconj<T>(cscale<T>(A, wm)), Pm);
-            const c2<T> cb = cmul<T>(cconj<T>(cscale<T>(B, wm)), Pm);
-            g[im] = mk<T>(ca.x - cb.y, ca.y + cb.x);                            // Ca + i Cb
-            if (ip != im) {
-                const c2<T> da = cmul<T>(cscale<T>(A, wp), Pp);
-                const c2<T> db = cmul<T>(cscale<T>(B, wp), Pp);
-                g[ip] = mk<T>(da.x - db.y, da.y + db.x);
-            }
-        }
-    }
-}
-
-template <typename T>
-cudaError_t launch_window_mult(c2<T>* grids, long long grid_stride, int n_grids, const c2<T>* pD, const T* inv_w,
-                               int n, cudaStream_t st) {
-    const int rows = (n / 2 + 1) * n;
-    int bx = rows < 152 * 8 ? rows : 152 * 8;
-    const int threads = n < 256 ? n : 256;
-    k_window_mult<T><<<dim3(bx, n_grids), threads, 0, st>>>(grids, grid_stride, pD, inv_w, n);
     return cudaGetLastError();
 }
 
@@ -173,10 +132,6 @@ cudaError_t launch_sbin(const SbinArgs<T>& a, int n_sm, cudaStream_t st) {
 
 template cudaError_t launch_window_partner<float>(const c2<float>*, c2<float>*, const float*, int, cudaStream_t);
 template cudaError_t launch_window_partner<double>(const c2<double>*, c2<double>*, const double*, int, cudaStream_t);
-template cudaError_t launch_window_mult<float>(c2<float>*, long long, int, const c2<float>*, const float*, int,
-                                               cudaStream_t);
-template cudaError_t launch_window_mult<double>(c2<double>*, long long, int, const c2<double>*, const double*, int,
-                                                cudaStream_t);
 template cudaError_t launch_sbin<float>(const SbinArgs<float>&, int, cudaStream_t);
 template cudaError_t launch_sbin<double>(const SbinArgs<double>&, int, cudaStream_t);
 
