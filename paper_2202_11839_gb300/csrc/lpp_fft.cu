@@ -2,12 +2,12 @@
 //
 // Each CTA transforms a tile of W pencils (n complex points each) with a mixed-radix
 // Stockham FFT (radix 8 stages, one leading radix-2 or -4 stage), every thread holding
-// 8 points per stage (FP32 grids of 64^3 and more: 8 points of two pencils, lpp_fft_pair.cuh), and
-// writes the pencils back in place.  Pencils along y and z are
-// read as rows of W consecutive x values, so every global access is a contiguous
-// W-element segment; the first stage takes its operands straight from those rows and
-// the last stage stores straight to them, so shared memory holds only the stages in
-// between.  x pencils are transposed into the same column layout in shared memory.
+// 8 points per stage (FP32 grids of 64^3 and more: 8 points of two pencils,
+// lpp_fft_pair.cuh), and writes the pencils back in place.  Pencils along y and z are read
+// as rows of W consecutive x values, so every global access is a contiguous W-element
+// segment; the first stage takes its operands straight from those rows and the last stage
+// stores straight to them, so shared memory holds only the stages in between.  x pencils
+// are transposed into the same column layout in shared memory.
 //
 // Passes can be pruned to the frequencies the shell binning needs: with a kept
 // range f in [-nk_neg, nk_pos] per axis, the x pass writes only kept x, the y pass
@@ -202,7 +202,8 @@ __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LO
 }
 
 // ---- FP32 passes on pencil pairs (lpp_fft_pair.cuh), 64 <= n <= 1024
-// One y (MODE 1) or z (MODE 2) tile of one grid, as pencil_tile.
+// One y (MODE 1) or z (MODE 2) tile of one grid, as pencil_tile.  MULT: the results take the factors
+// g.mult (the window multipoles on 256^3: z passes and products 2.12 -> 1.41 ms for 23 grids).
 template <int LOGN, int MODE, bool MULT>
 __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair* tw, cpair* tile, const FftGeom& g,
                                           int tile_id, int gi) {

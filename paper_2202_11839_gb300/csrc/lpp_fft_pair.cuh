@@ -1,16 +1,19 @@
 // FP32 pencil FFT on pairs of pencils with packed arithmetic (internal).
 //
 // With one pencil per thread the y and z passes were bound by instruction issue and by loads in
-// flight, not by DRAM.  Here a thread owns two neighbouring pencils: every value is a pair (re0, re1) or (im0, im1) in a 64-bit
-// register, added and multiplied by the packed FP32 instructions of sm_100 (add/sub/mul/fma.f32x2:
-// one issue slot for two results, the same FP32 rate), a global access is 16 bytes instead of
-// 8, a shared-memory access 16 bytes for two pencils, and a twiddle is read once for both.  The
-// tile holds N rows of W / 2 pairs {re0, re1, im0, im1}; eight consecutive lanes read 128
-// contiguous bytes of one row, so no padding is needed.  Same factorisation and order of
-// operations as lpp_fft_dev.cuh.  Eight grids of 256^3 to k = 0.995 k_Ny, y pass 414 -> 383 us, z pass 368 -> 320 us;
-// with the stores of ColumnBound and tiles of 16 columns 320 us (1.9 GB, 6.0 TB/s: bound by DRAM) and 246
-// us (1.4 GB, 5.7 TB/s).  512^3 stays bound by the latency of its five steps per tile, 32 warps per SM.  Grids below 64^3 keep one
-// pencil per thread: their passes take a few microseconds and have too few pencils to pair.
+// flight, not by DRAM.  Here a thread owns two neighbouring pencils: every value is a pair (re0, re1)
+// or (im0, im1) in a 64-bit register, added and multiplied by the packed FP32 instructions of sm_100
+// (add/sub/mul/fma.f32x2: one issue slot for two results, the same FP32 rate), a global access is
+// 16 bytes instead of 8, a shared-memory access 16 bytes for two pencils, and a twiddle is read once
+// for both.  The tile holds N rows of W / 2 pairs {re0, re1, im0, im1}; eight consecutive lanes read
+// 128 contiguous bytes of one row, so no padding is needed.  Same factorisation and order of
+// operations as lpp_fft_dev.cuh.
+//
+// Eight grids of 256^3 to k = 0.995 k_Ny: y pass 414 -> 383 us, z pass 368 -> 320 us; with the bounds of
+// ColumnBound and tiles of 16 columns 320 us (1.9 GB, 6.0 TB/s: bound by DRAM) and 246 us (1.4 GB,
+// 5.7 TB/s).  512^3 stays bound by the latency of its five steps per tile, 32 warps per SM (y pass 454
+// us, z pass 446 us for eight grids of a survey).  Grids below 64^3 keep one pencil per thread: their
+// passes take a few microseconds and have too few pencils to pair.
 #pragma once
 
 #include "lpp_fft_dev.cuh"
