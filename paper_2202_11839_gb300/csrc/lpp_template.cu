@@ -415,37 +415,24 @@ k_template(const __grid_constant__ TemplateArgs a) {
         const int k_lo = seg * (kSlab / kSegs), k_hi = k_lo + kSlab / kSegs;
 #pragma unroll
         for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = 0.0;
-        if (!png) {
-            for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
-                const double2 av = *reinterpret_cast<const double2*>(arow + k0);
-                double2 bv[NT];
+        // the response enters the density rows not at all, the cross rows once and the plus and
+        // minus rows twice; a tile may straddle two families, so every row takes the product
+        // with its own family's spectrum of the three
+        for (int pw = 0; pw < 3; ++pw) {
 #pragma unroll
-                for (int j = 0; j < NT; ++j) bv[j] = op[brow[j] + k0 / 2];
-#pragma unroll
-                for (int j = 0; j < NT; ++j) mma_f64(acc[j], av.x, bv[j].x);
-#pragma unroll
-                for (int j = 0; j < NT; ++j) mma_f64(acc[j], av.y, bv[j].y);
-            }
-        } else {
-            // the response enters the density rows not at all, the cross rows once and the plus and
-            // minus rows twice; a tile may straddle two families, so every row takes the product
-            // with its own family's spectrum of the three
-            for (int pw = 0; pw < 3; ++pw) {
-#pragma unroll
-                for (int j = 0; j < NT; ++j) {
-                    const int r8 = 8 * (wt + lanes * j);
-                    if (r8 >= rows) break;
-                    const int r = min(r8 + rl, rows - 1);
-                    const int sl = a.slot[r / nbl];
-                    const int want = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
-                    if (!__any_sync(0xffffffffu, want == pw)) continue;   // warp-uniform
-                    const double on = want == pw ? 1.0 : 0.0;
-                    for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
-                        const double2 av = *reinterpret_cast<const double2*>(arow + pw * kSets * kSlabPad + k0);
-                        const double2 bv = op[brow[j] + k0 / 2];
-                        mma_f64(acc[j], av.x, on * bv.x);
-                        mma_f64(acc[j], av.y, on * bv.y);
-                    }
+            for (int j = 0; j < NT; ++j) {
+                const int r8 = 8 * (wt + lanes * j);
+                if (r8 >= rows) break;
+                const int r = min(r8 + rl, rows - 1);
+                const int sl = a.slot[r / nbl];
+                const int want = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
+                if (!__any_sync(0xffffffffu, want == pw)) continue;   // warp-uniform
+                const double on = want == pw ? 1.0 : 0.0;
+                for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
+                    const double2 av = *reinterpret_cast<const double2*>(arow + pw * kSets * kSlabPad + k0);
+                    const double2 bv = op[brow[j] + k0 / 2];
+                    mma_f64(acc[j], av.x, on * bv.x);
+                    mma_f64(acc[j], av.y, on * bv.y);
                 }
             }
         }
