@@ -316,7 +316,8 @@ lpp_status lpp_convolve_template_eb(lpp_template_t tmpl, const double* params, i
  * layer inputs, back-propagated gradients) and accumulates in FP32 on the tensor cores;
  * Adam (beta 0.9, 0.999, eps 1e-8, bias-corrected) updates FP32 master weights.
  * Parameters travel as one FP32 host array: for each layer W [out][in] then b [out]
- * (in/out = 6/256, 256/256, 256/256, 256/256, 256/320). */
+ * (in/out = 6/256, 256/256, 256/256, 256/256, 256/320).  Device arrays need the alignment of
+ * their elements only. */
 typedef struct lpp_surrogate_s* lpp_surrogate_t;
 
 /* batch: training minibatch and inference chunk (multiple of 32). */

@@ -50,6 +50,20 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+// Two neighbouring floats of a caller's array, which may start at any float (rows of 320 keep the
+// address's remainder: the branch goes one way for a whole call).
+__device__ __forceinline__ float2 load2(const float* p) {
+    return ((uintptr_t)p & 7) == 0 ? *reinterpret_cast<const float2*>(p) : make_float2(p[0], p[1]);
+}
+__device__ __forceinline__ void store2(float* p, float a, float b) {
+    if (((uintptr_t)p & 7) == 0) {
+        *reinterpret_cast<float2*>(p) = make_float2(a, b);
+    } else {
+        p[0] = a;
+        p[1] = b;
+    }
+}
+
 // ---- weight streaming
 // The passes of a row chain: the forward layers 0..4, then (training) the activation gradients
 // through layers 4..1.  Pass p multiplies by w[p] [rows][K], K contiguous, in chunks of 32 K
@@ -315,7 +329,7 @@ k_train_rows(const __grid_constant__ TrainRowArgs a) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int r = r0 + g + 8 * h;
-                const float2 yv = *reinterpret_cast<const float2*>(a.y + (size_t)a.idx[r] * kNout + co);
+                const float2 yv = load2(a.y + (size_t)a.idx[r] * kNout + co);
                 const float d0 = (acc[j][2 * h] + b.x) - yv.x, d1 = (acc[j][2 * h + 1] + b.y) - yv.y;
                 part += (double)d0 * d0 + (double)d1 * d1;
                 const float2 gv = make_float2(sc * d0, sc * d1);
@@ -827,7 +841,7 @@ __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, c
             u = pair_mul(u, pr(c.isig));
             res[q] = __fadd_rn(u.hi, u.lo);
         }
-        *reinterpret_cast<float2*>(out + (size_t)r * kNout + 8 * tile + 2 * t) = make_float2(res[0], res[1]);
+        store2(out + (size_t)r * kNout + 8 * tile + 2 * t, res[0], res[1]);
     }
 }
 
@@ -909,8 +923,8 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_predict(const __grid_constan
             } else {
                 const int r = mt * 16 + g;
                 float* o = a.out + (size_t)(r0 + r) * kNout + c;
-                if (r < rows) *reinterpret_cast<float2*>(o) = make_float2(v.x, v.y);
-                if (r + 8 < rows) *reinterpret_cast<float2*>(o + 8 * kNout) = make_float2(v.z, v.w);
+                if (r < rows) store2(o, v.x, v.y);
+                if (r + 8 < rows) store2(o + 8 * kNout, v.z, v.w);
             }
         }
     }
@@ -981,8 +995,8 @@ k_predict_few(const __grid_constant__ PredictArgs a) {
             decode_tile<R>(a.map, wd, rc, cols - o0, 0, tile, rows, v, a.out + (size_t)r0 * kNout);
         } else {
             float* o = a.out + (size_t)(r0 + g) * kNout + co;
-            if (g < rows) *reinterpret_cast<float2*>(o) = make_float2(v[0], v[1]);
-            if (g + 8 < rows) *reinterpret_cast<float2*>(o + 8 * kNout) = make_float2(v[2], v[3]);
+            if (g < rows) store2(o, v[0], v[1]);
+            if (g + 8 < rows) store2(o + 8 * kNout, v[2], v[3]);
         }
     }
 }
