@@ -1111,6 +1111,7 @@ extern "C" lpp_status lpp_surrogate_set_workspace(lpp_surrogate_t s, void* dev, 
     if (bytes < s->need) return LPP_ERR_WORKSPACE;
     s->ws = (char*)dev;
     s->step = 0;
+    s->base_split = false;   // the digits of the map's base went with the old contents
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(s->ws, 0, s->need, st) != cudaSuccess) return LPP_ERR_CUDA;
     std::vector<float> wpad;
