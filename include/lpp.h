@@ -317,7 +317,8 @@ lpp_status lpp_convolve_template_eb(lpp_template_t tmpl, const double* params, i
  * Adam (beta 0.9, 0.999, eps 1e-8, bias-corrected) updates FP32 master weights.
  * Parameters travel as one FP32 host array: for each layer W [out][in] then b [out]
  * (in/out = 6/256, 256/256, 256/256, 256/256, 256/320).  Device arrays need the alignment of
- * their elements only. */
+ * their elements only.  The calls on one surrogate share its workspace: on more than one stream
+ * they have to be ordered by the caller. */
 typedef struct lpp_surrogate_s* lpp_surrogate_t;
 
 /* batch: training minibatch and inference chunk (multiple of 32). */

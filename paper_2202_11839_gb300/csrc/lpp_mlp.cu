@@ -1357,7 +1357,11 @@ extern "C" lpp_status lpp_surrogate_predict(lpp_surrogate_t s, const double* the
             k_base_digits<<<kNout / 8, 256, 0, st>>>(s->map.base, s->map.nodes * s->map.nodes,
                                                      (uint4*)(s->ws + s->digits), (int*)(s->ws + s->exponent));
             if (cudaGetLastError() != cudaSuccess) return LPP_ERR_CUDA;
-            s->base_split = true;
+            // a captured launch has not run yet: the graph forms the digits each time, and so does the
+            // next call outside of it
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return LPP_ERR_CUDA;
+            s->base_split = cap == cudaStreamCaptureStatusNone;
         }
     }
     PredictArgs a;

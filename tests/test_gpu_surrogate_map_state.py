@@ -40,3 +40,27 @@ def test_predict_after_a_new_workspace():
             C.c_void_p(net.stream.cuda_stream)) == L.LPP_OK
         assert np.array_equal(net.predict(theta).cpu().numpy(), want)
     net.close()
+
+
+def test_predict_after_a_capture():
+    """A first predict that is only captured forms nothing: the next one outside of the graph, before the graph
+    has run, and the graph itself give the same curves."""
+    import torch
+    _, ref, _, theta = _net()
+    want = ref.predict(theta).cpu().numpy()
+    ref.close()
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        _, net, _, theta = _net(stream=st)
+        out = torch.zeros((40, 320), dtype=torch.float32, device="cuda")
+        st.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            net.predict(theta, out=out)
+        eager = net.predict(theta)
+        st.synchronize()
+        assert np.array_equal(eager.cpu().numpy(), want)
+        graph.replay()
+        st.synchronize()
+        assert np.array_equal(out.cpu().numpy(), want)
+    net.close()
