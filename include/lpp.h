@@ -367,9 +367,11 @@ lpp_status lpp_surrogate_infer(lpp_surrogate_t net, const float* x, int n, float
  * device FP64 [320] or NULL (0, 1) standardise the prediction as (t - ref) / sigma, as
  * lpp_convolve_template_eb does.  The pointers are borrowed and must outlive the surrogate's
  * use of them; the first lpp_surrogate_predict after lpp_surrogate_set_map writes base into
- * the surrogate's workspace as 48-bit fixed-point digits for the decoding, which sums the
- * baseline by exact products of digits (the FP64 sum to about 2^-38 of its largest term), so a changed
- * base needs lpp_surrogate_set_map again.  nodes in 2..8. */
+ * the surrogate's workspace as 48-bit fixed-point digits for the decoding, so a changed
+ * base needs lpp_surrogate_set_map again.  The decoding sums the baseline by products of digits and
+ * the rest in pairs of floats where that gives the FP64 result to a quarter of its last FP32 place,
+ * and in FP64 elsewhere: a prediction is the FP64 value of the map to 3/4 of an FP32 place.  nodes in
+ * 2..8. */
 typedef struct {
     double lo[6], hi[6];
     int feed[6];

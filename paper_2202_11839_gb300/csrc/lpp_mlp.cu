@@ -565,16 +565,21 @@ __device__ __forceinline__ void lobatto_basis_fast(double x, const MapArgs& a, d
 
 // ---- exact products of the baseline on the tensor cores
 // The baseline sum_q w_q base_qj cancels: it needs more than the FP32 digits of its terms, and
-// GB300 runs FP64 at 1/64 of the FP32 rate.  Both factors are therefore written as kDigits signed
-// base-256 digits of a 48-bit fixed-point number (weights relative to the row's largest, base
-// values to the column's largest).  A digit is an integer of at most 128, exact in BF16; a sum of
-// 64 products of digits is an integer below 2^20, and one of up to six such sums below 2^23,
-// exact in the FP32 accumulators.  Products of digits i and j have weight 2^(-8 (i + j)): the sums
-// of equal i + j <= 6 share an accumulator (26 of the 36 products; the rest are below 2^-48 of
-// the largest term), and the seven accumulators are added in float pairs.
-constexpr int kDigits = 6, kOrders = 7;
+// GB300 runs FP64 at 1/64 of the FP32 rate.  Both factors are therefore written as signed base-256
+// digits of fixed-point numbers: base values with kDigits (48 bits) relative to the column's largest,
+// below 2^ec, weights with kWDigits (56 bits) relative to the row's largest, below 2^er.  A digit is
+// an integer of at most 128, exact in BF16; a sum of 64 products of digits is an integer below 2^20,
+// and one of up to six such sums below 2^23, exact in the FP32 accumulators.  Products of digits i
+// and j have weight 2^(-8 (i + j)): the sums of equal i + j <= 6 share an accumulator (27 of the 42
+// products), and the seven accumulators are added in float pairs.
+// The error is that of the base digits, 2^(ec - 48) sum |w_q|, and at most 2^(er + ec - 45) (64 times the
+// weight digits' 2^(er + ec - 56) and the dropped products' 5 x 2^(er + ec - 56), the last orders
+// added in one float 2^(er + ec - 46), the pairs).  It is small against the largest terms, not against every
+// sum: decode_tile decides output by output whether it is small enough.
+constexpr int kDigits = 6, kWDigits = 7, kOrders = 7;
 constexpr int kBaseKsteps = kMaxNodes * kMaxNodes / 16;            // 16 baseline terms per mma
 constexpr int kDigitWords = kDigits * (kNout / 8) * (kBaseKsteps / 2) * 32;   // uint4 of digit fragments
+constexpr int kZeroExponent = -(1 << 20);   // a column of zeros
 
 // v with |v| <= 2^e -> the kDigits digits d_i of v = 2^e sum_i d_i 2^(-8 i - 7) to 2^(e - 48).  One
 // FP64 multiply-add: v 2^(47 - e) + 1.5 2^52 holds the rounded integer in its low bits.
@@ -588,16 +593,28 @@ __device__ __forceinline__ void fixed_digits(double v, int e, int* d) {
     }
     d[0] = (int)q;
 }
+// v with |v| < 2^e -> kWDigits digits of v to 2^(e - 56).
+__device__ __forceinline__ void weight_digits(double v, int e, int* d) {
+    const double scale = __hiloint2double((55 - e + 1023) << 20, 0);
+    long long q = __double2ll_rn(v * scale);
+#pragma unroll
+    for (int i = kWDigits - 1; i > 0; --i) {
+        d[i] = (int)((q + 128) & 255) - 128;
+        q = (q - d[i]) >> 8;
+    }
+    d[0] = (int)q;
+}
 // The exponent e of the largest of the warp's values (two per lane): |v| < 2^e; kBadExponent for
-// an infinity, a NaN or values beyond 2^900; the smallest usable exponent for zeros.  Integer
-// instructions on the high words.
+// an infinity, a NaN or values beyond 2^900; kZeroExponent for zeros (and denormals below 2^-1042); the
+// smallest usable exponent for others below it.  Integer instructions on the high words.
 __device__ __forceinline__ int warp_exponent(double v0, double v1) {
     int h = max(__double2hiint(v0) & 0x7fffffff, __double2hiint(v1) & 0x7fffffff);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
     const int e = (h >> 20) - 1022;
-    return e > 900 ? kBadExponent : max(e, -900);
+    return h == 0 ? kZeroExponent : (e > 900 ? kBadExponent : max(e, -900));
 }
+__device__ __forceinline__ bool usable(int e) { return e >= -900 && e <= 900; }
 
 // base -> digits in the order in which a lane reads its operand fragments: word
 // ((digit 40 + column tile) 2 + k half) 32 + lane holds terms q = 32 half + {2t, 2t+1, 2t+8, 2t+9} + {0, 16}
@@ -615,7 +632,7 @@ __global__ void k_base_digits(const double* __restrict__ base, int nn, uint4* __
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         int d[kDigits];
-        fixed_digits(e == kBadExponent ? 0.0 : v[h], e == kBadExponent ? 0 : e, d);
+        fixed_digits(usable(e) ? v[h] : 0.0, usable(e) ? e : 0, d);
         // term q = 32 h + lane: k step of 16, position in it -> fragment register and half
         const int s16 = lane >> 4, p = lane & 15, t = (p & 7) >> 1;
         const int word = 2 * s16 + (p >> 3);   // of the uint4: {b0, b1} of two k steps
@@ -674,9 +691,7 @@ __device__ __forceinline__ float exp2i(int e) {   // 2^e for -126 <= e <= 127
     return __int_as_float((e + 127) << 23);
 }
 
-__device__ __forceinline__ float scale2(float v, int e) {   // v 2^e
-    return e > -100 && e < 100 ? v * exp2i(e) : ldexpf(v, e);
-}
+constexpr float kTiny = 7.174648137343064e-43f;   // 2^-140: low words may lose up to 2^-149 by underflow
 
 struct PredictArgs {
     Passes ps;
@@ -693,6 +708,7 @@ struct PredictArgs {
 // the map's arrays as they are at this call.
 struct ColumnConst {
     float2 mu, sd, shot, ref, isig;
+    float tiny;   // kTiny, 0 when shot and ref are zero
     int e;
 };
 __device__ __forceinline__ ColumnConst column_const(const MapArgs& m, int j) {
@@ -703,6 +719,7 @@ __device__ __forceinline__ ColumnConst column_const(const MapArgs& m, int j) {
     c.shot = as2(pair_of(m.shot[j]));
     c.ref = as2(pair_of(m.ref ? m.ref[j] : 0.0));
     c.isig = as2(pair_of(m.sigma ? 1.0 / m.sigma[j] : 1.0));
+    c.tiny = m.shot[j] != 0.0 || (m.ref && m.ref[j] != 0.0) ? kTiny : 0.f;
     c.e = m.base ? m.exponent[j] : 0;
     return c;
 }
@@ -715,12 +732,14 @@ __global__ void k_columns(MapArgs m, ColumnConst* __restrict__ out) {
 template <int R>
 struct RowConst {
     float2 amp[2][R], t5[R];   // A b sigma_8^2 (gE), A^2 sigma_8^2 (EE, BB); shot-noise scale
-    int e[R];
+    float tiny[2][R];          // kTiny, 0 when the amplitude is zero
+    int e[R];                  // exponent of the weights' digits
+    float wsum[R];             // sum of |w_q|
     double la[R][kMaxNodes], lb[R][kMaxNodes];
 };
 
 // The constants of R parameter rows and their Lagrange weights as digit fragments
-// wd[kDigits][R / 16][kBaseKsteps][32]; ends with a barrier.
+// wd[kWDigits][R / 16][kBaseKsteps][32]; ends with a barrier.
 template <int R>
 __device__ __forceinline__ void decode_rows(const MapArgs& m, const double* theta, int r0, int rows, RowConst<R>& rc,
                                             uint4* wd) {
@@ -733,8 +752,12 @@ __device__ __forceinline__ void decode_rows(const MapArgs& m, const double* thet
         const double* th = theta + (size_t)(r0 + r) * kNin;
         if (k == 0) {
             const double s2 = th[2] * th[2];
-            rc.amp[0][r] = as2(pair_of(s2 * (th[0] * th[1])));
-            rc.amp[1][r] = as2(pair_of(s2 * (th[0] * th[0])));
+            const double amp[2] = {s2 * (th[0] * th[1]), s2 * (th[0] * th[0])};
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                rc.amp[c][r] = as2(pair_of(amp[c]));
+                rc.tiny[c][r] = amp[c] != 0.0 ? kTiny : 0.f;
+            }
             rc.t5[r] = as2(pair_of(th[5]));
         } else if (m.base) {
             const int c = m.base_in[k - 1];
@@ -753,17 +776,23 @@ __device__ __forceinline__ void decode_rows(const MapArgs& m, const double* thet
             v[h] = (r < rows && q < nn) ? rc.la[r][q / m.nodes] * rc.lb[r][q % m.nodes] : 0.0;
         }
         const int e = warp_exponent(v[0], v[1]);
-        if (lane == 0) rc.e[r] = e;
+        float sum = (float)(fabs(v[0]) + fabs(v[1]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) {
+            rc.e[r] = e;
+            rc.wsum[r] = sum;
+        }
         const int mt = r >> 4, rr = r & 15;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            int d[kDigits];
-            fixed_digits(e == kBadExponent ? 0.0 : v[h], e == kBadExponent ? 0 : e, d);
+            int d[kWDigits];
+            weight_digits(usable(e) ? v[h] : 0.0, usable(e) ? e : 0, d);
             // term q = 32 h + lane = 16 ks + p: register (rr >> 3) + 2 (p >> 3) of lane 4 (rr & 7) + (p & 7) / 2
             const int ks = 2 * h + (lane >> 4), p = lane & 15;
             const int reg = (rr >> 3) + 2 * (p >> 3), ln = 4 * (rr & 7) + ((p & 7) >> 1);
 #pragma unroll
-            for (int i = 0; i < kDigits; ++i)
+            for (int i = 0; i < kWDigits; ++i)
                 wo[((((i * MT + mt) * kBaseKsteps + ks) * 32 + ln) * 4 + reg) * 2 + (p & 1)] =
                     __float2bfloat16_rn((float)d[i]);
         }
@@ -771,14 +800,39 @@ __device__ __forceinline__ void decode_rows(const MapArgs& m, const double* thet
     __syncthreads();
 }
 
+// One output of a parameter row th in FP64, by a whole warp: y the network's output j, la and lb the
+// row's Lagrange weights.
+__device__ __noinline__ float decode_exact(const MapArgs& m, const double* la, const double* lb, const double* th, int j,
+                                           float y) {
+    double b = 0.0;
+    if (m.base) {
+        for (int q = threadIdx.x & 31; q < m.nodes * m.nodes; q += 32)
+            b = fma(la[q / m.nodes] * lb[q % m.nodes], m.base[(size_t)q * kNout + j], b);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    const double amp = th[2] * th[2] * (j < 2 * (kNout / 8) ? th[0] * th[1] : th[0] * th[0]);
+    double v = amp * (m.mu[j] + b + m.sd[j] * (double)y) + th[5] * m.shot[j];
+    if (m.ref) v -= m.ref[j];
+    if (m.sigma) v /= m.sigma[j];
+    return (float)v;
+}
+
 // The decoding of one tile: rows 16 mt + {g, g + 8}, columns 8 tile + {2 t, 2 t + 1}, from the
-// network outputs y[4] on the mma accumulator's positions.
+// network outputs y[4] on the mma accumulator's positions; theta: the first row's parameters.
+//
+// The digit products and the float pairs bound their error (the terms' magnitudes times 2^-43, the
+// digits' bound above, and 2^-140 where a low word may underflow).  An output for which that is more than
+// a quarter of its last FP32 place, which is no number or whose exponents leave FP32's range is done
+// again in FP64 (decode_exact): the stored value is the FP64 one to 3/4 of a place, whatever the
+// map holds.  Curves of some hundred error bars around the reference repeat a fraction of a per cent.
 template <int R>
 __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, const RowConst<R>& rc,
                                             const ColumnConst* cc, int mt, int tile, int rows, const float y[4],
-                                            float* out) {
+                                            const double* theta, float* out) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     constexpr int MT = R / 16;
+    constexpr unsigned full = 0xffffffffu;
     auto pr = [](float2 v) { return fpair{v.x, v.y}; };
     float acc[kOrders][4];
 #pragma unroll
@@ -794,7 +848,7 @@ __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, c
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
-                for (int i = 0; i < kDigits; ++i) {
+                for (int i = 0; i < kWDigits; ++i) {
                     const uint4 av = wd[((i * MT + mt) * kBaseKsteps + 2 * h + k) * 32 + lane];
                     const uint32_t af[4] = {av.x, av.y, av.z, av.w};
 #pragma unroll
@@ -809,39 +863,58 @@ __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, c
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
         const int r = mt * 16 + g + 8 * hh;
-        if (r >= rows) continue;
         float res[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int v = 2 * hh + q;
             const ColumnConst& c = cq[q];
-            fpair u = pr(c.mu);
-            if (m.base) {
-                // sum_o acc_o 2^(-8 o): the first three orders exactly, the rest (below 2^-22 of the
-                // largest possible sum) in one float
-                const float low = fmaf(acc[6][v], exp2i(-48), fmaf(acc[5][v], exp2i(-40),
-                                       fmaf(acc[4][v], exp2i(-32), __fmul_rn(acc[3][v], exp2i(-24)))));
-                const fpair s1 = two_sum(acc[0][v], __fmul_rn(acc[1][v], exp2i(-8)));
-                const fpair s2 = two_sum(s1.hi, __fmul_rn(acc[2][v], exp2i(-16)));
-                fpair b = fast_two_sum(s2.hi, __fadd_rn(s2.lo, __fadd_rn(s1.lo, low)));
-                const int er = rc.e[r];
-                if (er == kBadExponent || c.e == kBadExponent) {
-                    b.hi = b.lo = NAN;
-                } else {
-                    const int e = er + c.e - 14;   // the digits' unit: 2^(e_r + e_c) 2^-14
-                    b.hi = scale2(b.hi, e);
-                    b.lo = scale2(b.lo, e);
+            bool done = r >= rows;
+            if (!done) {
+                fpair u = pr(c.mu);
+                float mag = fabsf(c.mu.x), eb = 0.f;   // the terms' magnitudes, the digits' error
+                bool range = true;
+                if (m.base && c.e != kZeroExponent) {
+                    // sum_o acc_o 2^(-8 o): the first four orders exactly, the rest in one float
+                    const float low = fmaf(acc[6][v], exp2i(-48), fmaf(acc[5][v], exp2i(-40), __fmul_rn(acc[4][v], exp2i(-32))));
+                    const fpair s1 = two_sum(acc[0][v], __fmul_rn(acc[1][v], exp2i(-8)));
+                    const fpair s2 = two_sum(s1.hi, __fmul_rn(acc[2][v], exp2i(-16)));
+                    const fpair s3 = two_sum(s2.hi, __fmul_rn(acc[3][v], exp2i(-24)));
+                    fpair b = fast_two_sum(s3.hi, __fadd_rn(s3.lo, __fadd_rn(s2.lo, __fadd_rn(s1.lo, low))));
+                    const int er = rc.e[r], ec = c.e;
+                    range = er > -50 && er < 50 && ec > -50 && ec < 50;
+                    const int e = range ? er + ec : 0;
+                    b.hi *= exp2i(e - 14);   // the digits' unit: 2^(e_r + e_c) 2^-14
+                    b.lo *= exp2i(e - 14);
+                    u = pair_add(u, b);
+                    mag += fabsf(b.hi);
+                    eb = fmaf(rc.wsum[r] * exp2i(-48), range ? exp2i(ec) : 0.f, exp2i(e - 14) * exp2i(-31));
                 }
-                u = pair_add(u, b);
+                const int ci = tile < 2 * (kNout / 8) / 8 ? 0 : 1;
+                const fpair amp = pr(rc.amp[ci][r]);
+                const float tiny = rc.tiny[ci][r];
+                const fpair net = pair_mul(pr(c.sd), y[v]), shot = pair_mul(pr(rc.t5[r]), pr(c.shot));
+                u = pair_add(u, net);
+                mag += fabsf(net.hi);
+                u = pair_mul(u, amp);
+                u = pair_add(u, shot);
+                u = pair_add(u, fpair{-c.ref.x, -c.ref.y});
+                const float all = fmaf(fabsf(amp.hi), mag, fabsf(shot.hi) + fabsf(c.ref.x));
+                u = pair_mul(u, pr(c.isig));
+                res[q] = __fadd_rn(u.hi, u.lo);
+                const float err = fmaf(fabsf(amp.hi), eb + tiny, fmaf(all, exp2i(-43), fmaf(mag, tiny, fmaxf(tiny, c.tiny))));
+                const float bound = fmaf(fabsf(c.isig.x), err, all * kTiny);
+                done = range && bound <= fabsf(res[q]) * exp2i(-26) && fabsf(res[q]) < INFINITY;
             }
-            u = pair_add(u, pair_mul(pr(c.sd), y[v]));
-            u = pair_mul(u, pr(rc.amp[tile < 2 * (kNout / 8) / 8 ? 0 : 1][r]));
-            u = pair_add(u, pair_mul(pr(rc.t5[r]), pr(c.shot)));
-            u = pair_add(u, fpair{-c.ref.x, -c.ref.y});
-            u = pair_mul(u, pr(c.isig));
-            res[q] = __fadd_rn(u.hi, u.lo);
+            unsigned again = __ballot_sync(full, !done);
+            while (again) {   // warp-uniform
+                const int src = __ffs(again) - 1, rs = mt * 16 + (src >> 2) + 8 * hh;
+                again &= again - 1;
+                const float x = decode_exact(m, rc.la[rs], rc.lb[rs], theta + (size_t)rs * kNin, 8 * tile + 2 * (src & 3) + q,
+                                             __shfl_sync(full, y[v], src));
+                if (lane == src) res[q] = x;
+            }
         }
-        store2(out + (size_t)r * kNout + 8 * tile + 2 * t, res[0], res[1]);
+        if (r < rows) store2(out + (size_t)r * kNout + 8 * tile + 2 * t, res[0], res[1]);
     }
 }
 
@@ -862,10 +935,13 @@ __device__ __forceinline__ void input_rows(const PredictArgs& a, int r0, int row
 // Forward pass of 32 rows per CTA and, with MAP, the whole prediction: the parameters' encoding
 // before it and the decoding after it
 //   (pre_c (mu + sum_q w_q base_q + sd y) + theta_5 shot - ref) / sigma,
-// the baseline by exact digit products (above), the rest in float pairs.
+// the baseline by exact digit products (above), the rest in float pairs, FP64 where those do not decide
+// the FP32 result.
 //
 // What bounds it: the GELUs' instructions and the mma issue.  8192 rows: 287 us as eight launches
-// with the decoding's last operations in FP64 -> 90 us.
+// with the decoding's last operations in FP64 -> 96 us (90 us without decode_tile's error bound and the
+// seventh weight digit; 104 us near a reference curve, where a per cent of the outputs are done
+// again).
 template <bool MAP>
 __global__ void __launch_bounds__(kRowThreads, 2) k_predict(const __grid_constant__ PredictArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -906,10 +982,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_predict(const __grid_constan
     __syncthreads();   // the ring and the activations are free
     // network outputs in shared memory on their accumulator positions [tile][mt][lane]: the decoding
     // loops over the tiles without unrolling (an unrolled one stalls on instruction fetches)
-    uint4* wd = reinterpret_cast<uint4*>(smem_raw);                     // [kDigits][MT][kBaseKsteps][32]
-    float4* ys = reinterpret_cast<float4*>(wd + kDigits * MT * kBaseKsteps * 32);   // [kNout / 8][MT][32]
+    uint4* wd = reinterpret_cast<uint4*>(smem_raw);                     // [kWDigits][MT][kBaseKsteps][32]
+    float4* ys = reinterpret_cast<float4*>(wd + kWDigits * MT * kBaseKsteps * 32);   // [kNout / 8][MT][32]
     RowConst<R>& rc = *reinterpret_cast<RowConst<R>*>(ys + (kNout / 8) * MT * 32);
-    static_assert(sizeof(uint4) * kDigits * MT * kBaseKsteps * 32 + sizeof(float4) * (kNout / 8) * MT * 32 +
+    static_assert(sizeof(uint4) * kWDigits * MT * kBaseKsteps * 32 + sizeof(float4) * (kNout / 8) * MT * 32 +
                       sizeof(RowConst<R>) <= kPredSmem, "the decoding fits in the forward pass's shared memory");
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
@@ -934,14 +1010,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_predict(const __grid_constan
         for (int i = warp * 5 * MT; i < (warp + 1) * 5 * MT; ++i) {
             const float4 v = ys[i * 32 + lane];
             const float yv[4] = {v.x, v.y, v.z, v.w};
-            decode_tile<R>(a.map, wd, rc, a.cols, i % MT, i / MT, rows, yv, a.out + (size_t)r0 * kNout);
+            decode_tile<R>(a.map, wd, rc, a.cols, i % MT, i / MT, rows, yv, a.theta + (size_t)r0 * kNin,
+                           a.out + (size_t)r0 * kNout);
         }
     }
 }
 
 // The same for few rows: 16 rows on a cluster of kSplit CTAs, each a quarter of every layer's columns
 // and of the outputs.  What bounds it: the latency of the dependent layers.  50 rows: 85 us as eight
-// launches, 49 us with one CTA per 16 rows -> 25 us.
+// launches, 49 us with one CTA per 16 rows -> 27 us.
 template <bool MAP>
 __global__ void __cluster_dims__(kSplit, 1, 1) __launch_bounds__(kRowThreads, 1)
 k_predict_few(const __grid_constant__ PredictArgs a) {
@@ -957,8 +1034,8 @@ k_predict_few(const __grid_constant__ PredictArgs a) {
     buf[1] = buf[0] + 16 * kActLd;
     // the decoding's rows and columns are prepared while the first weights arrive
     constexpr int R = 16;
-    uint4* wd = reinterpret_cast<uint4*>(smem_raw + kSliceSmem);                     // [kDigits][1][kBaseKsteps][32]
-    RowConst<R>& rc = *reinterpret_cast<RowConst<R>*>(wd + kDigits * kBaseKsteps * 32);
+    uint4* wd = reinterpret_cast<uint4*>(smem_raw + kSliceSmem);                     // [kWDigits][1][kBaseKsteps][32]
+    RowConst<R>& rc = *reinterpret_cast<RowConst<R>*>(wd + kWDigits * kBaseKsteps * 32);
     ColumnConst* cols = reinterpret_cast<ColumnConst*>(&rc + 1);                     // [kNout / kSplit]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const int r0 = (int)(blockIdx.x / kSplit) * R, rows = min(R, a.n - r0);
@@ -992,7 +1069,8 @@ k_predict_few(const __grid_constant__ PredictArgs a) {
         const float2 b = *reinterpret_cast<const float2*>(a.bias[kLayers - 1] + co);
         const float v[4] = {y[j][0] + b.x, y[j][1] + b.y, y[j][2] + b.x, y[j][3] + b.y};
         if constexpr (MAP) {
-            decode_tile<R>(a.map, wd, rc, cols - o0, 0, tile, rows, v, a.out + (size_t)r0 * kNout);
+            decode_tile<R>(a.map, wd, rc, cols - o0, 0, tile, rows, v, a.theta + (size_t)r0 * kNin,
+                           a.out + (size_t)r0 * kNout);
         } else {
             float* o = a.out + (size_t)(r0 + g) * kNout + co;
             if (g < rows) store2(o, v[0], v[1]);
@@ -1000,7 +1078,7 @@ k_predict_few(const __grid_constant__ PredictArgs a) {
         }
     }
 }
-constexpr size_t kFewSmem = kSliceSmem + sizeof(uint4) * kDigits * kBaseKsteps * 32 + sizeof(RowConst<16>) +
+constexpr size_t kFewSmem = kSliceSmem + sizeof(uint4) * kWDigits * kBaseKsteps * 32 + sizeof(RowConst<16>) +
                             sizeof(ColumnConst) * (kNout / kSplit);
 
 // training targets: derived curves u of native template slots [n][LPP_N_MOMENTS][40] (FP64, unit
