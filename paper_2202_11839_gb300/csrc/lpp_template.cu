@@ -463,10 +463,15 @@ k_template(const __grid_constant__ TemplateArgs a) {
 // 2^(-8 (i + j)): those of equal i + j <= 6 share an accumulator (28 mma instead of one FP64 product;
 // the dropped ones are below 2^-54 of the slab's largest product), and every 128 columns the
 // seven accumulators are added to two 64-bit integers.  The slabs are added in FP64.
+// A spectrum that varies by less than 2^kSpread against the reference within its slabs is so held to
+// 2^-53 of each of its values, as FP64 holds it; a set that varies more, in any slab, takes FP64
+// products there (tilts within 0.2 and Gamma within 0.1 to 0.3 vary by 2^1.5 at most; against the
+// magnitudes of the terms the digits of a tilt of 2 lost a factor 10, of 8 a factor 90).
 constexpr int kDigits = 7;
 constexpr int kManySets = 16;                 // sets per cluster: two column tiles of the mma
 constexpr int kManyTiles = 5;                 // row tiles of 16 per warp
 constexpr int kManyRows = 8 * 16 * kManyTiles;
+constexpr int kSpread = 3;
 // groups of sets from which a cluster is four CTAs of two slabs each: clusters of eight leave 40 of the 152
 // SMs idle (40 shells, nine slots, eight -> four CTAs: 16 sets 81 -> 153 us, 64 sets 165 -> 161, 256 sets
 // 306 -> 197, 8192 sets 4421 -> 3654)
@@ -547,7 +552,9 @@ k_template_many(const __grid_constant__ TemplateArgs a) {
     uint2* frag = reinterpret_cast<uint2*>(smem_raw);
     double* part = reinterpret_cast<double*>(frag + kDigits * 16 * 2 * 32);
     __shared__ double s8part[kManySets];
-    __shared__ int hmax[kManySets];
+    __shared__ int hmax[kManySets], hmin[kManySets];
+    __shared__ unsigned exact_sets;        // the sets of this slab that take FP64 products
+    __shared__ double exact_spec[kSlab];   // and the spectrum of one of them
     __shared__ double pw_hi[kManySets][16], pw_lo[kManySets][16], igam[kManySets];
     __shared__ double2 logtab[128];
     __shared__ double s8w[8][kManySets];
@@ -570,7 +577,10 @@ k_template_many(const __grid_constant__ TemplateArgs a) {
             }
         }
         if (tid < 128) logtab[tid] = a.logtab[tid];
-        if (tid < kManySets) hmax[tid] = 0;
+        if (tid < kManySets) {
+            hmax[tid] = 0;
+            hmin[tid] = 0x7fffffff;
+        }
         __syncthreads();
         // spectra of the sixteen sets at this thread's grid k, relative to the reference
         const int n = slab * kSlab + tid;
@@ -586,16 +596,28 @@ k_template_many(const __grid_constant__ TemplateArgs a) {
             const double s = warp_sum(sw * p[t]);
             if (lane == 0) s8w[warp][t] = s;
             p[t] *= ir;
-            int h = __double2hiint(p[t]) & 0x7fffffff;
+            int h = __double2hiint(p[t]) & 0x7fffffff, l = h;
     #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
-            if (lane == 0) atomicMax(&hmax[t], h);
+            for (int o = 16; o > 0; o >>= 1) {
+                h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
+                l = min(l, __shfl_xor_sync(0xffffffffu, l, o));
+            }
+            if (lane == 0) {
+                atomicMax(&hmax[t], h);
+                atomicMin(&hmin[t], l);
+            }
         }
         __syncthreads();
         if (tid < kManySets) {
             double s = 0.0;
             for (int w = 0; w < 8; ++w) s += s8w[w][tid];
             s8part[tid] = slab == rank * (8 / CL) ? s : s8part[tid] + s;
+        }
+        if (warp == 0) {
+            const int t = lane % kManySets, e = high_exponent(hmax[t]);
+            const unsigned b = __ballot_sync(0xffffffffu, lane < sets && (hmax[t] - hmin[t] >= kSpread << 20 || e == kBadExp ||
+                                                                          e <= -900));
+            if (lane == 0) exact_sets = b;
         }
         {   // column tid = 16 ks + 4 tt + 2 r + lo: register r, half lo of the lanes 4 g + tt
             const int ks = tid >> 4, tt = (tid & 15) >> 2, r = (tid >> 1) & 1, lo = tid & 1;
@@ -614,6 +636,7 @@ k_template_many(const __grid_constant__ TemplateArgs a) {
         __syncthreads();
         const int g = lane >> 2, tt = lane & 3;
         const int all_rows = kSlots * a.nb;
+        const unsigned exact = exact_sets;
         for (int tile = warp; tile * 16 < rows; tile += 8) {
             // the operator rows g and g + 8 of the tile (rows beyond the last repeat it and are not read back)
             int orow[2];
@@ -680,12 +703,32 @@ k_template_many(const __grid_constant__ TemplateArgs a) {
     #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const int t = 8 * c + 2 * tt + q, es = high_exponent(hmax[t]);
+                        if ((exact >> t) & 1u) continue;
                         double v = fma((double)vh[c][2 * h + q], 4294967296.0, (double)vl[c][2 * h + q]) * pow2(-62);
                         v = er == kBadExp || es == kBadExp ? NAN : v * pow2(er) * pow2(es);
                         double* d = part + r * kManySets + t;
                         *d = slab == rank * (8 / CL) ? v : *d + v;
                     }
             }
+        }
+        for (unsigned rest = exact; rest; rest &= rest - 1) {   // CTA-uniform
+            const int t = __ffs(rest) - 1;
+            exact_spec[tid] = bbks_value(k, ik, a.params[6 * (size_t)(t0 + t) + 4], igam[t],
+                                         pw_hi[t][tid >> 4] * pw_lo[t][tid & 15], logtab, nullptr);
+            __syncthreads();
+            for (int r = warp; r < rows; r += 8) {   // a warp per row: 8 columns per lane, then the lanes' sums
+                const int si = r / nbl;
+                const double* op = a.op + (size_t)(a.slot[si] * a.nb + b0 + (r - si * nbl)) * kNin + slab * kSlab;
+                double v = 0.0;
+    #pragma unroll
+                for (int i = 0; i < kSlab / 32; ++i) v = fma(op[lane + 32 * i], exact_spec[lane + 32 * i], v);
+                v = warp_sum(v);
+                if (lane == 0) {
+                    double* d = part + r * kManySets + t;
+                    *d = slab == rank * (8 / CL) ? v : *d + v;
+                }
+            }
+            __syncthreads();   // the next set rewrites the spectrum
         }
         __syncthreads();   // the next slab rewrites the tables and digits
     }
