@@ -416,24 +416,29 @@ k_template(const __grid_constant__ TemplateArgs a) {
 #pragma unroll
         for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = 0.0;
         // the response enters the density rows not at all, the cross rows once and the plus and
-        // minus rows twice; a tile may straddle two families, so every row takes the product
-        // with its own family's spectrum of the three
+        // minus rows twice; a tile may straddle two families: it is multiplied with the spectrum of
+        // each, and every row keeps the product with its own (not a sum with the others times
+        // zero, which an infinite spectrum would spoil)
+        auto power = [&](int r) {   // of row r's family
+            const int sl = a.slot[min(r, rows - 1) / nbl];
+            return sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
+        };
         for (int pw = 0; pw < 3; ++pw) {
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 const int r8 = 8 * (wt + lanes * j);
                 if (r8 >= rows) break;
-                const int r = min(r8 + rl, rows - 1);
-                const int sl = a.slot[r / nbl];
-                const int want = sl == 0 || sl == 10 || sl == 11 ? 0 : (sl <= 3 ? 1 : 2);
-                if (!__any_sync(0xffffffffu, want == pw)) continue;   // warp-uniform
-                const double on = want == pw ? 1.0 : 0.0;
+                if (!__any_sync(0xffffffffu, power(r8 + rl) == pw)) continue;   // warp-uniform
+                double v[2] = {0.0, 0.0};
                 for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
                     const double2 av = *reinterpret_cast<const double2*>(arow + pw * kSets * kSlabPad + k0);
                     const double2 bv = op[brow[j] + k0 / 2];
-                    mma_f64(acc[j], av.x, on * bv.x);
-                    mma_f64(acc[j], av.y, on * bv.y);
+                    mma_f64(v, av.x, bv.x);
+                    mma_f64(v, av.y, bv.y);
                 }
+#pragma unroll
+                for (int q = 0; q < 2; ++q)   // accumulator columns are rows of the operator
+                    if (power(r8 + cl + q) == pw) acc[j][q] = v[q];
             }
         }
         const bool first = seg < KPARTS;
