@@ -360,7 +360,8 @@ static cudaError_t launch_combine_mode(const CombineArgs<T>& a, int n_sm, cudaSt
     const int na = std::max(a.nk_pos, a.nk_neg) + 1;
     if (c.items == nullptr) c.n_items = a.nzi * na * ((na + 31) / 32);   // every segment of every row
     // one resident wave (the launch bounds' CTAs per SM)
-    cudaFuncSetAttribute(k_combine<T, PARTNER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k_combine<T, PARTNER>, kMaxShared);
+    if (e != cudaSuccess) return e;
     // lists that leave half of the resident warps idle take the two signs of fy as separate items
     // (64^3 to k = 0.8 k_Ny: 530 items for 2432 warps; an estimate 1.43 -> 1.37 ms)
     const int warps = n_sm * combine_ctas<T>() * kCombineWarps;

@@ -154,6 +154,16 @@ void eb_matrices(double N[2][3], double M[3][3]);
 // --------------------------------------------------------------------- device params
 struct DevTables;  // opaque pointer bundle filled by the C API
 
+// The dynamic shared memory that a kernel's launches may ask for.  The limit belongs to the function
+// on the device, not to a launch: a call that set it to its own need could lower it between another
+// thread's call and launch, so it is always the kernel's largest need or kMaxShared (227 KB a CTA less
+// 1 KB for the kernels' static arrays).
+constexpr size_t kMaxShared = 226 * 1024;
+template <typename K>
+cudaError_t allow_shared(K* kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Per-kernel timing bookkeeping (kernel kinds as in lpp_plan_kernel_stats).
 enum KernelKind { KK_ASSIGN = 0, KK_FFT = 1, KK_COMBINE = 2, KK_COEFF = 3, KK_PARTNER = 4, KK_OTHER = 5, KK_COUNT = 6 };
 

@@ -302,8 +302,7 @@ extern "C" lpp_status lpp_window_Q_pairs(const double* pos, const double* w, con
         a.copies = 32;
         while (a.copies > 4 && smem_of(a.copies) > 112 * 1024) a.copies /= 2;
         const size_t smem = smem_of(a.copies);
-        if (cudaFuncSetAttribute(k_pair_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return LPP_ERR_CUDA;
+        if (lpp::allow_shared(k_pair_sums, lpp::kMaxShared) != cudaSuccess) return LPP_ERR_CUDA;
         const long long tp = (long long)a.n_tiles * (a.n_tiles + 1) / 2;
         int dev = 0, sms = 152;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

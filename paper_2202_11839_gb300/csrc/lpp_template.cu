@@ -303,6 +303,8 @@ constexpr int kFewSets = 2;
 constexpr int kManyFrom = kFewSets + 1;
 constexpr int kMaxRows = 8 * 8 * kTiles;   // rows per cluster: 8 warps x kTiles tiles of 8
 constexpr int kSlabPad = kSlab + 2;        // the eight sets' rows start in different banks
+// the most dynamic shared memory of a launch: three spectra, kMaxRows rows (kSegs parts of at most 64 are fewer)
+constexpr size_t kTemplateSmem = ((size_t)3 * kSets * kSlabPad + (size_t)kMaxRows * kSets) * sizeof(double);
 
 // NT: tiles of 8 rows per warp, KPARTS: column segments taken by different warps (1 or kSegs);
 // compile-time, so that every tile of a warp is one unconditional product
@@ -477,6 +479,7 @@ constexpr int kManySets = 16;                 // sets per cluster: two column ti
 constexpr int kManyTiles = 5;                 // row tiles of 16 per warp
 constexpr int kManyRows = 8 * 16 * kManyTiles;
 constexpr int kSpread = 3;
+constexpr size_t kManySmem = (size_t)kDigits * 16 * 2 * 32 * sizeof(uint2) + (size_t)kManyRows * kManySets * sizeof(double);
 // groups of sets from which a cluster is four CTAs of two slabs each: clusters of eight leave 40 of the 152
 // SMs idle (40 shells, nine slots, eight -> four CTAs: 16 sets 81 -> 153 us, 64 sets 165 -> 161, 256 sets
 // 306 -> 197, 8192 sets 4421 -> 3654)
@@ -1122,12 +1125,11 @@ static lpp_status convolve(lpp_template_t t, const double* params, int n_templat
         const size_t smem = (size_t)kDigits * 16 * 2 * 32 * sizeof(uint2) +
                             (size_t)a.bins * a.n_slots * kManySets * sizeof(double);
         auto launch = [&](void (*kernel)(TemplateArgs)) {
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (lpp::allow_shared(kernel, kManySmem) != cudaSuccess) return LPP_ERR_CUDA;
             kernel<<<dim3(many * cl, groups), 256, smem, (cudaStream_t)stream>>>(a);
+            return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
         };
-        if (cl == 4) launch(k_template_many<4>);
-        else launch(k_template_many<8>);
-        return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
+        return cl == 4 ? launch(k_template_many<4>) : launch(k_template_many<8>);
     }
     // shells per cluster: at most kMaxRows rows, and enough clusters for every SM (2 x 19 clusters of 8)
     const int clusters = (n_templates + kSets - 1) / kSets, ns = a.n_slots > 0 ? a.n_slots : 1;
@@ -1142,29 +1144,27 @@ static lpp_status convolve(lpp_template_t t, const double* params, int n_templat
     const size_t smem = ((size_t)(t->png_amp != 0.0 ? 3 : 1) * kSets * kSlabPad + (size_t)kparts * rows * kSets) *
                         sizeof(double);
     auto launch = [&](void (*kernel)(TemplateArgs)) {
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (lpp::allow_shared(kernel, kTemplateSmem) != cudaSuccess) return LPP_ERR_CUDA;
         kernel<<<dim3(clusters * kCluster, groups), 256, smem, (cudaStream_t)stream>>>(a);
+        return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
     };
-    if (n_templates <= kFewSets) {
-        launch(k_template<1, 1, true>);
-    } else if (kparts == kSegs) {
+    if (n_templates <= kFewSets) return launch(k_template<1, 1, true>);
+    if (kparts == kSegs) {
         switch (nt) {
-            case 1: launch(k_template<1, kSegs>); break;
-            case 2: launch(k_template<2, kSegs>); break;
-            case 3: launch(k_template<3, kSegs>); break;
-            default: launch(k_template<4, kSegs>); break;
-        }
-    } else {
-        switch (nt) {
-            case 2: launch(k_template<2, 1>); break;
-            case 3: launch(k_template<3, 1>); break;
-            case 4: launch(k_template<4, 1>); break;
-            case 5: launch(k_template<5, 1>); break;
-            case 6: launch(k_template<6, 1>); break;
-            case 7: launch(k_template<7, 1>); break;
-            case 8: launch(k_template<8, 1>); break;
-            default: launch(k_template<9, 1>); break;
+            case 1: return launch(k_template<1, kSegs>);
+            case 2: return launch(k_template<2, kSegs>);
+            case 3: return launch(k_template<3, kSegs>);
+            default: return launch(k_template<4, kSegs>);
         }
     }
-    return cudaGetLastError() == cudaSuccess ? LPP_OK : LPP_ERR_CUDA;
+    switch (nt) {
+        case 2: return launch(k_template<2, 1>);
+        case 3: return launch(k_template<3, 1>);
+        case 4: return launch(k_template<4, 1>);
+        case 5: return launch(k_template<5, 1>);
+        case 6: return launch(k_template<6, 1>);
+        case 7: return launch(k_template<7, 1>);
+        case 8: return launch(k_template<8, 1>);
+        default: return launch(k_template<9, 1>);
+    }
 }

@@ -122,7 +122,8 @@ template <typename T>
 cudaError_t launch_sbin(const SbinArgs<T>& a, int n_sm, cudaStream_t st) {
     const int E = a.n_runs * a.nb * 2;
     const size_t smem = (size_t)kSbinWarps * E * Owned<T>::words * sizeof(T) + (size_t)(a.nb + 1) * sizeof(int);
-    cudaFuncSetAttribute(k_sbin<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k_sbin<T>, kMaxShared);
+    if (e != cudaSuccess) return e;
     const long long items = (long long)a.nks * a.nks * ((a.ns_pos + 32) / 32 + (a.ns_neg + 31) / 32);
     const int blocks = (int)std::max(1LL, std::min<long long>((long long)n_sm * (sizeof(T) == 4 ? 3 : 2),
                                                               (items + kSbinWarps - 1) / kSbinWarps));
