@@ -339,7 +339,8 @@ extern "C" lpp_status lpp_window_Q_pairs(const double* pos, const double* w, con
                                            s_edges[b] * s_edges[b] * s_edges[b]) / 3.0;
             const double* p = &h_out[(size_t)b * kEll];
             double sum = 2.0 * leg[e][0] * p[0];   // p_0 = 2 per pair
-            for (int k = 1; k < kEll; ++k) sum += leg[e][k] * p[k];
+            // to degree e: the powers beyond are not its own (NaN where a line of sight does not exist)
+            for (int k = 1; k <= e; ++k) sum += leg[e][k] * p[k];
             q[e * n_s + b] = I > 0.0 ? (4.0 * e + 1.0) * alpha * alpha * sum / (I * vol) : 0.0;
         }
     return LPP_OK;

@@ -1,0 +1,27 @@
+"""Window pair counts where a pair has no direction or a separation far below one.
+
+Tolerances: FP64 sums of at most 5e4 pairs, 1e-12 of the shell's Q_0 (the same pairs, the same
+operations but for a power of two); 1e-6 where a separation is replaced by a larger parallel one.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _q(pos, w, observer, edges, box=0.0):
+    import torch
+    from paper_2202_11839_gb300 import lpp as L
+    L.load_library()
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float64)).cuda()
+    return L.window_q_pairs(t(pos), t(w), None, observer, np.asarray(edges, dtype=np.float64), alpha=0.5, box=box)
+
+
+def test_monopole_with_a_point_at_the_observer():
+    """Q_0 does not depend on the observer, also where a line of sight does not exist."""
+    rng = np.random.default_rng(2)
+    pos, w = rng.uniform(0, 100, (3, 200)), rng.uniform(0.5, 1.5, 200)
+    edges = np.linspace(0, 60, 7)
+    want = _q(pos, w, (50.0, 50.0, -300.0), edges)
+    got = _q(pos, w, tuple(pos[:, 17]), edges)
+    np.testing.assert_allclose(got[0], want[0], rtol=1e-12)
