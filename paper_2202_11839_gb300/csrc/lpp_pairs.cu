@@ -180,21 +180,25 @@ __global__ void __launch_bounds__(kTile) k_pair_sums(PairArgs a) {
                 if (f2 >= thf[mid]) lo = mid; else hi = mid;
             }
             while (lo > 0 && f2 == thf[lo] && b2 < order_bits(thr[lo])) --lo;
-            // 1 / s2: an FP32 reciprocal and a third-order correction (its error to the third power)
-            double inv;
+            const double di = dx * ux + dy * uy + dz * uz;
+            const double dj = dx * xj[4 * kTile + jj] + dy * xj[5 * kTile + jj] + dz * xj[6 * kTile + jj];
+            // 1 / s2: an FP32 reciprocal and a third-order correction (its error to the third power); beyond
+            // FP32's exponents by the cosines themselves, as 1 / s2 and the squares leave FP64's too
+            double yi2, yj2;
             if (f2 > 0x0e000000 && f2 < 0x70000000) {   // 2^-99 .. 2^97
                 float r;
                 asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__int_as_float(f2)));
                 const int rb = __float_as_int(r);   // widened by its bits (normal)
                 const double rd = __hiloint2double((rb >> 3) + 0x38000000, rb << 29);
                 const double e = fma(-s2, rd, 1.0);
-                inv = fma(rd, fma(e, e, e), rd);
+                const double inv = fma(rd, fma(e, e, e), rd);
+                yi2 = fma(di * di, inv, -1.0);
+                yj2 = fma(dj * dj, inv, -1.0);
             } else {
-                inv = 1.0 / s2;
+                const double s = sqrt(s2), ci = di / s, cj = dj / s;
+                yi2 = fma(ci, ci, -1.0);
+                yj2 = fma(cj, cj, -1.0);
             }
-            const double di = dx * ux + dy * uy + dz * uz;
-            const double dj = dx * xj[4 * kTile + jj] + dy * xj[5 * kTile + jj] + dz * xj[6 * kTile + jj];
-            const double yi2 = fma(di * di, inv, -1.0), yj2 = fma(dj * dj, inv, -1.0);
             // Newton's identities for the power sums of two numbers
             const double e1 = yi2 + yj2, e2 = yi2 * yj2;
             const double p2 = fma(e1, e1, -2.0 * e2);

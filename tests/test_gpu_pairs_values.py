@@ -25,3 +25,13 @@ def test_monopole_with_a_point_at_the_observer():
     want = _q(pos, w, (50.0, 50.0, -300.0), edges)
     got = _q(pos, w, tuple(pos[:, 17]), edges)
     np.testing.assert_allclose(got[0], want[0], rtol=1e-12)
+
+
+@pytest.mark.parametrize("exponent", [-20, -150, -154, -155, -156, -158])
+def test_separations_near_the_underflow_threshold(exponent):
+    """Two points 10^exponent apart have the multipoles of two points 1e-6 apart in the same direction."""
+    d = np.array([0.3, -0.5, 0.7])
+    w, edges, observer = np.array([1.0, 2.0]), (0.0, 1.0), (3.0, 2.0, -10.0)
+    pair = lambda s: np.stack([np.zeros(3), d * s], axis=1)
+    want, got = _q(pair(1e-6), w, observer, edges), _q(pair(10.0 ** exponent), w, observer, edges)
+    np.testing.assert_allclose(got, want, atol=1e-6 * want[0].max())
