@@ -151,11 +151,12 @@ __global__ void __launch_bounds__(kTile) k_pair_sums(PairArgs a) {
         const long long jn = n - (long long)jt * kTile;
         const int j1 = jn < kTile ? (int)jn : kTile;
         // a pair whose FP32 separation exceeds the last edge by more than every rounding (2^-21 of the
-        // coordinates) is out of range
+        // coordinates) is out of range; below 1e-16 the squares would round among FP32's denormals and
+        // every pair is taken
         const float boxf = (float)a.box, ibox = a.box > 0.0 ? 1.0f / boxf : 0.0f;
         const float xif = (float)xi, yif = (float)yi, zif = (float)zi;
         const float edge = (float)a.s_max * 1.00001f + 4.8e-7f * (far_j + fabsf(xif) + fabsf(yif) + fabsf(zif) + boxf);
-        const float far = edge * edge;
+        const float far = edge >= 1e-16f ? edge * edge : INFINITY;
         for (int jj = 0; jj < j1; ++jj) {   // warp-uniform: the lanes take turns below
             bool in = live && jj >= j0;
             float fx = xf[jj] - xif, fy = xf[kTile + jj] - yif, fz = xf[2 * kTile + jj] - zif;

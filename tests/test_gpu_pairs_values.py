@@ -35,3 +35,15 @@ def test_separations_near_the_underflow_threshold(exponent):
     pair = lambda s: np.stack([np.zeros(3), d * s], axis=1)
     want, got = _q(pair(1e-6), w, observer, edges), _q(pair(10.0 ** exponent), w, observer, edges)
     np.testing.assert_allclose(got, want, atol=1e-6 * want[0].max())
+
+
+@pytest.mark.parametrize("power", [-40, -60, -70, -71, -72, -76])
+@pytest.mark.parametrize("periodic", [False, True])
+def test_shells_in_a_small_unit(power, periodic):
+    """Every length times a power of two: the same pairs in the same shells."""
+    rng = np.random.default_rng(5)
+    pos, w = rng.uniform(0, 1, (3, 300)), rng.uniform(0.5, 1.5, 300)
+    edges, observer, u = np.linspace(0, 0.45, 10), np.array([0.5, 0.4, -3.0]), 2.0 ** power
+    want = _q(pos, w, tuple(observer), edges, 1.0 if periodic else 0.0)
+    got = _q(pos * u, w, tuple(observer * u), edges * u, u if periodic else 0.0) * u ** 3
+    assert (np.abs(got - want) <= 1e-12 * np.abs(want[0])).all()
