@@ -165,15 +165,18 @@ __global__ void __launch_bounds__(256) k_coeffs(const __grid_constant__ CoeffArg
         sw += (double)w;
         sg += (double)w * (double)w * ((double)g1 * g1 + (double)g2 * g2);
         if (a.n_groups == 0) continue;
-        // angles of the estimator's line of sight in the grid's frame (phi = 0 on its z axis)
+        // angles of the estimator's line of sight in the grid's frame (phi = 0 on its z axis, and so
+        // close to it that the axis is the same direction to the last digit: there the squares may
+        // underflow, and a division by their root would not give a unit vector)
         T ct[LMAX + 1], st[LMAX + 1], cp[LMAX + 1], sp[LMAX + 1];
         ct[0] = cp[0] = (T)1;
         st[0] = sp[0] = (T)0;
         const T rho = sqrt(xe[0] * xe[0] + xe[1] * xe[1]);
         ct[1] = xe[2];
         st[1] = rho;
-        cp[1] = rho > (T)0 ? xe[0] / rho : (T)1;
-        sp[1] = rho > (T)0 ? xe[1] / rho : (T)0;
+        const bool off_axis = rho > (T)(sizeof(T) == 4 ? 1e-15 : 1e-100);
+        cp[1] = off_axis ? xe[0] / rho : (T)1;
+        sp[1] = off_axis ? xe[1] / rho : (T)0;
 #pragma unroll
         for (int j = 2; j <= LMAX; ++j) {
             ct[j] = ct[j - 1] * ct[1] - st[j - 1] * st[1];
