@@ -757,7 +757,6 @@ static lpp_status enqueue(lpp_plan_t plan, double* host_out, double* host_sums, 
     cb.nb = nb;
     cb.nk_pos = plan->nk_pos;
     cb.nk_neg = plan->nk_neg;
-    cb.nky = plan->nky;
     cb.nzi = plan->nzi;
     cb.out = out;
     cb.err = err;

@@ -129,7 +129,7 @@ __device__ __forceinline__ void pencil_tile(c2<T>* grid, const c2<T>* twg, c2<T>
     }
     if (twg)
         for (int k = tid; k < N; k += S::THREADS) tw[k] = twg[k];
-    fft_columns_io<T, LOGN, false, S::IPT, LD>(
+    fft_columns_io<T, LOGN, S::IPT, LD>(
         tile, c, u, tw,
         [&](int b, int e) { return ((live >> b) & 1u) ? gp[(size_t)e * ES] : mk<T>((T)0, (T)0); },
         [&](int e, c2<T> v) {
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(PassShape<LOGN>::THREADS, sizeof(T) == 4 ? (LO
             tile[e * LD + c] = base[e + c * N];
         }
         __syncthreads();
-        fft_columns<T, LOGN, false, S::IPT, LD>(tile, tid & (W - 1), tid >> S::LOGW, tw);
+        fft_columns<T, LOGN, S::IPT, LD>(tile, tid & (W - 1), tid >> S::LOGW, tw);
 #pragma unroll
         for (int k = 0; k < S::PER; ++k) {
             const int idx = tid + k * S::THREADS;
@@ -258,7 +258,7 @@ __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair
     auto twiddle = [](float2 w) { return cpair{pk2(w.x, w.x), pk2(-w.y, -w.y)}; };
     if (twg)
         for (int k = tid; k < N; k += S::THREADS) tw[k] = twiddle(twg[k]);
-    fft_pairs_io<LOGN, false>(
+    fft_pairs_io<LOGN>(
         tile, c, u, tw,
         [&](int b, int e) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -270,7 +270,7 @@ __device__ __forceinline__ void pair_tile(float2* grid, const float2* twg, cpair
             if constexpr (MULT) {
                 const float4 f = static_cast<const float4*>(
                     g.mult)[(gp - reinterpret_cast<float4*>(grid)) + (size_t)e * (ES / 2)];
-                v = pmul<true>(v, cpair{pk2(f.x, f.z), pk2(f.y, f.w)});
+                v = pmul_plain(v, cpair{pk2(f.x, f.z), pk2(f.y, f.w)});
             }
             float4 w;
             unpk2(v.re, w.x, w.z);

@@ -11,41 +11,34 @@
 
 namespace lpp {
 
-template <typename T, bool INV>
+template <typename T>
 __device__ __forceinline__ void dft4(c2<T>* v) {
     c2<T> a0 = cadd<T>(v[0], v[2]), a1 = csub<T>(v[0], v[2]);
     c2<T> b0 = cadd<T>(v[1], v[3]), b1 = csub<T>(v[1], v[3]);
-    b1 = INV ? mk<T>(-b1.y, b1.x) : mk<T>(b1.y, -b1.x);  // * (+i) or * (-i)
+    b1 = mk<T>(b1.y, -b1.x);  // * (-i)
     v[0] = cadd<T>(a0, b0);
     v[2] = csub<T>(a0, b0);
     v[1] = cadd<T>(a1, b1);
     v[3] = csub<T>(a1, b1);
 }
 
-template <typename T, bool INV>
+template <typename T>
 __device__ __forceinline__ void dft2(c2<T>* v) {
     c2<T> a = v[0];
     v[0] = cadd<T>(a, v[1]);
     v[1] = csub<T>(a, v[1]);
 }
 
-template <typename T, bool INV>
+template <typename T>
 __device__ __forceinline__ void dft8(c2<T>* v) {
     c2<T> e[4] = {v[0], v[2], v[4], v[6]};
     c2<T> o[4] = {v[1], v[3], v[5], v[7]};
-    dft4<T, INV>(e);
-    dft4<T, INV>(o);
+    dft4<T>(e);
+    dft4<T>(o);
     const T r = (T)0.70710678118654752440;
-    c2<T> t1, t2, t3;
-    if (!INV) {
-        t1 = mk<T>((o[1].x + o[1].y) * r, (o[1].y - o[1].x) * r);   // * (1 - i)/sqrt2
-        t2 = mk<T>(o[2].y, -o[2].x);                               // * (-i)
-        t3 = mk<T>((o[3].y - o[3].x) * r, -(o[3].x + o[3].y) * r);  // * (-1 - i)/sqrt2
-    } else {
-        t1 = mk<T>((o[1].x - o[1].y) * r, (o[1].x + o[1].y) * r);
-        t2 = mk<T>(-o[2].y, o[2].x);
-        t3 = mk<T>(-(o[3].x + o[3].y) * r, (o[3].x - o[3].y) * r);
-    }
+    const c2<T> t1 = mk<T>((o[1].x + o[1].y) * r, (o[1].y - o[1].x) * r);   // * (1 - i)/sqrt2
+    const c2<T> t2 = mk<T>(o[2].y, -o[2].x);                               // * (-i)
+    const c2<T> t3 = mk<T>((o[3].y - o[3].x) * r, -(o[3].x + o[3].y) * r);  // * (-1 - i)/sqrt2
     v[0] = cadd<T>(e[0], o[0]);
     v[4] = csub<T>(e[0], o[0]);
     v[1] = cadd<T>(e[1], t1);
@@ -63,7 +56,7 @@ __device__ __forceinline__ void dft8(c2<T>* v) {
 // touch 16 different banks pairs (no conflicts) and read the same twiddle (a broadcast).
 // LD and the stage's sub-transform length NS are compile-time, so every address is a
 // per-thread base plus an immediate offset; the first stage (NS = 1) has no twiddles.
-template <typename T, int N, int R, bool INV, int IPT, int LD, int NS>
+template <typename T, int N, int R, int IPT, int LD, int NS>
 __device__ __forceinline__ void stockham_stage(c2<T>* tile, int c, int u, const c2<T>* tw) {
     constexpr int Q = 8 / R;
     constexpr int US = N / (8 * IPT);
@@ -88,14 +81,13 @@ __device__ __forceinline__ void stockham_stage(c2<T>* tile, int c, int u, const 
                 const int step = jm * (N / (NS * R));
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    c2<T> w = tw[step * r];
-                    if (INV) w.y = -w.y;
+                    const c2<T> w = tw[step * r];
                     v[s][q * R + r] = cmul<T>(v[s][q * R + r], w);
                 }
             }
-            if (R == 8) dft8<T, INV>(v[s] + q * R);
-            else if (R == 4) dft4<T, INV>(v[s] + q * R);
-            else dft2<T, INV>(v[s] + q * R);
+            if (R == 8) dft8<T>(v[s] + q * R);
+            else if (R == 4) dft4<T>(v[s] + q * R);
+            else dft2<T>(v[s] + q * R);
             c2<T>* dst = tile + ((j - jm) * R + jm) * LD + c;
 #pragma unroll
             for (int r = 0; r < R; ++r) dst[r * NS * LD] = v[s][q * R + r];
@@ -104,29 +96,29 @@ __device__ __forceinline__ void stockham_stage(c2<T>* tile, int c, int u, const 
     __syncthreads();
 }
 
-template <typename T, int N, bool INV, int IPT, int LD, int NS>
+template <typename T, int N, int IPT, int LD, int NS>
 __device__ __forceinline__ void radix8_stages(c2<T>* tile, int c, int u, const c2<T>* tw) {
     if constexpr (NS < N) {
-        stockham_stage<T, N, 8, INV, IPT, LD, NS>(tile, c, u, tw);
-        radix8_stages<T, N, INV, IPT, LD, NS * 8>(tile, c, u, tw);
+        stockham_stage<T, N, 8, IPT, LD, NS>(tile, c, u, tw);
+        radix8_stages<T, N, IPT, LD, NS * 8>(tile, c, u, tw);
     }
 }
 
-// Forward (or inverse, unnormalised) FFT of length N = 2^LOGN along every pencil: one
+// Forward FFT of length N = 2^LOGN along every pencil: one
 // radix-2 or radix-4 stage when LOGN is not a multiple of 3, then radix-8 stages.
 // c = the thread's pencil, u = its first butterfly slot (0 .. N / (8 IPT) - 1).
-template <typename T, int LOGN, bool INV, int IPT, int LD>
+template <typename T, int LOGN, int IPT, int LD>
 __device__ __forceinline__ void fft_columns(c2<T>* tile, int c, int u, const c2<T>* tw) {
     constexpr int N = 1 << LOGN;
     constexpr int rem = LOGN % 3;
     if constexpr (rem == 1) {
-        stockham_stage<T, N, 2, INV, IPT, LD, 1>(tile, c, u, tw);
-        radix8_stages<T, N, INV, IPT, LD, 2>(tile, c, u, tw);
+        stockham_stage<T, N, 2, IPT, LD, 1>(tile, c, u, tw);
+        radix8_stages<T, N, IPT, LD, 2>(tile, c, u, tw);
     } else if constexpr (rem == 2) {
-        stockham_stage<T, N, 4, INV, IPT, LD, 1>(tile, c, u, tw);
-        radix8_stages<T, N, INV, IPT, LD, 4>(tile, c, u, tw);
+        stockham_stage<T, N, 4, IPT, LD, 1>(tile, c, u, tw);
+        radix8_stages<T, N, IPT, LD, 4>(tile, c, u, tw);
     } else {
-        radix8_stages<T, N, INV, IPT, LD, 1>(tile, c, u, tw);
+        radix8_stages<T, N, IPT, LD, 1>(tile, c, u, tw);
     }
 }
 
@@ -149,7 +141,7 @@ __device__ __forceinline__ int lead_row(int u, int b) {
 // Leading stage (NS = 1, no twiddles) with operand b of point e from load(b, e); results
 // to the tile.  INPLACE: load reads the tile itself (a barrier separates the reads from
 // the writes).  Ends with a barrier.
-template <typename T, int LOGN, bool INV, int IPT, int LD, bool INPLACE, class Load>
+template <typename T, int LOGN, int IPT, int LD, bool INPLACE, class Load>
 __device__ __forceinline__ void lead_stage(c2<T>* tile, int c, int u, Load&& load) {
     constexpr int N = 1 << LOGN, R = LeadRadix<LOGN>::R, Q = 8 / R, US = N / (8 * IPT);
     c2<T> v[IPT][8];
@@ -164,9 +156,9 @@ __device__ __forceinline__ void lead_stage(c2<T>* tile, int c, int u, Load&& loa
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int j = u + s * US + q * (N / 8);
-            if (R == 8) dft8<T, INV>(v[s] + q * R);
-            else if (R == 4) dft4<T, INV>(v[s] + q * R);
-            else dft2<T, INV>(v[s] + q * R);
+            if (R == 8) dft8<T>(v[s] + q * R);
+            else if (R == 4) dft4<T>(v[s] + q * R);
+            else dft2<T>(v[s] + q * R);
             c2<T>* dst = tile + j * R * LD + c;
 #pragma unroll
             for (int r = 0; r < R; ++r) dst[r * LD] = v[s][q * R + r];
@@ -175,17 +167,17 @@ __device__ __forceinline__ void lead_stage(c2<T>* tile, int c, int u, Load&& loa
     __syncthreads();
 }
 
-template <typename T, int N, bool INV, int IPT, int LD, int NS, int NS_END>
+template <typename T, int N, int IPT, int LD, int NS, int NS_END>
 __device__ __forceinline__ void radix8_until(c2<T>* tile, int c, int u, const c2<T>* tw) {
     if constexpr (NS < NS_END) {
-        stockham_stage<T, N, 8, INV, IPT, LD, NS>(tile, c, u, tw);
-        radix8_until<T, N, INV, IPT, LD, NS * 8, NS_END>(tile, c, u, tw);
+        stockham_stage<T, N, 8, IPT, LD, NS>(tile, c, u, tw);
+        radix8_until<T, N, IPT, LD, NS * 8, NS_END>(tile, c, u, tw);
     }
 }
 
 // Last radix-8 stage (NS = N/8) from the tile, results to store(e, value): the butterfly
 // at slot j writes points j + r N/8.  No barrier at the end.
-template <typename T, int N, bool INV, int IPT, int LD, class Store>
+template <typename T, int N, int IPT, int LD, class Store>
 __device__ __forceinline__ void last_stage(const c2<T>* tile, int c, int u, const c2<T>* tw, Store&& store) {
     constexpr int US = N / (8 * IPT);
     c2<T> v[IPT][8];
@@ -200,11 +192,10 @@ __device__ __forceinline__ void last_stage(const c2<T>* tile, int c, int u, cons
         const int j = u + s * US;
 #pragma unroll
         for (int r = 1; r < 8; ++r) {
-            c2<T> w = tw[j * r];
-            if (INV) w.y = -w.y;
+            const c2<T> w = tw[j * r];
             v[s][r] = cmul<T>(v[s][r], w);
         }
-        dft8<T, INV>(v[s]);
+        dft8<T>(v[s]);
 #pragma unroll
         for (int r = 0; r < 8; ++r) store(j + r * (N / 8), v[s][r]);
     }
@@ -215,7 +206,7 @@ __device__ __forceinline__ void last_stage(const c2<T>* tile, int c, int u, cons
 // hands to store(e, value) are consecutive across the warp (a coalesced store along the
 // pencil).  twr holds each leg's twiddles by slot, twr[(r - 1) N/8 + j] = w^(j r), so the
 // lanes read consecutive words.  No barrier at the end.
-template <typename T, int N, bool INV, int IPT, int LD, class Store>
+template <typename T, int N, int IPT, int LD, class Store>
 __device__ __forceinline__ void last_stage_warp(const c2<T>* tile, int c, int l, const c2<T>* twr, Store&& store) {
     static_assert(N / 8 == 32 * IPT, "one warp covers the N/8 butterfly slots of a pencil");
     c2<T> v[IPT][8];
@@ -229,11 +220,10 @@ __device__ __forceinline__ void last_stage_warp(const c2<T>* tile, int c, int l,
         const int j = l + 32 * s;
 #pragma unroll
         for (int r = 1; r < 8; ++r) {
-            c2<T> w = twr[(r - 1) * (N / 8) + j];
-            if (INV) w.y = -w.y;
+            const c2<T> w = twr[(r - 1) * (N / 8) + j];
             v[s][r] = cmul<T>(v[s][r], w);
         }
-        dft8<T, INV>(v[s]);
+        dft8<T>(v[s]);
 #pragma unroll
         for (int r = 0; r < 8; ++r) store(j + r * (N / 8), v[s][r]);
     }
@@ -248,9 +238,8 @@ __device__ __forceinline__ void last_stage_warp(const c2<T>* tile, int c, int l,
 // y1 sits at row 64 k0 + (m + 8 k0) % 64 and y2 at row 8 R1 n0 + (k0 + R1 k1 + 2 n0) % (8 R1),
 // so that with an odd LD the 16 lanes of every half-warp access 16 different bank pairs in
 // each pass.  load(e): point e of the input; store(k, value): output k (consecutive lanes
-// store consecutive k).  t1[(k0 - 1) 64 + m] = w^(m k0) and t2[(k1 - 1) 8 + n0] = w^(R1 n0 k1)
-// (forward twiddles; conjugated for INV).
-template <typename T, int LOGN, bool INV, int LD, bool ZERO = false, class Load, class Store>
+// store consecutive k).  t1[(k0 - 1) 64 + m] = w^(m k0) and t2[(k1 - 1) 8 + n0] = w^(R1 n0 k1).
+template <typename T, int LOGN, int LD, bool ZERO = false, class Load, class Store>
 __device__ __forceinline__ void fft_pencil_warp(c2<T>* tile, int c, int lane, const c2<T>* t1, const c2<T>* t2,
                                                 Load&& load, Store&& store) {
     constexpr int N = 1 << LOGN, R1 = N / 64, Q = 8 * R1, B = R1 / 4;
@@ -267,12 +256,11 @@ __device__ __forceinline__ void fft_pencil_warp(c2<T>* tile, int c, int lane, co
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int m = lane + 32 * h;
-            if (R1 == 8) dft8<T, INV>(v[h]);
-            else dft4<T, INV>(v[h]);
+            if (R1 == 8) dft8<T>(v[h]);
+            else dft4<T>(v[h]);
 #pragma unroll
             for (int k0 = 1; k0 < R1; ++k0) {
-                c2<T> w = t1[(k0 - 1) * 64 + m];
-                if (INV) w.y = -w.y;
+                const c2<T> w = t1[(k0 - 1) * 64 + m];
                 v[h][k0] = cmul<T>(v[h][k0], w);
             }
 #pragma unroll
@@ -291,11 +279,10 @@ __device__ __forceinline__ void fft_pencil_warp(c2<T>* tile, int c, int lane, co
 #pragma unroll
     for (int b = 0; b < B; ++b) {
         const int m2 = lane + 32 * b, n0 = m2 & 7, k0 = m2 >> 3;
-        dft8<T, INV>(v[b]);
+        dft8<T>(v[b]);
 #pragma unroll
         for (int k1 = 1; k1 < 8; ++k1) {
-            c2<T> w = t2[(k1 - 1) * 8 + n0];
-            if (INV) w.y = -w.y;
+            const c2<T> w = t2[(k1 - 1) * 8 + n0];
             v[b][k1] = cmul<T>(v[b][k1], w);
         }
 #pragma unroll
@@ -320,7 +307,7 @@ __device__ __forceinline__ void fft_pencil_warp(c2<T>* tile, int c, int lane, co
 #pragma unroll
     for (int b = 0; b < B; ++b) {
         const int q = lane + 32 * b;
-        dft8<T, INV>(v[b]);
+        dft8<T>(v[b]);
 #pragma unroll
         for (int k2 = 0; k2 < 8; ++k2) store(q + Q * k2, v[b][k2]);
     }
@@ -337,7 +324,7 @@ struct PencilWarpTw {
 // and the output handed to store(e, value) by the last: the tile holds only the
 // intermediate stages, so a pass moves each point through shared memory twice (not four
 // times) for N = 512.  The caller reuses the tile only after a barrier.
-template <typename T, int LOGN, bool INV, int IPT, int LD, class Load, class Store>
+template <typename T, int LOGN, int IPT, int LD, class Load, class Store>
 __device__ __forceinline__ void fft_columns_io(c2<T>* tile, int c, int u, const c2<T>* tw, Load&& load,
                                                Store&& store) {
     constexpr int N = 1 << LOGN;
@@ -345,13 +332,13 @@ __device__ __forceinline__ void fft_columns_io(c2<T>* tile, int c, int u, const 
         c2<T> v[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) v[k] = load(k, k);
-        dft8<T, INV>(v);
+        dft8<T>(v);
 #pragma unroll
         for (int k = 0; k < 8; ++k) store(k, v[k]);
     } else {
-        lead_stage<T, LOGN, INV, IPT, LD, false>(tile, c, u, load);
-        radix8_until<T, N, INV, IPT, LD, LeadRadix<LOGN>::R, N / 8>(tile, c, u, tw);
-        last_stage<T, N, INV, IPT, LD>(tile, c, u, tw, store);
+        lead_stage<T, LOGN, IPT, LD, false>(tile, c, u, load);
+        radix8_until<T, N, IPT, LD, LeadRadix<LOGN>::R, N / 8>(tile, c, u, tw);
+        last_stage<T, N, IPT, LD>(tile, c, u, tw, store);
     }
 }
 

@@ -55,61 +55,47 @@ struct __align__(16) cpair {
 };
 __device__ __forceinline__ cpair padd(cpair a, cpair b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
 __device__ __forceinline__ cpair psub(cpair a, cpair b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
-// v w (v conj w for INV), the twiddle stored as {(wx, wx), (-wy, -wy)}
-template <bool INV>
+// v w, the twiddle stored as {(wx, wx), (-wy, -wy)}
 __device__ __forceinline__ cpair pmul(cpair v, cpair w) {
-    if (!INV) return {fma2(v.im, w.im, mul2(v.re, w.re)), sub2(mul2(v.im, w.re), mul2(v.re, w.im))};
-    return {sub2(mul2(v.re, w.re), mul2(v.im, w.im)), fma2(v.re, w.im, mul2(v.im, w.re))};
+    return {fma2(v.im, w.im, mul2(v.re, w.re)), sub2(mul2(v.im, w.re), mul2(v.re, w.im))};
+}
+// v f of two complex values as they are
+__device__ __forceinline__ cpair pmul_plain(cpair v, cpair f) {
+    return {sub2(mul2(v.re, f.re), mul2(v.im, f.im)), fma2(v.re, f.im, mul2(v.im, f.re))};
 }
 
-template <bool INV>
 __device__ __forceinline__ void pdft4(cpair* v) {
     const cpair a0 = padd(v[0], v[2]), a1 = psub(v[0], v[2]);
     const cpair b0 = padd(v[1], v[3]), b1 = psub(v[1], v[3]);
     v[0] = padd(a0, b0);
     v[2] = psub(a0, b0);
     // a1 -+ i b1
-    v[INV ? 3 : 1] = {add2(a1.re, b1.im), sub2(a1.im, b1.re)};
-    v[INV ? 1 : 3] = {sub2(a1.re, b1.im), add2(a1.im, b1.re)};
+    v[1] = {add2(a1.re, b1.im), sub2(a1.im, b1.re)};
+    v[3] = {sub2(a1.re, b1.im), add2(a1.im, b1.re)};
 }
 
-template <bool INV>
 __device__ __forceinline__ void pdft2(cpair* v) {
     const cpair a = v[0];
     v[0] = padd(a, v[1]);
     v[1] = psub(a, v[1]);
 }
 
-template <bool INV>
 __device__ __forceinline__ void pdft8(cpair* v) {
     cpair e[4] = {v[0], v[2], v[4], v[6]};
     cpair o[4] = {v[1], v[3], v[5], v[7]};
-    pdft4<INV>(e);
-    pdft4<INV>(o);
+    pdft4(e);
+    pdft4(o);
     const f2x r = pk2(0.70710678118654752440f, 0.70710678118654752440f);
-    cpair t1, t3;
-    if (!INV) {
-        t1 = {mul2(add2(o[1].re, o[1].im), r), mul2(sub2(o[1].im, o[1].re), r)};   // * (1 - i)/sqrt2
-        t3 = {mul2(sub2(o[3].im, o[3].re), r), mul2(add2(o[3].re, o[3].im), r)};   // * (-1 - i)/sqrt2, im negated
-    } else {
-        t1 = {mul2(sub2(o[1].re, o[1].im), r), mul2(add2(o[1].re, o[1].im), r)};
-        t3 = {mul2(add2(o[3].re, o[3].im), r), mul2(sub2(o[3].re, o[3].im), r)};   // re negated
-    }
+    const cpair t1 = {mul2(add2(o[1].re, o[1].im), r), mul2(sub2(o[1].im, o[1].re), r)};   // * (1 - i)/sqrt2
+    const cpair t3 = {mul2(sub2(o[3].im, o[3].re), r), mul2(add2(o[3].re, o[3].im), r)};   // * (-1 - i)/sqrt2, im negated
     v[0] = padd(e[0], o[0]);
     v[4] = psub(e[0], o[0]);
     v[1] = padd(e[1], t1);
     v[5] = psub(e[1], t1);
-    if (!INV) {   // o2 * (-i) = (im, -re)
-        v[2] = {add2(e[2].re, o[2].im), sub2(e[2].im, o[2].re)};
-        v[6] = {sub2(e[2].re, o[2].im), add2(e[2].im, o[2].re)};
-        v[3] = {add2(e[3].re, t3.re), sub2(e[3].im, t3.im)};
-        v[7] = {sub2(e[3].re, t3.re), add2(e[3].im, t3.im)};
-    } else {
-        v[2] = {sub2(e[2].re, o[2].im), add2(e[2].im, o[2].re)};
-        v[6] = {add2(e[2].re, o[2].im), sub2(e[2].im, o[2].re)};
-        v[3] = {sub2(e[3].re, t3.re), add2(e[3].im, t3.im)};
-        v[7] = {add2(e[3].re, t3.re), sub2(e[3].im, t3.im)};
-    }
+    v[2] = {add2(e[2].re, o[2].im), sub2(e[2].im, o[2].re)};   // o2 * (-i) = (im, -re)
+    v[6] = {sub2(e[2].re, o[2].im), add2(e[2].im, o[2].re)};
+    v[3] = {add2(e[3].re, t3.re), sub2(e[3].im, t3.im)};
+    v[7] = {sub2(e[3].re, t3.re), add2(e[3].im, t3.im)};
 }
 
 // Pass shape: W pencils (128-byte segments; 64 bytes at n = 1024), half as many pencil pairs; one
@@ -134,7 +120,7 @@ struct PairShape {
 // FFT of length N along every pencil pair of the tile with operands from load(b, e) in the first stage
 // (point e, operand b as in lead_row) and results to store(e, value) in the last; c: the
 // thread's pair, u: its first butterfly slot.  The caller reuses the tile only after a barrier.
-template <int LOGN, bool INV, class Load, class Store>
+template <int LOGN, class Load, class Store>
 __device__ __forceinline__ void fft_pairs_io(cpair* tile, int c, int u, const cpair* tw, Load&& load, Store&& store) {
     using S = PairShape<LOGN>;
     constexpr int N = S::N, IPT = S::IPT, LD = S::CP, US = N / (8 * IPT), R = LeadRadix<LOGN>::R, Q = 8 / R;
@@ -148,9 +134,9 @@ __device__ __forceinline__ void fft_pairs_io(cpair* tile, int c, int u, const cp
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int j = u + s * US + q * (N / 8);
-            if (R == 8) pdft8<INV>(v[s] + q * R);
-            else if (R == 4) pdft4<INV>(v[s] + q * R);
-            else pdft2<INV>(v[s] + q * R);
+            if (R == 8) pdft8(v[s] + q * R);
+            else if (R == 4) pdft4(v[s] + q * R);
+            else pdft2(v[s] + q * R);
             cpair* dst = tile + j * R * LD + c;
 #pragma unroll
             for (int r = 0; r < R; ++r) dst[r * LD] = v[s][q * R + r];
@@ -169,8 +155,8 @@ __device__ __forceinline__ void fft_pairs_io(cpair* tile, int c, int u, const cp
         for (int s = 0; s < IPT; ++s) {
             const int j = u + s * US, jm = j & (ns - 1), step = jm * (N / (ns * 8));
 #pragma unroll
-            for (int r = 1; r < 8; ++r) v[s][r] = pmul<INV>(v[s][r], tw[step * r]);
-            pdft8<INV>(v[s]);
+            for (int r = 1; r < 8; ++r) v[s][r] = pmul(v[s][r], tw[step * r]);
+            pdft8(v[s]);
             cpair* dst = tile + ((j - jm) * 8 + jm) * LD + c;
 #pragma unroll
             for (int r = 0; r < 8; ++r) dst[r * ns * LD] = v[s][r];
@@ -186,8 +172,8 @@ __device__ __forceinline__ void fft_pairs_io(cpair* tile, int c, int u, const cp
     for (int s = 0; s < IPT; ++s) {
         const int j = u + s * US;
 #pragma unroll
-        for (int r = 1; r < 8; ++r) v[s][r] = pmul<INV>(v[s][r], tw[j * r]);
-        pdft8<INV>(v[s]);
+        for (int r = 1; r < 8; ++r) v[s][r] = pmul(v[s][r], tw[j * r]);
+        pdft8(v[s]);
 #pragma unroll
         for (int r = 0; r < 8; ++r) store(j + r * (N / 8), v[s][r]);
     }

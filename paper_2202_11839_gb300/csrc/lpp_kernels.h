@@ -311,7 +311,7 @@ struct CombineArgs {
     const c2<T>* phase;    // [n] per-index e^{-i pi f/n}
     const int* thr;        // [nb+1] thresholds on n^2
     int nb;
-    int nk_pos, nk_neg, nky, nzi;
+    int nk_pos, nk_neg, nzi;
     double* out;           // [rows][nb][2]
     // the work list (combine_items), or null: every segment of every row of the kept cube
     const int* items;
@@ -350,7 +350,7 @@ struct SbinArgs {
     const int* thr;   // [nb+1] thresholds on the integer |s|^2 / h^2
     int nb;
     int ns_pos, ns_neg, nks;
-    double scale;     // 1 / n^3 of the unnormalised inverse FFT
+    double scale;     // 1 / n^3 of the two transforms of the correlations
     double* out;      // [rows][nb][2]
 };
 template <typename T>

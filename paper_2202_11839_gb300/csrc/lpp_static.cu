@@ -170,7 +170,6 @@ lpp_status run_static(char* base, const Layout& lay, int n, double box, const do
     cb.nb = nb;
     cb.nk_pos = nk_pos;
     cb.nk_neg = nk_neg;
-    cb.nky = geom.nky;
     cb.nzi = nk_pos + 1 + (nk_neg == n / 2 ? 1 : 0);
     cb.out = reinterpret_cast<double*>(base + lay.out);
     int dev = 0, sms = 152;

@@ -109,10 +109,10 @@ struct TemplateArgs {
 // wk <- FFT(wk) * u ; FFT again (the log-Fourier transform between the two grids)
 __device__ void log_fourier(double2* wk, const double2* __restrict__ u, const double2* __restrict__ tw) {
     const int tid = threadIdx.x;
-    lpp::fft_columns<double, kLogN, false, 1, 1>(wk, 0, tid, tw);
+    lpp::fft_columns<double, kLogN, 1, 1>(wk, 0, tid, tw);
     for (int i = tid; i < kNfft; i += blockDim.x) wk[i] = lpp::cmul<double>(wk[i], u[i]);
     __syncthreads();
-    lpp::fft_columns<double, kLogN, false, 1, 1>(wk, 0, tid, tw);
+    lpp::fft_columns<double, kLogN, 1, 1>(wk, 0, tid, tw);
 }
 
 // One row (slot, shell) of the operator: out = sum_n op[n] P(k_n).  Forwards, a spectrum is

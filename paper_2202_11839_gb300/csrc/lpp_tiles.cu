@@ -476,7 +476,7 @@ __device__ __forceinline__ void x_transform(c2<T>* tile, int t, const c2<T>* tw,
             if constexpr (sizeof(T) == 4) {
                 if (fixed) {
                     const int2* ti = reinterpret_cast<const int2*>(tile) + pc;
-                    fft_pencil_warp<T, LOGN, false, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) {
+                    fft_pencil_warp<T, LOGN, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) {
                         const int2 q = ti[e * LD];
                         return mk<T>((T)((float)q.x * unit), (T)((float)q.y * unit));
                     }, store);
@@ -484,7 +484,7 @@ __device__ __forceinline__ void x_transform(c2<T>* tile, int t, const c2<T>* tw,
                 }
             }
             const c2<T>* col = tile + pc;
-            fft_pencil_warp<T, LOGN, false, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) { return col[e * LD]; },
+            fft_pencil_warp<T, LOGN, LD, ZERO>(tile, pc, lane, twr, twr + T1, [&](int e) { return col[e * LD]; },
                                                       store);
         }
     } else {
@@ -495,23 +495,23 @@ __device__ __forceinline__ void x_transform(c2<T>* tile, int t, const c2<T>* tw,
         if constexpr (sizeof(T) == 4) {
             if (fixed) {
                 const int2* ti = reinterpret_cast<const int2*>(tile) + c;
-                lead_stage<T, LOGN, false, IPT, LD, true>(tile, c, u, [&](int, int e) {
+                lead_stage<T, LOGN, IPT, LD, true>(tile, c, u, [&](int, int e) {
                     const int2 q = ti[e * LD];
                     return mk<T>((T)((float)q.x * unit), (T)((float)q.y * unit));
                 });
                 converted = true;
             }
         }
-        if (!converted) stockham_stage<T, N, R0, false, IPT, LD, 1>(tile, c, u, tw);
+        if (!converted) stockham_stage<T, N, R0, IPT, LD, 1>(tile, c, u, tw);
         if constexpr (S::WARP_OUT) {
-            radix8_until<T, N, false, IPT, LD, R0, N / 8>(tile, c, u, tw);
+            radix8_until<T, N, IPT, LD, R0, N / 8>(tile, c, u, tw);
             const int pc = t >> 5;
             c2<T>* po = out + ((size_t)(pc / TY) * N + (pc & (TY - 1))) * N;
-            last_stage_warp<T, N, false, IPT, LD>(tile, pc, t & 31, twr, [&](int e, c2<T> v) {
+            last_stage_warp<T, N, IPT, LD>(tile, pc, t & 31, twr, [&](int e, c2<T> v) {
                 if (kept(e, N, nk_pos, nk_neg)) po[e] = v;
             });
         } else {
-            radix8_until<T, N, false, IPT, LD, R0, N>(tile, c, u, tw);
+            radix8_until<T, N, IPT, LD, R0, N>(tile, c, u, tw);
             // LPL consecutive threads store one pencil (coalesced along x)
             constexpr int LPL = S::THREADS / W;
             const int cw = t / LPL;
