@@ -40,7 +40,7 @@ struct PairArgs {
     const double* thr;   // [nb + 1] thresholds on the squared separation
     double s_max;        // the last edge
     int nb;
-    int copies;          // lanes' private copies of a warp's shell sums: 32, 16, 8 or 4
+    int copies;          // lanes' private copies of a warp's shell sums: 32, 16, 8, 4, 2 or 1
     double* out;         // [nb][5] pair sums of w w' p_k (k = 0: of w w')
 };
 
@@ -86,8 +86,10 @@ __device__ __forceinline__ int float_bits(double v) {
 // What bounds it: the FP64 rate (1/64 of FP32 on GB300), about 35 operations a pair in range (110
 // with a square root, a division and two sets of polynomials per pair).  The sums need no
 // atomics (FP64 ones in shared memory are compare-and-swap loops): every lane adds to its own copy
-// of its warp's shells, copies[nb][5][32], and with fewer copies the lanes that share one take
-// turns; 4 warps per SM hide the FP64 latency.  20001 points, 40 shells: 37.9 -> 15.9 ms.
+// of its warp's shells, copies[nb][5][32], and with fewer copies the lanes that share one and meet on
+// a shell go one after the other (all lanes of a copy in fixed turns: 16.0 ms at 40 shells, 43.0 at
+// 256, more than atomics had taken there); 4 warps per SM hide the FP64 latency.  20000 points: 37.9 ->
+// 15.0 ms with 40 shells, 34.3 -> 15.8 with 256.
 __global__ void __launch_bounds__(kTile) k_pair_sums(PairArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nb = a.nb, C = a.copies;
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(kTile) k_pair_sums(PairArgs a) {
         const float xif = (float)xi, yif = (float)yi, zif = (float)zi;
         const float edge = (float)a.s_max * 1.00001f + 4.8e-7f * (far_j + fabsf(xif) + fabsf(yif) + fabsf(zif) + boxf);
         const float far = edge >= 1e-16f ? edge * edge : INFINITY;
-        for (int jj = 0; jj < j1; ++jj) {   // warp-uniform: the lanes take turns below
+        for (int jj = 0; jj < j1; ++jj) {   // warp-uniform: the lanes wait for one another below
             bool in = live && jj >= j0;
             float fx = xf[jj] - xif, fy = xf[kTile + jj] - yif, fz = xf[2 * kTile + jj] - zif;
             if (boxf > 0.f) {
@@ -206,16 +208,24 @@ __global__ void __launch_bounds__(kTile) k_pair_sums(PairArgs a) {
             const double p3 = fma(e1, p2, -e2 * e1);
             const double p4 = fma(e1, p3, -e2 * p2);
             const double ww = wi * xj[3 * kTile + jj];
-            for (int turn = 0; turn < 32; turn += C) {
-                if (in && (lane & ~(C - 1)) == turn) {
-                    double* q = h + lo * kEll * C;
-                    q[0] += ww;
-                    q[C] = fma(ww, e1, q[C]);
-                    q[2 * C] = fma(ww, p2, q[2 * C]);
-                    q[3 * C] = fma(ww, p3, q[3 * C]);
-                    q[4 * C] = fma(ww, p4, q[4 * C]);
+            auto add = [&]() {
+                double* q = h + lo * kEll * C;
+                q[0] += ww;
+                q[C] = fma(ww, e1, q[C]);
+                q[2 * C] = fma(ww, p2, q[2 * C]);
+                q[3 * C] = fma(ww, p3, q[3 * C]);
+                q[4 * C] = fma(ww, p4, q[4 * C]);
+            };
+            if (C == 32) {
+                if (in) add();
+            } else {
+                // the lanes that meet on one copy of one shell, one after the other
+                const unsigned peers = __match_any_sync(0xffffffffu, in ? lo * C + (lane & (C - 1)) : -1 - lane);
+                const int rank = __popc(peers & ((1u << lane) - 1u));
+                for (int turn = 0; __any_sync(0xffffffffu, in && rank >= turn); ++turn) {
+                    if (in && rank == turn) add();
+                    __syncwarp();
                 }
-                if (C < 32) __syncwarp();
             }
         }
     }
@@ -299,13 +309,14 @@ extern "C" lpp_status lpp_window_Q_pairs(const double* pos, const double* w, con
         a.nb = n_s;
         a.out = d_out;
         // copies of the shell sums: as many as leave room for two CTAs per SM (40 shells: 16 copies,
-        // 20.6 -> 15.9 ms against 32 copies and one CTA, whose four warps do not hide the FP64 latency)
+        // 20.6 -> 15.9 ms against 32 copies and one CTA, whose four warps do not hide the FP64 latency;
+        // 256 shells: two)
         auto smem_of = [&](int c) {
             return ((size_t)kWarps * n_s * kEll * c + 7 * kTile + n_s + 1) * sizeof(double) +
                    ((size_t)(n_s + 1) + 3 * kTile) * sizeof(float);
         };
         a.copies = 32;
-        while (a.copies > 4 && smem_of(a.copies) > 112 * 1024) a.copies /= 2;
+        while (a.copies > 1 && smem_of(a.copies) > 112 * 1024) a.copies /= 2;
         const size_t smem = smem_of(a.copies);
         if (lpp::allow_shared(k_pair_sums, lpp::kMaxShared) != cudaSuccess) return LPP_ERR_CUDA;
         const long long tp = (long long)a.n_tiles * (a.n_tiles + 1) / 2;
