@@ -791,9 +791,10 @@ std::complex<double> lgamma_c(std::complex<double> z) {
 }
 
 // u_alpha = (k_0 r_0)^{-i eta} M_l(q + i eta) / N, eta = 2 pi alpha / (N Delta), alpha in DFT order;
-// the Nyquist coefficient is kept real.
+// the Nyquist coefficient is kept real.  u_-alpha = conj u_alpha, which halves most of the time that a new
+// window's tables take.
 void fftlog_kernel(int ell, double q, double delta, double kr0, double2* u) {
-    for (int i = 0; i < kNfft; ++i) {
+    for (int i = 0; i <= kNfft / 2; ++i) {
         const int alpha = i < kNfft / 2 ? i : i - kNfft;
         const double eta = 2.0 * kPi * alpha / (kNfft * delta);
         const std::complex<double> s(q, eta);
@@ -802,6 +803,7 @@ void fftlog_kernel(int ell, double q, double delta, double kr0, double2* u) {
         std::complex<double> v = std::exp(lm - std::complex<double>(0.0, eta * log(kr0))) / double(kNfft);
         if (i == kNfft / 2) v = std::complex<double>(v.real(), 0.0);
         u[i] = make_double2(v.real(), v.imag());
+        if (i > 0 && i < kNfft / 2) u[kNfft - i] = make_double2(v.real(), -v.imag());
     }
 }
 
