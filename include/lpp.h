@@ -112,7 +112,9 @@ typedef struct {
     long long max_density;
     long long max_randoms;
     int host_inputs;         /* 1: reserve staging so lpp_assign accepts host catalogues       */
-    int batch;               /* complex grids per field pass; 0 = library default             */
+    int batch;               /* complex grids per field pass, 1..8, or 0 = library default: 16 for
+                                interlaced grids up to 256^3 (FP64 128^3), else 8; as many grids
+                                are reserved in the workspace (256^3 FP32: 128 MiB each)       */
     int fused_slots;         /* channel fields per CTA of the fused assignment + x-FFT pass:
                                 0 = library choice (two for FP32 interlaced grids of 64^3 to 512^3
                                 when a batch holds an even number), 1 = always one (a tuning knob;
@@ -284,7 +286,9 @@ lpp_status lpp_template_create(const double* q, const double* s, int n_s, const 
                                double shot_plus, lpp_template_t* tmpl);
 void lpp_template_destroy(lpp_template_t tmpl);
 lpp_status lpp_template_workspace_size(lpp_template_t tmpl, size_t* bytes);
-/* Device buffer (256-byte aligned, caller-owned); uploads the tables on `stream` and synchronises it. */
+/* Device buffer (256-byte aligned, caller-owned); uploads the tables on `stream`, forms the window's linear
+ * operator there (its rows and their digits take 22 x 2048 bytes per slot and shell: 25 MB with 40
+ * shells) and synchronises it. */
 lpp_status lpp_template_set_workspace(lpp_template_t tmpl, void* device_ptr, size_t bytes, void* stream);
 /* Spin-2 local primordial non-Gaussianity (Sec. 5): the shape response P -> [1 + 12 f_nl db_ia /
  * M(k)] P with M(k) = (2/3) k^2 T(k) D (c/H0)^2 / omega_m, T the BBKS transfer function of the
@@ -299,7 +303,9 @@ lpp_status lpp_template_set_png(lpp_template_t tmpl, double f_nl, double db_ia, 
  * LPP_N_MOMENTS.  Host-only. */
 lpp_status lpp_template_set_slots(lpp_template_t tmpl, unsigned mask);
 /* params: device [n_templates][6]; out: device [n_templates][LPP_N_MOMENTS][n_bins].
- * Asynchronous on `stream`. */
+ * Asynchronous on `stream`.  A set's values do not depend on the other sets, but the order of their sums
+ * depends on n_templates (one or two, three to 48, more): the last FP64 digits may differ between
+ * calls of different sizes. */
 lpp_status lpp_convolve_template(lpp_template_t tmpl, const double* params, int n_templates, double* out,
                                  void* stream);
 /* As lpp_convolve_template, and also the Legendre multipoles of the derived spectra
@@ -321,7 +327,7 @@ lpp_status lpp_convolve_template_eb(lpp_template_t tmpl, const double* params, i
  * they have to be ordered by the caller. */
 typedef struct lpp_surrogate_s* lpp_surrogate_t;
 
-/* batch: training minibatch and inference chunk (multiple of 32). */
+/* batch: training minibatch (multiple of 32). */
 lpp_status lpp_surrogate_create(int batch, lpp_surrogate_t* net);
 void lpp_surrogate_destroy(lpp_surrogate_t net);
 lpp_status lpp_surrogate_workspace_size(lpp_surrogate_t net, size_t* bytes);
@@ -348,7 +354,7 @@ lpp_status lpp_surrogate_train(lpp_surrogate_t net, const float* x, const float*
  * without changing the network: host grads in the parameter layout, host *loss.  Synchronous. */
 lpp_status lpp_surrogate_gradients(lpp_surrogate_t net, const float* x, const float* y, const int* idx,
                                    float* grads, double* loss, void* stream);
-/* Forward pass: device x [n][6] -> device y [n][320], in chunks of `batch` rows. */
+/* Forward pass: device x [n][6] -> device y [n][320]. */
 lpp_status lpp_surrogate_infer(lpp_surrogate_t net, const float* x, int n, float* y, void* stream);
 
 /* Map between template parameters and the network (the emulator of lpp_convolve_template_eb

@@ -12,8 +12,9 @@ device (torch's counter-based generator), so 64 mocks are ready in seconds.
 
 The grids per pass of each plan (its `batch`) and the fused pass's channel fields per CTA
 (`fused_slots`) are chosen by `autotune`: every combination is timed on a sample mock with the
-library's own kernel timers.  (The fused kernel's tile shape, 4 x 4 pencils, is fixed at
-compile time.)
+library's own kernel timers; a plan takes at most 8 grids per pass, and larger candidates are
+skipped.  (The fused kernel's tile shape, 4 x 4 pencils or 8 x 4 on FP32 grids of 128^3 and 256^3, is
+fixed at compile time.)
 """
 from __future__ import annotations
 

@@ -329,9 +329,10 @@ extern "C" lpp_status lpp_plan_create(const lpp_plan_desc* desc, lpp_plan_t* out
     plan->out_rows = (int)plan->channels.size() + 2;
 
     // batch: grids per field pass; the partner pass needs up to 3 (interlaced) grids
-    // interlaced grids up to 256^3 (FP64: 128^3, for the workspace) take 16: launches of 8 end before small
-    // grids fill the SMs evenly, and every combine launch reads the partner spectra again (an estimate,
-    // 8 -> 16: 64^3 969 -> 828 us, mocks on 64^3 and 128^3 18.3 -> 17.1 ms, 256^3 29.0 -> 28.1 ms)
+    // by default interlaced grids up to 256^3 (FP64: 128^3, for the workspace) take 16: launches of 8 end before
+    // small grids fill the SMs evenly, and every combine launch reads the partner spectra again (an estimate,
+    // 8 -> 16: 64^3 969 -> 828 us, mocks on 64^3 and 128^3 18.3 -> 17.1 ms, 256^3 29.0 -> 28.1 ms; a caller's
+    // own number stays at most 8)
     int batch = d.batch > 0 ? d.batch : (n <= (plan->fp64 ? 128 : 256) ? kMaxSlots : 8);
     const int per_grid = d.interlace ? 1 : 2;
     // shared-memory partials of the combine: channels x bins x 2 <= 8192 values

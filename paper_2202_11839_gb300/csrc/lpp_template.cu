@@ -293,8 +293,9 @@ __device__ __forceinline__ void finish_sets(const TemplateArgs& a, cooperative_g
 // is no faster here but issues and loads a quarter as much): 6.1 G multiply-adds of the products
 // are 11.6 ms of 8192 sets with nine slots and 40 shells, the model spectra (k^tilt from two
 // short tables of powers, log1p_table, rsqrt: about 50 operations a value) most of the rest.
-// 78.0 -> 15.0 ms against one CTA per set running its own transforms (24 FFTs of 4096 points);
-// without non-Gaussian factors such a batch takes k_template_many (3.7 ms).  One set, fourteen
+// With a non-Gaussian response, whose three spectra only the rows of their families read, 107 -> 15.4
+// ms against one CTA per set running its own transforms (FFTs of 4096 points); without one three and more
+// sets take k_template_many.  One set, fourteen
 // slots: 1.99 ms -> 24 us, the shells spread over the SMs by blockIdx.y; there an mma would idle
 // seven of its eight rows, and up to kFewSets sets take plain multiply-adds (FEW).
 constexpr int kFewSets = 2;
@@ -550,7 +551,8 @@ __global__ void __launch_bounds__(256) k_op_digits(const double* __restrict__ op
 // spectra's from shared memory in fragment order.
 //
 // What bounds it: the FP64 spectra (1.4 ms at the FP64 rate for 8192 sets) and the mma issue.
-// 8192 sets, nine slots, 40 shells: 15.0 -> 3.7 ms against the FP64 products (78.0 ms at first).
+// 8192 sets, nine slots, 40 shells: 15.0 -> 3.7 ms against the FP64 products (78.0 ms with transforms
+// per set).
 template <int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(256, 1)
 k_template_many(const __grid_constant__ TemplateArgs a) {
