@@ -208,6 +208,12 @@ __device__ __forceinline__ int fixed_round(float a, float b) {
 // run to the fixed bound 3 with a guard on P so the stencil stays in registers.  With addresses and
 // products per cell an atomic cost eight instructions: eight fields of 2 M galaxies on 256^3
 // 0.97 -> 0.91 ms with the x transform.
+//
+// The fixed-point fields take v wx once for the nine lines.  The others take v (wx wy wz): positions have few
+// bits below the cell (15 at u = 256), so v wx rounds alike for many particles, and with one v for all
+// randoms (-alpha) that is a bias of their total weight (3e-8 where all share an offset, 1e-10 in this
+// order) which data - alpha randoms magnifies: P_dd^(0) of a survey's lowest shell was off by rms 2.2e-7
+// instead of 1.1e-7.
 template <typename T, bool FIXED, int NS, int STRIDE, int LD, int TY, int TZ>
 __device__ __forceinline__ void scatter(T* tilef, int n, int P, T ux, T uy, T uz, T shift, int y0, int z0,
                                         const T* v, int im, int* err = nullptr) {
@@ -219,7 +225,7 @@ __device__ __forceinline__ void scatter(T* tilef, int n, int P, T ux, T uy, T uz
     // the stencil's first line relative to the tile, periodic: lines ry + ky in [0, TY) are the tile's
     const int ry = ((cy - y0 + 2) & (n - 1)) - 2, rz = ((cz - z0 + 2) & (n - 1)) - 2;
     T* base = tilef + 2 * ((cx + 1) * LD + rz * TY + ry) + im;
-    T vx[NS][3];
+    T vx[NS][3];   // FIXED
 #pragma unroll
     for (int q = 0; q < NS; ++q)
 #pragma unroll
@@ -234,6 +240,7 @@ __device__ __forceinline__ void scatter(T* tilef, int n, int P, T ux, T uy, T uz
 #pragma unroll
             for (int kx = 0; kx < 3; ++kx) {
                 if (kx >= P) continue;
+                const T ww = wyz * wx[kx];   // not FIXED
 #pragma unroll
                 for (int q = 0; q < NS; ++q) {
                     T* d = base + (2 * (kx * LD + kz * TY + ky) + q * STRIDE);
@@ -241,7 +248,7 @@ __device__ __forceinline__ void scatter(T* tilef, int n, int P, T ux, T uy, T uz
                         // v arrives pre-scaled to the tile's fixed-point unit
                         atomicAdd(reinterpret_cast<int*>(d), fixed_round((float)vx[q][kx], (float)wyz));
                     } else {
-                        atomicAdd(d, vx[q][kx] * wyz);
+                        atomicAdd(d, v[q] * ww);
                     }
                 }
             }
