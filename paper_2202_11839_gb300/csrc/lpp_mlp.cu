@@ -705,7 +705,9 @@ struct PredictArgs {
 };
 
 // The columns' constants of the decoding (float pairs) and the column exponents of the baseline, from
-// the map's arrays as they are at this call.
+// the map's arrays as they are at this call.  Each column is taken in the power-of-two unit of its baseline (else
+// of mu or sd), sigma with it: curves in any unit stay within FP32's exponents (without that 1e30
+// took 570 us for 8192 rows, all done again in FP64).
 struct ColumnConst {
     float2 mu, sd, shot, ref, isig;
     float tiny;   // kTiny, 0 when shot and ref are zero
@@ -714,13 +716,21 @@ struct ColumnConst {
 __device__ __forceinline__ ColumnConst column_const(const MapArgs& m, int j) {
     auto as2 = [](fpair p) { return make_float2(p.hi, p.lo); };
     ColumnConst c;
-    c.mu = as2(pair_of(m.mu[j]));
-    c.sd = as2(pair_of(m.sd[j]));
-    c.shot = as2(pair_of(m.shot[j]));
-    c.ref = as2(pair_of(m.ref ? m.ref[j] : 0.0));
-    c.isig = as2(pair_of(m.sigma ? 1.0 / m.sigma[j] : 1.0));
+    const int e = m.base ? m.exponent[j] : kZeroExponent;
+    const double mu = m.mu[j], sd = m.sd[j];
+    int k = e;
+    if (!usable(e)) {
+        const double big = fmax(fabs(mu), fabs(sd));
+        k = big > 1e-270 && big < 1e270 ? ((__double2hiint(big) >> 20) - 1022) : 0;
+    }
+    const double s = __hiloint2double((1023 - k) << 20, 0);   // 2^-k
+    c.mu = as2(pair_of(mu * s));
+    c.sd = as2(pair_of(sd * s));
+    c.shot = as2(pair_of(m.shot[j] * s));
+    c.ref = as2(pair_of(m.ref ? m.ref[j] * s : 0.0));
+    c.isig = as2(pair_of(1.0 / (m.sigma ? m.sigma[j] * s : s)));
     c.tiny = m.shot[j] != 0.0 || (m.ref && m.ref[j] != 0.0) ? kTiny : 0.f;
-    c.e = m.base ? m.exponent[j] : 0;
+    c.e = usable(e) ? 0 : e;   // relative to the unit
     return c;
 }
 __global__ void k_columns(MapArgs m, ColumnConst* __restrict__ out) {
@@ -800,16 +810,27 @@ __device__ __forceinline__ void decode_rows(const MapArgs& m, const double* thet
     __syncthreads();
 }
 
-// One output of a parameter row th in FP64, by a whole warp: y the network's output j, la and lb the
-// row's Lagrange weights.
+// One output of a parameter row th in FP64: y the network's output j, la and lb the row's Lagrange
+// weights.  WARP: by a whole warp (an FP64 instruction takes as long for one lane as for 32: 40 of them
+// instead of 110); else by each calling lane.
+template <bool WARP>
 __device__ __noinline__ float decode_exact(const MapArgs& m, const double* la, const double* lb, const double* th, int j,
                                            float y) {
     double b = 0.0;
     if (m.base) {
-        for (int q = threadIdx.x & 31; q < m.nodes * m.nodes; q += 32)
-            b = fma(la[q / m.nodes] * lb[q % m.nodes], m.base[(size_t)q * kNout + j], b);
+        const double* base = m.base + j;
+        if (WARP) {
+            for (int q = threadIdx.x & 31; q < m.nodes * m.nodes; q += 32)
+                b = fma(la[q / m.nodes] * lb[q % m.nodes], base[(size_t)q * kNout], b);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+            for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xffffffffu, b, o);
+        } else {
+            for (int p = 0; p < m.nodes; ++p) {
+                double row = 0.0;
+                for (int q = 0; q < m.nodes; ++q) row = fma(lb[q], base[(size_t)(p * m.nodes + q) * kNout], row);
+                b = fma(la[p], row, b);
+            }
+        }
     }
     const double amp = th[2] * th[2] * (j < 2 * (kNout / 8) ? th[0] * th[1] : th[0] * th[0]);
     double v = amp * (m.mu[j] + b + m.sd[j] * (double)y) + th[5] * m.shot[j];
@@ -824,8 +845,10 @@ __device__ __noinline__ float decode_exact(const MapArgs& m, const double* la, c
 // The digit products and the float pairs bound their error (the terms' magnitudes times 2^-43, the
 // digits' bound above, and 2^-140 where a low word may underflow).  An output for which that is more than
 // a quarter of its last FP32 place, which is no number or whose exponents leave FP32's range is done
-// again in FP64 (decode_exact): the stored value is the FP64 one to 3/4 of a place, whatever the
-// map holds.  Curves of some hundred error bars around the reference repeat a fraction of a per cent.
+// again in FP64 (decode_exact), one by one by the warp or, when they are more than two, each by its lane:
+// the stored value is the FP64 one to 3/4 of a place, whatever the map holds.  Curves of some hundred
+// error bars around the reference repeat a fraction of a per cent (8192 rows 98 -> 107 us); where a
+// baseline spans 2^17 and more nearly all are repeated (300 us, 280 in float pairs before).
 template <int R>
 __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, const RowConst<R>& rc,
                                             const ColumnConst* cc, int mt, int tile, int rows, const float y[4],
@@ -881,13 +904,13 @@ __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, c
                     const fpair s3 = two_sum(s2.hi, __fmul_rn(acc[3][v], exp2i(-24)));
                     fpair b = fast_two_sum(s3.hi, __fadd_rn(s3.lo, __fadd_rn(s2.lo, __fadd_rn(s1.lo, low))));
                     const int er = rc.e[r], ec = c.e;
-                    range = er > -50 && er < 50 && ec > -50 && ec < 50;
-                    const int e = range ? er + ec : 0;
+                    range = er > -50 && er < 50 && ec == 0;   // ec: 0, or kBadExponent
+                    const int e = range ? er : 0;
                     b.hi *= exp2i(e - 14);   // the digits' unit: 2^(e_r + e_c) 2^-14
                     b.lo *= exp2i(e - 14);
                     u = pair_add(u, b);
                     mag += fabsf(b.hi);
-                    eb = fmaf(rc.wsum[r] * exp2i(-48), range ? exp2i(ec) : 0.f, exp2i(e - 14) * exp2i(-31));
+                    eb = fmaf(rc.wsum[r], exp2i(-48), exp2i(e - 45));
                 }
                 const int ci = tile < 2 * (kNout / 8) / 8 ? 0 : 1;
                 const fpair amp = pr(rc.amp[ci][r]);
@@ -906,11 +929,16 @@ __device__ __forceinline__ void decode_tile(const MapArgs& m, const uint4* wd, c
                 done = range && bound <= fabsf(res[q]) * exp2i(-26) && fabsf(res[q]) < INFINITY;
             }
             unsigned again = __ballot_sync(full, !done);
-            while (again) {   // warp-uniform
+            if (__popc(again) > 2) {   // warp-uniform
+                if (!done)
+                    res[q] = decode_exact<false>(m, rc.la[r], rc.lb[r], theta + (size_t)r * kNin, 8 * tile + 2 * t + q, y[v]);
+                again = 0;
+            }
+            while (again) {
                 const int src = __ffs(again) - 1, rs = mt * 16 + (src >> 2) + 8 * hh;
                 again &= again - 1;
-                const float x = decode_exact(m, rc.la[rs], rc.lb[rs], theta + (size_t)rs * kNin, 8 * tile + 2 * (src & 3) + q,
-                                             __shfl_sync(full, y[v], src));
+                const float x = decode_exact<true>(m, rc.la[rs], rc.lb[rs], theta + (size_t)rs * kNin, 8 * tile + 2 * (src & 3) + q,
+                                                   __shfl_sync(full, y[v], src));
                 if (lane == src) res[q] = x;
             }
         }
@@ -939,8 +967,8 @@ __device__ __forceinline__ void input_rows(const PredictArgs& a, int r0, int row
 // the FP32 result.
 //
 // What bounds it: the GELUs' instructions and the mma issue.  8192 rows: 287 us as eight launches
-// with the decoding's last operations in FP64 -> 96 us (90 us without decode_tile's error bound and the
-// seventh weight digit; 104 us near a reference curve, where a per cent of the outputs are done
+// with the decoding's last operations in FP64 -> 98 us (90 us without decode_tile's error bound and the
+// seventh weight digit; 107 us near a reference curve, where a per cent of the outputs are done
 // again).
 template <bool MAP>
 __global__ void __launch_bounds__(kRowThreads, 2) k_predict(const __grid_constant__ PredictArgs a) {
